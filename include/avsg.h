@@ -91,10 +91,11 @@ extern "C" {
                                        as AVSG_XFER_SM_BALANCED                          */
 
 /* How Stage One finds the slot that holds an id (same results either way). */
-#define AVSG_INDEX_HASH   0u  /* open-addressing table in shared memory, rebuilt every step     */
-#define AVSG_INDEX_DIRECT 1u  /* one 16-bit entry per context position in device memory
-                                 (2 bytes x max_context per table, L2-resident); needs every
-                                 id < max_context                                              */
+#define AVSG_INDEX_HASH   0u  /* hash index in shared memory, rebuilt every step                */
+#define AVSG_INDEX_DIRECT 1u  /* needs every id < max_context.  Tables that a thread-block cluster
+                                 serves: one 16-bit entry per context position in device memory
+                                 (2 bytes x max_context per table, L2-resident); tables that fit
+                                 one block use the hash index, which is the quicker one there  */
 #define AVSG_INDEX_PAPER  2u  /* the paper's Hash-State table as printed (Eq. 2-4, Eq. 8-11,
                                  Alg. 2): packed 64-bit entries, double hashing with a retry
                                  budget, fingerprints, lazy reclamation.  LOSSY: a resident id

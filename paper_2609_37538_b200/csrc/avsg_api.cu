@@ -255,7 +255,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     // and the size of the direct index
     auto id_limit_of = [&](uint32_t i) -> uint32_t {
         uint32_t lim = a->kv_rows ? a->kv_rows[i] : 0x80000000u;
-        if (c->d_where && c->cfg.max_context < lim) lim = c->cfg.max_context;
+        if (c->cfg.index_mode == AVSG_INDEX_DIRECT && c->cfg.max_context < lim) lim = c->cfg.max_context;
         return lim;
     };
     // Stage One for tables [first, first + cnt) of the call, with the small or the large argument block
@@ -455,7 +455,7 @@ int avsg_create(const avsg_config* cfg, avsg_ctx** out)
         auto fits = [&](uint32_t C) -> bool {
             if (cfg->index_mode == AVSG_INDEX_PAPER)
                 return C == 1 && S <= 8192 && stage_one_paper_smem_bytes(S, K, L) <= (size_t)max_smem;
-            if (C == 1) return S <= 8192 && stage_one_smem_bytes(S, K, L, direct) <= (size_t)max_smem;
+            if (C == 1) return S <= 8192 && stage_one_smem_bytes(S, K, cfg->max_tokens) <= (size_t)max_smem;
             return S / C >= 32 && S / C <= 8192 && stage_one_cluster_smem_bytes(S, K, L, C, direct) <= (size_t)max_smem;
         };
         uint32_t C = cfg->stage_one_cluster;
@@ -495,7 +495,7 @@ int avsg_create(const avsg_config* cfg, avsg_ctx** out)
         ok = ok && cudaMalloc(&c->d_q, T * S * sizeof(uint32_t)) == cudaSuccess;
         ok = ok && cudaMalloc(&c->d_q_snap, T * S * sizeof(uint32_t)) == cudaSuccess;
     }
-    if (cfg->index_mode == AVSG_INDEX_DIRECT)
+    if (cfg->index_mode == AVSG_INDEX_DIRECT && c->s1_cluster > 1)     // (the single-block kernel builds its own index)
         ok = ok && cudaMalloc(&c->d_where, T * (size_t)cfg->max_context * sizeof(uint16_t)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_tok_snap, T * S * sizeof(int32_t)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_life_snap, T * S) == cudaSuccess;

@@ -182,7 +182,7 @@ struct ResetParams {             // stream-ordered reset of some tables: empty, 
 };
 cudaError_t launch_reset_tables(const ResetParams& p, uint32_t n_tables, cudaStream_t stream);
 
-size_t stage_one_smem_bytes(uint32_t S, uint32_t K, uint32_t L, bool direct = false);
+size_t stage_one_smem_bytes(uint32_t S, uint32_t K, uint32_t n_q);
 size_t stage_one_paper_smem_bytes(uint32_t S, uint32_t K, uint32_t L);
 uint32_t stage_one_threads(uint32_t S, uint32_t K);
 cudaError_t stage_one_prepare(size_t max_smem);

@@ -81,7 +81,7 @@ extern "C" int avsg_step_noalloc(const avsg_noalloc_args* a, void* cuda_stream)
     NoAllocScratch* sc = nullptr;
     int rc = setup_device(dev, &sc);
     if (rc != AVSG_OK) return rc;
-    if (stage_one_smem_bytes(a->buffer_slots, a->topk, (uint32_t)a->max_lifetime) > (size_t)g_max_smem[dev])
+    if (stage_one_smem_bytes(a->buffer_slots, a->topk, a->n_tokens) > (size_t)g_max_smem[dev])
         return AVSG_EUNSUPPORTED;
 
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);

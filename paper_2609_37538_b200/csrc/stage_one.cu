@@ -1,377 +1,372 @@
 // Stage One of the AVSG operator: match + reserve, one thread block per table.
 //
-// Follows Algorithm 1 (refresh / classify / allocate) with the lifetime
-// operations of Algorithm 3, for the N_q tokens of one iteration in order
-// (Algorithm 4), and the end-of-step invalidation of Algorithm 4.
-//
-// Two interchangeable id -> slot indexes (template parameter DIRECT):
-//   hash   (default) an open-addressing table in shared memory, rebuilt every step (described below);
-//   direct           one 16-bit slot number per context position in global memory (it stays L2-resident:
-//                    2 bytes x context per table).  An entry is only ever written when an id is installed
-//                    and is never cleared: a lookup masks it to a valid slot number and then compares the
-//                    slot's cached id, so stale or uninitialised entries simply miss.  No build, no probing.
+// Follows Algorithm 1 (refresh / classify / allocate) with the lifetime operations of Algorithm 3, for the N_q tokens
+// of one iteration in order (Algorithm 4), and the end-of-step invalidation of Algorithm 4.
 //
 // The whole table lives in shared memory for the step:
-//   s_tok[S]   cached id per slot            s_life[S]  lifetime per slot
-//   s_key[H], s_val[H]  open-addressing index id -> slot, H = 2S buckets,
-//                       rebuilt from s_tok at the start of every step
-// The index is private to this kernel (it is not part of the table state): a
-// hit is "some slot holds the id" (Eq. 1), whatever bucket found it.  Entries
-// are never deleted: when a slot is reclaimed its old key stays behind and is
-// recognised as stale because s_tok[slot] no longer equals the key; a later
-// insert of the same id re-uses that bucket, so a key occupies one bucket at
-// most.  The index is rebuilt when stale keys would push the load above 3/4.
+//   s_node[n]  {id, slot << 16 | next node}: node n < S is slot n with its cached id; an id that comes in before the
+//              last token gets a node of its own behind those, because its slot's node still hangs in the chain of the
+//              id that it replaces (where it is passed over, its id being another one); the last node closes every chain
+//   s_head[2S] the chains' first nodes: the index id -> slot, built from the cached ids at the start of every step
+//   s_life[S]  lifetime per slot, one signed byte;  s_bits: one bit per slot, set where it is dead (lifetime < 0)
+// The index is private to the kernel: a hit is "some slot holds the id" (Eq. 1), whatever node found it, so both
+// exact index modes of the interface run it (AVSG_INDEX_DIRECT only adds the bound on the ids).
 //
-// The decay loop of Algorithm 1 ("decay all, CollectDead, until enough slots
-// are dead") is evaluated in closed form: d = the smallest number of unit
-// decays after which at least n_g lifetimes are negative, read off a
-// histogram of the S lifetimes; the lifetimes then drop by d at once,
-// saturating at -1.  For L <= 30 the histogram is counted without atomics:
-// every thread bumps private byte counters (one column per thread, one row
-// per lifetime value) and one warp per value sums its row with dp4a.  Dead slots are compacted in increasing slot order and
-// the k-th miss in position order takes the k-th of them (ballot-free packed
-// byte arithmetic + warp/block prefix sums, no atomics, so the assignment is
-// deterministic).
+// What bounds it: nothing but latency.  A 32-table call touches 4 MB, 0.6 us of HBM time; the rest is a chain of
+// dependent passes over shared memory on one SM per table.  So the passes are few and short:
+//   * The index is chained and not open-addressed: an insert is one exchange whatever it meets, so a thread has all of
+//     its eight in flight, and a chain is 1.25 nodes long on average where linear probing at half load goes through
+//     clusters; what a warp pays for is the longest of its 32 lanes.  A step along a chain is one 8-byte read without a
+//     branch: a lane that is through reads the closing node again.
+//   * Three block barriers per token: lookups | misses and dead slots listed | install |.  Misses are ranked by ballots
+//     (a warp takes 32 consecutive positions at a time, so lane order is position order) and the block prefix is two
+//     warp reductions that every warp does for itself, over the warps' totals.  The dead slots of a warp are counted
+//     when lifetimes decay; hits that revive one and slots that are handed out are taken off.  Only the warps that
+//     hold some of the first n_g dead slots rank them, and the compacted misses are installed by a few warps: an SM
+//     issues instructions for 32 warps here, and what all of them execute is what takes the time.
+//   * The decay loop of Algorithm 1 ("decay all, CollectDead, until enough slots are dead") in closed form: d = the
+//     smallest number of unit decays after which n_g lifetimes are negative, found by counting the lifetimes below up
+//     to four candidate values at a time.
+//   * Only what changed is written back: installed ids, the lifetimes, and ids that verification makes empty.
+// Measured inside the kernel, 32 tables of 8192 slots, K = 2048, two tokens: 8.6 us.  With the open-addressing index of
+// 4-byte keys and 2-byte slots, eight barriers and a lifetime histogram it was 30.0 us, and 12.7 us with a table of one
+// 2-byte entry per context position in device memory; K = 256, S = 1024, one token: 2.5 us against 7.8.
 //
-// When Stage Two overlaps Stage One (S1Params::ready set), the block announces
-// every token as soon as its misses are placed: see publish_token().
+// When Stage Two overlaps Stage One (S1Params::flags set), the block announces every token as soon as its misses are
+// placed: see announce_token().
+#include <type_traits>
+
 #include "avsg_kernels.cuh"
 #include "stage_one_common.cuh"
 
 namespace avsg {
 namespace {
 
-struct Index {
-    int32_t*  key;
-    uint16_t* val;
-    const int32_t* tok;
-    uint32_t mask, logH;
+// Shared memory of one block, in bytes from its start (every part on a 16-byte boundary).
+struct S1Layout {
+    uint32_t head, life, bits, tot, ndead, cnt, sum, miss, pos, dead, total;
 };
-
-// Returns the slot holding x, or -1.  Bounded by the number of buckets.
-__device__ __forceinline__ int32_t index_find(const Index& ix, int32_t x, uint32_t* status)
+__host__ __device__ inline uint32_t align16(uint32_t n) { return (n + 15u) & ~15u; }
+__host__ __device__ inline S1Layout s1_layout(uint32_t S, uint32_t K, uint32_t n_q, uint32_t nt)
 {
-    uint32_t b = hash_id(x, ix.logH);
-    for (uint32_t it = 0; it <= ix.mask; ++it) {
-        const int32_t k = ix.key[b];
-        if (k == x) {
-            const uint32_t j = ix.val[b];
-            return ix.tok[j] == x ? (int32_t)j : -1;     // a stale key means the id was reclaimed this step
-        }
-        if (k == EMPTY) return -1;
-        b = (b + 1u) & ix.mask;
-    }
-    atomicOr(status, ST_PROBE_EXHAUSTED);
-    return -1;
+    S1Layout o;
+    uint32_t a = align16((S + (n_q - 1u) * K + 1u) * 8u);      // nodes first
+    o.head = a;  a += 2u * S * 4u;
+    o.life = a;  a += align16(S);
+    o.bits = a;  a += align16(2u * nt);
+    o.tot = a;   a += 2u * 32u * 4u;                           // warps' miss totals, by parity
+    o.ndead = a; a += 2u * 32u * 4u;                           // warps' dead slots, by parity
+    o.cnt = a;   a += 2u * 2u * 32u * 4u;                      // warps' counts of the decay search, by parity
+    o.sum = a;   a += 16u;                                     // valid ids of the call
+    o.miss = a;  a += align16(K * 4u);                         // misses in position order: ids,
+    o.pos = a;   a += align16(K * 2u);                         //   positions
+    o.dead = a;  a += align16(K * 2u);                         // dead slots in slot order
+    o.total = a;
+    return o;
 }
 
-// Installs x -> slot; re-uses the bucket that already carries x if there is one.
-__device__ __forceinline__ void index_insert(const Index& ix, int32_t x, uint32_t slot, uint32_t* status)
-{
-    uint32_t b = hash_id(x, ix.logH);
-    for (uint32_t it = 0; it <= ix.mask; ++it) {
-        const int32_t old = atomicCAS(&ix.key[b], EMPTY, x);
-        if (old == EMPTY || old == x) { ix.val[b] = (uint16_t)slot; return; }
-        b = (b + 1u) & ix.mask;
-    }
-    atomicOr(status, ST_PROBE_EXHAUSTED);
-}
+// Bits 0 .. 3: the sign bits of a word's four bytes.
+__device__ __forceinline__ uint32_t signs(uint32_t w) { return (((w >> 7) & 0x01010101u) * 0x10204080u) >> 28; }
 
-// Inserts the ids of the slots a thread owns.  The first compare-and-swap of every id is issued
-// before any result is inspected, so that a thread keeps up to eight shared-memory atomics in flight.
-__device__ __forceinline__ void build_index(const Index& ix, const int32_t* s_tok, uint32_t j0, uint32_t spt, bool own,
-                                            uint32_t* s_fill, uint32_t* status)
-{
-    uint32_t live = 0;
-    int32_t x[MAX_SPT], old[MAX_SPT];
-    uint32_t b[MAX_SPT];
-#pragma unroll
-    for (uint32_t k = 0; k < (uint32_t)MAX_SPT; ++k) {
-        x[k] = (own && k < spt) ? s_tok[j0 + k] : -1;
-        if (x[k] >= 0) {
-            b[k] = hash_id(x[k], ix.logH);
-            old[k] = atomicCAS(&ix.key[b[k]], EMPTY, x[k]);
-            ++live;
-        }
-    }
-#pragma unroll
-    for (uint32_t k = 0; k < (uint32_t)MAX_SPT; ++k) {
-        if (x[k] >= 0) {
-            if (old[k] == EMPTY || old[k] == x[k]) {
-                ix.val[b[k]] = (uint16_t)(j0 + k);
-            } else {
-                uint32_t bb = (b[k] + 1u) & ix.mask;
-                bool done = false;
-                for (uint32_t it = 0; it < ix.mask; ++it) {
-                    const int32_t o = atomicCAS(&ix.key[bb], EMPTY, x[k]);
-                    if (o == EMPTY || o == x[k]) { ix.val[bb] = (uint16_t)(j0 + k); done = true; break; }
-                    bb = (bb + 1u) & ix.mask;
-                }
-                if (!done) atomicOr(status, ST_PROBE_EXHAUSTED);
-            }
-        }
-    }
-    live = __reduce_add_sync(0xffffffffu, live);
-    if ((threadIdx.x & 31u) == 0 && live) atomicAdd(s_fill, live);
-}
-
-template <bool DIRECT, int CAP, bool ROUNDS>
+// SPT slots per thread (a power of two): S <= SPT * blockDim.x.  IPT: the most ids a thread has to look up per token
+// (K <= S, so SPT is always enough).  CAP: tables the argument block has room for.
+template <int SPT, int IPT, int CAP>
 __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_constant__ S1ParamsT<CAP> p)
 {
+    constexpr int NV = (SPT + 3) / 4;                    // 4-slot vectors of ids / words of lifetimes per thread
+    using bits_t = typename std::conditional<(SPT > 8), uint16_t, uint8_t>::type;       // a thread's dead bits
+    constexpr uint32_t PER_WORD = 4 / sizeof(bits_t);
     extern __shared__ __align__(16) unsigned char smem[];
-    const uint32_t S = p.S, K = p.K, H = DIRECT ? 0u : 1u << p.logH, Kp = (K + 7u) & ~7u;
-    const uint32_t tid = threadIdx.x, nt = blockDim.x;
-    const int32_t L = (int32_t)p.L;
+    const uint32_t S = p.S, K = p.K, H = 2u * S, L = p.L;
+    const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u, warp = tid >> 5, nw = nt >> 5;
+    const uint32_t below = (1u << lane) - 1u;            // the lanes before this one
+    const uint32_t NIL = S + (p.n_q - 1u) * K;           // the closing node
 
-    int32_t*  s_tok      = reinterpret_cast<int32_t*>(smem);
-    int32_t*  s_key      = s_tok + S;
-    int32_t*  s_miss_x   = s_key + H;
-    uint16_t* s_val      = reinterpret_cast<uint16_t*>(s_miss_x + Kp);
-    uint16_t* s_miss_pos = s_val + H;
-    uint16_t* s_dead     = s_miss_pos + Kp;
-    int8_t*   s_life     = reinterpret_cast<int8_t*>(s_dead + Kp);
-    uint32_t* s_hist     = reinterpret_cast<uint32_t*>(s_life + S);
-    uint32_t* s_scan_a   = s_hist + 128;
-    uint32_t* s_scan_b   = s_scan_a + 40;
-    uint32_t* s_fill     = s_scan_b + 40;
-    const uint32_t priv_stride = nt + 4u;                 // +4: rows start in different banks
-    uint8_t*  s_priv     = L <= PRIV_HIST_MAX_L ? reinterpret_cast<uint8_t*>(s_fill + 8) : nullptr;
+    const S1Layout lay = s1_layout(S, K, p.n_q, nt);
+    uint2*    s_node = reinterpret_cast<uint2*>(smem);
+    uint32_t* s_head = reinterpret_cast<uint32_t*>(smem + lay.head);
+    int8_t*   s_life = reinterpret_cast<int8_t*>(smem + lay.life);
+    bits_t*   s_bits = reinterpret_cast<bits_t*>(smem + lay.bits);
+    uint32_t* s_tot  = reinterpret_cast<uint32_t*>(smem + lay.tot);
+    uint32_t* s_ndead = reinterpret_cast<uint32_t*>(smem + lay.ndead);
+    uint32_t* s_cnt  = reinterpret_cast<uint32_t*>(smem + lay.cnt);
+    uint32_t* s_sum  = reinterpret_cast<uint32_t*>(smem + lay.sum);
+    int32_t*  s_miss = reinterpret_cast<int32_t*>(smem + lay.miss);
+    uint16_t* s_pos  = reinterpret_cast<uint16_t*>(smem + lay.pos);
+    uint16_t* s_dead = reinterpret_cast<uint16_t*>(smem + lay.dead);
+
+    auto clear_index = [&] {
+        for (uint32_t i = tid; i < H / 4; i += nt) reinterpret_cast<uint4*>(s_head)[i] = make_uint4(NIL, NIL, NIL, NIL);
+    };
+    // slot j is no longer dead (the count follows the bit, so that an id that comes twice is counted once)
+    auto revive = [&](uint32_t j, uint32_t par) {
+        const uint32_t owner = j / SPT, bit = 1u << ((owner % PER_WORD) * (32u / PER_WORD) + j % SPT);
+        if (atomicAnd(reinterpret_cast<uint32_t*>(s_bits) + owner / PER_WORD, ~bit) & bit)
+            atomicSub(&s_ndead[par + owner / 32u], 1u);
+    };
+    // the first table's arguments and the clearing come before the wait: under the previous kernel's tail
+    uint32_t bt = blockIdx.x, table = p.table_id[bt], id_limit = p.id_limit[bt];
+    int32_t N = p.verified_len[bt];
+    clear_index();
+    if (tid == 0) s_node[NIL] = make_uint2(0xFFFFFFFEu, NIL);          // an id that nobody looks for
 
     // Programmatic dependent launch: this grid may have been started while the previous kernel of the stream
     // was still running; nothing is read before that kernel has completed.  The next kernel (Stage Two) is
     // allowed to start its own prologue right away - it waits the same way before it reads the miss list.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (p.t_range && threadIdx.x == 0) atomicMin(p.t_range, global_ns());
+    if (p.t_range && tid == 0) atomicMin(p.t_range, global_ns());
     const uint32_t epoch = p.flags ? __ldcg(p.epoch) : 0u;      // the number of this overlapped call
 
-    // The grid usually has one block per table (ROUNDS = false: one pass, bt = blockIdx.x).  A call with many tables
-    // and an overlapped Stage Two is launched with fewer blocks than tables (ROUNDS = true): a block then serves the
-    // tables bt = blockIdx.x, blockIdx.x + gridDim.x, ... one after the other, so that Stage One stays on a few SMs
-    // and publishes its tables round by round while the transfer grid, resident on the other SMs, already copies
-    // the earlier rounds' misses.
-    auto one_table = [&](const uint32_t bt) {
-        const uint32_t ti = p.first + bt;            // table index within the call
-        const uint32_t table = p.table_id[bt];
+    const uint32_t ipt = (K + nt - 1) / nt;              // ids per thread
+    const uint32_t i0 = warp * ipt * 32u + lane;         // position of the thread's k-th id: i0 + 32 k, below i1
+    const uint32_t i1 = (warp + 1u) * ipt * 32u < K ? (warp + 1u) * ipt * 32u : K;
+    const uint32_t j0 = tid * SPT;                       // first of the thread's slots
+    const bool own = j0 < S;
+
+    // A block usually serves one table.  A call with many tables and an overlapped Stage Two is launched with fewer
+    // blocks than tables: a block then serves the tables bt = blockIdx.x, blockIdx.x + gridDim.x, ... one after the
+    // other, so that Stage One stays on a few SMs and publishes its tables round by round while the transfer grid,
+    // resident on the other SMs, already copies the earlier rounds' misses.
+    for (;;) {
+        const uint32_t ti = p.first + bt;                // table index within the call
         int32_t* g_tok = p.tok + (size_t)table * S;
         int8_t*  g_life = p.life + (size_t)table * S;
+        const int32_t* ids = p.indices + (size_t)ti * p.n_q * K;
 
-        const uint32_t spt = S >= nt ? S / nt : 1u;           // slots per thread, power of two <= 8
-        const uint32_t j0 = tid * spt;
-        const bool own = j0 < S;
-        const uint32_t ipt = (K + nt - 1) / nt;               // ids per thread, <= 8
-        const uint32_t i0 = tid * ipt;
+        // ---- every global load is issued first: cached ids, lifetimes, the first token's ids ----
+        int4 t4[NV];
+        uint32_t w[NV];
+        int32_t xs[IPT];
+        auto load_token = [&](uint32_t g) {
+#pragma unroll
+            for (int k = 0; k < IPT; ++k) xs[k] = i0 + 32u * k < i1 ? __ldcg(ids + (size_t)g * K + i0 + 32u * k) : -1;
+        };
+#pragma unroll
+        for (int q = 0; q < NV; ++q)
+            if (tid + q * nt < S / 4) t4[q] = __ldcg(reinterpret_cast<const int4*>(g_tok) + tid + q * nt);
+        life_words<SPT, true>(g_life + j0, own, w);
+        load_token(0);
+        if (p.verified_len_dev) N = __ldg(p.verified_len_dev + ti);
+        if (tid == 0) s_sum[0] = 0;
+        __syncthreads();                                 // the index is empty
 
-        Index ix{s_key, s_val, s_tok, H - 1u, p.logH};
-        uint16_t* where = DIRECT ? p.where + (size_t)table * p.max_context : nullptr;
-
-        // ---- issue every global load first: table state and the first token's ids ----
-        int4 t4[MAX_SPT / 4];
-        int32_t t1[3];
-        uint32_t lw0, lw1;
-        if (own) {
-            if ((spt & 3u) == 0) {
-    #pragma unroll
-                for (uint32_t q = 0; q < (uint32_t)MAX_SPT / 4; ++q)
-                    if (q < spt / 4) t4[q] = __ldg(reinterpret_cast<const int4*>(g_tok + j0) + q);
-            } else {
-    #pragma unroll
-                for (uint32_t k = 0; k < 3; ++k)
-                    if (k < spt) t1[k] = __ldg(g_tok + j0 + k);
+        // ---- ids to shared memory and into the index; global pre-decay of the lifetimes (Alg. 1 Pass 1) ----
+        bool stale_ids = false;                          // ids that are no longer verified (the caller took tokens back)
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            if (tid + q * nt < S / 4) {
+                const uint32_t j = 4u * (tid + q * nt);
+                const int32_t x[4] = {t4[q].x, t4[q].y, t4[q].z, t4[q].w};
+                uint32_t next[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    next[c] = x[c] >= 0 ? atomicExch(&s_head[hash_id(x[c], p.logH)], j + c) : NIL;
+                    stale_ids = stale_ids || x[c] >= N;
+                }
+#pragma unroll
+                for (int c = 0; c < 4; c += 2)
+                    reinterpret_cast<uint4*>(s_node)[(j + c) / 2] = make_uint4((uint32_t)x[c], (j + c) << 16 | next[c],
+                                                                               (uint32_t)x[c + 1], (j + c + 1) << 16 | next[c + 1]);
             }
         }
-        life_load(g_life, j0, spt, own, lw0, lw1);
-        int32_t xs[MAX_IPT];
-        load_ids(p.indices + (size_t)ti * p.n_q * K, i0, ipt, K, xs);
-        const uint32_t id_limit = p.id_limit[bt];
+        auto store_life = [&](uint32_t par) {            // the thread's lifetimes and dead bits, the warp's dead slots
+            uint32_t bits = 0;
+#pragma unroll
+            for (int q = 0; q < NV; ++q) bits |= signs(w[q]) << (4 * q);
+            life_words_store<SPT>(s_life + j0, own, w);
+            s_bits[tid] = (bits_t)bits;
+            const uint32_t n = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(bits));
+            if (lane == 0) s_ndead[par + warp] = n;
+        };
+        uint32_t high = 0;                               // lifetimes above L (only a caller's own state can have them)
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            if (own) high |= __vcmpgts4(w[q], L * 0x01010101u) & (SPT == 2 ? 0xFFFFu : 0xFFFFFFFFu);
+            w[q] = decay4(w[q], 1);
+        }
+        store_life(0);
+        const bool unusual = __syncthreads_or(high != 0);
 
-        if constexpr (!DIRECT) {
-            for (uint32_t i = tid; i < H / 4; i += nt)
-                reinterpret_cast<int4*>(s_key)[i] = make_int4(EMPTY, EMPTY, EMPTY, EMPTY);
-        }
-        if (s_priv)
-            for (uint32_t i = tid; i < ((uint32_t)(L + 2) * priv_stride + 15u) / 16u; i += nt)
-                reinterpret_cast<int4*>(s_priv)[i] = make_int4(0, 0, 0, 0);
-        if (tid == 0) *s_fill = 0;
-        if (own) {
-            if ((spt & 3u) == 0) {
-    #pragma unroll
-                for (uint32_t q = 0; q < (uint32_t)MAX_SPT / 4; ++q)
-                    if (q < spt / 4) reinterpret_cast<int4*>(s_tok + j0)[q] = t4[q];
-            } else {
-    #pragma unroll
-                for (uint32_t k = 0; k < 3; ++k)
-                    if (k < spt) s_tok[j0 + k] = t1[k];
-            }
-        }
-        // global pre-decay of the iteration's first token (Alg. 1 Pass 1)
-        life_store(s_life, j0, spt, own, decay4(lw0, 1), decay4(lw1, 1));
-        __syncthreads();
-        uint32_t fill_bound = 0;                              // hash index: non-empty buckets (upper bound)
-        if (!DIRECT) {
-            build_index(ix, s_tok, j0, spt, own, s_fill, p.status);
-            __syncthreads();
-            fill_bound = *s_fill;
-        }
-
-        uint32_t list_off = 0, sum_valid = 0, sum_miss = 0, sum_decay = 0;
+        uint32_t list_off = 0, sum_miss = 0, sum_decay = 0, valid = 0;
         int2* list = p.miss_list + (size_t)ti * p.list_stride;
 
-
         for (uint32_t g = 0; g < p.n_q; ++g) {
+            const bool last = g + 1 == p.n_q;
+            const uint32_t par = 32u * (g & 1u);
             const size_t row = ((size_t)ti * p.n_q + g) * K;
             int32_t* O = p.slots + row;
             uint8_t* Hm = p.hit ? p.hit + row : nullptr;
-            if (tid < 128) s_hist[tid] = 0;
 
-            // ---- Probe, refresh hits to L, emit hit slots (Pass 1 + Pass 2) ----
-            uint32_t missmask = 0, nmiss = 0, nvalid = 0;
-            uint32_t cand[MAX_IPT];                             // direct index: candidate slot per id
-            check_ids(xs, i0, ipt, K, id_limit, p.status);      // out-of-range ids become padding (id_limit <= max_context)
-            if (DIRECT) {
-    #pragma unroll
-                for (uint32_t k = 0; k < (uint32_t)MAX_IPT; ++k) {   // all loads are issued before any is used
-                    cand[k] = 0xFFFFFFFFu;
-                    if (k < ipt && i0 + k < K && xs[k] >= 0) cand[k] = __ldcg(where + xs[k]) & (S - 1u);
-                }
+            // ---- lookups; hits: lifetime <- L, slot and flag out (Pass 1 + Pass 2) ----
+            // (pass after pass over the thread's ids, so that their reads are in flight together)
+            uint32_t node[IPT], rank[IPT], missing = 0, wmiss = 0;
+            int32_t slot[IPT], was[IPT];
+            bool bad = false;
+#pragma unroll
+            for (int k = 0; k < IPT; ++k) {
+                const bool ok = (uint32_t)xs[k] < id_limit;
+                bad = bad || (!ok && xs[k] >= 0);
+                xs[k] = ok ? xs[k] : -1;
+                valid += ok;
+                slot[k] = -1;
+                node[k] = NIL;
+                if (ok) node[k] = s_head[hash_id(xs[k], p.logH)];
             }
-    #pragma unroll
-            for (uint32_t k = 0; k < (uint32_t)MAX_IPT; ++k) {
-                const uint32_t i = i0 + k;
-                if (k < ipt && i < K) {
-                    const int32_t x = xs[k];
-                    if (x >= 0 && (!DIRECT || cand[k] != 0xFFFFFFFFu)) {
-                        ++nvalid;
-                        int32_t j;
-                        if (DIRECT) j = s_tok[cand[k]] == x ? (int32_t)cand[k] : -1;
-                        else j = index_find(ix, x, p.status);
-                        if (j >= 0) {
-                            s_life[j] = (int8_t)L;
-                            O[i] = j;
-                            if (Hm) Hm[i] = 1;
-                        } else {
-                            missmask |= 1u << k;
-                            ++nmiss;
-                        }
-                    } else {
-                        O[i] = -1;
-                        if (Hm) Hm[i] = 0;
+            if (bad) atomicOr(p.status, ST_BAD_ID);                    // not fetched: reported and taken as padding
+            uint32_t open = 1;
+            for (uint32_t it = 0; open && it <= NIL; ++it) {           // all chains of the warp side by side
+                uint2 v[IPT];
+#pragma unroll
+                for (int k = 0; k < IPT; ++k) v[k] = s_node[node[k]];
+                open = 0;
+#pragma unroll
+                for (int k = 0; k < IPT; ++k) {
+                    const bool found = (int32_t)v[k].x == xs[k];
+                    slot[k] = found ? (int32_t)(v[k].y >> 16) : slot[k];
+                    node[k] = found ? NIL : v[k].y & 0xFFFFu;
+                    open |= node[k] ^ NIL;
+                }
+                open = __any_sync(0xffffffffu, open);
+            }
+            if (open) atomicOr(p.status, ST_PROBE_EXHAUSTED);
+            // with lifetimes above L on entry a slot reserved in this step may go to yet another id: its first node is stale
+            if (unusual) {
+#pragma unroll
+                for (int k = 0; k < IPT; ++k)
+                    if (slot[k] >= 0 && (int32_t)s_node[slot[k]].x != xs[k]) slot[k] = -1;
+            }
+#pragma unroll
+            for (int k = 0; k < IPT; ++k) was[k] = slot[k] >= 0 ? s_life[slot[k]] : 0;
+            bool revived = false;
+#pragma unroll
+            for (int k = 0; k < IPT; ++k) {
+                const bool miss = xs[k] >= 0 && slot[k] < 0, store = !miss && i0 + 32u * k < i1;
+                const uint32_t votes = __ballot_sync(0xffffffffu, miss);
+                rank[k] = wmiss + __popc(votes & below);               // within the warp, in position order
+                wmiss += __popc(votes);
+                missing |= miss ? 1u << k : 0u;
+                if (slot[k] >= 0) s_life[slot[k]] = (int8_t)L;
+                if (store) O[i0 + 32u * k] = slot[k];
+                if (store && Hm) Hm[i0 + 32u * k] = slot[k] >= 0;
+                revived = revived || was[k] < 0;
+            }
+            if (revived) {
+#pragma unroll
+                for (int k = 0; k < IPT; ++k)
+                    if (was[k] < 0) revive((uint32_t)slot[k], par);
+            }
+            if (last) {
+                valid = __reduce_add_sync(0xffffffffu, valid);
+                if (lane == 0 && valid) atomicAdd(s_sum, valid);
+            }
+            if (lane == 0) s_tot[par + warp] = wmiss;
+            __syncthreads();
+
+            // ---- CollectDead and the misses, each in order; the prefix over the warps: lane l looks at warp l ----
+            uint32_t t = lane < nw ? s_ndead[par + lane] | s_tot[par + lane] << 16 : 0u;
+            const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? t : 0u);
+            const uint32_t all = __reduce_add_sync(0xffffffffu, t);
+            const uint32_t n_g = all >> 16;
+            uint32_t dtotal = all & 0xFFFFu, dead_before = before & 0xFFFFu, d = 0;
+            sum_miss += n_g;
+            if (tid == 0 && p.miss_count) p.miss_count[(size_t)ti * p.n_q + g] = (int32_t)n_g;
+            if (missing) {
+#pragma unroll
+                for (int k = 0; k < IPT; ++k) {
+                    if (missing & (1u << k)) {
+                        s_miss[(before >> 16) + rank[k]] = xs[k];
+                        s_pos[(before >> 16) + rank[k]] = (uint16_t)(i0 + 32u * k);
                     }
                 }
             }
-            // order-preserving compaction of the misses: t = x[not m]
-            uint32_t total;
-            uint32_t off = block_excl_scan(nmiss | (nvalid << 16), s_scan_a, total) & 0xFFFFu;
-            const uint32_t n_g = total & 0xFFFFu;
-            sum_valid += total >> 16;
-            sum_miss += n_g;
-    #pragma unroll
-            for (uint32_t k = 0; k < (uint32_t)MAX_IPT; ++k) {
-                if (missmask & (1u << k)) {
-                    s_miss_x[off] = xs[k];
-                    s_miss_pos[off] = (uint16_t)(i0 + k);
-                    ++off;
-                }
-            }
-            // the next token's ids travel while this token's misses are placed
-            if (g + 1 < p.n_q) load_ids(p.indices + row + K, i0, ipt, K, xs);
-            if (tid == 0 && p.miss_count) p.miss_count[(size_t)ti * p.n_q + g] = (int32_t)n_g;
-            if (n_g == 0) { __syncthreads(); publish_token(p, ti, table, g, 0, bt, epoch); continue; }
-            __syncthreads();
+            if (!last) load_token(g + 1);                              // arrives while this token's misses are placed
 
-            // ---- Pass 3: CollectDead; if fewer than n_g slots are dead, decay until enough are ----
-            uint32_t w0, w1;
-            life_load(s_life, j0, spt, own, w0, w1);
-            uint32_t sg0 = w0 & 0x80808080u, sg1 = w1 & 0x80808080u;       // sign bits = dead slots
-            uint32_t dtotal, d = 0;
-            uint32_t doff = block_excl_scan(__popc(sg0) + __popc(sg1), s_scan_b, dtotal);
+            // Pass 3, the while-loop of Alg. 1: decay until n_g slots are dead
             if (dtotal < n_g) {
-                // the while-loop of Alg. 1 in closed form: d = fewest unit decays after which n_g slots are dead,
-                // read off the histogram of the lifetimes (only needed on this, the rarer, path)
-                count_lifetimes(w0, w1, spt, own, L, s_priv, priv_stride, s_hist);
+                life_words<SPT>(s_life + j0, own, w);
+                uint32_t lo = 0, hi = L + 1u, buf = 0;   // lo decays are too few, hi are enough (lifetimes are <= L)
+                while (hi - lo > 1u) {                   // (L >= 1: at least once, so every warp has read the old counts)
+                    uint32_t c[4];                       // candidates in (lo, hi), ascending; small ones first
+#pragma unroll
+                    for (uint32_t i = 0; i < 4; ++i) {
+                        c[i] = lo == 0 ? 1u << i : lo + ((i + 1u) * (hi - lo)) / 5u;
+                        c[i] = c[i] <= lo ? lo + 1u : (c[i] >= hi ? hi - 1u : c[i]);
+                    }
+                    uint32_t n01 = 0, n23 = 0;
+#pragma unroll
+                    for (int q = 0; q < NV; ++q) {
+                        n01 += __popc(__vsubss4(w[q], c[0] * 0x01010101u) & 0x80808080u) |
+                               (__popc(__vsubss4(w[q], c[1] * 0x01010101u) & 0x80808080u) << 16);
+                        n23 += __popc(__vsubss4(w[q], c[2] * 0x01010101u) & 0x80808080u) |
+                               (__popc(__vsubss4(w[q], c[3] * 0x01010101u) & 0x80808080u) << 16);
+                    }
+                    n01 = __reduce_add_sync(0xffffffffu, n01);
+                    n23 = __reduce_add_sync(0xffffffffu, n23);
+                    if (lane == 0) { s_cnt[buf + warp] = n01; s_cnt[buf + 32u + warp] = n23; }
+                    __syncthreads();
+                    n01 = __reduce_add_sync(0xffffffffu, lane < nw ? s_cnt[buf + lane] : 0u);
+                    n23 = __reduce_add_sync(0xffffffffu, lane < nw ? s_cnt[buf + 32u + lane] : 0u);
+                    const uint32_t n[4] = {n01 & 0xFFFFu, n01 >> 16, n23 & 0xFFFFu, n23 >> 16};
+#pragma unroll
+                    for (int i = 3; i >= 0; --i) if (n[i] >= n_g) hi = c[i];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) if (n[i] < n_g) lo = c[i];
+                    buf ^= 64u;
+                }
+                d = hi;
+#pragma unroll
+                for (int q = 0; q < NV; ++q) w[q] = decay4(w[q], d);
+                store_life(par);
                 __syncthreads();
-                uint32_t cum = 0;
-                bool found = false;
-                d = (uint32_t)L + 1u;
-                for (uint32_t b = 0; b <= (uint32_t)L + 1u; ++b) {   // bin b counts lifetime b-1; dead after b decays
-                    cum += s_hist[b];
-                    if (cum >= n_g) { d = b; found = true; break; }
-                }
-                if (!found && tid == 0) atomicOr(p.status, ST_NO_DEAD_SLOTS);
-                w0 = decay4(w0, d);
-                w1 = decay4(w1, d);
-                life_store(s_life, j0, spt, own, w0, w1);
-                sg0 = w0 & 0x80808080u; sg1 = w1 & 0x80808080u;
-                doff = block_excl_scan(__popc(sg0) + __popc(sg1), s_scan_b, dtotal);
+                t = lane < nw ? s_ndead[par + lane] : 0u;
+                dead_before = __reduce_add_sync(0xffffffffu, lane < warp ? t : 0u);
+                dtotal = __reduce_add_sync(0xffffffffu, t);
+                if (dtotal < n_g && tid == 0) atomicOr(p.status, ST_NO_DEAD_SLOTS);
             }
-            // dead slots in increasing order; the first n_g are handed out
-    #pragma unroll
-            for (uint32_t k = 0; k < (uint32_t)MAX_SPT; ++k) {
-                const uint32_t bit = k < 4 ? (sg0 >> (8 * k + 7)) & 1u : (sg1 >> (8 * (k - 4) + 7)) & 1u;
-                if (bit) {
-                    if (doff < n_g) s_dead[doff] = (uint16_t)(j0 + k);
-                    ++doff;
-                }
+            const uint32_t n_take = n_g < dtotal ? n_g : dtotal;
+            if (dead_before < n_take) {                  // some of the first n_g dead slots are this warp's
+                uint32_t bits = s_bits[tid], r, unused;
+                warp_rank<SPT>(__popc(bits), below, r, unused);
+                for (r += dead_before; bits && r < n_take; bits &= bits - 1u, ++r) s_dead[r] = (uint16_t)(j0 + __ffs((int)bits) - 1);
+                s_bits[tid] = (bits_t)bits;              // what is handed out is dead no more
             }
+            uint32_t left = __shfl_sync(0xffffffffu, t & 0xFFFFu, (int)warp);          // the warp's dead slots for the next token
+            if (dead_before < n_take) left = left > n_take - dead_before ? left - (n_take - dead_before) : 0u;
+            if (lane == 0) s_ndead[32u - par + warp] = left;
             __syncthreads();
 
-            // ---- install the misses: k-th miss takes the k-th dead slot ----
-            const bool rebuild = !DIRECT && fill_bound + n_g > (H / 4u) * 3u;
-            const uint32_t n_take = n_g < dtotal ? n_g : dtotal;
-            for (uint32_t k = tid; k < n_take; k += nt) {
-                const uint32_t j = s_dead[k];
-                const int32_t x = s_miss_x[k];
-                const uint32_t i = s_miss_pos[k];
-                if (j < S && i < K) {
-                    s_tok[j] = x;
+            // ---- install: the k-th miss in position order takes the k-th dead slot ----
+            for (uint32_t k = tid; k < n_g; k += nt) {
+                const uint32_t i = s_pos[k];
+                const int32_t x = s_miss[k];
+                const int32_t j = k < n_take ? s_dead[k] : -1;
+                if (k < n_take) {
+                    s_node[j].x = (uint32_t)x;
                     s_life[j] = (int8_t)L;
-                    O[i] = (int32_t)j;
-                    if (Hm) Hm[i] = 0;
-                    list[list_off + k] = make_int2(x, (int32_t)j);
-                    if (DIRECT) __stcg(where + x, (uint16_t)j);
-                    else if (!rebuild) index_insert(ix, x, j, p.status);
-                } else {
-                    list[list_off + k] = make_int2(-1, -1);          // Stage Two skips it
-                    atomicOr(p.status, ST_BAD_SLOT);
+                    list[list_off + k] = make_int2(x, j);
+                    g_tok[j] = x >= N ? -1 : x;                        // speculative ids are forgotten (end of Alg. 4)
+                    if (!last) {
+                        const uint32_t n = S + list_off + k;
+                        s_node[n] = make_uint2((uint32_t)x, (uint32_t)j << 16 | atomicExch(&s_head[hash_id(x, p.logH)], n));
+                    }
                 }
+                O[i] = j;
+                if (Hm) Hm[i] = 0;
             }
             list_off += n_take;
             sum_decay += d;
-            if (!rebuild) {
-                fill_bound += n_g;
-                __syncthreads();
-            } else if constexpr (!DIRECT) {
-                __syncthreads();
-                for (uint32_t i = tid; i < H / 4; i += nt)
-                    reinterpret_cast<int4*>(s_key)[i] = make_int4(EMPTY, EMPTY, EMPTY, EMPTY);
-                if (tid == 0) *s_fill = 0;
-                __syncthreads();
-                build_index(ix, s_tok, j0, spt, own, s_fill, p.status);
-                __syncthreads();
-                fill_bound = *s_fill;
-            }
-            publish_token(p, ti, table, g, n_take, bt, epoch);
+            __syncthreads();
+            announce_token(p, ti, table, g, n_take, bt, epoch);
         }
 
-        // ---- write the table back; speculative entries (id >= N) become empty (Alg. 4) ----
-        const int32_t N = p.verified_len_dev ? __ldg(p.verified_len_dev + ti) : p.verified_len[bt];
-        if (own) {
-            if ((spt & 3u) == 0) {
-                for (uint32_t q = 0; q < spt / 4; ++q) {
-                    int4 v = reinterpret_cast<const int4*>(s_tok + j0)[q];
-                    v.x = v.x >= N ? -1 : v.x; v.y = v.y >= N ? -1 : v.y;
-                    v.z = v.z >= N ? -1 : v.z; v.w = v.w >= N ? -1 : v.w;
-                    reinterpret_cast<int4*>(g_tok + j0)[q] = v;
-                }
-            } else {
-                for (uint32_t k = 0; k < spt; ++k) {
-                    const int32_t v = s_tok[j0 + k];
-                    g_tok[j0 + k] = v >= N ? -1 : v;
-                }
-            }
-            uint32_t w0, w1;
-            life_load(s_life, j0, spt, own, w0, w1);
-            life_store(g_life, j0, spt, own, w0, w1);
+        // ---- write back: lifetimes; resident ids that are no longer verified become empty (Alg. 4) ----
+        life_words<SPT>(s_life + j0, own, w);
+        life_words_store<SPT>(g_life + j0, own, w);
+        if (stale_ids) {
+            for (uint32_t q = 0; q < NV; ++q)
+                for (uint32_t j = 4u * (tid + q * nt); j < 4u * (tid + q * nt) + 4u && j < S; ++j)
+                    if ((int32_t)s_node[j].x >= N) g_tok[j] = -1;
         }
         if (tid == 0) {
             SegDesc sd;
@@ -381,22 +376,19 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
             sd.count = list_off;
             sd.pad = 0;
             p.seg[ti] = sd;
-            TableStats* st = p.stats + table;
-            st->steps += 1;
-            st->tokens += p.n_q;
-            st->hits += sum_valid - sum_miss;
-            st->misses += sum_miss;
-            st->rows += list_off;
-            st->extra_decays += sum_decay;
+            TableStats* st = p.stats + table;            // (reductions: nothing waits for the old values)
+            atomicAdd(&st->steps, 1ull);
+            atomicAdd(&st->tokens, (unsigned long long)p.n_q);
+            atomicAdd(&st->hits, (unsigned long long)(s_sum[0] - sum_miss));
+            atomicAdd(&st->misses, (unsigned long long)sum_miss);
+            atomicAdd(&st->rows, (unsigned long long)list_off);
+            atomicAdd(&st->extra_decays, (unsigned long long)sum_decay);
         }
-    };
-    if constexpr (ROUNDS) {
-        for (uint32_t bt = blockIdx.x; bt < p.n_launch; bt += gridDim.x) {
-            if (bt != blockIdx.x) __syncthreads();        // the previous table's last reads of shared memory are over
-            one_table(bt);
-        }
-    } else {
-        one_table(blockIdx.x);
+        bt += gridDim.x;
+        if (bt >= p.n_launch) break;
+        table = p.table_id[bt]; id_limit = p.id_limit[bt]; N = p.verified_len[bt];
+        __syncthreads();                                 // this table's last reads of shared memory are over
+        clear_index();
     }
     if (p.t_range) {
         __syncthreads();
@@ -742,43 +734,50 @@ __global__ void __launch_bounds__(256) avsg_all_k_prepare_kernel(const __grid_co
 
 }  // namespace
 
-size_t stage_one_smem_bytes(uint32_t S, uint32_t K, uint32_t L, bool direct)
+size_t stage_one_smem_bytes(uint32_t S, uint32_t K, uint32_t n_q)
 {
-    const size_t H = direct ? 0 : 2ull * S, Kp = (K + 7u) & ~7u;
-    size_t n = S * 4 + H * 4 + Kp * 4 + H * 2 + Kp * 2 + Kp * 2 + S + (128 + 40 + 40 + 8) * 4;
-    if ((int32_t)L <= PRIV_HIST_MAX_L) n += ((size_t)(L + 2) * (stage_one_threads(S, K) + 4) + 15) / 16 * 16;
-    (void)direct;
-    return n;
+    return s1_layout(S, K, n_q, stage_one_threads(S, K)).total;
+}
+
+static uint32_t stage_one_paper_threads(uint32_t S)
+{
+    const uint32_t t = S / 2;
+    return t < 128 ? 128 : (t > 1024 ? 1024 : t);
 }
 
 size_t stage_one_paper_smem_bytes(uint32_t S, uint32_t K, uint32_t L)
 {
     const size_t Kp = (K + 7u) & ~7u;
     size_t n = S * 12 + Kp * 4 + Kp * 2 * 3 + (128 + 40 + 40) * 4;
-    if ((int32_t)L <= PRIV_HIST_MAX_L) n += ((size_t)(L + 2) * (stage_one_threads(S, K) + 4) + 15) / 16 * 16;
+    if ((int32_t)L <= PRIV_HIST_MAX_L) n += ((size_t)(L + 2) * (stage_one_paper_threads(S) + 4) + 15) / 16 * 16;
     return n;
 }
 
+// Eight slots per thread when that leaves a thread at most two ids of a token, else four (at most 1024 threads).
+// Measured inside the kernel, eight / four slots per thread: S = 4096, K = 1000: 3.9 / 4.5 us; S = 2048, K = 512, two
+// tokens: 4.8 / 5.0; S = 4096, K = 2048, two tokens: 13.1 / 10.7; S = K = 2048: 8.3 / 6.8; S = 1024, K = 512, two
+// tokens: 8.4 / 5.6 (two slots per thread: 6.4).
 uint32_t stage_one_threads(uint32_t S, uint32_t K)
 {
-    (void)K;
-    uint32_t t = S / 2;
-    if (t < 128) t = 128;
-    if (t > 1024) t = 1024;
-    return t;
+    const uint32_t t = K <= S / 4 ? S / 8 : S / 4;
+    return t < 128 ? 128 : (t > 1024 ? 1024 : t);
 }
 
 cudaError_t stage_one_prepare(size_t max_smem)
 {
     const void* kernels[] = {
-        reinterpret_cast<const void*>(avsg_stage_one_kernel<false, S1_MAX_TABLES, false>),
-        reinterpret_cast<const void*>(avsg_stage_one_kernel<true, S1_MAX_TABLES, false>),
-        reinterpret_cast<const void*>(avsg_stage_one_kernel<false, S1_BIG_TABLES, false>),
-        reinterpret_cast<const void*>(avsg_stage_one_kernel<true, S1_BIG_TABLES, false>),
-        reinterpret_cast<const void*>(avsg_stage_one_kernel<false, S1_MAX_TABLES, true>),
-        reinterpret_cast<const void*>(avsg_stage_one_kernel<true, S1_MAX_TABLES, true>),
-        reinterpret_cast<const void*>(avsg_stage_one_kernel<false, S1_BIG_TABLES, true>),
-        reinterpret_cast<const void*>(avsg_stage_one_kernel<true, S1_BIG_TABLES, true>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<2, 2, S1_MAX_TABLES>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<4, 2, S1_MAX_TABLES>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<4, 4, S1_MAX_TABLES>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 2, S1_MAX_TABLES>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 4, S1_MAX_TABLES>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 8, S1_MAX_TABLES>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<2, 2, S1_BIG_TABLES>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<4, 2, S1_BIG_TABLES>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<4, 4, S1_BIG_TABLES>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 2, S1_BIG_TABLES>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 4, S1_BIG_TABLES>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 8, S1_BIG_TABLES>),
         reinterpret_cast<const void*>(avsg_stage_one_paper_kernel)};
     for (const void* k : kernels) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem);
@@ -800,24 +799,27 @@ cudaError_t stage_one_prepare(size_t max_smem)
 
 namespace {
 template <int CAP>
-cudaError_t launch_stage_one_t(const S1ParamsT<CAP>& p, uint32_t n_tables, cudaStream_t stream)
+cudaError_t launch_stage_one_t(const S1ParamsT<CAP>& p, uint32_t n_blocks, cudaStream_t stream)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n_tables);
+    cfg.gridDim = dim3(n_blocks);
     cfg.blockDim = dim3(stage_one_threads(p.S, p.K));
-    const bool direct = p.where != nullptr;
-    cfg.dynamicSmemBytes = stage_one_smem_bytes(p.S, p.K, p.L, direct);
+    cfg.dynamicSmemBytes = stage_one_smem_bytes(p.S, p.K, p.n_q);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (n_tables < p.n_launch)              // fewer blocks than tables: the blocks serve the tables in rounds
-        return direct ? cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<true, CAP, true>, p)
-                      : cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<false, CAP, true>, p);
-    return direct ? cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<true, CAP, false>, p)
-                  : cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<false, CAP, false>, p);
+    const uint32_t ipt = (p.K + cfg.blockDim.x - 1) / cfg.blockDim.x;      // ids per thread
+    switch (p.S / cfg.blockDim.x) {
+        case 8:  return ipt <= 2 ? cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<8, 2, CAP>, p)
+                      : ipt <= 4 ? cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<8, 4, CAP>, p)
+                                 : cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<8, 8, CAP>, p);
+        case 4:  return ipt <= 2 ? cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<4, 2, CAP>, p)
+                                 : cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<4, 4, CAP>, p);
+        default: return cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<2, 2, CAP>, p);
+    }
 }
 }  // namespace
 
@@ -826,7 +828,7 @@ cudaError_t launch_stage_one(const S1Params& p, uint32_t n_tables, cudaStream_t 
     if (p.qword == nullptr) return launch_stage_one_t(p, n_tables, stream);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_tables);
-    cfg.blockDim = dim3(stage_one_threads(p.S, p.K));
+    cfg.blockDim = dim3(stage_one_paper_threads(p.S));
     cfg.dynamicSmemBytes = stage_one_paper_smem_bytes(p.S, p.K, p.L);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];

@@ -41,6 +41,45 @@ __device__ __forceinline__ uint32_t decay4(uint32_t w, uint32_t d)
     return __vmaxs4(__vsubss4(w, d * 0x01010101u), 0xFFFFFFFFu);
 }
 
+// The same for SPT consecutive slots (2, 4 or 8), four to a word.  GLOBAL: from global memory, past L1.
+template <int SPT, bool GLOBAL = false>
+__device__ __forceinline__ void life_words(const int8_t* at, bool own, uint32_t (&w)[(SPT + 3) / 4])
+{
+#pragma unroll
+    for (int q = 0; q < (SPT + 3) / 4; ++q) w[q] = 0x7F7F7F7Fu;
+    if (!own) return;
+    if constexpr (SPT == 8) {
+        const uint2 v = GLOBAL ? __ldcg(reinterpret_cast<const uint2*>(at)) : *reinterpret_cast<const uint2*>(at);
+        w[0] = v.x; w[1] = v.y;
+    } else if constexpr (SPT == 4) {
+        w[0] = GLOBAL ? __ldcg(reinterpret_cast<const uint32_t*>(at)) : *reinterpret_cast<const uint32_t*>(at);
+    } else {
+        w[0] = 0x7F7F0000u | (GLOBAL ? __ldcg(reinterpret_cast<const uint16_t*>(at)) : *reinterpret_cast<const uint16_t*>(at));
+    }
+}
+
+template <int SPT>
+__device__ __forceinline__ void life_words_store(int8_t* at, bool own, const uint32_t (&w)[(SPT + 3) / 4])
+{
+    if (!own) return;
+    if constexpr (SPT == 8) *reinterpret_cast<uint2*>(at) = make_uint2(w[0], w[1]);
+    else if constexpr (SPT == 4) *reinterpret_cast<uint32_t*>(at) = w[0];
+    else *reinterpret_cast<uint16_t*>(at) = (uint16_t)w[0];
+}
+
+// Exclusive prefix over the lanes and total of a count 0 .. MAX that every lane of the warp has: one ballot per bit.
+template <int MAX>
+__device__ __forceinline__ void warp_rank(uint32_t n, uint32_t below, uint32_t& rank, uint32_t& total)
+{
+    rank = total = 0;
+#pragma unroll
+    for (int bit = 0; (1 << bit) <= MAX; ++bit) {
+        const uint32_t v = __ballot_sync(0xffffffffu, (n >> bit) & 1u);
+        rank += __popc(v & below) << bit;
+        total += __popc(v) << bit;
+    }
+}
+
 // The ids a thread handles for one token: positions i0 .. i0+ipt-1.
 __device__ __forceinline__ void load_ids(const int32_t* X, uint32_t i0, uint32_t ipt, uint32_t K, int32_t (&xs)[MAX_IPT])
 {
@@ -119,44 +158,47 @@ __device__ __forceinline__ void count_lifetimes(uint32_t w0, uint32_t w1, uint32
 
 // Overlapped Stage Two only (p.flags set): tells the transfer kernel, which is already resident, that token g of
 // this table is placed - `count` more entries of the table's miss list are final.  Called by every thread of the
-// block: the block meets after its list writes; one thread then fences (the barrier makes the fence cover the whole
+// block after a barrier behind the list writes; one thread then fences (the barrier makes the fence cover the whole
 // block's earlier writes, as in a grid-wide barrier) and writes the table's flag of token g: the call's number
 // (read once when the kernel starts) in the upper half, the count in the lower.
 template <typename P>
-__device__ __forceinline__ void publish_token(const P& p, uint32_t ti, uint32_t table, uint32_t g, uint32_t count,
-                                              uint32_t bt,      // bt: the table's index within this launch
-                                              uint32_t epoch)
+__device__ __forceinline__ void announce_token(const P& p, uint32_t ti, uint32_t table, uint32_t g, uint32_t count,
+                                               uint32_t bt,      // bt: the table's index within this launch
+                                               uint32_t epoch)
 {
     const bool announce = p.done_seq && g + 1 == p.n_q;
-    if (!p.flags && !announce) return;
-    const uint32_t tid = threadIdx.x;
-    if (tid == 0 && p.flags) {
-        if (g == 0) {
-            SegDesc sd;
-            sd.src_base = p.kv_base[bt];
-            sd.src_stride = p.kv_stride[bt];
-            sd.dst_base = reinterpret_cast<uint64_t>(p.buffer + (size_t)table * p.S * p.row_bytes);
-            sd.count = 0;
-            sd.pad = 0;
-            p.seg[ti] = sd;
-        }
+    if ((!p.flags && !announce) || threadIdx.x != 0) return;
+    if (p.flags && g == 0) {
+        SegDesc sd;
+        sd.src_base = p.kv_base[bt];
+        sd.src_stride = p.kv_stride[bt];
+        sd.dst_base = reinterpret_cast<uint64_t>(p.buffer + (size_t)table * p.S * p.row_bytes);
+        sd.count = 0;
+        sd.pad = 0;
+        p.seg[ti] = sd;
     }
-    __syncthreads();
-    if (tid == 0) {
+    __threadfence();
+    if (p.flags)
+        *reinterpret_cast<volatile unsigned long long*>(p.flags + (size_t)ti * p.n_q + g) =
+            ((unsigned long long)epoch << 32) | count;
+    // calls that asked for it (host buffers in the overlapped mode, or a caller's own signal word): the table
+    // that arrives last after the call's last token announces that every table of the call has written its
+    // slot table, hit mask and miss counts.  The arrivals are counted in a word of their own that wraps to
+    // zero by itself (atomicInc), whatever state the transfer kernel leaves the per-token counters in.
+    if (announce && atomicInc(p.done_ctr, p.expect - 1u) == p.expect - 1u) {
         __threadfence();
-        if (p.flags)
-            *reinterpret_cast<volatile unsigned long long*>(p.flags + (size_t)ti * p.n_q + g) =
-                ((unsigned long long)epoch << 32) | count;
-        // calls that asked for it (host buffers in the overlapped mode, or a caller's own signal word): the table
-        // that arrives last after the call's last token announces that every table of the call has written its
-        // slot table, hit mask and miss counts.  The arrivals are counted in a word of their own that wraps to
-        // zero by itself (atomicInc), whatever state the transfer kernel leaves the per-token counters in.
-        if (announce && atomicInc(p.done_ctr, p.expect - 1u) == p.expect - 1u) {
-            __threadfence();
-            *reinterpret_cast<volatile unsigned long long*>(p.done_seq) = p.host_seq;
-        }
+        *reinterpret_cast<volatile unsigned long long*>(p.done_seq) = p.host_seq;
     }
 }
 
+// The same with the barrier in front.
+template <typename P>
+__device__ __forceinline__ void publish_token(const P& p, uint32_t ti, uint32_t table, uint32_t g, uint32_t count,
+                                              uint32_t bt, uint32_t epoch)
+{
+    if (!p.flags && !(p.done_seq && g + 1 == p.n_q)) return;
+    __syncthreads();
+    announce_token(p, ti, table, g, count, bt, epoch);
+}
 
 }  // namespace avsg

@@ -1,0 +1,99 @@
+"""Stage One with one block per table at the sizes where its split of slots and ids over threads changes, with ids that
+share one chain of its index, and with states only a caller's own table can have; compared with the oracle after every
+call (whole numbers: nothing to tolerate)."""
+import numpy as np
+import pytest
+
+import avsg_traces as tr
+from oracle import OracleTable
+
+pytestmark = pytest.mark.gpu
+RB, CTX = 32, 40000
+
+
+def _same_bucket_ids(S, n, bucket):
+    """n ids whose multiplicative hash falls into one of the 2 S buckets."""
+    x = np.arange(1 << 22, dtype=np.uint64)
+    h = ((x * 2654435769) & 0xFFFFFFFF) >> np.uint64(32 - int(2 * S).bit_length() + 1)
+    return x[h == bucket][:n].astype(np.int32)
+
+
+# S below four warps' slots; K around S / 4 (the number of threads changes); one and two ids per thread and more;
+# K = S; the smallest K; as many nodes as fit one SM (N_q K = S)
+@pytest.mark.parametrize("S,K,n_q", [(32, 32, 1), (32, 1, 8), (64, 31, 2), (256, 64, 4), (256, 65, 3), (1024, 256, 2),
+                                     (1024, 257, 3), (2048, 2048, 1), (4096, 1024, 4), (4096, 1025, 3), (8192, 1, 8),
+                                     (8192, 2047, 4), (8192, 2049, 3), (8192, 4097, 1), (8192, 1024, 8)])
+def test_splits_of_slots_and_ids(S, K, n_q):
+    import torch
+    import paper_2609_37538_b200 as avsg
+    T, n, L = 6, 2, 3
+    rng = np.random.default_rng([S, K, n_q])
+    kv = avsg.pinned_empty(CTX * RB)
+    tr.fill_kv(kv.data_ptr(), 1, 0, CTX, RB)
+    ctx = avsg.Context(n, S, RB, K, n_q, L)
+    orc = [OracleTable(S, RB, L) for _ in range(n)]
+    for t in range(T):
+        span = min(CTX, 3 * S // 2 + K)               # a good share of the ids comes back
+        X = np.stack([[rng.choice(span, K, replace=False) for _ in range(n_q)] for _ in range(n)]).astype(np.int32)
+        X[:, :, K // 2] = -1                          # padding in the middle
+        N = [span - 7 * t for _ in range(n)]          # shrinks: resident ids become unverified
+        out = ctx.step(list(range(n)), torch.from_numpy(X).cuda(), [kv] * n, N)
+        slots, hit, mc = out.slots.cpu().numpy(), out.hit.cpu().numpy(), out.miss_count.cpu().numpy()
+        for i in range(n):
+            r = orc[i].step(X[i], N[i], kv.numpy(), RB)
+            assert (slots[i] == r.O).all() and (hit[i] == r.M).all() and (mc[i] == r.n).all(), (t, i)
+            tok, life = ctx.export_state(i)
+            c, l = orc[i].export_state()
+            assert (tok == c).all() and (life == l).all(), (t, i)
+            assert (ctx.buffer(i).cpu().numpy() == orc[i].rows()).all(), (t, i)
+            ts, oc = ctx.table_stats(i), orc[i].counters()
+            assert all(ts[k] == oc[k] for k in ("hits", "misses", "rows_copied", "extra_decays")), (t, i)
+    assert ctx.sync_status() == 0
+
+
+def test_ids_of_one_chain():
+    """Every id hashes to the same bucket: one chain holds the whole table and the ids that come in."""
+    import torch
+    import paper_2609_37538_b200 as avsg
+    S, K, n_q, L = 128, 32, 4, 4
+    ids = _same_bucket_ids(S, 256, 77)
+    rows = int(ids.max()) + 1
+    kv = avsg.pinned_empty(rows * 16)
+    kv.numpy()[:] = np.random.default_rng(5).integers(0, 256, rows * 16, dtype=np.uint8)
+    ctx, orc = avsg.Context(1, S, 16, K, n_q, L), OracleTable(S, 16, L)
+    rng = np.random.default_rng(6)
+    for t in range(12):
+        X = np.stack([rng.choice(ids, K, replace=False) for _ in range(n_q)])
+        out = ctx.step([0], torch.from_numpy(X[None]).cuda(), [kv], [rows])
+        r = orc.step(X, rows, kv.numpy(), 16)
+        assert (out.slots.cpu().numpy()[0] == r.O).all() and (out.hit.cpu().numpy()[0] == r.M).all(), t
+    assert (ctx.buffer(0).cpu().numpy() == orc.rows()).all() and ctx.sync_status() == 0
+
+
+def test_lifetimes_above_the_maximum():
+    """Caller-owned state from a longer maximum lifetime: slots reserved early in a call are reclaimed later in it, and
+    an id that was reserved and lost within the call is missed again."""
+    import torch
+    import paper_2609_37538_b200 as avsg
+    S, K, n_q, L = 64, 16, 4, 3
+    kv = avsg.pinned_empty(4000 * RB)
+    tr.fill_kv(kv.data_ptr(), 3, 0, 4000, RB)
+    rng = np.random.default_rng(9)
+    tok = np.full(S, -1, np.int32)
+    life = np.full(S, -1, np.int8)
+    tok[::2], life[::2] = np.arange(1000, 1000 + S // 2), 90          # half of the table outlives the call
+    orc = OracleTable(S, RB, L)
+    orc.import_state(tok, life)
+    d = dict(device="cuda")
+    tok_d, life_d = torch.from_numpy(tok[None]).to(**d), torch.from_numpy(life[None]).to(**d)
+    buf, status = torch.zeros((1, S, RB), dtype=torch.uint8, **d), torch.zeros(1, dtype=torch.int32, **d)
+    slots, hit = torch.empty((1, n_q, K), dtype=torch.int32, **d), torch.empty((1, n_q, K), dtype=torch.uint8, **d)
+    for t in range(4):
+        X = np.stack([rng.choice(70, K, replace=False) for _ in range(n_q)]).astype(np.int32)
+        avsg.step_noalloc(tok_d, life_d, buf, torch.from_numpy(X[None]).cuda(), [kv], [4000], max_lifetime=L, slots=slots,
+                          hit=hit, status=status)
+        r = orc.step(X, 4000, kv.numpy(), RB)
+        c, l = orc.export_state()
+        assert (slots[0].cpu().numpy() == r.O).all() and (hit[0].cpu().numpy() == r.M).all(), t
+        assert (tok_d[0].cpu().numpy() == c).all() and (life_d[0].cpu().numpy() == l).all(), t
+        assert int(status.item()) == 0
