@@ -7,8 +7,10 @@ any use raises: there is no CPU fallback.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
+import struct
 from typing import List, Optional, Sequence, Union
 
 import numpy as np
@@ -177,10 +179,27 @@ def _addr(x) -> int:
     raise TypeError("expected a tensor, an array or an address, got %r" % type(x))
 
 
+_current_stream_fn = None
+
+
+def _current_stream() -> int:
+    """Handle of the current device's current stream.  torch.cuda.current_stream() builds a Stream object (3.2 us); the
+    functions beneath it give the handle in 0.2 us, where the installed torch has them."""
+    global _current_stream_fn
+    if _current_stream_fn is None:
+        import torch
+        torch.cuda.init()
+        raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if raw is not None and dev is not None:
+            _current_stream_fn = lambda: raw(dev())
+        else:
+            _current_stream_fn = lambda: torch.cuda.current_stream().cuda_stream
+    return _current_stream_fn()
+
+
 def _stream_handle(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream or None
+        return _current_stream() or None
     if isinstance(stream, int):
         return stream or None
     return stream.cuda_stream or None
@@ -215,6 +234,7 @@ class PreparedCall:
         self._kv = (ctypes.c_void_p * n)(*[_addr(k) for k in kv])
         self._stride = (ctypes.c_uint64 * n)(*[int(s) for s in row_stride]) if row_stride is not None else None
         self._vlen = (ctypes.c_int32 * n)()
+        self._pack_vlen = struct.Struct("=%di" % n).pack_into
         self._rows = (ctypes.c_uint32 * n)(*[int(r) for r in kv_rows]) if kv_rows is not None else None
         a = AvsgStepArgs()
         a.n, a.n_tokens, a.topk = n, n_tokens, topk
@@ -224,6 +244,7 @@ class PreparedCall:
         a.verified_len = ctypes.addressof(self._vlen)
         a.kv_rows = ctypes.addressof(self._rows) if self._rows is not None else None
         self.args = a
+        self._ref = ctypes.byref(a)
 
     def run(self, indices, verified_len: Sequence[int], slots, hit=None, miss_count=None, stream=None,
             host: bool = False, stage_one_done=None, arriving=None) -> None:
@@ -243,13 +264,17 @@ class PreparedCall:
             a.verified_len_dev = verified_len.data_ptr()
         else:
             a.verified_len_dev = None
-            self._vlen[:] = [int(v) for v in verified_len]
+            try:
+                self._pack_vlen(self._vlen, 0, *verified_len)
+            except struct.error:                         # not n integers that fit: as the element type converts them
+                self._vlen[:] = [int(v) for v in verified_len]
         a.indices, a.slots = _addr(indices), _addr(slots)
         a.hit = _addr(hit) if hit is not None else None
         a.miss_count = _addr(miss_count) if miss_count is not None else None
         lib = self.ctx._lib
-        fn = lib.avsg_step_host if host else lib.avsg_step
-        _check(fn(self.ctx._h, ctypes.byref(a), _stream_handle(stream)), "avsg_step")
+        rc = (lib.avsg_step_host if host else lib.avsg_step)(self.ctx._h, self._ref, _stream_handle(stream))
+        if rc != OK:
+            _check(rc, "avsg_step")
 
 
 class Context:
@@ -400,6 +425,24 @@ class Context:
         return {name: getattr(s, name) for name, _ in AvsgStats._fields_ if not name.startswith("last_")}
 
 
+_CTYPES = {"Q": ctypes.c_uint64, "I": ctypes.c_uint32, "i": ctypes.c_int32}
+
+
+def _c_array(kind: str, values, n: int):
+    """(owner, address) of a C array of n integers; None: no array.  array.array fills from Python integers at a third of
+    a ctypes array's cost; what it does not take (other numbers, another count, values that wrap) goes that way."""
+    if values is None:
+        return None, None
+    try:
+        out = array.array(kind, values)
+        if len(out) == n:
+            return out, out.buffer_info()[0]
+    except (TypeError, OverflowError):
+        pass
+    out = (_CTYPES[kind] * n)(*[int(v) for v in values])
+    return out, ctypes.addressof(out)
+
+
 def step_noalloc(tok, life, buffer, indices, kv, verified_len, *, max_lifetime: int = 16, slots, hit=None,
                  miss_count=None, status=None, row_stride=None, stream=None, kv_rows=None) -> None:
     """avsg_step_noalloc: one decode iteration on caller-owned state, for callers that cannot allocate
@@ -413,20 +456,17 @@ def step_noalloc(tok, life, buffer, indices, kv, verified_len, *, max_lifetime: 
     """
     n, S = tok.shape
     _, n_q, K = indices.shape
-    kv_arr = (ctypes.c_void_p * n)(*[_addr(k) for k in kv])
-    vlen = (ctypes.c_int32 * n)(*[int(v) for v in verified_len])
-    stride = (ctypes.c_uint64 * n)(*[int(s) for s in row_stride]) if row_stride is not None else None
+    kv_arr, kv_at = _c_array("Q", [_addr(k) for k in kv], n)
+    vlen, vlen_at = _c_array("i", verified_len, n)
+    stride, stride_at = _c_array("Q", row_stride, n)
+    rows, rows_at = _c_array("I", kv_rows, n)
     a = AvsgNoAllocArgs()
     a.n, a.n_tokens, a.topk, a.buffer_slots = n, n_q, K, S
     a.row_bytes, a.max_lifetime = buffer.shape[-1], max_lifetime
     a.tok, a.life, a.buffer, a.indices = _addr(tok), _addr(life), _addr(buffer), _addr(indices)
-    a.kv_base = ctypes.addressof(kv_arr)
-    a.row_stride = ctypes.addressof(stride) if stride is not None else None
-    a.verified_len = ctypes.addressof(vlen)
+    a.kv_base, a.row_stride, a.verified_len, a.kv_rows = kv_at, stride_at, vlen_at, rows_at
     a.slots = _addr(slots)
     a.hit = _addr(hit) if hit is not None else None
     a.miss_count = _addr(miss_count) if miss_count is not None else None
     a.status = _addr(status) if status is not None else None
-    rows = (ctypes.c_uint32 * n)(*[int(r) for r in kv_rows]) if kv_rows is not None else None
-    a.kv_rows = ctypes.addressof(rows) if rows is not None else None
     _check(load_library().avsg_step_noalloc(ctypes.byref(a), _stream_handle(stream)), "avsg_step_noalloc")
