@@ -60,8 +60,8 @@ extern "C" {
                                              with the direct index (taken as padding)          */
 #define AVSG_STATUS_WAIT_TIMEOUT    0x20u /* overlapped Stage Two gave up waiting for Stage One:
                                              rows of THAT call were not copied.  Later calls are
-                                             not affected (the hand-over flags carry the number
-                                             of their call)                                     */
+                                             not affected (each takes the hand-over flags down
+                                             before its transfer kernel can start)              */
 #define AVSG_STATUS_LAUNCH_FAILED   0x40u /* a Stage Two launch failed after Stage One had run:
                                              slots were reserved whose rows were never copied  */
 

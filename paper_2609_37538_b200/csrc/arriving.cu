@@ -26,13 +26,7 @@ __global__ void __launch_bounds__(512) avsg_arriving_kernel(const __grid_constan
     const uint32_t tid = threadIdx.x, nt = blockDim.x, words = (p.S + 31u) / 32u;
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    uint32_t epoch = 0;
-    if (p.flags) {
-        // the number of this overlapped call: final before Stage One, which this grid was launched behind, started
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(epoch) : "l"(p.epoch) : "memory");
-    } else {
-        asm volatile("griddepcontrol.wait;" ::: "memory");   // Stage One is complete: slot tables and lists are final
-    }
+    if (!p.flags) asm volatile("griddepcontrol.wait;" ::: "memory");   // Stage One is complete: slot tables and lists are final
     const bool vec = (p.per_table & 3u) == 0 && (reinterpret_cast<uint64_t>(p.slots) & 15u) == 0 &&
                      (reinterpret_cast<uint64_t>(p.arriving) & 3u) == 0;
 
@@ -44,16 +38,15 @@ __global__ void __launch_bounds__(512) avsg_arriving_kernel(const __grid_constan
                 // the table's last token is placed: its slot table is final, and so are the list entries the flags count
                 uint32_t count = 0;
                 for (uint32_t g = p.n_q; g-- > 0 && s_ok;) {          // last token first: the others are there by then
-                    const unsigned long long* f = p.flags + (size_t)ti * p.n_q + g;
-                    unsigned long long v = 0;
-                    uint32_t spin = 0;
+                    const uint32_t* f = p.flags + (size_t)ti * p.n_q + g;
+                    uint32_t v = 0, spin = 0;
                     for (; spin < OVERLAP_SPIN_LIMIT; ++spin) {
-                        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(f) : "memory");
-                        if ((uint32_t)(v >> 32) == epoch) break;
+                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
+                        if (v) break;
                         __nanosleep(64);
                     }
                     if (spin == OVERLAP_SPIN_LIMIT) { s_ok = 0; atomicOr(p.status, ST_WAIT_TIMEOUT); }
-                    count += (uint32_t)v;
+                    count += v - (v ? 1u : 0u);
                 }
                 s_count = count;
             } else {
@@ -93,6 +86,8 @@ __global__ void __launch_bounds__(512) avsg_arriving_kernel(const __grid_constan
             *reinterpret_cast<volatile unsigned long long*>(p.done_seq) = p.value;
         }
     }
+    // the next grid's wait for this one has to cover Stage One too, whose write-back goes on behind its last flag
+    if (p.flags) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace

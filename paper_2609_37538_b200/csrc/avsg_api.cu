@@ -12,6 +12,10 @@
 
 using namespace avsg;
 
+namespace {
+constexpr size_t FLAG_BYTES = ((size_t)OVERLAP_MAX_TABLES * OVERLAP_MAX_TOKENS + 1) * sizeof(uint32_t);
+}
+
 struct avsg_ctx {
     avsg_config cfg;
     uint32_t logS = 0, logH = 0;
@@ -26,12 +30,12 @@ struct avsg_ctx {
     int8_t* d_life = nullptr;
     uint8_t* d_buffer = nullptr;
     TableStats* d_stats = nullptr;
-    unsigned long long* d_flags = nullptr;         // overlapped Stage Two: per-(table of the call, token) flags
-                                                   //   (call number << 32 | miss count) [OVERLAP_MAX_TABLES x TOKENS]
-    unsigned long long* d_sync = nullptr;          //   [0] the call number, [1] transfer blocks that are through,
-                                                   //   [2] sequence number of the last host-buffer call,
+    uint32_t* d_flags = nullptr;                   // hand-over flags per (table of the call, token) (1 + miss count)
+                                                   //   [OVERLAP_MAX_TABLES x TOKENS], and one that is never raised
+    unsigned long long* d_sync = nullptr;          //   [2] sequence number of the last host-buffer call,
                                                    //   [3] arrivals after a host-buffer call's last token
-    S1ParamsBig* big_args = nullptr;               // host: the large Stage One argument block, built in place per call
+    S1ParamsBig* big_args = nullptr;               // host: the large argument blocks, built in place per call
+    XferOverlapParamsBig* big_xfer_args = nullptr;
     unsigned long long* d_trange = nullptr;        // [8] time marks of the last timed call, then [8] their initial values
     unsigned long long* d_trange_init = nullptr;
     int2* d_list = nullptr;
@@ -91,6 +95,7 @@ void free_all(avsg_ctx* c)
     cudaFree(c->d_tok); cudaFree(c->d_life); cudaFree(c->d_buffer); cudaFree(c->d_stats); cudaFree(c->d_trange);
     cudaFree(c->d_flags); cudaFree(c->d_sync);
     delete c->big_args;
+    delete c->big_xfer_args;
     cudaFree(c->d_list); cudaFree(c->d_seg); cudaFree(c->d_status); cudaFree(c->d_where); cudaFree(c->d_q); cudaFree(c->d_q_snap);
     cudaFree(c->d_tok_snap); cudaFree(c->d_life_snap);
     cudaFree(c->d_idx_stage); cudaFree(c->d_slots_stage); cudaFree(c->d_hit_stage); cudaFree(c->d_mc_stage);
@@ -186,6 +191,16 @@ int copy_engine_transfer(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stre
     return AVSG_OK;
 }
 
+// The transfer kernel's arguments but for the tables' own.
+template <typename X>
+void overlap_params(avsg_ctx* c, X& x, uint32_t n, uint32_t n_q, uint32_t round_size)
+{
+    x.miss_list = c->d_list; x.status = c->d_status; x.buffer = c->d_buffer;
+    x.flags = c->d_flags;
+    x.n = n; x.n_q = n_q; x.list_stride = c->list_stride; x.row_bytes = c->cfg.row_bytes; x.S = c->cfg.buffer_slots;
+    x.round_size = round_size; x.t_range = nullptr;
+}
+
 int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool host_io)
 {
     int rc = check_args(c, a);
@@ -236,7 +251,8 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
             mode = AVSG_XFER_SM_BALANCED;
     }
     // host buffers in the overlapped mode: no event between the two grids, the download waits for a sequence number
-    const bool wait_on_sequence = host_io && mode == AVSG_XFER_SM_OVERLAP && c->wait_value64 != nullptr;
+    const bool overlap = mode == AVSG_XFER_SM_OVERLAP;
+    const bool wait_on_sequence = host_io && overlap && c->wait_value64 != nullptr;
     // the position-level comparator reads the hit mask: use the library's own buffer if the caller wants none
     if (mode == AVSG_XFER_POSITION_LEVEL && !hit) hit = c->d_hit_stage;
     if (c->timing) {
@@ -266,15 +282,13 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
         p.S = c->cfg.buffer_slots; p.logH = c->logH; p.row_bytes = c->cfg.row_bytes;
         p.K = K; p.n_q = n_q; p.L = (uint32_t)c->cfg.max_lifetime;
         p.first = first; p.list_stride = c->list_stride;
-        p.n_launch = cnt; p.round_size = round_size;
+        p.n_launch = cnt;
         p.where = c->d_where; p.max_context = c->cfg.max_context;
         p.qword = c->d_q; p.probe_retries = c->cfg.probe_retries; p.hash_a1 = c->cfg.hash_a1; p.hash_a2 = c->cfg.hash_a2;
         p.t_range = c->timing ? c->d_trange : nullptr;
         p.verified_len_dev = a->verified_len_dev;
         // (every field is assigned: the large block is re-used from call to call)
-        const bool overlap = mode == AVSG_XFER_SM_OVERLAP;
         p.flags = overlap ? c->d_flags : nullptr;
-        p.epoch = reinterpret_cast<const uint32_t*>(c->d_sync);
         // the caller's word: written by Stage One itself, or by the `arriving` kernel behind it when that output
         // is asked for too (the word then also covers it)
         p.done_seq = wait_on_sequence ? c->d_sync + 2
@@ -323,8 +337,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
         q.done_ctr = reinterpret_cast<uint32_t*>(c->d_sync + 3);
         q.value = a->stage_one_done_value;
         q.n = n; q.per_table = n_q * K; q.S = c->cfg.buffer_slots; q.list_stride = c->list_stride;
-        q.flags = mode == AVSG_XFER_SM_OVERLAP ? c->d_flags : nullptr;
-        q.epoch = reinterpret_cast<const uint32_t*>(c->d_sync);
+        q.flags = overlap ? c->d_flags : nullptr;
         q.n_q = n_q; q.status = c->d_status;
         CU(launch_arriving(q, (uint32_t)c->sm_count, stream));
     }
@@ -354,20 +367,26 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
         q.seg = c->d_seg; q.indices = indices; q.slots = slots; q.hit = hit; q.status = c->d_status;
         q.n = n; q.per_table = n_q * K; q.row_bytes = c->cfg.row_bytes; q.S = c->cfg.buffer_slots;
         CU(launch_transfer_positions(q, c->xfer_blocks ? c->xfer_blocks : (uint32_t)c->sm_count, c->xfer_threads, stream));
-    } else if (mode == AVSG_XFER_SM_OVERLAP) {
-        XferOverlapParams x;
-        x.seg = c->d_seg; x.miss_list = c->d_list; x.status = c->d_status;
-        x.flags = c->d_flags; x.epoch = reinterpret_cast<uint32_t*>(c->d_sync);
-        x.done = reinterpret_cast<uint32_t*>(c->d_sync + 1);
-        x.n = n; x.n_q = n_q; x.list_stride = c->list_stride; x.row_bytes = c->cfg.row_bytes; x.S = c->cfg.buffer_slots;
-        x.round_size = round_size; x.expect_extra = 0;
-        x.t_range = c->timing ? c->d_trange + 2 : nullptr;
-        if (launch_transfer_overlap(x, c->xfer_blocks ? c->xfer_blocks : (uint32_t)c->sm_count, c->xfer_threads, stream)
-            != cudaSuccess) {
-            // Stage One has run and written flags with the current call number, which nothing will advance: wipe
-            // them here, in stream order, and remember that this call reserved slots whose rows were never copied
-            cudaGetLastError();
-            cudaMemsetAsync(c->d_flags, 0, (size_t)OVERLAP_MAX_TABLES * OVERLAP_MAX_TOKENS * sizeof(unsigned long long), stream);
+    } else if (overlap) {
+        auto launch = [&](auto& x) -> cudaError_t {
+            overlap_params(c, x, n, n_q, round_size);
+            x.t_range = c->timing ? c->d_trange + 2 : nullptr;
+            for (uint32_t i = 0; i < n; ++i) {
+                x.table_id[i] = a->table_ids[i];
+                x.kv_base[i] = c->call_kv_dev[i];
+                x.kv_stride[i] = a->row_stride ? a->row_stride[i] : c->cfg.row_bytes;
+            }
+            return launch_transfer_overlap(x, c->xfer_blocks ? c->xfer_blocks : (uint32_t)c->sm_count, c->xfer_threads, stream);
+        };
+        cudaError_t e;
+        if (n <= (uint32_t)S1_MAX_TABLES) {
+            XferOverlapParams x;
+            e = launch(x);
+        } else {
+            e = launch(*c->big_xfer_args);
+        }
+        if (e != cudaSuccess) {
+            cudaGetLastError();                  // this call reserved slots whose rows were never copied
             c->host_status |= AVSG_STATUS_LAUNCH_FAILED;
             return AVSG_ECUDA;
         }
@@ -484,10 +503,11 @@ int avsg_create(const avsg_config* cfg, avsg_ctx** out)
     ok = ok && cudaMalloc(&c->d_buffer, T * S * cfg->row_bytes) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_stats, T * sizeof(TableStats)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_trange, 16 * sizeof(unsigned long long)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->d_flags, (size_t)OVERLAP_MAX_TABLES * OVERLAP_MAX_TOKENS * sizeof(unsigned long long)) == cudaSuccess;
+    ok = ok && cudaMalloc(&c->d_flags, FLAG_BYTES) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_sync, 8 * sizeof(unsigned long long)) == cudaSuccess;
     c->big_args = new (std::nothrow) S1ParamsBig();
-    ok = ok && c->big_args != nullptr;
+    c->big_xfer_args = new (std::nothrow) XferOverlapParamsBig();
+    ok = ok && c->big_args != nullptr && c->big_xfer_args != nullptr;
     ok = ok && cudaMalloc(&c->d_list, n_ids * sizeof(int2)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_seg, T * sizeof(SegDesc)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_status, 256) == cudaSuccess;
@@ -527,13 +547,12 @@ int avsg_create(const avsg_config* cfg, avsg_ctx** out)
     {
         // [0] Stage One first start, [1] its last end; Stage Two: [2] first start, [3] last end, [4] first copy loop,
         // [5] first row in, [6] first block done; minima start at "never", maxima at 0
-        const unsigned long long never = ~0ull, first_epoch = 1;      // call numbers start at 1: a zeroed flag is never valid
+        const unsigned long long never = ~0ull;
         const unsigned long long init[16] = {never, 0, never, 0, never, never, never, 0, never, 0, never, 0, never, never, never, 0};
         c->d_trange_init = c->d_trange + 8;
         if (cudaMemcpy(c->d_trange, init, sizeof(init), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemset(c->d_flags, 0, (size_t)OVERLAP_MAX_TABLES * OVERLAP_MAX_TOKENS * sizeof(unsigned long long)) != cudaSuccess ||
-            cudaMemset(c->d_sync, 0, 8 * sizeof(unsigned long long)) != cudaSuccess ||
-            cudaMemcpy(c->d_sync, &first_epoch, sizeof(first_epoch), cudaMemcpyHostToDevice) != cudaSuccess) {
+            cudaMemset(c->d_flags, 0, FLAG_BYTES) != cudaSuccess ||
+            cudaMemset(c->d_sync, 0, 8 * sizeof(unsigned long long)) != cudaSuccess) {
             free_all(c); delete c; return AVSG_ECUDA;
         }
     }
@@ -677,10 +696,8 @@ int avsg_clear_status(avsg_ctx* c)
     if (!guard.ok) return AVSG_ECUDA;
     CU(cudaDeviceSynchronize());
     CU(cudaMemset(c->d_status, 0, sizeof(uint32_t)));
-    // a transfer kernel that gave up may have left the per-token counters of the overlapped mode raised
-    // (the flags of the overlapped mode carry their call's number and need no clearing; the two arrival counters
-    // wrap to zero by themselves unless a grid was lost half way)
-    CU(cudaMemset(c->d_sync + 1, 0, sizeof(unsigned long long)));
+    // (every call takes its hand-over flags down itself; the arrival counter wraps to zero by itself unless a grid was
+    // lost half way)
     CU(cudaMemset(c->d_sync + 3, 0, sizeof(unsigned long long)));
     c->host_status = 0;
     return AVSG_OK;
@@ -692,11 +709,9 @@ int avsg_probe_wait_limit(avsg_ctx* c, void* cuda_stream)
     DeviceGuard guard(c->cfg.device);
     if (!guard.ok) return AVSG_ECUDA;
     XferOverlapParams x;
-    x.seg = c->d_seg; x.miss_list = c->d_list; x.status = c->d_status;
-    x.flags = c->d_flags; x.epoch = reinterpret_cast<uint32_t*>(c->d_sync);
-    x.done = reinterpret_cast<uint32_t*>(c->d_sync + 1);
-    x.n = 1; x.n_q = 1; x.list_stride = c->list_stride; x.row_bytes = c->cfg.row_bytes; x.S = c->cfg.buffer_slots;
-    x.round_size = 1; x.expect_extra = 0x40000000u;     // a call number no Stage One will ever write: the wait must run out
+    overlap_params(c, x, 1, 1, 1);
+    x.table_id[0] = 0; x.kv_base[0] = 0; x.kv_stride[0] = 0;
+    x.flags = c->d_flags + (size_t)OVERLAP_MAX_TABLES * OVERLAP_MAX_TOKENS;      // never raised: the wait must run out
     CU(launch_transfer_overlap(x, c->xfer_blocks ? c->xfer_blocks : (uint32_t)c->sm_count, c->xfer_threads,
                                static_cast<cudaStream_t>(cuda_stream)));
     return AVSG_OK;

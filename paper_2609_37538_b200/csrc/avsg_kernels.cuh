@@ -91,18 +91,15 @@ struct S1ParamsT {
     uint32_t S, logH, row_bytes, K, n_q, L;
     uint32_t first;              // index within the call of this launch's first table
     uint32_t n_launch;           // tables of this launch (the grid may have fewer blocks: a block then serves several)
-    uint32_t round_size;         // overlapped Stage Two: tables per publication round (= grid size of Stage One)
     uint32_t list_stride;        // entries per segment of miss_list
     uint32_t max_context;        // direct index: entries per table
     uint16_t* where;             // direct index [num_tables][max_context], or null for the hash index
     uint32_t* qword;             // paper-literal mode: packed metadata words [num_tables][S], else null
     uint32_t probe_retries, hash_a1, hash_a2;   // paper-literal mode: R, a1, a2
     unsigned long long* t_range = nullptr;      // timing on: [0] earliest block start, [1] latest block end (ns)
-    // overlapped Stage Two (null otherwise): flags[ti * n_q + g] = (epoch << 32) | misses of token g of the ti-th
-    // table of the call, written when that token is placed; *epoch is the number of the current overlapped call
-    // (the transfer grid advances it when it is through), so flags of earlier calls never look valid
-    unsigned long long* flags = nullptr;
-    const uint32_t*     epoch = nullptr;
+    // overlapped Stage Two (null otherwise): flags[ti * n_q + g] = 1 + misses of token g of the ti-th table of the call,
+    // written when that token is placed; zero until then (see take_flags_down())
+    uint32_t* flags = nullptr;
     // calls with host buffers in that mode (null otherwise): the table that places the call's last token last
     // writes the call's sequence number to *done_seq, which the output download waits for
     unsigned long long* done_seq = nullptr;
@@ -135,18 +132,23 @@ constexpr uint32_t S1_ROUND_BLOCKS = 32;             // Stage One blocks of a ca
 constexpr int OVERLAP_MAX_TABLES = S1_BIG_TABLES;   // one Stage One launch
 constexpr uint32_t OVERLAP_SPIN_LIMIT = 1u << 18;   // polls before the wait gives up; a poll is an L2 round trip plus a 64 ns sleep, ~0.8 us measured: ~0.2 s
 
-struct XferOverlapParams {       // Stage Two that starts on token g's misses while Stage One places token g+1
-    const SegDesc* seg;          // bases written by Stage One before it publishes token 0
+// Stage Two that is resident while Stage One runs and starts on misses as they are announced (see the kernel).
+// The tables' bases come as kernel arguments, CAP tables' worth.
+template <int CAP>
+struct XferOverlapParamsT {
     const int2*    miss_list;
     uint32_t*      status;
-    const unsigned long long* flags;   // [n][n_q] (epoch << 32) | miss count, written by Stage One per placed token
-    uint32_t*      epoch;        // number of the current overlapped call; advanced by the last block of this grid
-    uint32_t*      done;         // blocks of this grid that are through; wraps to zero by itself
+    const uint32_t* flags;       // [n][n_q] 1 + miss count, written by Stage One
+    uint8_t*       buffer;       // [num_tables][S * row_bytes]
     uint32_t n, n_q, list_stride, row_bytes, S;
     uint32_t round_size;         // tables per round (n: one round)
-    uint32_t expect_extra;       // added to what a counter must reach: 0, or 1 for the wait-limit diagnostic
     unsigned long long* t_range = nullptr;
+    uint32_t table_id[CAP];
+    uint64_t kv_base[CAP];
+    uint64_t kv_stride[CAP];
 };
+using XferOverlapParams = XferOverlapParamsT<S1_MAX_TABLES>;
+using XferOverlapParamsBig = XferOverlapParamsT<S1_BIG_TABLES>;
 
 struct PosParams {               // comparator S2: equal top-K position partition
     const SegDesc* seg;          // per table: host base, stride, buffer base
@@ -201,6 +203,7 @@ cudaError_t launch_direct_index_from_state(const int32_t* tok, uint16_t* where, 
 cudaError_t launch_all_k_prepare(const AllKParams& p, uint32_t n_tables, cudaStream_t stream);
 cudaError_t launch_transfer(const XferParams& p, uint32_t blocks, uint32_t threads, cudaStream_t stream);
 cudaError_t launch_transfer_overlap(const XferOverlapParams& p, uint32_t blocks, uint32_t threads, cudaStream_t stream);
+cudaError_t launch_transfer_overlap(const XferOverlapParamsBig& p, uint32_t blocks, uint32_t threads, cudaStream_t stream);
 cudaError_t launch_transfer_positions(const PosParams& p, uint32_t blocks, uint32_t threads, cudaStream_t stream);
 
 // Optional output of a call (latency hiding, Sec. 6 with Sec. 3.6): which positions' rows come with THIS call's
@@ -216,9 +219,8 @@ struct ArrivingParams {
     uint32_t*      done_ctr;         // wraps to zero at the grid size
     unsigned long long value;
     uint32_t n, per_table, S, list_stride;
-    // overlapped Stage Two: Stage One's hand-over flags and the call number (see S1ParamsT), else null
-    const unsigned long long* flags;
-    const uint32_t* epoch;
+    // overlapped Stage Two: Stage One's hand-over flags (see S1ParamsT), else null
+    const uint32_t* flags;
     uint32_t n_q;
     uint32_t* status;
 };

@@ -111,12 +111,9 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
     if (tid == 0) s_node[NIL] = make_uint2(0xFFFFFFFEu, NIL);          // an id that nobody looks for
 
     // Programmatic dependent launch: this grid may have been started while the previous kernel of the stream
-    // was still running; nothing is read before that kernel has completed.  The next kernel (Stage Two) is
-    // allowed to start its own prologue right away - it waits the same way before it reads the miss list.
+    // was still running; nothing is read before that kernel has completed.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (p.t_range && tid == 0) atomicMin(p.t_range, global_ns());
-    const uint32_t epoch = p.flags ? __ldcg(p.epoch) : 0u;      // the number of this overlapped call
 
     const uint32_t ipt = (K + nt - 1) / nt;              // ids per thread
     const uint32_t i0 = warp * ipt * 32u + lane;         // position of the thread's k-th id: i0 + 32 k, below i1
@@ -148,6 +145,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
         life_words<SPT, true>(g_life + j0, own, w);
         load_token(0);
         if (p.verified_len_dev) N = __ldg(p.verified_len_dev + ti);
+        const uint32_t seen = bt == blockIdx.x ? take_flags_down(p, bt, gridDim.x, p.n_launch) : 0u;
         if (tid == 0) s_sum[0] = 0;
         __syncthreads();                                 // the index is empty
 
@@ -261,6 +259,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
                 if (lane == 0 && valid) atomicAdd(s_sum, valid);
             }
             if (lane == 0) s_tot[par + warp] = wmiss;
+            if (g == 0 && bt == blockIdx.x) start_dependents(seen);
             __syncthreads();
 
             // ---- CollectDead and the misses, each in order; the prefix over the warps: lane l looks at warp l ----
@@ -357,7 +356,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
             list_off += n_take;
             sum_decay += d;
             __syncthreads();
-            announce_token(p, ti, table, g, n_take, bt, epoch);
+            announce_token(p, ti, g, n_take);
         }
 
         // ---- write back: lifetimes; resident ids that are no longer verified become empty (Alg. 4) ----
@@ -491,10 +490,9 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_paper_kernel(const __g
     const uint32_t ipt = (K + nt - 1) / nt, i0 = tid * ipt;
 
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (p.t_range && threadIdx.x == 0) atomicMin(p.t_range, global_ns());
-    const uint32_t epoch = p.flags ? __ldcg(p.epoch) : 0u;
 
+    start_dependents(take_flags_down(p, blockIdx.x, gridDim.x, p.n_launch));
     // ---- load the table; global pre-decay ----
     if (own)
         for (uint32_t k = 0; k < spt; ++k) {
@@ -571,7 +569,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_paper_kernel(const __g
         }
         if (g + 1 < p.n_q) load_ids(p.indices + row + K, i0, ipt, K, xs);
         if (tid == 0 && p.miss_count) p.miss_count[(size_t)ti * p.n_q + g] = (int32_t)n_g;
-        if (n_g == 0) { __syncthreads(); publish_token(p, ti, table, g, 0, blockIdx.x, epoch); continue; }
+        if (n_g == 0) { __syncthreads(); publish_token(p, ti, g, 0); continue; }
         __syncthreads();
 
         // ---- CollectDead / decay until n_g slots are dead ----
@@ -653,7 +651,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_paper_kernel(const __g
         list_off += n_take;
         sum_decay += d;
         __syncthreads();
-        publish_token(p, ti, table, g, n_take, blockIdx.x, epoch);
+        publish_token(p, ti, g, n_take);
     }
 
     // ---- write back; speculative entries (id >= N) become empty ----

@@ -220,9 +220,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_cluster_kernel(const _
     };
 
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (p.t_range && tid == 0) atomicMin(p.t_range, global_ns());
-    const uint32_t epoch = p.flags ? __ldcg(p.epoch) : 0u;      // the number of this overlapped call
 
     // ---- issue every global load first: this block's part of the table state and of the first token's ids ----
     int4 t4[MAX_SPT / 4];
@@ -242,6 +240,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_cluster_kernel(const _
     life_load(g_life, j0, spt, own, lw0, lw1);
     int32_t xs[MAX_IPT];
     load_ids(p.indices + (size_t)ti * p.n_q * K + k_base, i0, ipt, Kl, xs);
+    const uint32_t seen = take_flags_down(p, bt, gridDim.x, rank == 0 ? p.n_launch : 0u);      // (a cluster serves one table)
 
     if (s_priv)
         for (uint32_t i = tid; i < ((uint32_t)(L + 2) * priv_stride + 15u) / 16u; i += nt)
@@ -257,6 +256,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_cluster_kernel(const _
                 if (k < spt) s_tok[j0 + k] = t1[k];
         }
     }
+    start_dependents(seen);
     // global pre-decay of the iteration's first token (Alg. 1 Pass 1)
     life_store(s_life, j0, spt, own, decay4(lw0, 1), decay4(lw1, 1));
     uint32_t fill_bound = 0;                              // hash index: occupied buckets (upper bound), cluster-wide
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_cluster_kernel(const _
         sum_miss += n_g;
         if (rank == 0 && tid == 0 && p.miss_count) p.miss_count[(size_t)ti * p.n_q + g] = (int32_t)n_g;
         if (n_g == 0) {                                   // the same decision in every block of the cluster
-            if (rank == 0) publish_token(p, ti, table, g, 0, bt, epoch);
+            if (rank == 0) publish_token(p, ti, g, 0);
             continue;
         }
 
@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_cluster_kernel(const _
         } else if constexpr (!DIRECT) {
             fill_bound = build();
         }
-        if (rank == 0) publish_token(p, ti, table, g, n_take, bt, epoch);
+        if (rank == 0) publish_token(p, ti, g, n_take);
     }
 
     // ---- write this block's slots back; speculative entries (id >= N) become empty (Alg. 4) ----

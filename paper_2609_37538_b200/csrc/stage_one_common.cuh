@@ -156,35 +156,43 @@ __device__ __forceinline__ void count_lifetimes(uint32_t w0, uint32_t w1, uint32
     }
 }
 
-// Overlapped Stage Two only (p.flags set): tells the transfer kernel, which is already resident, that token g of
-// this table is placed - `count` more entries of the table's miss list are final.  Called by every thread of the
-// block after a barrier behind the list writes; one thread then fences (the barrier makes the fence cover the whole
-// block's earlier writes, as in a grid-wide barrier) and writes the table's flag of token g: the call's number
-// (read once when the kernel starts) in the upper half, the count in the lower.
+// Takes down the hand-over flags of the block's tables, once the previous call of the context has completed
+// (griddepcontrol.wait); `tables` of this launch, every `step`-th from `from` on.  The next kernel of the stream may start
+// when every block has called start_dependents() with what this returned: so no flag of an earlier call is ever seen, and
+// nothing has to be counted or zeroed behind a call.  Atomic exchanges, because their results say that they are done: a
+// store and a fence in their place held up the block's first warp, and so its first barrier, by 0.5 us.
 template <typename P>
-__device__ __forceinline__ void announce_token(const P& p, uint32_t ti, uint32_t table, uint32_t g, uint32_t count,
-                                               uint32_t bt,      // bt: the table's index within this launch
-                                               uint32_t epoch)
+__device__ __forceinline__ uint32_t take_flags_down(const P& p, uint32_t from, uint32_t step, uint32_t tables)
+{
+    uint32_t seen = 0;
+    if (p.flags && threadIdx.x < 32u) {                  // lane: (table, token); at most eight tokens
+        const uint32_t at_once = 32u / p.n_q, i = threadIdx.x / p.n_q, g = threadIdx.x % p.n_q;
+        if (i < at_once)
+            for (uint32_t bt = from + i * step; bt < tables; bt += at_once * step)
+                seen |= atomicExch(p.flags + (size_t)(p.first + bt) * p.n_q + g, 0u);
+    }
+    return seen;
+}
+
+__device__ __forceinline__ void start_dependents(uint32_t seen)
+{
+    if (threadIdx.x < 32u && __all_sync(0xffffffffu, seen != 0xFFFFFFFFu) && threadIdx.x == 0)     // (no flag has that value)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Tells the overlapped transfer kernel, which is already resident (p.flags set), that token g of this table is placed:
+// `count` more entries of the table's miss list are final.  Called by every thread of the block after a barrier behind the list writes; one thread then fences (the
+// barrier makes the fence cover the whole block's earlier writes, as in a grid-wide barrier) and raises the table's flag.
+template <typename P>
+__device__ __forceinline__ void announce_token(const P& p, uint32_t ti, uint32_t g, uint32_t count)
 {
     const bool announce = p.done_seq && g + 1 == p.n_q;
     if ((!p.flags && !announce) || threadIdx.x != 0) return;
-    if (p.flags && g == 0) {
-        SegDesc sd;
-        sd.src_base = p.kv_base[bt];
-        sd.src_stride = p.kv_stride[bt];
-        sd.dst_base = reinterpret_cast<uint64_t>(p.buffer + (size_t)table * p.S * p.row_bytes);
-        sd.count = 0;
-        sd.pad = 0;
-        p.seg[ti] = sd;
-    }
     __threadfence();
-    if (p.flags)
-        *reinterpret_cast<volatile unsigned long long*>(p.flags + (size_t)ti * p.n_q + g) =
-            ((unsigned long long)epoch << 32) | count;
-    // calls that asked for it (host buffers in the overlapped mode, or a caller's own signal word): the table
-    // that arrives last after the call's last token announces that every table of the call has written its
-    // slot table, hit mask and miss counts.  The arrivals are counted in a word of their own that wraps to
-    // zero by itself (atomicInc), whatever state the transfer kernel leaves the per-token counters in.
+    if (p.flags) *reinterpret_cast<volatile uint32_t*>(p.flags + (size_t)ti * p.n_q + g) = 1u + count;
+    // calls that asked for it (host buffers in the overlapped mode, or a caller's own signal word): the table that arrives last after the
+    // call's last token announces that every table of the call has written its slot table, hit mask and miss counts.
+    // The arrivals are counted in a word of their own that wraps to zero by itself (atomicInc).
     if (announce && atomicInc(p.done_ctr, p.expect - 1u) == p.expect - 1u) {
         __threadfence();
         *reinterpret_cast<volatile unsigned long long*>(p.done_seq) = p.host_seq;
@@ -193,12 +201,11 @@ __device__ __forceinline__ void announce_token(const P& p, uint32_t ti, uint32_t
 
 // The same with the barrier in front.
 template <typename P>
-__device__ __forceinline__ void publish_token(const P& p, uint32_t ti, uint32_t table, uint32_t g, uint32_t count,
-                                              uint32_t bt, uint32_t epoch)
+__device__ __forceinline__ void publish_token(const P& p, uint32_t ti, uint32_t g, uint32_t count)
 {
     if (!p.flags && !(p.done_seq && g + 1 == p.n_q)) return;
     __syncthreads();
-    announce_token(p, ti, table, g, count, bt, epoch);
+    announce_token(p, ti, g, count);
 }
 
 }  // namespace avsg

@@ -141,96 +141,115 @@ __global__ void __launch_bounds__(1024, 1) avsg_transfer_kernel(const __grid_con
     }
 }
 
-// Stage Two that overlaps Stage One (the latency-hiding direction of App. G).  The grid is launched with
-// programmatic stream serialization and does NOT wait for Stage One to complete: its blocks become resident
-// once every Stage One block has started, then wait - with a bound - until all tables of a round have
-// placed token g (Stage One writes a flag per table and token, carrying the number of the call and the
-// token's miss count, after making that token's miss-list entries visible; every thread polls one table's
-// flag), cut that token's misses evenly over the blocks (Eq. 6 per round and token) and copy them while
-// Stage One places the next token or the next round of tables.  A call is one round unless it has so many
-// tables that Stage One, with a block per table, would take most of the SMs: then Stage One runs with
-// round_size blocks that serve the tables round by round, and this grid follows them.  Every Stage One block
-// is resident before this grid starts and never waits for it, so it always makes progress; if a wait still
-// runs out the block sets ST_WAIT_TIMEOUT and stops copying.  Before leaving, every block waits for the
-// completion of the Stage One grid, so that the completion of this grid implies it; the last block to leave
-// then advances the call number, so that no flag of this call can be taken for one of the next - nothing has
-// to be zeroed between calls, and the kernel arguments hold nothing that changes from call to call (a
-// captured call can be replayed).  All reads of data written by the running Stage One go to L2 (ld.cg /
-// acquire).
-__global__ void __launch_bounds__(1024, 1) avsg_transfer_overlap_kernel(const __grid_constant__ XferOverlapParams p)
-{
-    __shared__ uint32_t s_pref[OVERLAP_MAX_TABLES + 1];
-    __shared__ uint32_t s_off[OVERLAP_MAX_TABLES];
-    __shared__ uint64_t s_src[OVERLAP_MAX_TABLES], s_stride[OVERLAP_MAX_TABLES], s_dst[OVERLAP_MAX_TABLES];
-    __shared__ uint32_t s_w[40];
+// Stage Two that overlaps Stage One (the latency-hiding direction of App. G).  The grid is launched with programmatic
+// stream serialization and does NOT wait for Stage One to complete: its blocks become resident once every Stage One
+// block has started, and copy each token's misses as soon as Stage One has placed that token of all tables.  Stage One
+// raises a flag per table and token, carrying the miss count, after making those miss-list entries visible; it has taken
+// all flags down before this grid could start.
+//
+// A call is walked in phases, one per token.  The last warp of a block polls the phase's flags - with a bound -,
+// prefix-sums the counts over the tables and raises s_ready; the other warps copy (Eq. 6 per phase: the misses are cut
+// evenly over the blocks, and a block's over its warps).  In a small call no barrier ties the warps together and phases
+// go round over the blocks and warps: a row is a round trip of 2 us, and a warp without one in this phase is already at
+// work on the next (one request, 230 rows in two tokens: 17.3 us a call where the block met after every phase and found
+// its last block with a counter, 15.8 now).  With more rows per block than warps the copying warps do meet: rows of a
+// later phase that mix with this one's cost 1 % where the link is the limit (128 tables in one call: 392 us against
+// 394), and 5 % where translations on the way to 11 GB of host memory are.
+//
+// A call is one round unless it has so many tables that Stage One, with a block per table, would take most of the SMs:
+// then Stage One runs with round_size blocks that serve the tables round by round, and this grid follows them.  Every
+// Stage One block is resident before this grid starts and never waits for it, so it always makes progress; if a wait
+// still runs out the block sets ST_WAIT_TIMEOUT and stops copying.  Before leaving, every block waits for the
+// completion of the Stage One grid, so that the completion of this grid implies it.  The kernel arguments hold nothing
+// that changes from call to call (a captured call can be replayed).  All reads of data written by the running Stage One go to L2 (ld.cg / acquire).
+constexpr uint32_t GAVE_UP = 0xFFFFFFFFu;
+constexpr uint32_t READY_SPIN_LIMIT = 1u << 24;              // far above the polling warp's own limit
 
-    const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u;
-    const uint32_t n = p.n, rounds = (n + p.round_size - 1u) / p.round_size;
+template <int CAP>
+__global__ void __launch_bounds__(1024, 1) avsg_transfer_overlap_kernel(const __grid_constant__ XferOverlapParamsT<CAP> p)
+{
+    extern __shared__ uint32_t s_phase[];        // per phase: prefix sums [round_size + 1], first list entries [round_size]
+    __shared__ volatile uint32_t s_ready;        // phases whose prefix sums are there
+    __shared__ uint32_t s_copied;
+
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, W = (blockDim.x >> 5) - 1u;   // W warps copy
+    const uint32_t n = p.n, rounds = (n + p.round_size - 1u) / p.round_size, phases = rounds * p.n_q;
+    const uint32_t stride = 2u * p.round_size + 1u;
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (p.t_range && tid == 0) atomicMin(p.t_range, global_ns());
-    // the number of this call: the previous overlapped call's grid advanced it before this call's Stage One,
-    // which this grid was launched behind, could start
-    uint32_t epoch;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(epoch) : "l"(p.epoch) : "memory");
-    for (uint32_t i = tid; i < n; i += nt) s_off[i] = 0;
+    if (tid == 0) { s_ready = 0; s_copied = 0; }
     __syncthreads();
 
-    const uint32_t cpr = p.row_bytes >> 4;
-    bool first_row = p.t_range != nullptr, copied = false, gave_up = false;
-    for (uint32_t r = 0; r < rounds && !gave_up; ++r) {
-        const uint32_t base = r * p.round_size;                        // tables [base, base + nr) of the call
-        const uint32_t nr = n - base < p.round_size ? n - base : p.round_size;
-        for (uint32_t g = 0; g < p.n_q; ++g) {
-            // every thread waits for the flag of one table of the round (of several, if the block is small)
-            int ok = 1;
-            for (uint32_t i = tid; i < nr; i += nt) {
-                const unsigned long long* f = p.flags + (size_t)(base + i) * p.n_q + g;
-                unsigned long long v = 0;
-                uint32_t spin = 0;
-                for (; spin < OVERLAP_SPIN_LIMIT; ++spin) {
-                    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(f) : "memory");
-                    if ((uint32_t)(v >> 32) == epoch + p.expect_extra) break;
-                    __nanosleep(64);
-                }
-                if (spin == OVERLAP_SPIN_LIMIT) { ok = 0; atomicOr(p.status, ST_WAIT_TIMEOUT); break; }
-                s_pref[i] = (uint32_t)v;                               // the table's miss count of this token
-            }
-            if (!__syncthreads_and(ok)) { gave_up = true; break; }     // same decision in every thread
-            if (g == 0)                                                // a table's bases are published with its token 0
-                for (uint32_t i = base + tid; i < base + nr; i += nt) {
-                    s_src[i] = __ldcg(&p.seg[i].src_base);
-                    s_stride[i] = __ldcg(&p.seg[i].src_stride);
-                    s_dst[i] = __ldcg(&p.seg[i].dst_base);
-                }
-
-            // prefix sum of token g's miss counts over the tables of the round (the counts came with the flags)
+    if (warp == W) {
+        for (uint32_t ph = 0, base = 0, g = 0; ph < phases; ++ph) {
+            const uint32_t nr = n - base < p.round_size ? n - base : p.round_size;       // tables [base, base + nr)
+            uint32_t* pref = s_phase + ph * stride;
+            uint32_t* off = pref + p.round_size + 1u;
             uint32_t running = 0;
-            for (uint32_t b0 = 0; b0 < nr; b0 += nt) {
-                const uint32_t i = b0 + tid;
-                const uint32_t c = i < nr ? s_pref[i] : 0u;
-                uint32_t total;
-                const uint32_t excl = block_excl_scan(c, s_w, total);
-                if (i < nr) s_pref[i] = running + excl;
-                running += total;
-                __syncthreads();
+            bool ok = true;
+            for (uint32_t i = lane; i - lane < nr && ok; i += 32u) {
+                uint32_t c = 0, spin = 0;
+                if (i < nr) {
+                    const uint32_t* f = p.flags + (size_t)(base + i) * p.n_q + g;
+                    for (; spin < OVERLAP_SPIN_LIMIT; ++spin) {
+                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(f) : "memory");
+                        if (c) break;
+                        __nanosleep(64);
+                    }
+                    c -= c ? 1u : 0u;                                   // the table's misses of this phase
+                }
+                ok = __all_sync(0xffffffffu, spin < OVERLAP_SPIN_LIMIT);
+                const uint32_t incl = warp_incl_scan(c, lane);
+                if (i < nr) {
+                    pref[i] = running + incl - c;
+                    off[i] = g == 0 ? 0u : off[(int)i - (int)stride] + pref[(int)i + 1 - (int)stride] - pref[(int)i - (int)stride];
+                }
+                running += __shfl_sync(0xffffffffu, incl, 31);
             }
-            if (tid == 0) s_pref[nr] = running;
-            __syncthreads();
-
-            const uint32_t C = gridDim.x, cb = blockIdx.x, q = running / C, rem = running % C;
-            const uint32_t m0 = cb * q + (cb < rem ? cb : rem);
-            const uint32_t m1 = m0 + q + (cb < rem ? 1u : 0u);
-            if (first_row && tid == 0 && m1 > m0) atomicMin(p.t_range + 2, global_ns());
-            copied = copied || m1 > m0;
-            for (uint32_t m = m0 + (tid >> 5); m < m1; m += nt >> 5) {
-                uint32_t lo = 0, hi = nr;                              // largest lo with s_pref[lo] <= m
+            if (!ok) {
+                if (lane == 0) { atomicOr(p.status, ST_WAIT_TIMEOUT); s_ready = GAVE_UP; }
+                break;
+            }
+            if (lane == 0) pref[nr] = running;
+            __threadfence_block();
+            __syncwarp();
+            if (lane == 0) s_ready = ph + 1u;
+            if (++g == p.n_q) { g = 0; base += p.round_size; }
+        }
+    } else {
+        const uint32_t C = gridDim.x, cpr = p.row_bytes >> 4;
+        bool first_row = p.t_range != nullptr;
+        uint32_t block_from = 0, warp_from = 0;                        // where the next phase's shares start
+        for (uint32_t ph = 0, base = 0, g = 0; ph < phases; ++ph) {
+            const uint32_t nr = n - base < p.round_size ? n - base : p.round_size;
+            const uint32_t* pref = s_phase + ph * stride;
+            const uint32_t* off = pref + p.round_size + 1u;
+            uint32_t ready = s_ready;
+            for (uint32_t spin = 0; ready <= ph && spin < READY_SPIN_LIMIT; ++spin) {
+                __nanosleep(32);
+                ready = s_ready;
+            }
+            ready = __shfl_sync(0xffffffffu, ready, 0);                // one decision for the warp
+            if (ready <= ph || ready == GAVE_UP) {
+                if (ready != GAVE_UP && lane == 0) atomicOr(p.status, ST_WAIT_TIMEOUT);
+                break;
+            }
+            __threadfence_block();
+            const uint32_t total = pref[nr], q = total / C, rem = total % C;
+            const uint32_t cb = blockIdx.x >= block_from ? blockIdx.x - block_from : blockIdx.x + C - block_from;
+            const uint32_t m0 = cb * q + (cb < rem ? cb : rem), count = q + (cb < rem ? 1u : 0u);
+            block_from = q > 0 ? 0u : block_from + rem < C ? block_from + rem : block_from + rem - C;
+            if (first_row && lane == 0 && count) { atomicMin(p.t_range + 2, global_ns()); s_copied = 1; }
+            for (uint32_t k = warp >= warp_from ? warp - warp_from : warp + W - warp_from; k < count; k += W) {
+                const uint32_t m = m0 + k;
+                uint32_t lo = 0, hi = nr;                              // largest lo with pref[lo] <= m
                 while (hi - lo > 1) {
                     const uint32_t mid = (lo + hi) >> 1;
-                    if (s_pref[mid] <= m) lo = mid; else hi = mid;
+                    if (pref[mid] <= m) lo = mid; else hi = mid;
                 }
                 const uint32_t t = base + lo;                          // the table, within the call
-                const uint32_t local = s_off[t] + (m - s_pref[lo]);    // entry of the table's miss list
+                const uint32_t local = off[lo] + (m - pref[lo]);       // entry of the table's miss list
                 if (local >= p.list_stride) {
                     if (lane == 0) atomicOr(p.status, ST_BAD_SEGMENT);
                     continue;
@@ -241,35 +260,30 @@ __global__ void __launch_bounds__(1024, 1) avsg_transfer_overlap_kernel(const __
                     if (lane == 0) atomicOr(p.status, ST_BAD_SLOT);
                     continue;
                 }
-                const uint64_t src = s_src[t] + (uint64_t)(uint32_t)e.x * s_stride[t];
-                const uint64_t dst = s_dst[t] + (uint64_t)(uint32_t)e.y * p.row_bytes;
+                const uint64_t src = p.kv_base[t] + (uint64_t)(uint32_t)e.x * p.kv_stride[t];
+                const uint64_t dst = reinterpret_cast<uint64_t>(p.buffer) +
+                                     ((uint64_t)p.table_id[t] * p.S + (uint32_t)e.y) * p.row_bytes;
                 copy_row(src, dst, cpr, lane);
                 if (first_row) {
-                    if (tid == 0) atomicMin(p.t_range + 3, global_ns());
+                    if (lane == 0) atomicMin(p.t_range + 3, global_ns());
                     first_row = false;
                 }
             }
-            __syncthreads();
-            for (uint32_t i = tid; i < nr; i += nt) s_off[base + i] += s_pref[i + 1] - s_pref[i];
-            __syncthreads();
+            if (q < W) {
+                warp_from = (warp_from + count) % W;
+            } else {
+                warp_from = 0;
+                asm volatile("bar.sync 1, %0;" :: "r"(W * 32u) : "memory");        // (q is the same in all of them)
+            }
+            if (++g == p.n_q) { g = 0; base += p.round_size; }
         }
     }
-    unsigned long long t_copied = 0;
-    if (p.t_range) {
-        __syncthreads();
-        t_copied = global_ns();
-    }
+    __syncthreads();
+    const unsigned long long t_copied = p.t_range ? global_ns() : 0ull;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (p.t_range && tid == 0) {
-        atomicMax(p.t_range + 1, global_ns());                     // the block's end, the wait for Stage One included
-        if (copied) atomicMin(p.t_range + 4, t_copied);
-    }
-    // Stage One is complete (the wait above), so no flag of this call will be written any more: the last block to
-    // arrive here advances the call number (0 is never used: the flags start out as zero)
-    __syncthreads();
-    if (tid == 0 && atomicInc(p.done, gridDim.x - 1u) == gridDim.x - 1u) {
-        const uint32_t next = epoch + 1u ? epoch + 1u : 1u;
-        asm volatile("st.release.gpu.global.u32 [%0], %1;" :: "l"(p.epoch), "r"(next) : "memory");
+        atomicMax(p.t_range + 1, global_ns());                         // the block's end, the wait for Stage One included
+        if (s_copied) atomicMin(p.t_range + 4, t_copied);
     }
 }
 
@@ -306,19 +320,33 @@ cudaError_t launch_transfer_positions(const PosParams& p, uint32_t blocks, uint3
     return cudaGetLastError();
 }
 
-cudaError_t launch_transfer_overlap(const XferOverlapParams& p, uint32_t blocks, uint32_t threads, cudaStream_t stream)
+namespace {
+template <int CAP>
+cudaError_t launch_transfer_overlap_t(const XferOverlapParamsT<CAP>& p, uint32_t blocks, uint32_t threads, cudaStream_t stream)
 {
+    const uint32_t phases = (p.n + p.round_size - 1) / p.round_size * p.n_q;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = 0;
+    cfg.blockDim = dim3(threads + 32 < 1024 ? threads + 32 : 1024);        // the copying warps and the one that polls
+    cfg.dynamicSmemBytes = phases * (2 * p.round_size + 1) * sizeof(uint32_t);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, avsg_transfer_overlap_kernel, p);
+    return cudaLaunchKernelEx(&cfg, avsg_transfer_overlap_kernel<CAP>, p);
+}
+}  // namespace
+
+cudaError_t launch_transfer_overlap(const XferOverlapParams& p, uint32_t blocks, uint32_t threads, cudaStream_t stream)
+{
+    return launch_transfer_overlap_t(p, blocks, threads, stream);
+}
+
+cudaError_t launch_transfer_overlap(const XferOverlapParamsBig& p, uint32_t blocks, uint32_t threads, cudaStream_t stream)
+{
+    return launch_transfer_overlap_t(p, blocks, threads, stream);
 }
 
 cudaError_t launch_transfer(const XferParams& p, uint32_t blocks, uint32_t threads, cudaStream_t stream)
@@ -339,12 +367,20 @@ cudaError_t launch_transfer(const XferParams& p, uint32_t blocks, uint32_t threa
 // Loads this file's kernels (see stage_one_prepare() on why that is not left to their first launch).
 cudaError_t transfer_prepare()
 {
-    const void* kernels[] = {reinterpret_cast<const void*>(avsg_transfer_kernel),
-                             reinterpret_cast<const void*>(avsg_transfer_overlap_kernel),
+    const void* kernels[] = {reinterpret_cast<const void*>(avsg_transfer_overlap_kernel<S1_MAX_TABLES>),
+                             reinterpret_cast<const void*>(avsg_transfer_overlap_kernel<S1_BIG_TABLES>),
+                             reinterpret_cast<const void*>(avsg_transfer_kernel),
                              reinterpret_cast<const void*>(avsg_transfer_positions_kernel)};
     for (const void* k : kernels) {
         cudaFuncAttributes fa;
         cudaError_t e = cudaFuncGetAttributes(&fa, k);
+        if (e != cudaSuccess) return e;
+    }
+    // a call in 32 rounds of 32 tables and eight tokens has 256 phases
+    for (int k = 0; k < 2; ++k) {
+        cudaError_t e = cudaFuncSetAttribute(kernels[k], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(OVERLAP_MAX_TABLES / S1_ROUND_BLOCKS * OVERLAP_MAX_TOKENS *
+                                                   (2 * S1_ROUND_BLOCKS + 1) * sizeof(uint32_t)));
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
