@@ -265,8 +265,10 @@ int avsg_reset_async(avsg_ctx *ctx, const uint32_t *table_ids, uint32_t n, void 
 int avsg_step(avsg_ctx *ctx, const avsg_step_args *args, void *cuda_stream);
 
 /* Same operation (Algorithm 4), but indices / slots / hit / miss_count are HOST pointers (pinned for
- * asynchrony); the library stages them through its own device buffers on the
- * stream: one upload of the ids, one download per requested output. */
+ * asynchrony), and the ids are in place when the call is made.  Pinned buffers are read and
+ * written by the kernels themselves (one block per table, AVSG_XFER_SM_BALANCED or _OVERLAP);
+ * otherwise the library stages them through its own device buffers: one upload of the ids, one
+ * download per requested output. */
 int avsg_step_host(avsg_ctx *ctx, const avsg_step_args *args, void *cuda_stream);
 
 /* Sec. 3.1: the S-slot device buffer that sparse attention reads through the

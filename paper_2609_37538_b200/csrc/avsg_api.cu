@@ -201,6 +201,15 @@ void overlap_params(avsg_ctx* c, X& x, uint32_t n, uint32_t n_q, uint32_t round_
     x.round_size = round_size; x.t_range = nullptr;
 }
 
+// Device-visible address of a caller's host buffer (page-locked and mapped), or null.
+template <typename T>
+T* mapped(T* p)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    return at.type == cudaMemoryTypeHost ? static_cast<T*>(at.devicePointer) : nullptr;
+}
+
 int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool host_io)
 {
     int rc = check_args(c, a);
@@ -217,6 +226,27 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     int32_t* slots = a->slots;
     uint8_t* hit = a->hit;
     int32_t* miss_count = a->miss_count;
+    // Host buffers.  Page-locked ones are used by the kernels themselves: Stage One reads the ids in place and Stage Two
+    // writes the outputs back, so that the calls of a stream follow one another as launches do, without an event between
+    // them (measured with 32 tables: see put_outputs()).  Pageable ones, the cluster and paper-literal kernels and the
+    // comparators go through copies on a side stream.
+    HostOut out;
+    bool host_ids = false;
+    if (host_io && c->s1_cluster == 1 && c->cfg.index_mode != AVSG_INDEX_PAPER &&
+        (c->cfg.transfer_mode == AVSG_XFER_SM_BALANCED || c->cfg.transfer_mode == AVSG_XFER_SM_OVERLAP)) {
+        const int32_t* ids = mapped(a->indices);
+        out.host_slots = mapped(a->slots);
+        out.host_hit = a->hit ? mapped(a->hit) : nullptr;
+        out.host_count = a->miss_count ? mapped(a->miss_count) : nullptr;
+        if (ids && out.host_slots && !a->hit == !out.host_hit && !a->miss_count == !out.host_count) {
+            host_ids = true;
+            host_io = false;
+            indices = ids;
+            out.slots = slots = c->d_slots_stage; out.n_slots = (uint32_t)n_ids;
+            out.hit = hit = a->hit ? c->d_hit_stage : nullptr; out.n_hit = a->hit ? (uint32_t)n_ids : 0u;
+            out.count = miss_count = a->miss_count ? c->d_mc_stage : nullptr; out.n_count = a->miss_count ? n * n_q : 0u;
+        }
+    }
     if (host_io) {
         // The ids go up on the side stream, where they queue behind the previous call's output download (and
         // therefore behind its Stage One, the last reader of the staging buffer) but not behind its Stage Two:
@@ -279,6 +309,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
         p.tok = c->d_tok; p.life = c->d_life; p.buffer = c->d_buffer; p.stats = c->d_stats;
         p.miss_list = c->d_list; p.seg = c->d_seg; p.status = c->d_status;
         p.indices = indices; p.slots = slots; p.hit = hit; p.miss_count = miss_count;
+        p.host_ids = host_ids;
         p.S = c->cfg.buffer_slots; p.logH = c->logH; p.row_bytes = c->cfg.row_bytes;
         p.K = K; p.n_q = n_q; p.L = (uint32_t)c->cfg.max_lifetime;
         p.first = first; p.list_stride = c->list_stride;
@@ -370,6 +401,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     } else if (overlap) {
         auto launch = [&](auto& x) -> cudaError_t {
             overlap_params(c, x, n, n_q, round_size);
+            x.out = out;
             x.t_range = c->timing ? c->d_trange + 2 : nullptr;
             for (uint32_t i = 0; i < n; ++i) {
                 x.table_id[i] = a->table_ids[i];
@@ -402,6 +434,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
         x.seg = c->d_seg; x.miss_list = c->d_list; x.status = c->d_status;
         x.n_seg = n; x.list_stride = c->list_stride; x.row_bytes = c->cfg.row_bytes;
         x.request_level = mode == AVSG_XFER_REQUEST_LEVEL; x.S = c->cfg.buffer_slots;
+        x.out = out;
         x.t_range = c->timing ? c->d_trange + 2 : nullptr;
         const uint32_t blocks = x.request_level ? n : (c->xfer_blocks ? c->xfer_blocks : (uint32_t)c->sm_count);
         if (launch_transfer(x, blocks, c->xfer_threads, stream) != cudaSuccess) {

@@ -106,6 +106,7 @@ struct S1ParamsT {
     uint32_t*           done_ctr = nullptr;     // arrivals after the call's last token; wraps to zero at `expect`
     unsigned long long  host_seq = 0;
     uint32_t            expect = 0;             // tables of the call
+    uint32_t            host_ids = 0;           // indices is mapped host memory that holds the ids when the call is made
     const int32_t* verified_len_dev = nullptr;  // [n] of the call: read instead of verified_len[] when set
     uint32_t table_id[CAP];
     int32_t  verified_len[CAP];
@@ -117,11 +118,20 @@ using S1Params = S1ParamsT<S1_MAX_TABLES>;
 using S1ParamsBig = S1ParamsT<S1_BIG_TABLES>;
 static_assert(sizeof(S1ParamsBig) <= 32764, "kernel argument block too large");
 
+// Calls with host buffers: Stage Two writes the call's outputs from the library's device buffers (256-byte aligned) into
+// the caller's mapped host memory, which the GPU's side of the link that the gather leaves free carries.
+struct HostOut {
+    const int32_t* slots = nullptr;  int32_t* host_slots = nullptr;  uint32_t n_slots = 0;
+    const uint8_t* hit = nullptr;    uint8_t* host_hit = nullptr;    uint32_t n_hit = 0;           // none: 0
+    const int32_t* count = nullptr;  int32_t* host_count = nullptr;  uint32_t n_count = 0;
+};
+
 struct XferParams {
     const SegDesc* seg;
     const int2*    miss_list;
     uint32_t*      status;
     uint32_t n_seg, list_stride, row_bytes, request_level, S;
+    HostOut out;
     // timing on: [0] earliest block start, [1] latest block end, [2] earliest start of a block's copy loop,
     // [3] earliest arrival of a block's first row, [4] earliest end of a block that copied something (ns)
     unsigned long long* t_range = nullptr;
@@ -142,6 +152,7 @@ struct XferOverlapParamsT {
     uint8_t*       buffer;       // [num_tables][S * row_bytes]
     uint32_t n, n_q, list_stride, row_bytes, S;
     uint32_t round_size;         // tables per round (n: one round)
+    HostOut out;
     unsigned long long* t_range = nullptr;
     uint32_t table_id[CAP];
     uint64_t kv_base[CAP];

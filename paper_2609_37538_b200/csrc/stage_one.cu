@@ -104,20 +104,30 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
         if (atomicAnd(reinterpret_cast<uint32_t*>(s_bits) + owner / PER_WORD, ~bit) & bit)
             atomicSub(&s_ndead[par + owner / 32u], 1u);
     };
+    const uint32_t ipt = (K + nt - 1) / nt;              // ids per thread
+    const uint32_t i0 = warp * ipt * 32u + lane;         // position of the thread's k-th id: i0 + 32 k, below i1
+    const uint32_t i1 = (warp + 1u) * ipt * 32u < K ? (warp + 1u) * ipt * 32u : K;
+    int32_t xs[IPT];
+    auto load_token = [&](uint32_t ti, uint32_t g) {
+        const int32_t* ids = p.indices + ((size_t)ti * p.n_q + g) * K;
+#pragma unroll
+        for (int k = 0; k < IPT; ++k)
+            xs[k] = i0 + 32u * k < i1 ? (p.host_ids ? __ldcv(ids + i0 + 32u * k) : __ldcg(ids + i0 + 32u * k)) : -1;
+    };
     // the first table's arguments and the clearing come before the wait: under the previous kernel's tail
     uint32_t bt = blockIdx.x, table = p.table_id[bt], id_limit = p.id_limit[bt];
     int32_t N = p.verified_len[bt];
     clear_index();
     if (tid == 0) s_node[NIL] = make_uint2(0xFFFFFFFEu, NIL);          // an id that nobody looks for
+    // Ids in host memory are there when the call is made, and nothing on the device writes them: a call that queues
+    // behind another fetches its first ones while that one's rows travel (32 tables: 5 us of link time and a round trip).
+    if (p.host_ids) load_token(p.first + bt, 0);
 
     // Programmatic dependent launch: this grid may have been started while the previous kernel of the stream
-    // was still running; nothing is read before that kernel has completed.
+    // was still running; nothing that the device writes is read before that kernel has completed.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (p.t_range && tid == 0) atomicMin(p.t_range, global_ns());
 
-    const uint32_t ipt = (K + nt - 1) / nt;              // ids per thread
-    const uint32_t i0 = warp * ipt * 32u + lane;         // position of the thread's k-th id: i0 + 32 k, below i1
-    const uint32_t i1 = (warp + 1u) * ipt * 32u < K ? (warp + 1u) * ipt * 32u : K;
     const uint32_t j0 = tid * SPT;                       // first of the thread's slots
     const bool own = j0 < S;
 
@@ -129,21 +139,15 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
         const uint32_t ti = p.first + bt;                // table index within the call
         int32_t* g_tok = p.tok + (size_t)table * S;
         int8_t*  g_life = p.life + (size_t)table * S;
-        const int32_t* ids = p.indices + (size_t)ti * p.n_q * K;
 
         // ---- every global load is issued first: cached ids, lifetimes, the first token's ids ----
         int4 t4[NV];
         uint32_t w[NV];
-        int32_t xs[IPT];
-        auto load_token = [&](uint32_t g) {
-#pragma unroll
-            for (int k = 0; k < IPT; ++k) xs[k] = i0 + 32u * k < i1 ? __ldcg(ids + (size_t)g * K + i0 + 32u * k) : -1;
-        };
 #pragma unroll
         for (int q = 0; q < NV; ++q)
             if (tid + q * nt < S / 4) t4[q] = __ldcg(reinterpret_cast<const int4*>(g_tok) + tid + q * nt);
         life_words<SPT, true>(g_life + j0, own, w);
-        load_token(0);
+        if (!p.host_ids || bt != blockIdx.x) load_token(ti, 0);
         if (p.verified_len_dev) N = __ldg(p.verified_len_dev + ti);
         const uint32_t seen = bt == blockIdx.x ? take_flags_down(p, bt, gridDim.x, p.n_launch) : 0u;
         if (tid == 0) s_sum[0] = 0;
@@ -279,7 +283,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
                     }
                 }
             }
-            if (!last) load_token(g + 1);                              // arrives while this token's misses are placed
+            if (!last) load_token(ti, g + 1);                              // arrives while this token's misses are placed
 
             // Pass 3, the while-loop of Alg. 1: decay until n_g slots are dead
             if (dtotal < n_g) {

@@ -65,6 +65,29 @@ __device__ __forceinline__ void copy_row(uint64_t src, uint64_t dst, uint32_t cp
     }
 }
 
+// The share of worker w of W (32 threads each) of the call's outputs, to host memory: 16 bytes a lane where the caller's
+// pointer allows it.  The stores are posted: nothing waits for them but the end of the grid.  One 32-table call (0.5 MB of
+// slots, 131 KB of flags) with ids read and outputs written by the kernels: 130.4 us where the calls queue, 145 alone;
+// with copies and events on a side stream 147.4 and 154.  (Stage One writing them to the host itself: 165, its hand-over
+// fences wait for the link.)
+__device__ __forceinline__ void put_out(const uint8_t* src, uint8_t* dst, uint32_t bytes, uint32_t w, uint32_t W, uint32_t lane)
+{
+    const uint32_t wide = (reinterpret_cast<uint64_t>(dst) & 15u) == 0 ? bytes / 16u : 0u;
+    for (uint32_t i = w * 32u + lane; i < wide; i += W * 32u)
+        reinterpret_cast<int4*>(dst)[i] = __ldcg(reinterpret_cast<const int4*>(src) + i);
+    const uint32_t words = (reinterpret_cast<uint64_t>(dst) & 3u) == 0 ? bytes / 4u : 0u;
+    for (uint32_t i = wide * 4u + w * 32u + lane; i < words; i += W * 32u)
+        reinterpret_cast<int32_t*>(dst)[i] = __ldcg(reinterpret_cast<const int32_t*>(src) + i);
+    for (uint32_t i = (words ? words * 4u : wide * 16u) + w * 32u + lane; i < bytes; i += W * 32u) dst[i] = __ldcg(src + i);
+}
+__device__ __forceinline__ void put_outputs(const HostOut& o, uint32_t w, uint32_t W, uint32_t lane)
+{
+    put_out(reinterpret_cast<const uint8_t*>(o.slots), reinterpret_cast<uint8_t*>(o.host_slots), o.n_slots * 4u, w, W, lane);
+    if (o.n_hit) put_out(o.hit, o.host_hit, o.n_hit, w, W, lane);
+    if (o.n_count)
+        put_out(reinterpret_cast<const uint8_t*>(o.count), reinterpret_cast<uint8_t*>(o.host_count), o.n_count * 4u, w, W, lane);
+}
+
 __global__ void __launch_bounds__(1024, 1) avsg_transfer_kernel(const __grid_constant__ XferParams p)
 {
     __shared__ uint32_t s_pref[XFER_MAX_SEG + 1];
@@ -78,6 +101,8 @@ __global__ void __launch_bounds__(1024, 1) avsg_transfer_kernel(const __grid_con
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (p.t_range && tid == 0) atomicMin(p.t_range, global_ns());
+
+    if (p.out.n_slots) put_outputs(p.out, blockIdx.x * (nt >> 5) + (tid >> 5), gridDim.x * (nt >> 5), lane);
 
     // global miss prefix sum (every block computes the same one)
     uint32_t running = 0;
@@ -236,6 +261,8 @@ __global__ void __launch_bounds__(1024, 1) avsg_transfer_overlap_kernel(const __
                 break;
             }
             __threadfence_block();
+            if (p.out.n_slots && ph + 1u == phases)                    // the call's last token is placed: outputs are final
+                put_outputs(p.out, blockIdx.x * W + warp, C * W, lane);
             const uint32_t total = pref[nr], q = total / C, rem = total % C;
             const uint32_t cb = blockIdx.x >= block_from ? blockIdx.x - block_from : blockIdx.x + C - block_from;
             const uint32_t m0 = cb * q + (cb < rem ? cb : rem), count = q + (cb < rem ? 1u : 0u);
