@@ -1,27 +1,23 @@
-// Stage One of the AVSG operator across a thread-block cluster: one table per cluster of C blocks (C = 1, 2, 4, 8).
+// Stage One of the AVSG operator across a thread-block cluster: one table per cluster of C blocks (C = 2, 4, 8), for
+// tables that one SM's shared memory does not hold (S up to 32768 slots).
 //
 // Same results as the single-block kernel (Algorithm 1 with the lifetime operations of Algorithm 3, the tokens of an
-// iteration in order as in Algorithm 4, the end-of-step invalidation), for tables that do not fit one SM's shared
-// memory (S up to 32768 slots) and with a shorter critical path for the ones that do.
+// iteration in order as in Algorithm 4, the end-of-step invalidation), and the same index, bits and passes; see there.
 //
-// Block r of the cluster owns the slots [r S/C, (r+1) S/C) - their cached ids and lifetimes live in its shared
-// memory for the step - and looks up the positions [r Kc, (r+1) Kc), Kc = ceil(K/C), of every token.  What a block
-// needs from another one goes through distributed shared memory with plain ld / st / atom.shared::cluster (no
-// multicast, no TMA):
-//   * Match: the slot an index entry points at may belong to another block: its cached id is read, and on a hit its
-//     lifetime is set to L, in that block's shared memory.  With the hash index (2S buckets, block r holds buckets
-//     [r 2S/C, (r+1) 2S/C)) the probes read remote buckets the same way.
-//   * Order-preserving compaction of the misses and of the dead slots (Eq. 12): a block prefix sum, then every block
-//     sends its total to all blocks and a cluster barrier turns the totals into cluster-wide offsets.  Position
-//     order is block order, then thread order, so "the k-th miss in position order" and "the k-th dead slot in slot
-//     order" are well defined across blocks.
-//   * Closed-form decay (the while-loop of Algorithm 1): when the dead slots do not cover the misses, every block
-//     sends its lifetime histogram to all blocks; all compute the same d.
-//   * Install: the OWNER of the k-th dead slot fetches the k-th miss (id and position) from the block that
-//     compacted it and writes the id, the lifetime L, the slot-table entry, the transfer-list entry and the index.
-// Three cluster barriers per token (match -> dead-slot scan -> install -> next token), one or two more when a decay
-// is needed.  Every decision that changes the control flow (n_g = 0, decay or not, index rebuild) is taken on
-// exchanged, cluster-wide values, so all blocks of a cluster reach the same barriers.
+// What bounds it is again latency, and here above all what crosses blocks.  So block r of the cluster owns the slots
+// [r S/C, (r+1) S/C) with an index of its own over the ids in them, and looks up EVERY position of a token in it: no
+// lookup, hit or install touches another block's shared memory.  (Before, positions were split over the blocks and ids,
+// lifetimes and buckets of other blocks were read and written through distributed shared memory, with three cluster
+// barriers per token.)  What the blocks tell one another, once per token, goes by remote stores and additions that
+// nobody waits for, followed by ONE cluster barrier:
+//   * a bit per position that is a hit in the block (block 0 also sets those of padding): what no block has set is a
+//     miss, and every block sees the whole token's misses in position order;
+//   * the number of dead slots that the block's hits have revived.  The dead slots of every block are known to all at
+//     any time: a decay announces them anew, and how many of them a token takes follows from the same numbers.
+// So every block computes for itself how many slots have to be taken and which of the misses are its own: the k-th dead
+// slot in slot order (block order, then the block's) takes the k-th miss in position order, and the block that owns the
+// slot selects that miss from the bits and installs it.  A decay adds a barrier per four candidate values of d and one
+// for the new dead counts; an overlapped Stage Two one more per token, behind which block 0 announces it.
 #include "avsg_kernels.cuh"
 #include "stage_one_common.cuh"
 
@@ -29,6 +25,7 @@ namespace avsg {
 namespace {
 
 constexpr uint32_t MAX_CL = 8;          // largest cluster (the portable limit)
+constexpr uint32_t SMEM_LIMIT = 227u << 10;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t cluster_rank()
@@ -44,399 +41,380 @@ __device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank)
 {
     uint32_t r; asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank)); return r;
 }
-__device__ __forceinline__ int32_t ldc_s32(uint32_t a)
-{
-    int32_t v; asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(a) : "memory"); return v;
-}
-__device__ __forceinline__ uint32_t ldc_u16(uint32_t a)
-{
-    uint16_t v; asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory"); return v;
-}
 __device__ __forceinline__ void stc_u32(uint32_t a, uint32_t v)
 {
     asm volatile("st.shared::cluster.u32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
 }
-__device__ __forceinline__ void stc_u16(uint32_t a, uint32_t v)
+__device__ __forceinline__ void addc_u32(uint32_t a, uint32_t v)
 {
-    asm volatile("st.shared::cluster.u16 [%0], %1;" :: "r"(a), "h"((uint16_t)v) : "memory");
-}
-__device__ __forceinline__ void stc_u8(uint32_t a, uint32_t v)
-{
-    asm volatile("st.shared::cluster.u8 [%0], %1;" :: "r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ int32_t casc_s32(uint32_t a, int32_t cmp, int32_t val)
-{
-    int32_t old;
-    asm volatile("atom.shared::cluster.cas.b32 %0, [%1], %2, %3;" : "=r"(old) : "r"(a), "r"(cmp), "r"(val) : "memory");
-    return old;
+    asm volatile("red.shared::cluster.add.u32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
 }
 // All threads of all blocks of the cluster; earlier (distributed) shared-memory and global writes of the cluster
 // are visible to every thread of the cluster afterwards.
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
 
-// Shared-memory layout of one block (the same in every block of the cluster, so that a location's address in
-// another block follows from the local one).
+// Shared-memory layout of one block (the same in every block of the cluster, so that a location's address in another
+// block follows from the local one).  Nodes come first; a call takes each of the block's slots once at most.
 struct Layout {
-    uint32_t tok, key, miss_x, val, miss_pos, life, hist, xhist, xch, scan_a, scan_b, fill, priv, total;
+    uint32_t heads, nil;                                        // numbers, not offsets: chains, the closing node
+    uint32_t head, life, bits, ndead, dead, pref, mask, rev, cnt, sum, total;
 };
-__host__ __device__ inline Layout make_layout(uint32_t S, uint32_t K, uint32_t L, uint32_t C, bool direct, uint32_t nt)
+__host__ __device__ inline uint32_t align16(uint32_t n) { return (n + 15u) & ~15u; }
+__host__ __device__ inline Layout make_layout(uint32_t S, uint32_t K, uint32_t n_q, uint32_t C, uint32_t nt)
 {
-    const uint32_t Sc = S / C, Hc = direct ? 0u : 2u * Sc, Kc = (K + C - 1) / C, Kcp = (Kc + 7u) & ~7u;
+    const uint32_t Sc = S / C, W = (K + 31u) / 32u, extra = (n_q - 1u) * K < Sc ? (n_q - 1u) * K : Sc;
     Layout o;
-    uint32_t a = 0;
-    o.tok = a;      a += Sc * 4;
-    o.key = a;      a += Hc * 4;
-    o.miss_x = a;   a += Kcp * 4;
-    o.val = a;      a += Hc * 2;
-    o.miss_pos = a; a += Kcp * 2;
-    o.life = a;     a += (Sc + 15u) & ~15u;
-    o.hist = a;     a += 128 * 4;
-    o.xhist = a;    a += MAX_CL * 128 * 4;          // lifetime histograms of all blocks
-    o.xch = a;      a += 4 * 2 * MAX_CL * 4;        // totals of all blocks: [kind][token parity][block]
-    o.scan_a = a;   a += 40 * 4;
-    o.scan_b = a;   a += 40 * 4;
-    o.fill = a;     a += 16;
-    o.priv = a;
-    if ((int32_t)L <= PRIV_HIST_MAX_L) a += ((L + 2u) * (nt + 4u) + 15u) & ~15u;
-    o.total = a;
-    return o;
+    o.heads = 2u * Sc;
+    o.nil = Sc + extra;
+    for (;;) {
+        uint32_t a = align16((o.nil + 1u) * 8u);
+        o.head = a;  a += o.heads * 4u;
+        o.life = a;  a += align16(Sc);
+        o.bits = a;  a += align16(nt);
+        o.ndead = a; a += 2u * 32u * 4u;                        // warps' dead slots, by parity
+        o.dead = a;  a += align16((K < Sc ? K : Sc) * 2u);      // the block's dead slots that are taken
+        o.pref = a;  a += align16(W * 2u);                      // misses before each word of the mask
+        o.mask = a;  a += align16(2u * C * W * 4u);             // received: positions that are no miss [parity][block][word]
+        o.rev = a;   a += 2u * MAX_CL * 4u;                     // received: revived slots [parity][block]
+        o.cnt = a;   a += 3u * (2u + MAX_CL) * 4u;              // received: counts of the decay search, dead slots, in turn
+        o.sum = a;   a += 16u;
+        o.total = a;
+        if (a <= SMEM_LIMIT || o.heads <= Sc) return o;
+        o.heads = Sc;                                           // (longer chains where the rest needs the room)
+    }
 }
 
-enum : uint32_t { XCH_MISS = 0, XCH_DEAD = 1, XCH_DEAD2 = 2, XCH_FILL = 3 };
+// Bits 0 .. 3: the sign bits of a word's four bytes.
+__device__ __forceinline__ uint32_t signs(uint32_t w) { return (((w >> 7) & 0x01010101u) * 0x10204080u) >> 28; }
 
-template <bool DIRECT, int CAP>
+constexpr int IPT = 2;                  // words of 32 positions that a warp looks up at a time
+
+// SPT: the block's slots per thread (a power of two); CAP: tables the argument block has room for.
+template <int SPT, int CAP>
 __global__ void __launch_bounds__(1024, 1) avsg_stage_one_cluster_kernel(const __grid_constant__ S1ParamsT<CAP> p)
 {
+    constexpr int NV = (SPT + 3) / 4;
     extern __shared__ __align__(16) unsigned char smem[];
-    const uint32_t S = p.S, K = p.K, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u;
-    const int32_t L = (int32_t)p.L;
     const uint32_t rank = cluster_rank(), C = cluster_size();
-    const uint32_t Sc = S / C, logSc = 31u - (uint32_t)__clz((int)Sc);
-    const uint32_t Hc = DIRECT ? 0u : 2u * Sc, logHc = logSc + 1u, H = 2u * S;
-    const uint32_t Kc = (K + C - 1) / C;
-    const uint32_t k_base = rank * Kc;                                       // first position this block looks up
-    const uint32_t Kl = k_base < K ? (K - k_base < Kc ? K - k_base : Kc) : 0u;   // how many
-    const uint32_t j_base = rank * Sc;                                       // first slot this block owns
+    const uint32_t S = p.S, K = p.K, L = p.L, Sc = S / C, W = (K + 31u) / 32u;
+    const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u, warp = tid >> 5, nw = nt >> 5;
+    const uint32_t below = (1u << lane) - 1u;
+    const uint32_t j_base = rank * Sc;                           // the block's first slot
 
-    const Layout lay = make_layout(S, K, p.L, C, DIRECT, nt);
-    int32_t*  s_tok      = reinterpret_cast<int32_t*>(smem + lay.tok);
-    int32_t*  s_key      = reinterpret_cast<int32_t*>(smem + lay.key);
-    int32_t*  s_miss_x   = reinterpret_cast<int32_t*>(smem + lay.miss_x);
-    uint16_t* s_val      = reinterpret_cast<uint16_t*>(smem + lay.val);
-    uint16_t* s_miss_pos = reinterpret_cast<uint16_t*>(smem + lay.miss_pos);
-    int8_t*   s_life     = reinterpret_cast<int8_t*>(smem + lay.life);
-    uint32_t* s_hist     = reinterpret_cast<uint32_t*>(smem + lay.hist);
-    uint32_t* s_xhist    = reinterpret_cast<uint32_t*>(smem + lay.xhist);
-    uint32_t* s_xch      = reinterpret_cast<uint32_t*>(smem + lay.xch);
-    uint32_t* s_scan_a   = reinterpret_cast<uint32_t*>(smem + lay.scan_a);
-    uint32_t* s_scan_b   = reinterpret_cast<uint32_t*>(smem + lay.scan_b);
-    uint32_t* s_fill     = reinterpret_cast<uint32_t*>(smem + lay.fill);
-    const uint32_t priv_stride = nt + 4u;
-    uint8_t*  s_priv     = L <= PRIV_HIST_MAX_L ? smem + lay.priv : nullptr;
-    const uint32_t a_tok = smem_u32(s_tok), a_key = smem_u32(s_key), a_val = smem_u32(s_val), a_life = smem_u32(s_life),
-                   a_mx = smem_u32(s_miss_x), a_mp = smem_u32(s_miss_pos), a_xch = smem_u32(s_xch),
-                   a_xhist = smem_u32(s_xhist);
+    const Layout lay = make_layout(S, K, p.n_q, C, nt);
+    const uint32_t NIL = lay.nil, logH = 31u - (uint32_t)__clz((int)lay.heads);
+    uint2*    s_node = reinterpret_cast<uint2*>(smem);
+    uint32_t* s_head = reinterpret_cast<uint32_t*>(smem + lay.head);
+    int8_t*   s_life = reinterpret_cast<int8_t*>(smem + lay.life);
+    uint8_t*  s_bits = smem + lay.bits;
+    uint32_t* s_ndead = reinterpret_cast<uint32_t*>(smem + lay.ndead);
+    uint16_t* s_dead = reinterpret_cast<uint16_t*>(smem + lay.dead);
+    uint16_t* s_pref = reinterpret_cast<uint16_t*>(smem + lay.pref);
+    uint32_t* s_mask = reinterpret_cast<uint32_t*>(smem + lay.mask);
+    uint32_t* s_rev  = reinterpret_cast<uint32_t*>(smem + lay.rev);
+    uint32_t* s_cnt  = reinterpret_cast<uint32_t*>(smem + lay.cnt);
+    uint32_t* s_sum  = reinterpret_cast<uint32_t*>(smem + lay.sum);
 
-    const uint32_t bt = blockIdx.x / C;                   // table of this cluster within the launch
-    const uint32_t ti = p.first + bt;                     // ... within the call
-    const uint32_t table = p.table_id[bt];
+    const uint32_t bt = blockIdx.x / C;                          // table of this cluster within the launch
+    const uint32_t ti = p.first + bt, table = p.table_id[bt], id_limit = p.id_limit[bt];
+    int32_t N = p.verified_len[bt];
     int32_t* g_tok = p.tok + (size_t)table * S + j_base;
     int8_t*  g_life = p.life + (size_t)table * S + j_base;
-
-    const uint32_t spt = Sc >= nt ? Sc / nt : 1u;         // slots per thread, power of two <= 8
-    const uint32_t j0 = tid * spt;                        // local slot number
+    const int32_t* ids = p.indices + (size_t)ti * p.n_q * K;
+    const uint32_t j0 = tid * SPT;                               // first of the thread's slots, counted in the block
     const bool own = j0 < Sc;
-    const uint32_t ipt = (Kc + nt - 1) / nt;              // ids per thread, <= 8
-    const uint32_t i0 = tid * ipt;                        // local position
-    uint16_t* where = DIRECT ? p.where + (size_t)table * p.max_context : nullptr;
-    const uint32_t id_limit = p.id_limit[bt];
 
-    // cached id / lifetime byte of slot j (any block's)
-    auto tok_of = [&](uint32_t j) { return ldc_s32(map_rank(a_tok + 4u * (j & (Sc - 1u)), j >> logSc)); };
-    auto refresh = [&](uint32_t j) { stc_u8(map_rank(a_life + (j & (Sc - 1u)), j >> logSc), (uint32_t)L); };
-    // sends v to slot [kind][parity][rank] of every block's exchange array
-    auto send_total = [&](uint32_t kind, uint32_t parity, uint32_t v) {
-        if (tid < C) stc_u32(map_rank(a_xch + 4u * ((kind * 2u + parity) * MAX_CL + rank), tid), v);
-    };
-    auto totals = [&](uint32_t kind, uint32_t parity, uint32_t& before, uint32_t& all) {
-        before = all = 0;
-        for (uint32_t q = 0; q < C; ++q) {
-            const uint32_t v = s_xch[(kind * 2u + parity) * MAX_CL + q];
-            if (q < rank) before += v;
-            all += v;
+    int32_t xs[IPT];
+    auto load_ids = [&](uint32_t g, uint32_t w0) {               // positions of the words w0 + warp IPT + k
+#pragma unroll
+        for (int k = 0; k < IPT; ++k) {
+            const uint32_t i = (w0 + warp * IPT + k) * 32u + lane;
+            xs[k] = i < K ? (p.host_ids ? __ldcv(ids + (size_t)g * K + i) : __ldcg(ids + (size_t)g * K + i)) : -1;
         }
+    };
+    auto revive = [&](uint32_t j, uint32_t par) -> bool {        // the slot is no longer dead; false: it was not
+        const uint32_t owner = j / SPT, bit = 1u << ((owner & 3u) * 8u + j % SPT);
+        if (!(atomicAnd(reinterpret_cast<uint32_t*>(s_bits) + owner / 4u, ~bit) & bit)) return false;
+        atomicSub(&s_ndead[par + owner / 32u], 1u);
+        return true;
     };
 
-    // hash index over the whole cluster: bucket b lives in block b / Hc
-    auto find = [&](int32_t x) -> int32_t {
-        uint32_t b = hash_id(x, logHc + (31u - (uint32_t)__clz((int)C)));
-        for (uint32_t it = 0; it < H; ++it) {
-            const uint32_t q = b >> logHc, l = b & (Hc - 1u);
-            const int32_t k = ldc_s32(map_rank(a_key + 4u * l, q));
-            if (k == x) {
-                const uint32_t j = ldc_u16(map_rank(a_val + 2u * l, q));
-                return tok_of(j) == x ? (int32_t)j : -1;      // a stale key: the id was reclaimed this step
-            }
-            if (k == EMPTY) return -1;
-            b = (b + 1u) & (H - 1u);
-        }
-        atomicOr(p.status, ST_PROBE_EXHAUSTED);
-        return -1;
-    };
-    auto insert = [&](int32_t x, uint32_t slot) {
-        uint32_t b = hash_id(x, logHc + (31u - (uint32_t)__clz((int)C)));
-        for (uint32_t it = 0; it < H; ++it) {
-            const uint32_t q = b >> logHc, l = b & (Hc - 1u);
-            const int32_t old = casc_s32(map_rank(a_key + 4u * l, q), EMPTY, x);
-            if (old == EMPTY || old == x) { stc_u16(map_rank(a_val + 2u * l, q), slot); return; }
-            b = (b + 1u) & (H - 1u);
-        }
-        atomicOr(p.status, ST_PROBE_EXHAUSTED);
-    };
-    // (re)builds the index from the cached ids; returns the cluster-wide number of occupied buckets
-    auto build = [&]() -> uint32_t {
-        if constexpr (!DIRECT)
-            for (uint32_t i = tid; i < Hc / 4; i += nt)
-                reinterpret_cast<int4*>(s_key)[i] = make_int4(EMPTY, EMPTY, EMPTY, EMPTY);
-        if (tid == 0) *s_fill = 0;
-        cluster_sync();                                   // every block's buckets are empty, every block's ids in place
-        uint32_t live = 0;
-        if (own)
-            for (uint32_t k = 0; k < spt; ++k) {
-                const int32_t x = s_tok[j0 + k];
-                if (x >= 0) { insert(x, j_base + j0 + k); ++live; }
-            }
-        live = __reduce_add_sync(0xffffffffu, live);
-        if (lane == 0 && live) atomicAdd(s_fill, live);
-        __syncthreads();
-        send_total(XCH_FILL, 0, *s_fill);
-        cluster_sync();
-        uint32_t before, all;
-        totals(XCH_FILL, 0, before, all);
-        return all;
-    };
+    for (uint32_t i = tid; i < lay.heads / 4; i += nt) reinterpret_cast<uint4*>(s_head)[i] = make_uint4(NIL, NIL, NIL, NIL);
+    if (tid == 0) { s_node[NIL] = make_uint2(0xFFFFFFFEu, NIL); s_sum[0] = 0; }      // an id that nobody looks for
+    if (tid < 2u * MAX_CL) s_rev[tid] = 0;
+    if (tid < 3u * (2u + MAX_CL)) s_cnt[tid] = 0;
+    cluster_arrive();                                            // what the other blocks write to is ready (waited for below)
+    if (p.host_ids) load_ids(0, 0);                              // (see the single-block kernel)
 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (p.t_range && tid == 0) atomicMin(p.t_range, global_ns());
 
-    // ---- issue every global load first: this block's part of the table state and of the first token's ids ----
-    int4 t4[MAX_SPT / 4];
-    int32_t t1[3];
-    uint32_t lw0, lw1;
-    if (own) {
-        if ((spt & 3u) == 0) {
+    // ---- every global load is issued first: the block's cached ids and lifetimes, the first token's ids ----
+    int4 t4[NV];
+    uint32_t w[NV];
 #pragma unroll
-            for (uint32_t q = 0; q < (uint32_t)MAX_SPT / 4; ++q)
-                if (q < spt / 4) t4[q] = __ldg(reinterpret_cast<const int4*>(g_tok + j0) + q);
-        } else {
-#pragma unroll
-            for (uint32_t k = 0; k < 3; ++k)
-                if (k < spt) t1[k] = __ldg(g_tok + j0 + k);
-        }
-    }
-    life_load(g_life, j0, spt, own, lw0, lw1);
-    int32_t xs[MAX_IPT];
-    load_ids(p.indices + (size_t)ti * p.n_q * K + k_base, i0, ipt, Kl, xs);
+    for (int q = 0; q < NV; ++q)
+        if (tid + q * nt < Sc / 4) t4[q] = __ldcg(reinterpret_cast<const int4*>(g_tok) + tid + q * nt);
+    life_words<SPT, true>(g_life + j0, own, w);
+    if (!p.host_ids) load_ids(0, 0);
+    if (p.verified_len_dev) N = __ldg(p.verified_len_dev + ti);
     const uint32_t seen = take_flags_down(p, bt, gridDim.x, rank == 0 ? p.n_launch : 0u);      // (a cluster serves one table)
+    cluster_wait();                                              // (the index is empty, too)
 
-    if (s_priv)
-        for (uint32_t i = tid; i < ((uint32_t)(L + 2) * priv_stride + 15u) / 16u; i += nt)
-            reinterpret_cast<int4*>(s_priv)[i] = make_int4(0, 0, 0, 0);
-    if (own) {
-        if ((spt & 3u) == 0) {
+    // ---- ids to shared memory and into the index; global pre-decay of the lifetimes (Alg. 1 Pass 1) ----
+    bool stale_ids = false;                                      // ids that are no longer verified
 #pragma unroll
-            for (uint32_t q = 0; q < (uint32_t)MAX_SPT / 4; ++q)
-                if (q < spt / 4) reinterpret_cast<int4*>(s_tok + j0)[q] = t4[q];
-        } else {
+    for (int q = 0; q < NV; ++q) {
+        if (tid + q * nt < Sc / 4) {
+            const uint32_t j = 4u * (tid + q * nt);
+            const int32_t x[4] = {t4[q].x, t4[q].y, t4[q].z, t4[q].w};
+            uint32_t next[4];
 #pragma unroll
-            for (uint32_t k = 0; k < 3; ++k)
-                if (k < spt) s_tok[j0 + k] = t1[k];
+            for (int c = 0; c < 4; ++c) {
+                next[c] = x[c] >= 0 ? atomicExch(&s_head[hash_id(x[c], logH)], j + c) : NIL;
+                stale_ids = stale_ids || x[c] >= N;
+            }
+#pragma unroll
+            for (int c = 0; c < 4; c += 2)
+                reinterpret_cast<uint4*>(s_node)[(j + c) / 2] = make_uint4((uint32_t)x[c], (j + c) << 16 | next[c],
+                                                                           (uint32_t)x[c + 1], (j + c + 1) << 16 | next[c + 1]);
         }
     }
-    start_dependents(seen);
-    // global pre-decay of the iteration's first token (Alg. 1 Pass 1)
-    life_store(s_life, j0, spt, own, decay4(lw0, 1), decay4(lw1, 1));
-    uint32_t fill_bound = 0;                              // hash index: occupied buckets (upper bound), cluster-wide
-    if constexpr (!DIRECT) fill_bound = build();          // (two cluster barriers inside)
-    else cluster_sync();                                  // every block's ids and lifetimes are in place
+    // the block's dead slots are added up in the s_cnt buffers of all blocks; buffers take turns so that one can be
+    // zeroed while the next is in use: `turn` counts their uses, with a cluster barrier behind each
+    uint32_t turn = 0;
+    auto cnt_of = [&](uint32_t t) { return (t % 3u) * (2u + MAX_CL); };
+    auto store_life = [&](uint32_t par) {                        // lifetimes, dead bits, dead slots of warp and block
+        uint32_t bits = 0;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) bits |= signs(w[q]) << (4 * q);
+        life_words_store<SPT>(s_life + j0, own, w);
+        s_bits[tid] = (uint8_t)bits;
+        const uint32_t n = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(bits));
+        if (lane == 0) s_ndead[par + warp] = n;
+        if (lane < C && n) addc_u32(map_rank(smem_u32(s_cnt + cnt_of(turn) + 2u + rank), lane), n);
+        if (tid < 2u + MAX_CL) s_cnt[cnt_of(turn + 1u) + tid] = 0;
+        ++turn;
+    };
+#pragma unroll
+    for (int q = 0; q < NV; ++q) w[q] = decay4(w[q], 1);
+    store_life(0);
+    __syncthreads();
 
-    uint32_t list_off = 0, sum_valid = 0, sum_miss = 0, sum_decay = 0;
+    uint32_t list_off = 0, sum_miss = 0, sum_decay = 0, valid = 0;
+    uint32_t dead_of = 0;                                        // lane q < C: dead slots of block q; set after the barrier
+    bool fresh = true;                                           // ... from s_cnt, the first time
     int2* list = p.miss_list + (size_t)ti * p.list_stride;
 
     for (uint32_t g = 0; g < p.n_q; ++g) {
-        const uint32_t par = g & 1u;
+        const bool last = g + 1 == p.n_q;
+        const uint32_t par = 32u * (g & 1u);
         const size_t row = ((size_t)ti * p.n_q + g) * K;
         int32_t* O = p.slots + row;
         uint8_t* Hm = p.hit ? p.hit + row : nullptr;
-        if (tid < 128) s_hist[tid] = 0;
+        uint32_t* mask = s_mask + (g & 1u) * C * W;
 
-        // ---- Probe, refresh hits to L, emit hit slots (Pass 1 + Pass 2) ----
-        uint32_t missmask = 0, nmiss = 0, nvalid = 0;
-        uint32_t cand[MAX_IPT];
-        check_ids(xs, i0, ipt, Kl, id_limit, p.status);
-        if (DIRECT) {
+        // ---- lookups of all positions in the block's own index; hits: lifetime <- L, slot and flag out ----
+        for (uint32_t w0 = 0; w0 < W; w0 += nw * IPT) {
+            if (w0) load_ids(g, w0);
+            uint32_t node[IPT], revived = 0;
+            int32_t slot[IPT], was[IPT];
+            bool bad = false;
 #pragma unroll
-            for (uint32_t k = 0; k < (uint32_t)MAX_IPT; ++k) {   // all loads are issued before any is used
-                cand[k] = 0xFFFFFFFFu;
-                if (k < ipt && i0 + k < Kl && xs[k] >= 0) cand[k] = __ldcg(where + xs[k]) & (S - 1u);
+            for (int k = 0; k < IPT; ++k) {
+                const bool ok = (uint32_t)xs[k] < id_limit;
+                bad = bad || (!ok && xs[k] >= 0);
+                xs[k] = ok ? xs[k] : -1;
+                valid += ok;
+                slot[k] = -1;
+                node[k] = NIL;
+                if (ok) node[k] = s_head[hash_id(xs[k], logH)];
             }
-        }
+            if (bad && rank == 0) atomicOr(p.status, ST_BAD_ID);       // not fetched: reported and taken as padding
+            uint32_t open = 1;
+            for (uint32_t it = 0; open && it <= NIL; ++it) {           // all chains of the warp side by side
+                uint2 v[IPT];
 #pragma unroll
-        for (uint32_t k = 0; k < (uint32_t)MAX_IPT; ++k) {
-            const uint32_t i = k_base + i0 + k;           // position within the token
-            if (k < ipt && i0 + k < Kl) {
-                const int32_t x = xs[k];
-                if (x >= 0) {
-                    ++nvalid;
-                    int32_t j;
-                    if (DIRECT) j = tok_of(cand[k]) == x ? (int32_t)cand[k] : -1;
-                    else j = find(x);
-                    if (j >= 0) {
-                        refresh((uint32_t)j);
-                        O[i] = j;
-                        if (Hm) Hm[i] = 1;
-                    } else {
-                        missmask |= 1u << k;
-                        ++nmiss;
-                    }
-                } else {
-                    O[i] = -1;
-                    if (Hm) Hm[i] = 0;
+                for (int k = 0; k < IPT; ++k) v[k] = s_node[node[k]];
+                open = 0;
+#pragma unroll
+                for (int k = 0; k < IPT; ++k) {
+                    const bool found = (int32_t)v[k].x == xs[k];
+                    slot[k] = found ? (int32_t)(v[k].y >> 16) : slot[k];
+                    node[k] = found ? NIL : v[k].y & 0xFFFFu;
+                    open |= node[k] ^ NIL;
                 }
+                open = __any_sync(0xffffffffu, open);
             }
-        }
-        // order-preserving compaction of the misses: t = x[not m]; block order, then thread order
-        uint32_t total;
-        uint32_t off = block_excl_scan(nmiss | (nvalid << 16), s_scan_a, total) & 0xFFFFu;
+            if (open) atomicOr(p.status, ST_PROBE_EXHAUSTED);
 #pragma unroll
-        for (uint32_t k = 0; k < (uint32_t)MAX_IPT; ++k) {
-            if (missmask & (1u << k)) {
-                s_miss_x[off] = xs[k];
-                s_miss_pos[off] = (uint16_t)(k_base + i0 + k);
-                ++off;
+            for (int k = 0; k < IPT; ++k) was[k] = slot[k] >= 0 ? s_life[slot[k]] : 0;
+#pragma unroll
+            for (int k = 0; k < IPT; ++k) {
+                const uint32_t wi = w0 + warp * IPT + k, i = wi * 32u + lane;
+                const bool hit = slot[k] >= 0, pad = xs[k] < 0 && rank == 0;
+                const uint32_t votes = __ballot_sync(0xffffffffu, hit || pad);
+                if (lane < C && wi < W) stc_u32(map_rank(smem_u32(mask + rank * W + wi), lane), votes);
+                if (hit) s_life[slot[k]] = (int8_t)L;
+                if ((hit || pad) && i < K) {
+                    O[i] = hit ? (int32_t)j_base + slot[k] : -1;
+                    if (Hm) Hm[i] = hit;
+                }
+                const bool back = hit && was[k] < 0 && revive((uint32_t)slot[k], par);
+                revived += __popc(__ballot_sync(0xffffffffu, back));
+            }
+            if (revived && lane < C) addc_u32(map_rank(smem_u32(s_rev + (g & 1u) * MAX_CL + rank), lane), revived);
+        }
+        if (last && rank == 0) {
+            valid = __reduce_add_sync(0xffffffffu, valid);
+            if (lane == 0 && valid) atomicAdd(s_sum, valid);
+        }
+        if (!last) load_ids(g + 1, 0);                                 // arrives while this token's misses are placed
+        if (g == 0) start_dependents(seen);
+        cluster_sync();
+
+        // ---- the token's misses, and the dead slots of the blocks ----
+        uint32_t n_g = 0;
+        for (uint32_t w0 = 0; w0 < W; w0 += 32u) {
+            const uint32_t wi = w0 + lane;
+            uint32_t m = 0xFFFFFFFFu;
+            if (wi < W) {
+                m = 0;
+                for (uint32_t q = 0; q < C; ++q) m |= mask[q * W + wi];
+            }
+            const uint32_t c = __popc(~m);
+            if (warp == 0) {                                           // (the other warps need the sum alone)
+                const uint32_t incl = warp_incl_scan(c, lane);
+                if (wi < W) s_pref[wi] = (uint16_t)(n_g + incl - c);
+                n_g += __shfl_sync(0xffffffffu, incl, 31);
+            } else {
+                n_g += __reduce_add_sync(0xffffffffu, c);
             }
         }
-        send_total(XCH_MISS, par, total);
-        // the next token's ids travel while this token's misses are placed
-        if (g + 1 < p.n_q) load_ids(p.indices + row + K + k_base, i0, ipt, Kl, xs);
-        cluster_sync();                                   // (1) hits refreshed everywhere, miss totals exchanged
-        uint32_t m_before_packed, m_all_packed;
-        totals(XCH_MISS, par, m_before_packed, m_all_packed);
-        const uint32_t n_g = m_all_packed & 0xFFFFu;
-        sum_valid += m_all_packed >> 16;
+        if (fresh) dead_of = lane < C ? s_cnt[cnt_of(turn - 1u) + 2u + lane] : 0u;
+        fresh = false;
+        if (lane < C) dead_of -= s_rev[(g & 1u) * MAX_CL + lane];
+        uint32_t dtotal = __reduce_add_sync(0xffffffffu, dead_of), d = 0;
         sum_miss += n_g;
         if (rank == 0 && tid == 0 && p.miss_count) p.miss_count[(size_t)ti * p.n_q + g] = (int32_t)n_g;
-        if (n_g == 0) {                                   // the same decision in every block of the cluster
-            if (rank == 0) publish_token(p, ti, g, 0);
-            continue;
-        }
 
-        // ---- Pass 3: CollectDead; if fewer than n_g slots are dead, decay until enough are ----
-        uint32_t w0, w1;
-        life_load(s_life, j0, spt, own, w0, w1);
-        uint32_t sg0 = w0 & 0x80808080u, sg1 = w1 & 0x80808080u;       // sign bits = dead slots
-        uint32_t dloc, d = 0;
-        uint32_t doff = block_excl_scan(__popc(sg0) + __popc(sg1), s_scan_b, dloc);
-        send_total(XCH_DEAD, par, dloc);
-        cluster_sync();                                   // (2) dead-slot totals exchanged
-        uint32_t d_before, dtotal;
-        totals(XCH_DEAD, par, d_before, dtotal);
-        if (dtotal < n_g) {                               // same decision everywhere
-            // the while-loop of Alg. 1 in closed form: d = fewest unit decays after which n_g slots are dead, read
-            // off the histogram of the lifetimes of the whole table (every block sends its own to all blocks)
-            count_lifetimes(w0, w1, spt, own, L, s_priv, priv_stride, s_hist);
-            __syncthreads();
-            for (uint32_t i = tid; i < C * ((uint32_t)L + 2u); i += nt) {
-                const uint32_t q = i / ((uint32_t)L + 2u), b = i % ((uint32_t)L + 2u);
-                stc_u32(map_rank(a_xhist + 4u * (rank * 128u + b), q), s_hist[b]);
-            }
-            cluster_sync();
-            uint32_t cum = 0;
-            bool found = false;
-            d = (uint32_t)L + 1u;
-            for (uint32_t b = 0; b <= (uint32_t)L + 1u; ++b) {   // bin b counts lifetime b-1; dead after b decays
-                for (uint32_t q = 0; q < C; ++q) cum += s_xhist[q * 128u + b];
-                if (cum >= n_g) { d = b; found = true; break; }
-            }
-            if (!found && rank == 0 && tid == 0) atomicOr(p.status, ST_NO_DEAD_SLOTS);
-            w0 = decay4(w0, d);
-            w1 = decay4(w1, d);
-            life_store(s_life, j0, spt, own, w0, w1);
-            sg0 = w0 & 0x80808080u; sg1 = w1 & 0x80808080u;
-            doff = block_excl_scan(__popc(sg0) + __popc(sg1), s_scan_b, dloc);
-            send_total(XCH_DEAD2, par, dloc);
-            cluster_sync();
-            totals(XCH_DEAD2, par, d_before, dtotal);
-        }
-
-        // ---- install: the owner of the k-th dead slot (slot order) takes the k-th miss (position order) ----
-        const bool rebuild = !DIRECT && fill_bound + n_g > (H / 4u) * 3u;
-        const uint32_t n_take = n_g < dtotal ? n_g : dtotal;
-        uint32_t kk = d_before + doff;                    // cluster-wide rank of this thread's first dead slot
+        // Pass 3, the while-loop of Alg. 1: decay until n_g slots are dead (every block takes the same decisions)
+        if (dtotal < n_g) {
+            life_words<SPT>(s_life + j0, own, w);
+            uint32_t lo = 0, hi = L + 1u;                // lo decays are too few, hi are enough
+            while (hi - lo > 1u) {
+                uint32_t c[4];                           // candidates in (lo, hi), ascending; small ones first
 #pragma unroll
-        for (uint32_t k = 0; k < (uint32_t)MAX_SPT; ++k) {
-            const uint32_t bit = k < 4 ? (sg0 >> (8 * k + 7)) & 1u : (sg1 >> (8 * (k - 4) + 7)) & 1u;
-            if (bit) {
-                if (kk < n_take) {
-                    // the block that compacted miss kk, and the miss's place in its list
-                    uint32_t q = 0, base = 0;
-                    for (; q + 1 < C; ++q) {
-                        const uint32_t c = s_xch[(XCH_MISS * 2u + par) * MAX_CL + q] & 0xFFFFu;
-                        if (kk < base + c) break;
-                        base += c;
-                    }
-                    const int32_t x = ldc_s32(map_rank(a_mx + 4u * (kk - base), q));
-                    const uint32_t i = ldc_u16(map_rank(a_mp + 2u * (kk - base), q));
-                    const uint32_t jl = j0 + k, j = j_base + jl;
-                    if (i < K) {
-                        s_tok[jl] = x;
-                        s_life[jl] = (int8_t)L;
-                        O[i] = (int32_t)j;
-                        if (Hm) Hm[i] = 0;
-                        list[list_off + kk] = make_int2(x, (int32_t)j);
-                        if (DIRECT) __stcg(where + x, (uint16_t)j);
-                        else if (!rebuild) insert(x, j);
-                    } else {
-                        list[list_off + kk] = make_int2(-1, -1);         // Stage Two skips it
-                        atomicOr(p.status, ST_BAD_SLOT);
-                    }
+                for (uint32_t i = 0; i < 4; ++i) {
+                    c[i] = lo == 0 ? 1u << i : lo + ((i + 1u) * (hi - lo)) / 5u;
+                    c[i] = c[i] <= lo ? lo + 1u : (c[i] >= hi ? hi - 1u : c[i]);
                 }
-                ++kk;
+                uint32_t n01 = 0, n23 = 0;
+#pragma unroll
+                for (int q = 0; q < NV; ++q) {
+                    n01 += __popc(__vsubss4(w[q], c[0] * 0x01010101u) & 0x80808080u) |
+                           (__popc(__vsubss4(w[q], c[1] * 0x01010101u) & 0x80808080u) << 16);
+                    n23 += __popc(__vsubss4(w[q], c[2] * 0x01010101u) & 0x80808080u) |
+                           (__popc(__vsubss4(w[q], c[3] * 0x01010101u) & 0x80808080u) << 16);
+                }
+                n01 = __reduce_add_sync(0xffffffffu, n01);
+                n23 = __reduce_add_sync(0xffffffffu, n23);
+                uint32_t* cnt = s_cnt + cnt_of(turn);
+                if (lane < C && n01) addc_u32(map_rank(smem_u32(cnt), lane), n01);           // (S <= 32768: 16 bits are enough)
+                if (lane < C && n23) addc_u32(map_rank(smem_u32(cnt + 1), lane), n23);
+                if (tid < 2u + MAX_CL) s_cnt[cnt_of(turn + 1u) + tid] = 0;
+                ++turn;
+                cluster_sync();
+                const uint32_t n[4] = {cnt[0] & 0xFFFFu, cnt[0] >> 16, cnt[1] & 0xFFFFu, cnt[1] >> 16};
+#pragma unroll
+                for (int i = 3; i >= 0; --i) if (n[i] >= n_g) hi = c[i];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) if (n[i] < n_g) lo = c[i];
             }
+            d = hi;
+#pragma unroll
+            for (int q = 0; q < NV; ++q) w[q] = decay4(w[q], d);
+            store_life(par);
+            cluster_sync();
+            dead_of = lane < C ? s_cnt[cnt_of(turn - 1u) + 2u + lane] : 0u;
+            dtotal = __reduce_add_sync(0xffffffffu, dead_of);
+            if (dtotal < n_g && rank == 0 && tid == 0) atomicOr(p.status, ST_NO_DEAD_SLOTS);
+        }
+        const uint32_t n_take = n_g < dtotal ? n_g : dtotal;
+        const uint32_t first = __reduce_add_sync(0xffffffffu, lane < rank ? dead_of : 0u);       // dead slots of the blocks before
+        {   // what the token takes of every block's dead slots
+            const uint32_t before = warp_incl_scan(dead_of, lane) - dead_of;
+            const uint32_t taken = before < n_take ? (n_take - before < dead_of ? n_take - before : dead_of) : 0u;
+            dead_of -= taken;
+        }
+        // the block's dead slots that are taken, in increasing order
+        const uint32_t t = lane < nw ? s_ndead[par + lane] : 0u;
+        const uint32_t dead_before = first + __reduce_add_sync(0xffffffffu, lane < warp ? t : 0u);
+        if (dead_before < n_take) {
+            uint32_t bits = s_bits[tid], r, unused;
+            warp_rank<SPT>(__popc(bits), below, r, unused);
+            for (r += dead_before; bits && r < n_take; bits &= bits - 1u, ++r) s_dead[r - first] = (uint16_t)(j0 + __ffs((int)bits) - 1);
+            s_bits[tid] = (uint8_t)bits;                 // what is handed out is dead no more
+        }
+        uint32_t left = __shfl_sync(0xffffffffu, t, (int)warp);        // the warp's dead slots for the next token
+        if (dead_before < n_take) left = left > n_take - dead_before ? left - (n_take - dead_before) : 0u;
+        if (lane == 0) s_ndead[32u - par + warp] = left;
+        __syncthreads();
+        if (tid < MAX_CL) s_rev[(g & 1u) * MAX_CL + tid] = 0;          // (read by all; added to again two tokens on)
+
+        // ---- install: the k-th miss in position order takes the k-th dead slot ----
+        const uint32_t own_total = __reduce_add_sync(0xffffffffu, t);
+        const uint32_t mine = first < n_take ? (n_take - first < own_total ? n_take - first : own_total) : 0u;
+        for (uint32_t k = tid; k < mine + (rank == 0 ? n_g - n_take : 0u); k += nt) {
+            const uint32_t r = k < mine ? first + k : n_take + (k - mine);
+            uint32_t lo = 0, hi = W;                                   // largest lo with s_pref[lo] <= r
+            while (hi - lo > 1u) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (s_pref[mid] <= r) lo = mid; else hi = mid;
+            }
+            uint32_t m = 0;
+            for (uint32_t q = 0; q < C; ++q) m |= mask[q * W + lo];
+            m = ~m;
+            for (uint32_t skip = r - s_pref[lo]; skip && m; --skip) m &= m - 1u;
+            const uint32_t i = lo * 32u + (uint32_t)__ffs((int)m) - 1u;
+            if (m == 0 || i >= K) { atomicOr(p.status, ST_BAD_SLOT); continue; }
+            int32_t j = -1;
+            if (k < mine) {
+                const int32_t x = p.host_ids ? __ldcv(ids + (size_t)g * K + i) : __ldcg(ids + (size_t)g * K + i);
+                const uint32_t jl = s_dead[k];
+                j = (int32_t)(j_base + jl);
+                s_node[jl].x = (uint32_t)x;
+                s_life[jl] = (int8_t)L;
+                list[list_off + r] = make_int2(x, j);
+                g_tok[jl] = x >= N ? -1 : x;                           // speculative ids are forgotten (end of Alg. 4)
+                if (!last) {                                           // a node of its own: the slot's is in the old id's chain
+                    const uint32_t n = atomicAdd(&s_sum[1], 1u) + Sc;
+                    if (n < NIL) s_node[n] = make_uint2((uint32_t)x, jl << 16 | atomicExch(&s_head[hash_id(x, logH)], n));
+                    else atomicOr(p.status, ST_PROBE_EXHAUSTED);
+                }
+            }
+            O[i] = j;
+            if (Hm) Hm[i] = 0;
         }
         list_off += n_take;
         sum_decay += d;
-        if (!rebuild) {
-            fill_bound += n_g;
-            cluster_sync();                               // (3) the new ids are visible to every block's next lookups
-        } else if constexpr (!DIRECT) {
-            fill_bound = build();
+        if (p.flags || (p.done_seq && last)) {
+            cluster_sync();                                            // every block has installed its misses
+            if (rank == 0) announce_token(p, ti, g, n_take);
+        } else {
+            __syncthreads();
         }
-        if (rank == 0) publish_token(p, ti, g, n_take);
     }
 
-    // ---- write this block's slots back; speculative entries (id >= N) become empty (Alg. 4) ----
-    const int32_t N = p.verified_len_dev ? __ldg(p.verified_len_dev + ti) : p.verified_len[bt];
-    if (own) {
-        if ((spt & 3u) == 0) {
-            for (uint32_t q = 0; q < spt / 4; ++q) {
-                int4 v = reinterpret_cast<const int4*>(s_tok + j0)[q];
-                v.x = v.x >= N ? -1 : v.x; v.y = v.y >= N ? -1 : v.y;
-                v.z = v.z >= N ? -1 : v.z; v.w = v.w >= N ? -1 : v.w;
-                reinterpret_cast<int4*>(g_tok + j0)[q] = v;
-            }
-        } else {
-            for (uint32_t k = 0; k < spt; ++k) {
-                const int32_t v = s_tok[j0 + k];
-                g_tok[j0 + k] = v >= N ? -1 : v;
-            }
-        }
-        uint32_t w0, w1;
-        life_load(s_life, j0, spt, own, w0, w1);
-        life_store(g_life, j0, spt, own, w0, w1);
+    // ---- write back: lifetimes; resident ids that are no longer verified become empty (Alg. 4) ----
+    life_words<SPT>(s_life + j0, own, w);
+    life_words_store<SPT>(g_life + j0, own, w);
+    if (stale_ids) {
+        for (uint32_t q = 0; q < NV; ++q)
+            for (uint32_t j = 4u * (tid + q * nt); j < 4u * (tid + q * nt) + 4u && j < Sc; ++j)
+                if ((int32_t)s_node[j].x >= N) g_tok[j] = -1;
     }
     if (rank == 0 && tid == 0) {
         SegDesc sd;
@@ -447,93 +425,89 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_cluster_kernel(const _
         sd.pad = 0;
         p.seg[ti] = sd;
         TableStats* st = p.stats + table;
-        st->steps += 1;
-        st->tokens += p.n_q;
-        st->hits += sum_valid - sum_miss;
-        st->misses += sum_miss;
-        st->rows += list_off;
-        st->extra_decays += sum_decay;
+        atomicAdd(&st->steps, 1ull);
+        atomicAdd(&st->tokens, (unsigned long long)p.n_q);
+        atomicAdd(&st->hits, (unsigned long long)(s_sum[0] - sum_miss));
+        atomicAdd(&st->misses, (unsigned long long)sum_miss);
+        atomicAdd(&st->rows, (unsigned long long)list_off);
+        atomicAdd(&st->extra_decays, (unsigned long long)sum_decay);
     }
     if (p.t_range) {
         __syncthreads();
         if (tid == 0) atomicMax(p.t_range + 1, global_ns());
     }
-    // no block leaves while another one may still read its shared memory
-    cluster_sync();
+    // (nothing is written to another block's shared memory behind the last token's barrier: a block may leave)
+}
+
+template <int CAP>
+const void* kernel_of(uint32_t Sc, uint32_t nt)
+{
+    switch (Sc / nt) {
+        case 8:  return reinterpret_cast<const void*>(avsg_stage_one_cluster_kernel<8, CAP>);
+        case 4:  return reinterpret_cast<const void*>(avsg_stage_one_cluster_kernel<4, CAP>);
+        default: return reinterpret_cast<const void*>(avsg_stage_one_cluster_kernel<2, CAP>);
+    }
 }
 
 }  // namespace
 
-uint32_t stage_one_cluster_threads(uint32_t S, uint32_t C)
+// Every block looks up all K ids of a token, so the threads follow from the block's slots and K as for a table of S / C.
+size_t stage_one_cluster_smem_bytes(uint32_t S, uint32_t K, uint32_t n_q, uint32_t C)
 {
-    uint32_t t = S / C / 4;
-    if (t < 128) t = 128;
-    if (t > 1024) t = 1024;
-    return t;
-}
-
-size_t stage_one_cluster_smem_bytes(uint32_t S, uint32_t K, uint32_t L, uint32_t C, bool direct)
-{
-    return make_layout(S, K, L, C, direct, stage_one_cluster_threads(S, C)).total;
+    return make_layout(S, K, n_q, C, stage_one_threads(S / C, K)).total;
 }
 
 cudaError_t stage_one_cluster_prepare(size_t max_smem)
 {
-    const void* kernels[] = {
-        reinterpret_cast<const void*>(avsg_stage_one_cluster_kernel<false, S1_MAX_TABLES>),
-        reinterpret_cast<const void*>(avsg_stage_one_cluster_kernel<true, S1_MAX_TABLES>),
-        reinterpret_cast<const void*>(avsg_stage_one_cluster_kernel<false, S1_BIG_TABLES>),
-        reinterpret_cast<const void*>(avsg_stage_one_cluster_kernel<true, S1_BIG_TABLES>)};
-    for (const void* k : kernels) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem);
-        if (e != cudaSuccess) return e;
-    }
+    for (uint32_t spt : {2u, 4u, 8u})
+        for (const void* k : {kernel_of<S1_MAX_TABLES>(spt, 1), kernel_of<S1_BIG_TABLES>(spt, 1)}) {
+            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem);
+            if (e != cudaSuccess) return e;
+        }
     return cudaSuccess;
 }
 
 namespace {
-template <int CAP>
-cudaError_t launch_cluster_t(const S1ParamsT<CAP>& p, uint32_t n_tables, uint32_t C, cudaStream_t stream)
+void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, uint32_t n_tables, uint32_t S, uint32_t K, uint32_t n_q,
+                    uint32_t C)
 {
-    cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_tables * C);
-    cfg.blockDim = dim3(stage_one_cluster_threads(p.S, C));
-    const bool direct = p.where != nullptr;
-    cfg.dynamicSmemBytes = stage_one_cluster_smem_bytes(p.S, p.K, p.L, C, direct);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = C;
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    return direct ? cudaLaunchKernelEx(&cfg, avsg_stage_one_cluster_kernel<true, CAP>, p)
-                  : cudaLaunchKernelEx(&cfg, avsg_stage_one_cluster_kernel<false, CAP>, p);
-}
-}  // namespace
-
-// How many clusters of this shape the device can hold at once (0: the shape cannot be launched at all).
-int stage_one_cluster_max_active(uint32_t S, uint32_t K, uint32_t L, uint32_t C, bool direct)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(stage_one_cluster_threads(S, C));
-    cfg.dynamicSmemBytes = stage_one_cluster_smem_bytes(S, K, L, C, direct);
-    cudaLaunchAttribute attr[1];
+    cfg.blockDim = dim3(stage_one_threads(S / C, K));
+    cfg.dynamicSmemBytes = stage_one_cluster_smem_bytes(S, K, n_q, C);
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = C;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+}
+
+template <int CAP>
+cudaError_t launch_cluster_t(const S1ParamsT<CAP>& p, uint32_t n_tables, uint32_t C, cudaStream_t stream)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    cluster_config(cfg, attr, n_tables, p.S, p.K, p.n_q, C);
+    cfg.stream = stream;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+    void* args[] = {const_cast<S1ParamsT<CAP>*>(&p)};
+    return cudaLaunchKernelExC(&cfg, kernel_of<CAP>(p.S / C, cfg.blockDim.x), args);
+}
+}  // namespace
+
+// How many clusters of this shape the device can hold at once (0: the shape cannot be launched at all).
+int stage_one_cluster_max_active(uint32_t S, uint32_t K, uint32_t n_q, uint32_t C)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    cluster_config(cfg, attr, 1, S, K, n_q, C);
     int n = 0;
-    const cudaError_t e = direct
-        ? cudaOccupancyMaxActiveClusters(&n, avsg_stage_one_cluster_kernel<true, S1_MAX_TABLES>, &cfg)
-        : cudaOccupancyMaxActiveClusters(&n, avsg_stage_one_cluster_kernel<false, S1_MAX_TABLES>, &cfg);
-    if (e != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaOccupancyMaxActiveClusters(&n, kernel_of<S1_MAX_TABLES>(S / C, cfg.blockDim.x), &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
     return n;
 }
 
