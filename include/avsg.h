@@ -92,10 +92,9 @@ extern "C" {
 
 /* How Stage One finds the slot that holds an id (same results either way). */
 #define AVSG_INDEX_HASH   0u  /* hash index in shared memory, rebuilt every step                */
-#define AVSG_INDEX_DIRECT 1u  /* needs every id < max_context.  Tables that a thread-block cluster
-                                 serves: one 16-bit entry per context position in device memory
-                                 (2 bytes x max_context per table, L2-resident); tables that fit
-                                 one block use the hash index, which is the quicker one there  */
+#define AVSG_INDEX_DIRECT 1u  /* the same with a bound on the ids: one >= max_context is taken as
+                                 padding and reported.  (It once had an entry per context position
+                                 in device memory; the index in shared memory is quicker)      */
 #define AVSG_INDEX_PAPER  2u  /* the paper's Hash-State table as printed (Eq. 2-4, Eq. 8-11,
                                  Alg. 2): packed 64-bit entries, double hashing with a retry
                                  budget, fingerprints, lazy reclamation.  LOSSY: a resident id
@@ -266,7 +265,7 @@ int avsg_step(avsg_ctx *ctx, const avsg_step_args *args, void *cuda_stream);
 
 /* Same operation (Algorithm 4), but indices / slots / hit / miss_count are HOST pointers (pinned for
  * asynchrony), and the ids are in place when the call is made.  Pinned buffers are read and
- * written by the kernels themselves (one block per table, AVSG_XFER_SM_BALANCED or _OVERLAP);
+ * written by the kernels themselves (AVSG_XFER_SM_BALANCED or _OVERLAP, not AVSG_INDEX_PAPER);
  * otherwise the library stages them through its own device buffers: one upload of the ids, one
  * download per requested output. */
 int avsg_step_host(avsg_ctx *ctx, const avsg_step_args *args, void *cuda_stream);

@@ -41,7 +41,6 @@ struct avsg_ctx {
     int2* d_list = nullptr;
     SegDesc* d_seg = nullptr;
     uint32_t* d_status = nullptr;
-    uint16_t* d_where = nullptr;       // direct index, or null
     uint32_t* d_q = nullptr;           // paper-literal mode: packed words, or null
     uint32_t* d_q_snap = nullptr;
     int32_t* d_tok_snap = nullptr;
@@ -96,7 +95,7 @@ void free_all(avsg_ctx* c)
     cudaFree(c->d_flags); cudaFree(c->d_sync);
     delete c->big_args;
     delete c->big_xfer_args;
-    cudaFree(c->d_list); cudaFree(c->d_seg); cudaFree(c->d_status); cudaFree(c->d_where); cudaFree(c->d_q); cudaFree(c->d_q_snap);
+    cudaFree(c->d_list); cudaFree(c->d_seg); cudaFree(c->d_status); cudaFree(c->d_q); cudaFree(c->d_q_snap);
     cudaFree(c->d_tok_snap); cudaFree(c->d_life_snap);
     cudaFree(c->d_idx_stage); cudaFree(c->d_slots_stage); cudaFree(c->d_hit_stage); cudaFree(c->d_mc_stage);
     if (c->h_seg) cudaFreeHost(c->h_seg);
@@ -228,11 +227,11 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     int32_t* miss_count = a->miss_count;
     // Host buffers.  Page-locked ones are used by the kernels themselves: Stage One reads the ids in place and Stage Two
     // writes the outputs back, so that the calls of a stream follow one another as launches do, without an event between
-    // them (measured with 32 tables: see put_outputs()).  Pageable ones, the cluster and paper-literal kernels and the
-    // comparators go through copies on a side stream.
+    // them (measured with 32 tables: see put_outputs()).  Pageable ones, the paper-literal kernel and the comparators
+    // go through copies on a side stream.
     HostOut out;
     bool host_ids = false;
-    if (host_io && c->s1_cluster == 1 && c->cfg.index_mode != AVSG_INDEX_PAPER &&
+    if (host_io && c->cfg.index_mode != AVSG_INDEX_PAPER &&
         (c->cfg.transfer_mode == AVSG_XFER_SM_BALANCED || c->cfg.transfer_mode == AVSG_XFER_SM_OVERLAP)) {
         const int32_t* ids = mapped(a->indices);
         out.host_slots = mapped(a->slots);
@@ -314,7 +313,6 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
         p.K = K; p.n_q = n_q; p.L = (uint32_t)c->cfg.max_lifetime;
         p.first = first; p.list_stride = c->list_stride;
         p.n_launch = cnt;
-        p.where = c->d_where; p.max_context = c->cfg.max_context;
         p.qword = c->d_q; p.probe_retries = c->cfg.probe_retries; p.hash_a1 = c->cfg.hash_a1; p.hash_a2 = c->cfg.hash_a2;
         p.t_range = c->timing ? c->d_trange : nullptr;
         p.verified_len_dev = a->verified_len_dev;
@@ -502,13 +500,12 @@ int avsg_create(const avsg_config* cfg, avsg_ctx** out)
     // Blocks per table in Stage One: what the configuration asks for, else the single-block kernel while the table
     // fits one SM's shared memory and the smallest cluster that holds it above that.
     {
-        const bool direct = cfg->index_mode == AVSG_INDEX_DIRECT;
         const uint32_t S = cfg->buffer_slots, K = cfg->max_topk, L = (uint32_t)cfg->max_lifetime;
         auto fits = [&](uint32_t C) -> bool {
             if (cfg->index_mode == AVSG_INDEX_PAPER)
                 return C == 1 && S <= 8192 && stage_one_paper_smem_bytes(S, K, L) <= (size_t)max_smem;
             if (C == 1) return S <= 8192 && stage_one_smem_bytes(S, K, cfg->max_tokens) <= (size_t)max_smem;
-            return S / C >= 32 && S / C <= 8192 && stage_one_cluster_smem_bytes(S, K, L, C, direct) <= (size_t)max_smem;
+            return S / C >= 32 && S / C <= 8192 && stage_one_cluster_smem_bytes(S, K, cfg->max_tokens, C) <= (size_t)max_smem;
         };
         uint32_t C = cfg->stage_one_cluster;
         if (C == 0)
@@ -524,8 +521,7 @@ int avsg_create(const avsg_config* cfg, avsg_ctx** out)
     }
     // a cluster shape that fits on paper may still find no home on the device (blocks of one cluster share a GPC)
     if (c->s1_cluster > 1 &&
-        stage_one_cluster_max_active(cfg->buffer_slots, cfg->max_topk, (uint32_t)cfg->max_lifetime, c->s1_cluster,
-                                     cfg->index_mode == AVSG_INDEX_DIRECT) < 1) {
+        stage_one_cluster_max_active(cfg->buffer_slots, cfg->max_topk, cfg->max_tokens, c->s1_cluster) < 1) {
         delete c; return AVSG_EUNSUPPORTED;
     }
 
@@ -548,8 +544,6 @@ int avsg_create(const avsg_config* cfg, avsg_ctx** out)
         ok = ok && cudaMalloc(&c->d_q, T * S * sizeof(uint32_t)) == cudaSuccess;
         ok = ok && cudaMalloc(&c->d_q_snap, T * S * sizeof(uint32_t)) == cudaSuccess;
     }
-    if (cfg->index_mode == AVSG_INDEX_DIRECT && c->s1_cluster > 1)     // (the single-block kernel builds its own index)
-        ok = ok && cudaMalloc(&c->d_where, T * (size_t)cfg->max_context * sizeof(uint16_t)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_tok_snap, T * S * sizeof(int32_t)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_life_snap, T * S) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_idx_stage, n_ids * sizeof(int32_t)) == cudaSuccess;
@@ -589,8 +583,7 @@ int avsg_create(const avsg_config* cfg, avsg_ctx** out)
             free_all(c); delete c; return AVSG_ECUDA;
         }
     }
-    if ((c->d_where && cudaMemset(c->d_where, 0xFF, T * (size_t)cfg->max_context * sizeof(uint16_t)) != cudaSuccess) ||
-        cudaMemset(c->d_status, 0, 256) != cudaSuccess || cudaMemset(c->d_seg, 0, T * sizeof(SegDesc)) != cudaSuccess ||
+    if (cudaMemset(c->d_status, 0, 256) != cudaSuccess || cudaMemset(c->d_seg, 0, T * sizeof(SegDesc)) != cudaSuccess ||
         init_tables(c, 0, (uint32_t)T) != AVSG_OK || cudaDeviceSynchronize() != cudaSuccess) {
         free_all(c); delete c; return AVSG_ECUDA;
     }
@@ -773,10 +766,6 @@ int avsg_import_state(avsg_ctx* c, uint32_t table_id, const int32_t* tok, const 
     CU(cudaDeviceSynchronize());
     CU(cudaMemcpy(c->d_tok + table_id * S, tok, S * sizeof(int32_t), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(c->d_life + table_id * S, life, S, cudaMemcpyHostToDevice));
-    if (c->d_where) {
-        CU(launch_direct_index_from_state(c->d_tok, c->d_where, table_id, 1, c->cfg.buffer_slots, c->cfg.max_context, nullptr));
-        CU(cudaDeviceSynchronize());
-    }
     if (c->d_q) {                                           // ids and lifetimes kept, every mapping invalid
         std::vector<uint32_t> q(S);
         for (size_t j = 0; j < S; ++j) q[j] = ((uint32_t)(uint8_t)life[j] << 24) | 0x00800000u;
@@ -838,9 +827,6 @@ int avsg_restore_state(avsg_ctx* c, void* stream)
     CU(cudaMemcpyAsync(c->d_tok, c->d_tok_snap, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
     CU(cudaMemcpyAsync(c->d_life, c->d_life_snap, n, cudaMemcpyDeviceToDevice, s));
     if (c->d_q) CU(cudaMemcpyAsync(c->d_q, c->d_q_snap, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
-    if (c->d_where)
-        CU(launch_direct_index_from_state(c->d_tok, c->d_where, 0, c->cfg.num_tables, c->cfg.buffer_slots,
-                                          c->cfg.max_context, s));
     return AVSG_OK;
 }
 

@@ -92,8 +92,6 @@ struct S1ParamsT {
     uint32_t first;              // index within the call of this launch's first table
     uint32_t n_launch;           // tables of this launch (the grid may have fewer blocks: a block then serves several)
     uint32_t list_stride;        // entries per segment of miss_list
-    uint32_t max_context;        // direct index: entries per table
-    uint16_t* where;             // direct index [num_tables][max_context], or null for the hash index
     uint32_t* qword;             // paper-literal mode: packed metadata words [num_tables][S], else null
     uint32_t probe_retries, hash_a1, hash_a2;   // paper-literal mode: R, a1, a2
     unsigned long long* t_range = nullptr;      // timing on: [0] earliest block start, [1] latest block end (ns)
@@ -203,14 +201,11 @@ cudaError_t stage_one_prepare(size_t max_smem);
 cudaError_t launch_stage_one(const S1Params& p, uint32_t n_blocks, cudaStream_t stream);
 cudaError_t launch_stage_one(const S1ParamsBig& p, uint32_t n_blocks, cudaStream_t stream);   // hash / direct index only
 // Stage One with one table per thread-block cluster of C blocks (C = 2, 4 or 8; hash / direct index only)
-uint32_t stage_one_cluster_threads(uint32_t S, uint32_t C);
-size_t stage_one_cluster_smem_bytes(uint32_t S, uint32_t K, uint32_t L, uint32_t C, bool direct);
+size_t stage_one_cluster_smem_bytes(uint32_t S, uint32_t K, uint32_t n_q, uint32_t C);
 cudaError_t stage_one_cluster_prepare(size_t max_smem);
-int stage_one_cluster_max_active(uint32_t S, uint32_t K, uint32_t L, uint32_t C, bool direct);   // after ..._prepare
+int stage_one_cluster_max_active(uint32_t S, uint32_t K, uint32_t n_q, uint32_t C);   // after ..._prepare
 cudaError_t launch_stage_one_cluster(const S1Params& p, uint32_t n_tables, uint32_t C, cudaStream_t stream);
 cudaError_t launch_stage_one_cluster(const S1ParamsBig& p, uint32_t n_tables, uint32_t C, cudaStream_t stream);
-cudaError_t launch_direct_index_from_state(const int32_t* tok, uint16_t* where, uint32_t first_table, uint32_t n_tables,
-                                           uint32_t S, uint32_t max_context, cudaStream_t stream);
 cudaError_t launch_all_k_prepare(const AllKParams& p, uint32_t n_tables, cudaStream_t stream);
 cudaError_t launch_transfer(const XferParams& p, uint32_t blocks, uint32_t threads, cudaStream_t stream);
 cudaError_t launch_transfer_overlap(const XferOverlapParams& p, uint32_t blocks, uint32_t threads, cudaStream_t stream);

@@ -399,24 +399,8 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
     }
 }
 
-// Direct index: points every resident id at its slot again, after the table state was replaced from outside
-// (import, restore of a snapshot).  One thread per slot; ids are unique within a table.
-__global__ void avsg_direct_index_from_state_kernel(const int32_t* __restrict__ tok, uint16_t* where,
-                                                    uint32_t first_table, uint32_t n_tables, uint32_t S,
-                                                    uint32_t max_context)
-{
-    const size_t n = (size_t)n_tables * S;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const uint32_t t = first_table + (uint32_t)(i / S), j = (uint32_t)(i % S);
-        const int32_t x = tok[(size_t)t * S + j];
-        if (x >= 0 && (uint32_t)x < max_context) where[(size_t)t * max_context + x] = (uint16_t)j;
-    }
-}
-
-
 // A request ended: its tables become empty (id -1) and dead (lifetime -1) again, their counters and rows zero;
-// in the paper-literal mode every bucket word returns to (lifetime -1, invalid, fingerprint 0, slot 0).  The
-// direct index needs no reset: its entries are verified against the cached ids.  Grid (blocks per table, tables).
+// in the paper-literal mode every bucket word returns to (lifetime -1, invalid, fingerprint 0, slot 0).  Grid (blocks per table, tables).
 __global__ void avsg_reset_tables_kernel(const __grid_constant__ ResetParams p)
 {
     const uint32_t table = p.table_id[blockIdx.y];
@@ -789,8 +773,7 @@ cudaError_t stage_one_prepare(size_t max_smem)
     // have to wait for every stream of the device - forever, if a stream is waiting for something that very launch
     // would produce (a caller who arms a wait for a call's stage_one_done word before its first call).
     const void* others[] = {reinterpret_cast<const void*>(avsg_all_k_prepare_kernel),
-                            reinterpret_cast<const void*>(avsg_reset_tables_kernel),
-                            reinterpret_cast<const void*>(avsg_direct_index_from_state_kernel)};
+                            reinterpret_cast<const void*>(avsg_reset_tables_kernel)};
     for (const void* k : others) {
         cudaFuncAttributes fa;
         cudaError_t e = cudaFuncGetAttributes(&fa, k);
@@ -844,15 +827,6 @@ cudaError_t launch_stage_one(const S1Params& p, uint32_t n_tables, cudaStream_t 
 cudaError_t launch_stage_one(const S1ParamsBig& p, uint32_t n_tables, cudaStream_t stream)
 {
     return launch_stage_one_t(p, n_tables, stream);
-}
-
-cudaError_t launch_direct_index_from_state(const int32_t* tok, uint16_t* where, uint32_t first_table, uint32_t n_tables,
-                                           uint32_t S, uint32_t max_context, cudaStream_t stream)
-{
-    const size_t n = (size_t)n_tables * S;
-    const uint32_t blocks = (uint32_t)((n + 255) / 256 < 1184 ? (n + 255) / 256 : 1184);
-    avsg_direct_index_from_state_kernel<<<blocks, 256, 0, stream>>>(tok, where, first_table, n_tables, S, max_context);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_reset_tables(const ResetParams& p, uint32_t n_tables, cudaStream_t stream)

@@ -13,35 +13,14 @@ __device__ __forceinline__ uint32_t hash_id(int32_t x, uint32_t logH)
     return ((uint32_t)x * 2654435769u) >> (32u - logH);
 }
 
-// The lifetimes of the slots a thread owns, packed one signed byte each into
-// two words; unused lanes carry 0x7F (never counted, never dead).
-__device__ __forceinline__ void life_load(const int8_t* base, uint32_t j0, uint32_t spt, bool own,
-                                          uint32_t& w0, uint32_t& w1)
-{
-    w0 = w1 = 0x7F7F7F7Fu;
-    if (!own) return;
-    if (spt == 8) { const uint2 v = *reinterpret_cast<const uint2*>(base + j0); w0 = v.x; w1 = v.y; }
-    else if (spt == 4) { w0 = *reinterpret_cast<const uint32_t*>(base + j0); }
-    else if (spt == 2) { w0 = 0x7F7F0000u | *reinterpret_cast<const uint16_t*>(base + j0); }
-    else { w0 = 0x7F7F7F00u | (uint8_t)base[j0]; }
-}
-
-__device__ __forceinline__ void life_store(int8_t* base, uint32_t j0, uint32_t spt, bool own, uint32_t w0, uint32_t w1)
-{
-    if (!own) return;
-    if (spt == 8) { *reinterpret_cast<uint2*>(base + j0) = make_uint2(w0, w1); }
-    else if (spt == 4) { *reinterpret_cast<uint32_t*>(base + j0) = w0; }
-    else if (spt == 2) { *reinterpret_cast<uint16_t*>(base + j0) = (uint16_t)w0; }
-    else { base[j0] = (int8_t)(w0 & 0xFFu); }
-}
-
 // life <- max(life - d, -1) on four packed signed bytes
 __device__ __forceinline__ uint32_t decay4(uint32_t w, uint32_t d)
 {
     return __vmaxs4(__vsubss4(w, d * 0x01010101u), 0xFFFFFFFFu);
 }
 
-// The same for SPT consecutive slots (2, 4 or 8), four to a word.  GLOBAL: from global memory, past L1.
+// The lifetimes of a thread's SPT consecutive slots (2, 4 or 8), packed one signed byte each, four to a word; unused
+// bytes carry 0x7F (never counted, never dead).  GLOBAL: from global memory, past L1.
 template <int SPT, bool GLOBAL = false>
 __device__ __forceinline__ void life_words(const int8_t* at, bool own, uint32_t (&w)[(SPT + 3) / 4])
 {

@@ -1,4 +1,4 @@
-"""Stage One with one block per table at the sizes where its split of slots and ids over threads changes, with ids that
+"""Stage One at the sizes where its split of slots and ids over threads changes, with ids that
 share one chain of its index, and with states only a caller's own table can have; compared with the oracle after every
 call (whole numbers: nothing to tolerate)."""
 import numpy as np
@@ -8,7 +8,7 @@ import avsg_traces as tr
 from oracle import OracleTable
 
 pytestmark = pytest.mark.gpu
-RB, CTX = 32, 40000
+RB, CTX = 32, 60000
 
 
 def _same_bucket_ids(S, n, bucket):
@@ -24,19 +24,33 @@ def _same_bucket_ids(S, n, bucket):
                                      (1024, 257, 3), (2048, 2048, 1), (4096, 1024, 4), (4096, 1025, 3), (8192, 1, 8),
                                      (8192, 2047, 4), (8192, 2049, 3), (8192, 4097, 1), (8192, 1024, 8)])
 def test_splits_of_slots_and_ids(S, K, n_q):
+    _steps(S, K, n_q, 0, 3)
+
+
+# a cluster's blocks with fewer slots than threads, with words of positions that no block or only some warps have, with
+# several passes over the positions, with more ids coming in than a block has slots; L = 1: the shortest decay search
+@pytest.mark.parametrize("S,K,n_q,C,L", [(256, 256, 1, 8, 3), (256, 31, 8, 8, 1), (512, 170, 3, 4, 2), (2048, 1025, 1, 2, 126),
+                                         (4096, 1024, 4, 4, 1), (16384, 2047, 8, 0, 3), (16384, 5000, 3, 4, 5),
+                                         (32768, 4097, 2, 8, 30)])
+def test_splits_over_a_cluster(S, K, n_q, C, L):
+    _steps(S, K, n_q, C, L)
+
+
+def _steps(S, K, n_q, cluster, L):
     import torch
     import paper_2609_37538_b200 as avsg
-    T, n, L = 6, 2, 3
+    T, n = 6, 2
     rng = np.random.default_rng([S, K, n_q])
     kv = avsg.pinned_empty(CTX * RB)
     tr.fill_kv(kv.data_ptr(), 1, 0, CTX, RB)
-    ctx = avsg.Context(n, S, RB, K, n_q, L)
+    ctx = avsg.Context(n, S, RB, K, n_q, L, stage_one_cluster=cluster)
     orc = [OracleTable(S, RB, L) for _ in range(n)]
     for t in range(T):
         span = min(CTX, 3 * S // 2 + K)               # a good share of the ids comes back
         X = np.stack([[rng.choice(span, K, replace=False) for _ in range(n_q)] for _ in range(n)]).astype(np.int32)
         X[:, :, K // 2] = -1                          # padding in the middle
         N = [span - 7 * t for _ in range(n)]          # shrinks: resident ids become unverified
+        ctx.set_transfer_mode(avsg.XFER_SM_OVERLAP if t % 2 else avsg.XFER_SM_BALANCED)
         out = ctx.step(list(range(n)), torch.from_numpy(X).cuda(), [kv] * n, N)
         slots, hit, mc = out.slots.cpu().numpy(), out.hit.cpu().numpy(), out.miss_count.cpu().numpy()
         for i in range(n):
