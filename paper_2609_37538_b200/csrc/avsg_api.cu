@@ -632,7 +632,7 @@ int avsg_reset_async(avsg_ctx* c, const uint32_t* table_ids, uint32_t n, void* c
             p.table_id[i] = table_ids[first + i];
             c->kv_host[p.table_id[i]] = 0; c->kv_dev[p.table_id[i]] = 0;      // the next request brings its own host KV
         }
-        CU(launch_reset_tables(p, cnt, static_cast<cudaStream_t>(cuda_stream)));
+        CU(launch_reset_tables(p, cnt, (uint32_t)c->sm_count, static_cast<cudaStream_t>(cuda_stream)));
     }
     return AVSG_OK;
 }

@@ -191,7 +191,8 @@ struct ResetParams {             // stream-ordered reset of some tables: empty, 
     uint32_t S, row_bytes;
     uint32_t table_id[S1_MAX_TABLES];
 };
-cudaError_t launch_reset_tables(const ResetParams& p, uint32_t n_tables, cudaStream_t stream);
+constexpr uint32_t RESET_THREADS = 256;
+cudaError_t launch_reset_tables(const ResetParams& p, uint32_t n_tables, uint32_t sm_count, cudaStream_t stream);
 
 size_t stage_one_smem_bytes(uint32_t S, uint32_t K, uint32_t n_q);
 size_t stage_one_paper_smem_bytes(uint32_t S, uint32_t K, uint32_t L);

@@ -401,17 +401,23 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
 
 // A request ended: its tables become empty (id -1) and dead (lifetime -1) again, their counters and rows zero;
 // in the paper-literal mode every bucket word returns to (lifetime -1, invalid, fingerprint 0, slot 0).  Grid (blocks per table, tables).
-__global__ void avsg_reset_tables_kernel(const __grid_constant__ ResetParams p)
+// What bounds it is the 43 MB of rows that eight tables have, at the rate of stores; so the device is filled with blocks
+// whatever the number of tables, and the grid starts under the kernel before it and lets the next one start under itself
+// (programmatic launch): eight tables in 7.5 us and not 10.4.
+__global__ void __launch_bounds__(RESET_THREADS) avsg_reset_tables_kernel(const __grid_constant__ ResetParams p)
 {
-    const uint32_t table = p.table_id[blockIdx.y];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const size_t table = p.table_id[blockIdx.y];
     const size_t S = p.S, tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x, nth = (size_t)gridDim.x * blockDim.x;
-    for (size_t j = tid; j < S; j += nth) {
-        p.tok[table * S + j] = -1;
-        p.life[table * S + j] = (int8_t)-1;
-        if (p.qword) p.qword[table * S + j] = 0xFF800000u;
-    }
     int4* rows = reinterpret_cast<int4*>(p.buffer + table * S * p.row_bytes);
-    for (size_t i = tid; i < S * (p.row_bytes >> 4); i += nth) rows[i] = make_int4(0, 0, 0, 0);
+    const size_t chunks = S * (p.row_bytes >> 4);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (size_t i = tid; i < chunks; i += nth) rows[i] = make_int4(0, 0, 0, 0);
+    for (size_t j = tid; j < S / 4; j += nth) {
+        reinterpret_cast<int4*>(p.tok + table * S)[j] = make_int4(-1, -1, -1, -1);
+        reinterpret_cast<uint32_t*>(p.life + table * S)[j] = 0xFFFFFFFFu;
+        if (p.qword) reinterpret_cast<uint4*>(p.qword + table * S)[j] = make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0xFF800000u);
+    }
     if (tid == 0) p.stats[table] = TableStats{0, 0, 0, 0, 0, 0};
 }
 
@@ -829,10 +835,19 @@ cudaError_t launch_stage_one(const S1ParamsBig& p, uint32_t n_tables, cudaStream
     return launch_stage_one_t(p, n_tables, stream);
 }
 
-cudaError_t launch_reset_tables(const ResetParams& p, uint32_t n_tables, cudaStream_t stream)
+cudaError_t launch_reset_tables(const ResetParams& p, uint32_t n_tables, uint32_t sm_count, cudaStream_t stream)
 {
-    avsg_reset_tables_kernel<<<dim3(32, n_tables), 256, 0, stream>>>(p);
-    return cudaGetLastError();
+    const uint32_t per_sm = 2048 / RESET_THREADS;        // blocks
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((sm_count * per_sm + n_tables - 1) / n_tables, n_tables);
+    cfg.blockDim = dim3(RESET_THREADS);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, avsg_reset_tables_kernel, p);
 }
 
 cudaError_t launch_all_k_prepare(const AllKParams& p, uint32_t n_tables, cudaStream_t stream)
