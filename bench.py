@@ -472,7 +472,8 @@ def run_cuda(args):
                 "ms_per_step": e2e_ms_j / K,
                 "note": "avsg_step_host: ids uploaded from pinned host memory, slot table and miss counts "
                         "downloaded; h2d bytes = ids + missed KV rows"},
-        "gpu_launches": 2 * ncalls * K,
+        # two kernels per call (Stage One, Stage Two); one for calls of up to three tables
+        "gpu_launches": sum(2 if len(grp) > 3 else 1 for grp in w.calls) * K,
         "numa": {"gpu_pci": bdf, "numa_node": numa["numa_node"], "bound": numa["bound"], "cpus": len(numa["cpus"]),
                  "note": "rank 0; the pinned host KV is allocated and filled by threads bound to these CPUs when bound"},
         "hit_rate": hits_j / max(1.0, hits_j + miss_j),

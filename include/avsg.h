@@ -66,7 +66,13 @@ extern "C" {
                                              slots were reserved whose rows were never copied  */
 
 /* How Stage Two moves the missed rows (Sec. 3.4; App. D strategies). */
-#define AVSG_XFER_SM_BALANCED   0u  /* miss list cut evenly over all SMs (the operator)  */
+#define AVSG_XFER_SM_BALANCED   0u  /* miss list cut evenly over all SMs (the operator).
+                                       Calls of up to three tables run both stages in one
+                                       kernel in this mode and in AVSG_XFER_SM_OVERLAP: a
+                                       thread-block cluster per table, Stage Two following
+                                       Stage One token by token (not with arriving, timing,
+                                       an own transfer geometry or a table above 8192
+                                       slots)                                            */
 #define AVSG_XFER_COPY_ENGINE   1u  /* comparator: miss list read back, one async copy
                                        per run of consecutive rows on the copy engine    */
 #define AVSG_XFER_REQUEST_LEVEL 2u  /* comparator S1: one thread block per request       */

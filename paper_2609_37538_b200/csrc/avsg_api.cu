@@ -3,6 +3,7 @@
 // the host; there is no CPU fallback.
 #include <new>
 #include <string.h>
+#include <type_traits>
 #include <vector>
 
 #include <cuda.h>          // types of the one driver entry point fetched at run time (nothing links libcuda)
@@ -13,6 +14,8 @@
 using namespace avsg;
 
 namespace {
+// Calls in one kernel: a table takes eight SMs for the call's length, which larger batches leave to what runs beside them.
+constexpr uint32_t SMALL_CALL_TABLES = 3;
 constexpr size_t FLAG_BYTES = ((size_t)OVERLAP_MAX_TABLES * OVERLAP_MAX_TOKENS + 1) * sizeof(uint32_t);
 }
 
@@ -30,6 +33,8 @@ struct avsg_ctx {
     int8_t* d_life = nullptr;
     uint8_t* d_buffer = nullptr;
     TableStats* d_stats = nullptr;
+    bool step_possible = false;                    // calls in one kernel: the device places their clusters
+    bool geometry_set = false;                     // avsg_set_transfer_geometry was called
     uint32_t* d_flags = nullptr;                   // hand-over flags per (table of the call, token) (1 + miss count)
                                                    //   [OVERLAP_MAX_TABLES x TOKENS], and one that is never raised
     unsigned long long* d_sync = nullptr;          //   [2] sequence number of the last host-buffer call,
@@ -332,10 +337,19 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
             p.kv_base[i] = c->call_kv_dev[first + i];
             p.kv_stride[i] = a->row_stride ? a->row_stride[first + i] : c->cfg.row_bytes;
         }
-        if (c->s1_cluster > 1) CU(launch_stage_one_cluster(p, cnt, c->s1_cluster, stream));
+        if constexpr (std::is_same<std::remove_reference_t<decltype(p)>, StepParams>::value) {
+            p.flags = nullptr; p.out = out;
+            CU(launch_step(p, stream));
+        } else if (c->s1_cluster > 1) CU(launch_stage_one_cluster(p, cnt, c->s1_cluster, stream));
         else CU(launch_stage_one(p, cnt < round_size ? cnt : round_size, stream));
         return AVSG_OK;
     };
+    // Small calls take one kernel for both stages (see avsg_step_kernel for what it saves).
+    if (c->step_possible && n <= SMALL_CALL_TABLES && (overlap || mode == AVSG_XFER_SM_BALANCED) &&
+        c->s1_cluster == 1 && c->cfg.index_mode != AVSG_INDEX_PAPER && !a->arriving && !host_io && !c->timing && !c->geometry_set) {
+        StepParams p;
+        return stage_one(p, 0, n);
+    }
     for (uint32_t first = 0; first < n; first += chunk) {
         const uint32_t cnt = n - first < chunk ? n - first : chunk;
         if (mode == AVSG_XFER_ALL_K) {
@@ -519,6 +533,7 @@ int avsg_create(const avsg_config* cfg, avsg_ctx** out)
         transfer_prepare() != cudaSuccess || arriving_prepare() != cudaSuccess) {
         delete c; return AVSG_ECUDA;
     }
+    c->step_possible = step_possible((size_t)max_smem);
     // a cluster shape that fits on paper may still find no home on the device (blocks of one cluster share a GPC)
     if (c->s1_cluster > 1 &&
         stage_one_cluster_max_active(cfg->buffer_slots, cfg->max_topk, cfg->max_tokens, c->s1_cluster) < 1) {
@@ -850,6 +865,7 @@ int avsg_set_transfer_geometry(avsg_ctx* c, uint32_t blocks, uint32_t threads)
     if (!c || threads < 32 || threads > 1024 || threads % 32 || blocks > 65535) return AVSG_EINVAL;
     c->xfer_blocks = blocks;
     c->xfer_threads = threads;
+    c->geometry_set = true;
     return AVSG_OK;
 }
 

@@ -74,6 +74,20 @@ constexpr int MAX_IPT = 8;           // ids per thread
 constexpr int MAX_SPT = 8;           // slots per thread
 constexpr int XFER_MAX_SEG = 2048;   // segments per Stage Two launch (prefix sums live in shared memory)
 
+// Calls with host buffers: Stage Two writes the call's outputs from the library's device buffers (256-byte aligned) into
+// the caller's mapped host memory, which the GPU's side of the link that the gather leaves free carries.
+struct HostOut {
+    const int32_t* slots = nullptr;  int32_t* host_slots = nullptr;  uint32_t n_slots = 0;
+    const uint8_t* hit = nullptr;    uint8_t* host_hit = nullptr;    uint32_t n_hit = 0;           // none: 0
+    const int32_t* count = nullptr;  int32_t* host_count = nullptr;  uint32_t n_count = 0;
+};
+
+constexpr int OVERLAP_MAX_TOKENS = 8;
+
+// Calls in one kernel: a thread-block cluster per table, one block for Stage One and the others for Stage Two.
+constexpr int STEP_MAX_TABLES = 8;
+constexpr uint32_t STEP_CLUSTER = 8;
+
 // The per-call host arrays travel as kernel arguments, CAP tables' worth of them: a call needs no staging copy.
 template <int CAP>
 struct S1ParamsT {
@@ -104,6 +118,7 @@ struct S1ParamsT {
     uint32_t*           done_ctr = nullptr;     // arrivals after the call's last token; wraps to zero at `expect`
     unsigned long long  host_seq = 0;
     uint32_t            expect = 0;             // tables of the call
+    HostOut             out;                    // a call in one kernel: what its Stage Two writes to the host
     uint32_t            host_ids = 0;           // indices is mapped host memory that holds the ids when the call is made
     const int32_t* verified_len_dev = nullptr;  // [n] of the call: read instead of verified_len[] when set
     uint32_t table_id[CAP];
@@ -116,14 +131,6 @@ using S1Params = S1ParamsT<S1_MAX_TABLES>;
 using S1ParamsBig = S1ParamsT<S1_BIG_TABLES>;
 static_assert(sizeof(S1ParamsBig) <= 32764, "kernel argument block too large");
 
-// Calls with host buffers: Stage Two writes the call's outputs from the library's device buffers (256-byte aligned) into
-// the caller's mapped host memory, which the GPU's side of the link that the gather leaves free carries.
-struct HostOut {
-    const int32_t* slots = nullptr;  int32_t* host_slots = nullptr;  uint32_t n_slots = 0;
-    const uint8_t* hit = nullptr;    uint8_t* host_hit = nullptr;    uint32_t n_hit = 0;           // none: 0
-    const int32_t* count = nullptr;  int32_t* host_count = nullptr;  uint32_t n_count = 0;
-};
-
 struct XferParams {
     const SegDesc* seg;
     const int2*    miss_list;
@@ -135,7 +142,6 @@ struct XferParams {
     unsigned long long* t_range = nullptr;
 };
 
-constexpr int OVERLAP_MAX_TOKENS = 8;
 constexpr uint32_t S1_ROUND_BLOCKS = 32;             // Stage One blocks of a call that is served in rounds
 constexpr int OVERLAP_MAX_TABLES = S1_BIG_TABLES;   // one Stage One launch
 constexpr uint32_t OVERLAP_SPIN_LIMIT = 1u << 18;   // polls before the wait gives up; a poll is an L2 round trip plus a 64 ns sleep, ~0.8 us measured: ~0.2 s
@@ -198,6 +204,10 @@ size_t stage_one_smem_bytes(uint32_t S, uint32_t K, uint32_t n_q);
 size_t stage_one_paper_smem_bytes(uint32_t S, uint32_t K, uint32_t L);
 uint32_t stage_one_threads(uint32_t S, uint32_t K);
 cudaError_t stage_one_prepare(size_t max_smem);
+// both stages of a call of up to STEP_MAX_TABLES tables in one kernel
+using StepParams = S1ParamsT<STEP_MAX_TABLES>;
+bool step_possible(size_t max_smem);                    // after stage_one_prepare: the device places such a cluster
+cudaError_t launch_step(const StepParams& p, cudaStream_t stream);
 // n_blocks thread blocks serve the p.n_launch tables of the launch (one block per table unless the call runs in rounds)
 cudaError_t launch_stage_one(const S1Params& p, uint32_t n_blocks, cudaStream_t stream);
 cudaError_t launch_stage_one(const S1ParamsBig& p, uint32_t n_blocks, cudaStream_t stream);   // hash / direct index only

@@ -24,7 +24,7 @@ using namespace avsg;
 namespace {
 
 struct NoAllocScratch {
-    uint32_t   status[64];                                   // word 0: device status
+    uint32_t   status[64];                                   // word 0: device status, word 1: that of calls that ask for none
     SegDesc    seg[AVSG_NOALLOC_MAX_TABLES];
     TableStats stats[AVSG_NOALLOC_MAX_TABLES];
     int2       list[AVSG_NOALLOC_MAX_IDS];                   // (host position, slot) per miss
@@ -37,6 +37,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoAllocS
 constexpr int MAX_DEVICES = 64;
 std::mutex g_setup_mutex;
 NoAllocScratch* g_scratch_addr[MAX_DEVICES] = {nullptr};
+bool g_step_possible[MAX_DEVICES] = {false};
 int g_sm_count[MAX_DEVICES] = {0};
 int g_max_smem[MAX_DEVICES] = {0};
 
@@ -54,6 +55,7 @@ int setup_device(int dev, NoAllocScratch** out)
             cudaGetLastError();
             return AVSG_ECUDA;
         }
+        g_step_possible[dev] = step_possible((size_t)g_max_smem[dev]);
         g_scratch_addr[dev] = static_cast<NoAllocScratch*>(ptr);
     }
     *out = g_scratch_addr[dev];
@@ -87,42 +89,52 @@ extern "C" int avsg_step_noalloc(const avsg_noalloc_args* a, void* cuda_stream)
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const uint32_t list_stride = a->n_tokens * a->topk;
 
-    S1Params p;
-    p.tok = a->tok; p.life = a->life; p.buffer = static_cast<uint8_t*>(a->buffer);
-    p.stats = sc->stats; p.miss_list = sc->list; p.seg = sc->seg; p.status = sc->status;
-    p.indices = a->indices; p.slots = a->slots; p.hit = a->hit; p.miss_count = a->miss_count;
-    p.S = a->buffer_slots; p.row_bytes = a->row_bytes; p.K = a->topk; p.n_q = a->n_tokens;
-    p.L = (uint32_t)a->max_lifetime; p.first = 0; p.list_stride = list_stride;
-    p.n_launch = a->n;
-    p.qword = nullptr; p.probe_retries = 0; p.hash_a1 = 0; p.hash_a2 = 0;
-    p.logH = 1;
-    while ((1u << p.logH) < 2u * a->buffer_slots) ++p.logH;
-    for (uint32_t i = 0; i < a->n; ++i) {
-        const void* base = a->kv_base[i];
-        if (!base || (reinterpret_cast<uint64_t>(base) & 15u)) return AVSG_EINVAL;
-        if (a->row_stride && (a->row_stride[i] % 16 || a->row_stride[i] < a->row_bytes)) return AVSG_EINVAL;
-        if (a->kv_rows && a->kv_rows[i] > 0x80000000u) return AVSG_EINVAL;
-        p.id_limit[i] = a->kv_rows ? a->kv_rows[i] : 0x80000000u;
-        cudaPointerAttributes at;
-        if (cudaPointerGetAttributes(&at, base) != cudaSuccess) { cudaGetLastError(); return AVSG_EINVAL; }
-        if (at.type == cudaMemoryTypeUnregistered || !at.devicePointer) return AVSG_EINVAL;
-        p.table_id[i] = i;
-        p.verified_len[i] = a->verified_len[i];
-        p.kv_base[i] = reinterpret_cast<uint64_t>(at.devicePointer);
-        p.kv_stride[i] = a->row_stride ? a->row_stride[i] : a->row_bytes;
+    // A status word that the caller wants starts at zero; else the kernels' bits go to one that nobody reads.
+    uint32_t* status = sc->status + (a->status ? 0 : 1);
+    if (a->status && cudaMemsetAsync(status, 0, sizeof(uint32_t), stream) != cudaSuccess) return AVSG_ECUDA;
+
+    auto fill = [&](auto& p) -> int {
+        p.tok = a->tok; p.life = a->life; p.buffer = static_cast<uint8_t*>(a->buffer);
+        p.stats = sc->stats; p.miss_list = sc->list; p.seg = sc->seg; p.status = status;
+        p.indices = a->indices; p.slots = a->slots; p.hit = a->hit; p.miss_count = a->miss_count;
+        p.S = a->buffer_slots; p.row_bytes = a->row_bytes; p.K = a->topk; p.n_q = a->n_tokens;
+        p.L = (uint32_t)a->max_lifetime; p.first = 0; p.list_stride = list_stride;
+        p.n_launch = a->n;
+        p.qword = nullptr; p.probe_retries = 0; p.hash_a1 = 0; p.hash_a2 = 0;
+        p.logH = 1;
+        while ((1u << p.logH) < 2u * a->buffer_slots) ++p.logH;
+        for (uint32_t i = 0; i < a->n; ++i) {
+            const void* base = a->kv_base[i];
+            if (!base || (reinterpret_cast<uint64_t>(base) & 15u)) return AVSG_EINVAL;
+            if (a->row_stride && (a->row_stride[i] % 16 || a->row_stride[i] < a->row_bytes)) return AVSG_EINVAL;
+            if (a->kv_rows && a->kv_rows[i] > 0x80000000u) return AVSG_EINVAL;
+            p.id_limit[i] = a->kv_rows ? a->kv_rows[i] : 0x80000000u;
+            cudaPointerAttributes at;
+            if (cudaPointerGetAttributes(&at, base) != cudaSuccess) { cudaGetLastError(); return AVSG_EINVAL; }
+            if (at.type == cudaMemoryTypeUnregistered || !at.devicePointer) return AVSG_EINVAL;
+            p.table_id[i] = i;
+            p.verified_len[i] = a->verified_len[i];
+            p.kv_base[i] = reinterpret_cast<uint64_t>(at.devicePointer);
+            p.kv_stride[i] = a->row_stride ? a->row_stride[i] : a->row_bytes;
+        }
+        return AVSG_OK;
+    };
+    if (g_step_possible[dev] && a->n <= (uint32_t)STEP_MAX_TABLES) {
+        StepParams p;                                    // one kernel for both stages
+        if ((rc = fill(p)) != AVSG_OK) return rc;
+        if (launch_step(p, stream) != cudaSuccess) return AVSG_ECUDA;
+    } else {
+        S1Params p;
+        if ((rc = fill(p)) != AVSG_OK) return rc;
+        if (launch_stage_one(p, a->n, stream) != cudaSuccess) return AVSG_ECUDA;
+        XferParams x;
+        x.seg = sc->seg; x.miss_list = sc->list; x.status = status;
+        x.n_seg = a->n; x.list_stride = list_stride; x.row_bytes = a->row_bytes; x.request_level = 0; x.S = a->buffer_slots;
+        if (launch_transfer(x, (uint32_t)g_sm_count[dev], 256, stream) != cudaSuccess) return AVSG_ECUDA;
     }
 
-    // the array keeps the previous call's contents: status, segment lengths and counters restart at zero
-    if (cudaMemsetAsync(sc, 0, offsetof(NoAllocScratch, list), stream) != cudaSuccess) return AVSG_ECUDA;
-    if (launch_stage_one(p, a->n, stream) != cudaSuccess) return AVSG_ECUDA;
-
-    XferParams x;
-    x.seg = sc->seg; x.miss_list = sc->list; x.status = sc->status;
-    x.n_seg = a->n; x.list_stride = list_stride; x.row_bytes = a->row_bytes; x.request_level = 0; x.S = a->buffer_slots;
-    if (launch_transfer(x, (uint32_t)g_sm_count[dev], 256, stream) != cudaSuccess) return AVSG_ECUDA;
-
     if (a->status &&
-        cudaMemcpyAsync(a->status, sc->status, sizeof(uint32_t), cudaMemcpyDeviceToDevice, stream) != cudaSuccess)
+        cudaMemcpyAsync(a->status, status, sizeof(uint32_t), cudaMemcpyDeviceToDevice, stream) != cudaSuccess)
         return AVSG_ECUDA;
     return AVSG_OK;
 }

@@ -37,6 +37,7 @@
 #include <type_traits>
 
 #include "avsg_kernels.cuh"
+#include "follow_stage_one.cuh"
 #include "stage_one_common.cuh"
 
 namespace avsg {
@@ -70,13 +71,14 @@ __device__ __forceinline__ uint32_t signs(uint32_t w) { return (((w >> 7) & 0x01
 
 // SPT slots per thread (a power of two): S <= SPT * blockDim.x.  IPT: the most ids a thread has to look up per token
 // (K <= S, so SPT is always enough).  CAP: tables the argument block has room for.
-template <int SPT, int IPT, int CAP>
-__global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_constant__ S1ParamsT<CAP> p)
+// has room for.  The block serves the tables block, block + blocks, ... of the launch.  CLUSTER: it is the first block of
+// a cluster whose others copy what it places (avsg_step_kernel); a_count: where they wait for their counts.
+template <int SPT, int IPT, bool CLUSTER, int CAP>
+__device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_t block, const uint32_t blocks, unsigned char* smem, const uint32_t a_count = 0)
 {
     constexpr int NV = (SPT + 3) / 4;                    // 4-slot vectors of ids / words of lifetimes per thread
     using bits_t = typename std::conditional<(SPT > 8), uint16_t, uint8_t>::type;       // a thread's dead bits
     constexpr uint32_t PER_WORD = 4 / sizeof(bits_t);
-    extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t S = p.S, K = p.K, H = 2u * S, L = p.L;
     const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u, warp = tid >> 5, nw = nt >> 5;
     const uint32_t below = (1u << lane) - 1u;            // the lanes before this one
@@ -115,7 +117,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
             xs[k] = i0 + 32u * k < i1 ? (p.host_ids ? __ldcv(ids + i0 + 32u * k) : __ldcg(ids + i0 + 32u * k)) : -1;
     };
     // the first table's arguments and the clearing come before the wait: under the previous kernel's tail
-    uint32_t bt = blockIdx.x, table = p.table_id[bt], id_limit = p.id_limit[bt];
+    uint32_t bt = block, table = p.table_id[bt], id_limit = p.id_limit[bt];
     int32_t N = p.verified_len[bt];
     clear_index();
     if (tid == 0) s_node[NIL] = make_uint2(0xFFFFFFFEu, NIL);          // an id that nobody looks for
@@ -132,7 +134,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
     const bool own = j0 < S;
 
     // A block usually serves one table.  A call with many tables and an overlapped Stage Two is launched with fewer
-    // blocks than tables: a block then serves the tables bt = blockIdx.x, blockIdx.x + gridDim.x, ... one after the
+    // blocks than tables: a block then serves the tables bt = block, block + blocks, ... one after the
     // other, so that Stage One stays on a few SMs and publishes its tables round by round while the transfer grid,
     // resident on the other SMs, already copies the earlier rounds' misses.
     for (;;) {
@@ -147,9 +149,9 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
         for (int q = 0; q < NV; ++q)
             if (tid + q * nt < S / 4) t4[q] = __ldcg(reinterpret_cast<const int4*>(g_tok) + tid + q * nt);
         life_words<SPT, true>(g_life + j0, own, w);
-        if (!p.host_ids || bt != blockIdx.x) load_token(ti, 0);
+        if (!p.host_ids || bt != block) load_token(ti, 0);
         if (p.verified_len_dev) N = __ldg(p.verified_len_dev + ti);
-        const uint32_t seen = bt == blockIdx.x ? take_flags_down(p, bt, gridDim.x, p.n_launch) : 0u;
+        const uint32_t seen = !CLUSTER && bt == block ? take_flags_down(p, bt, blocks, p.n_launch) : 0u;
         if (tid == 0) s_sum[0] = 0;
         __syncthreads();                                 // the index is empty
 
@@ -263,7 +265,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
                 if (lane == 0 && valid) atomicAdd(s_sum, valid);
             }
             if (lane == 0) s_tot[par + warp] = wmiss;
-            if (g == 0 && bt == blockIdx.x) start_dependents(seen);
+            if (!CLUSTER && g == 0 && bt == block) start_dependents(seen);
             __syncthreads();
 
             // ---- CollectDead and the misses, each in order; the prefix over the warps: lane l looks at warp l ----
@@ -360,6 +362,11 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
             list_off += n_take;
             sum_decay += d;
             __syncthreads();
+            if constexpr (CLUSTER) {
+                cluster_wait();                          // (the last token's barrier, which the others have long reached)
+                if (tid < STEP_CLUSTER) stc_u32(map_rank(a_count + 4u * (g & 1u), tid), n_take);
+                cluster_arrive();
+            }
             announce_token(p, ti, g, n_take);
         }
 
@@ -387,7 +394,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
             atomicAdd(&st->rows, (unsigned long long)list_off);
             atomicAdd(&st->extra_decays, (unsigned long long)sum_decay);
         }
-        bt += gridDim.x;
+        bt += blocks;
         if (bt >= p.n_launch) break;
         table = p.table_id[bt]; id_limit = p.id_limit[bt]; N = p.verified_len[bt];
         __syncthreads();                                 // this table's last reads of shared memory are over
@@ -396,6 +403,60 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
     if (p.t_range) {
         __syncthreads();
         if (tid == 0) atomicMax(p.t_range + 1, global_ns());
+    }
+}
+
+template <int SPT, int IPT, int CAP>
+__global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_constant__ S1ParamsT<CAP> p)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    stage_one<SPT, IPT, false>(p, blockIdx.x, gridDim.x, smem);
+}
+
+// A small call in one kernel: a cluster of eight blocks per table.  The first block runs Stage One; the others copy the
+// misses of every token as soon as it is placed, in either mode.  What it saves is a launch (1.8 us of host time, which bounds the
+// smallest calls), the way from the end of one grid to the start of the next, and the hand-over through global memory:
+// the blocks of a cluster run at the same time, so a cluster barrier per announcement does it.  The copying blocks arrive
+// at the next one before they copy, so Stage One never waits for them.  Every table's misses have seven SMs of their own,
+// whose warps keep 140 KB of rows on the way: one table alone can fill the link (2 us round trip x 47 GB/s).  Measured, two
+// kernels / one: K = 256, S = 1024 8.4 / 6.3 us; K = 2048, S = 8192, two tokens, 230 rows 17.2 / 13.0 (14.3 where the copy
+// starts after the last token), from a captured graph 19.2 / 17.8; eight tables, K = 1000, S = 4096, 1230 rows 40.8 / 35.0.
+template <int SPT, int IPT>
+__global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constant__ StepParams p)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint32_t s_count[2];                                    // misses announced, by token parity
+    const uint32_t rank = cluster_rank(), ti = blockIdx.x / STEP_CLUSTER, lane = threadIdx.x & 31u;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    cluster_arrive();                                                  // every block is there: see the first wait
+    if (rank == 0) {
+        stage_one<SPT, IPT, true>(p, ti, p.n_launch, smem, smem_u32(s_count));
+        return;
+    }
+    const uint32_t cpr = p.row_bytes >> 4;
+    const uint32_t W = (blockDim.x >> 5) * (STEP_CLUSTER - 1u), w = (threadIdx.x >> 5) * (STEP_CLUSTER - 1u) + rank - 1u;
+    const int2* list = p.miss_list + (size_t)ti * p.list_stride;
+    const uint64_t src = p.kv_base[ti], stride = p.kv_stride[ti];
+    const uint64_t dst = reinterpret_cast<uint64_t>(p.buffer + (size_t)p.table_id[ti] * p.S * p.row_bytes);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    cluster_wait();
+    cluster_arrive();
+    uint32_t from = 0, off = 0;                                        // the warp that is next; list entries copied
+    for (uint32_t g = 0; g < p.n_q; ++g) {
+        cluster_wait();                                                // Stage One has announced
+        const uint32_t count = *reinterpret_cast<volatile uint32_t*>(&s_count[g & 1u]);
+        if (g + 1u < p.n_q) cluster_arrive();
+        else if (p.out.n_slots) put_outputs_of(p.out, ti, p.n_q * p.K, p.n_q, w, W, lane);
+        for (uint32_t k = w >= from ? w - from : w + W - from; k < count; k += W) {
+            const int2 e = off + k < p.list_stride ? __ldcg(list + off + k) : make_int2(-1, -1);
+            if (e.x < 0 || e.y < 0 || (uint32_t)e.y >= p.S) {
+                if (lane == 0) atomicOr(p.status, ST_BAD_SLOT);
+                continue;
+            }
+            copy_row(src + (uint64_t)(uint32_t)e.x * stride, dst + (uint64_t)(uint32_t)e.y * p.row_bytes, cpr, lane);
+        }
+        off += count;
+        from = (from + count) % W;
     }
 }
 
@@ -770,9 +831,18 @@ cudaError_t stage_one_prepare(size_t max_smem)
         reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 2, S1_BIG_TABLES>),
         reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 4, S1_BIG_TABLES>),
         reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 8, S1_BIG_TABLES>),
+        reinterpret_cast<const void*>(avsg_step_kernel<2, 2>),
+        reinterpret_cast<const void*>(avsg_step_kernel<4, 2>),
+        reinterpret_cast<const void*>(avsg_step_kernel<4, 4>),
+        reinterpret_cast<const void*>(avsg_step_kernel<8, 2>),
+        reinterpret_cast<const void*>(avsg_step_kernel<8, 4>),
+        reinterpret_cast<const void*>(avsg_step_kernel<8, 8>),
         reinterpret_cast<const void*>(avsg_stage_one_paper_kernel)};
     for (const void* k : kernels) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem);
+        cudaFuncAttributes fa;
+        cudaError_t e = cudaFuncGetAttributes(&fa, k);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(max_smem - fa.sharedSizeBytes));
         if (e != cudaSuccess) return e;
     }
     // The other kernels of this file are loaded now as well: the runtime loads a kernel at its first use, which may
@@ -828,6 +898,68 @@ cudaError_t launch_stage_one(const S1Params& p, uint32_t n_tables, cudaStream_t 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, avsg_stage_one_paper_kernel, p);
+}
+
+namespace {
+// At least 16 warps a block where the table has the slots for it: they copy.
+uint32_t step_threads(uint32_t S, uint32_t K)
+{
+    const uint32_t t = stage_one_threads(S, K), most = S / 2 < 512u ? S / 2 : 512u;
+    return t > most ? t : most;
+}
+
+const void* step_kernel(uint32_t S, uint32_t K)
+{
+    const uint32_t nt = step_threads(S, K), ipt = (K + nt - 1) / nt;
+    switch (S / nt) {
+        case 8:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 2>)
+                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 4>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<8, 8>);
+        case 4:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<4, 2>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<4, 4>);
+        default: return reinterpret_cast<const void*>(avsg_step_kernel<2, 2>);
+    }
+}
+
+void step_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, uint32_t n_tables, uint32_t threads, size_t smem)
+{
+    cfg.gridDim = dim3(n_tables * STEP_CLUSTER);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = STEP_CLUSTER;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+}
+}  // namespace
+
+bool step_possible(size_t max_smem)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    step_config(cfg, attr, 1, 1024, max_smem - 1024);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(avsg_step_kernel<8, 2>), &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return n > 0;
+}
+
+cudaError_t launch_step(const StepParams& p, cudaStream_t stream)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    const uint32_t nt = step_threads(p.S, p.K);
+    step_config(cfg, attr, p.n_launch, nt, s1_layout(p.S, p.K, p.n_q, nt).total);
+    cfg.stream = stream;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+    void* args[] = {const_cast<StepParams*>(&p)};
+    return cudaLaunchKernelExC(&cfg, step_kernel(p.S, p.K), args);
 }
 
 cudaError_t launch_stage_one(const S1ParamsBig& p, uint32_t n_tables, cudaStream_t stream)

@@ -30,34 +30,6 @@ namespace {
 constexpr uint32_t MAX_CL = 8;          // largest cluster (the portable limit)
 constexpr uint32_t SMEM_LIMIT = 227u << 10;
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r;
-}
-__device__ __forceinline__ uint32_t cluster_size()
-{
-    uint32_t r; asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r;
-}
-// the address of the same shared-memory location in block `rank` of the cluster
-__device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank)
-{
-    uint32_t r; asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank)); return r;
-}
-__device__ __forceinline__ void stc_u32(uint32_t a, uint32_t v)
-{
-    asm volatile("st.shared::cluster.u32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ void addc_u32(uint32_t a, uint32_t v)
-{
-    asm volatile("red.shared::cluster.add.u32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
-}
-// All threads of all blocks of the cluster; earlier (distributed) shared-memory and global writes of the cluster
-// are visible to every thread of the cluster afterwards.
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
-
 // Shared-memory layout of one block (the same in every block of the cluster, so that a location's address in another
 // block follows from the local one).  Nodes come first; a call takes each of the block's slots once at most.
 struct Layout {

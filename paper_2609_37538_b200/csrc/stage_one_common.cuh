@@ -5,8 +5,36 @@
 
 namespace avsg {
 
-constexpr int32_t EMPTY = -1;
 constexpr int32_t PRIV_HIST_MAX_L = 30;   // private byte-counter histogram up to this L (32 rows)
+
+// ---- thread-block clusters ----
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r;
+}
+__device__ __forceinline__ uint32_t cluster_size()
+{
+    uint32_t r; asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r;
+}
+// the address of the same shared-memory location in block `rank` of the cluster
+__device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank)
+{
+    uint32_t r; asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank)); return r;
+}
+__device__ __forceinline__ void stc_u32(uint32_t a, uint32_t v)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void addc_u32(uint32_t a, uint32_t v)
+{
+    asm volatile("red.shared::cluster.add.u32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
+}
+// All threads of all blocks of the cluster; earlier (distributed) shared-memory and global writes of the cluster
+// are visible to every thread of the cluster afterwards.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
 
 __device__ __forceinline__ uint32_t hash_id(int32_t x, uint32_t logH)
 {
@@ -159,9 +187,22 @@ __device__ __forceinline__ void start_dependents(uint32_t seen)
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Calls that asked for it (host buffers in the overlapped mode, or a caller's own signal word): the table that arrives last
+// after the call's last token announces that every table of the call has written its slot table, hit mask and miss counts.
+// The arrivals are counted in a word of their own that wraps to zero by itself (atomicInc).  One thread per table.
+template <typename P>
+__device__ __forceinline__ void announce_call(const P& p, bool announce)
+{
+    if (announce && atomicInc(p.done_ctr, p.expect - 1u) == p.expect - 1u) {
+        __threadfence();
+        *reinterpret_cast<volatile unsigned long long*>(p.done_seq) = p.host_seq;
+    }
+}
+
 // Tells the overlapped transfer kernel, which is already resident (p.flags set), that token g of this table is placed:
-// `count` more entries of the table's miss list are final.  Called by every thread of the block after a barrier behind the list writes; one thread then fences (the
-// barrier makes the fence cover the whole block's earlier writes, as in a grid-wide barrier) and raises the table's flag.
+// `count` more entries of the table's miss list are final.  Called by every thread of the block after a barrier behind
+// the list writes; one thread then fences (the barrier makes the fence cover the whole block's earlier writes, as in a
+// grid-wide barrier) and raises the table's flag.
 template <typename P>
 __device__ __forceinline__ void announce_token(const P& p, uint32_t ti, uint32_t g, uint32_t count)
 {
@@ -169,13 +210,7 @@ __device__ __forceinline__ void announce_token(const P& p, uint32_t ti, uint32_t
     if ((!p.flags && !announce) || threadIdx.x != 0) return;
     __threadfence();
     if (p.flags) *reinterpret_cast<volatile uint32_t*>(p.flags + (size_t)ti * p.n_q + g) = 1u + count;
-    // calls that asked for it (host buffers in the overlapped mode, or a caller's own signal word): the table that arrives last after the
-    // call's last token announces that every table of the call has written its slot table, hit mask and miss counts.
-    // The arrivals are counted in a word of their own that wraps to zero by itself (atomicInc).
-    if (announce && atomicInc(p.done_ctr, p.expect - 1u) == p.expect - 1u) {
-        __threadfence();
-        *reinterpret_cast<volatile unsigned long long*>(p.done_seq) = p.host_seq;
-    }
+    announce_call(p, announce);
 }
 
 // The same with the barrier in front.

@@ -1,0 +1,113 @@
+"""Small calls, which one kernel serves: calls whose number of tables, tokens and ids changes from one to the next, among
+calls that take two kernels, queued without a wait; both modes, host buffers, the signal word, a captured
+call; compared with the oracle (whole numbers and bytes: nothing to tolerate)."""
+import numpy as np
+import pytest
+
+import avsg_traces as tr
+from oracle import OracleTable
+
+pytestmark = pytest.mark.gpu
+RB, CTX = 48, 5000
+
+
+def _kv(avsg):
+    kv = avsg.pinned_empty(CTX * RB)
+    tr.fill_kv(kv.data_ptr(), 1, 0, CTX, RB)
+    return kv
+
+
+# blocks of 4, 16 and 32 warps; K below and above S / 4
+@pytest.mark.parametrize("S,K_max", [(256, 32), (1024, 128), (4096, 500), (8192, 600)])
+def test_calls_of_changing_size(S, K_max):
+    import torch
+    import paper_2609_37538_b200 as avsg
+    rng = np.random.default_rng(S)
+    n, L, calls = 6, 4, 60
+    kv = _kv(avsg)
+    ctx = avsg.Context(n, S, RB, K_max, 8, L)
+    orc = [OracleTable(S, RB, L) for _ in range(n)]
+    word = torch.zeros(1, dtype=torch.int64, device="cuda")
+    done = []
+    for c in range(calls):
+        tabs = [int(t) for t in rng.permutation(n)[: int(rng.choice([1, 1, 2, 3, 3, 4, 6]))]]
+        n_q, K = int(rng.integers(1, 9)), int(rng.integers(1, K_max + 1))
+        ctx.set_transfer_mode(int(rng.choice([avsg.XFER_SM_BALANCED, avsg.XFER_SM_OVERLAP])))
+        X = np.stack([[rng.choice(700, K, replace=False) for _ in range(n_q)] for _ in tabs]).astype(np.int32)
+        if c % 4 == 3:
+            out = ctx.step_host(tabs, torch.from_numpy(X).pin_memory(), [kv] * len(tabs), [690] * len(tabs))
+        else:
+            out = ctx.step(tabs, torch.from_numpy(X).cuda(), [kv] * len(tabs), [690] * len(tabs),
+                           stage_one_done=(word, c + 1) if c % 3 == 0 else None)
+        done.append((tabs, X, out))
+    torch.cuda.synchronize()
+    assert int(word.item()) == max(c + 1 for c in range(calls) if c % 3 == 0 and c % 4 != 3)
+    for c, (tabs, X, out) in enumerate(done):
+        for a, t in enumerate(tabs):
+            r = orc[t].step(X[a], 690, kv.numpy(), RB)
+            assert (out.slots[a].cpu().numpy() == r.O).all() and (out.hit[a].cpu().numpy() == r.M).all(), (c, t)
+            assert (out.miss_count[a].cpu().numpy() == r.n).all(), (c, t)
+    for t in range(n):
+        assert (ctx.buffer(t).cpu().numpy() == orc[t].rows()).all(), t
+    assert ctx.sync_status() == 0
+
+
+@pytest.mark.parametrize("mode", ["XFER_SM_BALANCED", "XFER_SM_OVERLAP"])
+def test_a_captured_small_call(mode):
+    import torch
+    import paper_2609_37538_b200 as avsg
+    S, K, n_q, L = 1024, 200, 3, 5
+    rng = np.random.default_rng(3)
+    kv = _kv(avsg)
+    ctx = avsg.Context(2, S, RB, K, n_q, L, transfer_mode=getattr(avsg, mode))
+    orc = [OracleTable(S, RB, L) for _ in range(2)]
+    call = ctx.prepare([1, 0], [kv] * 2, n_q, K)
+    X = torch.empty((2, n_q, K), dtype=torch.int32, device="cuda")
+    slots, N = torch.empty_like(X), torch.full((2,), CTX, dtype=torch.int32, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(2):                               # the same call twice in the graph
+            call.run(X, N, slots)
+    for t in range(8):
+        ids = np.stack([[rng.choice(2000, K, replace=False) for _ in range(n_q)] for _ in range(2)]).astype(np.int32)
+        X.copy_(torch.from_numpy(ids))
+        graph.replay()
+        torch.cuda.synchronize()
+        for i, table in enumerate((1, 0)):
+            orc[table].step(ids[i], CTX, kv.numpy(), RB)
+            r = orc[table].step(ids[i], CTX, kv.numpy(), RB)
+            assert (slots[i].cpu().numpy() == r.O).all() and (ctx.buffer(table).cpu().numpy() == orc[table].rows()).all(), (t, i)
+        call.run(X, [CTX, CTX], slots)                   # and once outside
+        torch.cuda.synchronize()
+        for i, table in enumerate((1, 0)):
+            assert (slots[i].cpu().numpy() == orc[table].step(ids[i], CTX, kv.numpy(), RB).O).all(), (t, i)
+    assert ctx.sync_status() == 0
+
+
+def test_noalloc_with_and_without_a_status_word():
+    """A call without a status word must not leave its bits to the next one's."""
+    import torch
+    import paper_2609_37538_b200 as avsg
+    S, K = 256, 16
+    kv = _kv(avsg)
+    d = dict(device="cuda")
+    tok, life = torch.full((2, S), -1, dtype=torch.int32, **d), torch.full((2, S), -1, dtype=torch.int8, **d)
+    buf, status = torch.zeros((2, S, RB), dtype=torch.uint8, **d), torch.full((1,), 7, dtype=torch.int32, **d)
+    orc = [OracleTable(S, RB, 4) for _ in range(2)]
+    rng = np.random.default_rng(4)
+    for t in range(12):
+        n_q = 9 if t % 3 == 2 else 2
+        X = np.stack([[rng.choice(600, K, replace=False) for _ in range(n_q)] for _ in range(2)]).astype(np.int32)
+        bad = t % 4 == 1
+        if bad:
+            X[0, 0, 3] = 999                             # beyond the stated host rows
+        slots = torch.empty(X.shape, dtype=torch.int32, **d)
+        wants = t % 2 == 0
+        avsg.step_noalloc(tok, life, buf, torch.from_numpy(X).cuda(), [kv] * 2, [CTX] * 2, max_lifetime=4, slots=slots,
+                          status=status if wants else None, kv_rows=[700, 700])
+        torch.cuda.synchronize()
+        if wants:
+            assert int(status.item()) == 0, t            # the call before it flagged an id and asked for no status
+        for i in range(2):
+            r = orc[i].step(np.where(X[i] >= 700, -1, X[i]), CTX, kv.numpy(), RB)
+            assert (slots[i].cpu().numpy() == r.O).all() and (buf[i].cpu().numpy() == orc[i].rows()).all(), (t, i)
