@@ -1,5 +1,5 @@
 """Small calls, which one kernel serves: calls whose number of tables, tokens and ids changes from one to the next, among
-calls that take two kernels, queued without a wait; both modes, host buffers, the signal word, a captured
+calls that take two kernels, resets and a restored snapshot, queued without a wait; both modes, host buffers, the signal word, a captured
 call; compared with the oracle (whole numbers and bytes: nothing to tolerate)."""
 import numpy as np
 import pytest
@@ -19,13 +19,14 @@ def _kv(avsg):
 
 # blocks of 4, 16 and 32 warps; K below and above S / 4
 @pytest.mark.parametrize("S,K_max", [(256, 32), (1024, 128), (4096, 500), (8192, 600)])
-def test_calls_of_changing_size(S, K_max):
+@pytest.mark.parametrize("cluster", [0, 2])
+def test_calls_of_changing_size(S, K_max, cluster):
     import torch
     import paper_2609_37538_b200 as avsg
     rng = np.random.default_rng(S)
     n, L, calls = 6, 4, 60
     kv = _kv(avsg)
-    ctx = avsg.Context(n, S, RB, K_max, 8, L)
+    ctx = avsg.Context(n, S, RB, K_max, 8, L, stage_one_cluster=cluster)
     orc = [OracleTable(S, RB, L) for _ in range(n)]
     word = torch.zeros(1, dtype=torch.int64, device="cuda")
     done = []
@@ -34,21 +35,38 @@ def test_calls_of_changing_size(S, K_max):
         n_q, K = int(rng.integers(1, 9)), int(rng.integers(1, K_max + 1))
         ctx.set_transfer_mode(int(rng.choice([avsg.XFER_SM_BALANCED, avsg.XFER_SM_OVERLAP])))
         X = np.stack([[rng.choice(700, K, replace=False) for _ in range(n_q)] for _ in tabs]).astype(np.int32)
+        gone = [int(t) for t in rng.permutation(n)[:2]] if c % 7 == 4 else []
+        if gone:
+            ctx.reset_async(gone)                        # in the stream's order, between two calls
+        if c == 21:
+            ctx.save_state()
+        if c == 40:
+            ctx.restore_state()
         if c % 4 == 3:
             out = ctx.step_host(tabs, torch.from_numpy(X).pin_memory(), [kv] * len(tabs), [690] * len(tabs))
         else:
             out = ctx.step(tabs, torch.from_numpy(X).cuda(), [kv] * len(tabs), [690] * len(tabs),
-                           stage_one_done=(word, c + 1) if c % 3 == 0 else None)
-        done.append((tabs, X, out))
+                           stage_one_done=(word, c + 1) if c % 3 == 0 else None, want_arriving=c % 5 == 0)
+        done.append((tabs, X, gone, out))
     torch.cuda.synchronize()
     assert int(word.item()) == max(c + 1 for c in range(calls) if c % 3 == 0 and c % 4 != 3)
-    for c, (tabs, X, out) in enumerate(done):
+    for c, (tabs, X, gone, out) in enumerate(done):
+        for t in gone:
+            orc[t].reset()
+        if c == 21:
+            saved = [o.export_state() for o in orc]
+        if c == 40:
+            for o, state in zip(orc, saved):
+                o.import_state(*state)                   # (ids and lifetimes; rows are fetched again where they are missed)
         for a, t in enumerate(tabs):
             r = orc[t].step(X[a], 690, kv.numpy(), RB)
             assert (out.slots[a].cpu().numpy() == r.O).all() and (out.hit[a].cpu().numpy() == r.M).all(), (c, t)
             assert (out.miss_count[a].cpu().numpy() == r.n).all(), (c, t)
+            assert c % 5 or c % 4 == 3 or (out.arriving[a].cpu().numpy() == r.arriving).all(), (c, t)
     for t in range(n):
         assert (ctx.buffer(t).cpu().numpy() == orc[t].rows()).all(), t
+        tok, life = ctx.export_state(t)
+        assert (tok == orc[t].export_state()[0]).all() and (life == orc[t].export_state()[1]).all(), t
     assert ctx.sync_status() == 0
 
 
