@@ -345,7 +345,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
         return AVSG_OK;
     };
     // Small calls take one kernel for both stages (see avsg_step_kernel for what it saves).
-    if (c->step_possible && n <= SMALL_CALL_TABLES && (overlap || mode == AVSG_XFER_SM_BALANCED) &&
+    if (c->step_possible && n <= SMALL_CALL_TABLES && n_q <= STEP_MAX_TOKENS && (overlap || mode == AVSG_XFER_SM_BALANCED) &&
         c->s1_cluster == 1 && c->cfg.index_mode != AVSG_INDEX_PAPER && !a->arriving && !host_io && !c->timing && !c->geometry_set) {
         StepParams p;
         return stage_one(p, 0, n);

@@ -86,7 +86,8 @@ constexpr int OVERLAP_MAX_TOKENS = 8;
 
 // Calls in one kernel: a thread-block cluster per table, one block for Stage One and the others for Stage Two.
 constexpr int STEP_MAX_TABLES = 8;
-constexpr uint32_t STEP_CLUSTER = 8;
+constexpr uint32_t STEP_CLUSTER = 8, STEP_COPYING = STEP_CLUSTER - 1;
+constexpr uint32_t STEP_MAX_TOKENS = 64;
 
 // The per-call host arrays travel as kernel arguments, CAP tables' worth of them: a call needs no staging copy.
 template <int CAP>

@@ -119,7 +119,7 @@ extern "C" int avsg_step_noalloc(const avsg_noalloc_args* a, void* cuda_stream)
         }
         return AVSG_OK;
     };
-    if (g_step_possible[dev] && a->n <= (uint32_t)STEP_MAX_TABLES) {
+    if (g_step_possible[dev] && a->n <= (uint32_t)STEP_MAX_TABLES && a->n_tokens <= STEP_MAX_TOKENS) {
         StepParams p;                                    // one kernel for both stages
         if ((rc = fill(p)) != AVSG_OK) return rc;
         if (launch_step(p, stream) != cudaSuccess) return AVSG_ECUDA;

@@ -69,12 +69,17 @@ __host__ __device__ inline S1Layout s1_layout(uint32_t S, uint32_t K, uint32_t n
 // Bits 0 .. 3: the sign bits of a word's four bytes.
 __device__ __forceinline__ uint32_t signs(uint32_t w) { return (((w >> 7) & 0x01010101u) * 0x10204080u) >> 28; }
 
+constexpr uint32_t STEP_SPIN_LIMIT = 1u << 20;            // waits of a microsecond or so each (the hardware suspends the warp)
+
+// Words of eight bytes that a copying block of a cluster gets per token, at most.
+__device__ __forceinline__ uint32_t step_rows(uint32_t K) { return 1u + (K + STEP_COPYING - 1u) / STEP_COPYING; }
+
 // SPT slots per thread (a power of two): S <= SPT * blockDim.x.  IPT: the most ids a thread has to look up per token
 // (K <= S, so SPT is always enough).  CAP: tables the argument block has room for.
 // has room for.  The block serves the tables block, block + blocks, ... of the launch.  CLUSTER: it is the first block of
-// a cluster whose others copy what it places (avsg_step_kernel); a_count: where they wait for their counts.
+// a cluster whose others copy what it places (avsg_step_kernel); a_mbar: their mbarriers, one per token.
 template <int SPT, int IPT, bool CLUSTER, int CAP>
-__device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_t block, const uint32_t blocks, unsigned char* smem, const uint32_t a_count = 0)
+__device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_t block, const uint32_t blocks, unsigned char* smem, const uint32_t a_mbar = 0)
 {
     constexpr int NV = (SPT + 3) / 4;                    // 4-slot vectors of ids / words of lifetimes per thread
     using bits_t = typename std::conditional<(SPT > 8), uint16_t, uint8_t>::type;       // a thread's dead bits
@@ -341,6 +346,15 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
             if (lane == 0) s_ndead[32u - par + warp] = left;
             __syncthreads();
 
+            if constexpr (CLUSTER) {                     // what the copying blocks get of this token: a head and their rows
+                if (g == 0) cluster_wait();              // (their mbarriers are ready)
+                if (tid < STEP_COPYING) {
+                    const uint32_t n = (n_take + STEP_COPYING - 1u - tid) / STEP_COPYING, mbar = map_rank(a_mbar + 8u * g, tid + 1u);
+                    send_async(map_rank(smem_u32(smem) + 8u * g * step_rows(K), tid + 1u), (int32_t)n, 0, mbar);
+                    arrive_expect(mbar, 8u * (n + 1u));
+                }
+            }
+
             // ---- install: the k-th miss in position order takes the k-th dead slot ----
             for (uint32_t k = tid; k < n_g; k += nt) {
                 const uint32_t i = s_pos[k];
@@ -349,7 +363,13 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
                 if (k < n_take) {
                     s_node[j].x = (uint32_t)x;
                     s_life[j] = (int8_t)L;
-                    list[list_off + k] = make_int2(x, j);
+                    if constexpr (CLUSTER) {
+                        const uint32_t to = 1u + k % STEP_COPYING;
+                        send_async(map_rank(smem_u32(smem) + 8u * (g * step_rows(K) + 1u + k / STEP_COPYING), to), x, j,
+                                   map_rank(a_mbar + 8u * g, to));
+                    } else {
+                        list[list_off + k] = make_int2(x, j);
+                    }
                     g_tok[j] = x >= N ? -1 : x;                        // speculative ids are forgotten (end of Alg. 4)
                     if (!last) {
                         const uint32_t n = S + list_off + k;
@@ -362,11 +382,6 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
             list_off += n_take;
             sum_decay += d;
             __syncthreads();
-            if constexpr (CLUSTER) {
-                cluster_wait();                          // (the last token's barrier, which the others have long reached)
-                if (tid < STEP_CLUSTER) stc_u32(map_rank(a_count + 4u * (g & 1u), tid), n_take);
-                cluster_arrive();
-            }
             announce_token(p, ti, g, n_take);
         }
 
@@ -414,49 +429,61 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
 }
 
 // A small call in one kernel: a cluster of eight blocks per table.  The first block runs Stage One; the others copy the
-// misses of every token as soon as it is placed, in either mode.  What it saves is a launch (1.8 us of host time, which bounds the
-// smallest calls), the way from the end of one grid to the start of the next, and the hand-over through global memory:
-// the blocks of a cluster run at the same time, so a cluster barrier per announcement does it.  The copying blocks arrive
-// at the next one before they copy, so Stage One never waits for them.  Every table's misses have seven SMs of their own,
-// whose warps keep 140 KB of rows on the way: one table alone can fill the link (2 us round trip x 47 GB/s).  Measured, two
-// kernels / one: K = 256, S = 1024 8.4 / 6.3 us; K = 2048, S = 8192, two tokens, 230 rows 17.2 / 13.0 (14.3 where the copy
-// starts after the last token), from a captured graph 19.2 / 17.8; eight tables, K = 1000, S = 4096, 1230 rows 40.8 / 35.0.
+// misses of every token as soon as it is placed, in either mode.  What it saves is a launch (1.8 us of host time, which
+// bounds the smallest calls), the way from the end of one grid to the start of the next, and the hand-over through global
+// memory with its fences: Stage One sends every miss (id, slot) straight into the shared memory of the block that will copy
+// it, where an mbarrier per token counts the bytes, and goes on.  Every table's misses have seven SMs of their own, whose
+// warps keep 140 KB of rows on the way: one table alone can fill the link (2 us round trip x 47 GB/s).  Measured with
+// two kernels / in one whose blocks met at a cluster barrier per token / in this one: K = 256, S = 1024 8.4 / 6.5 / 5.8 us;
+// K = 2048, S = 8192, two tokens, 230 rows 17.2 / 13.3 / 12.2, from a captured graph 19.8 / 19.3 / 18.3; eight tables,
+// K = 1000, S = 4096, 1230 rows of 1152 bytes 40.8 / 36.0 / 35.3.
 template <int SPT, int IPT>
 __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constant__ StepParams p)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ uint32_t s_count[2];                                    // misses announced, by token parity
+    extern __shared__ __align__(16) unsigned char smem[];              // of a copying block: the words that it gets, by token
+    __shared__ __align__(8) unsigned long long s_mbar[STEP_MAX_TOKENS];
     const uint32_t rank = cluster_rank(), ti = blockIdx.x / STEP_CLUSTER, lane = threadIdx.x & 31u;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    cluster_arrive();                                                  // every block is there: see the first wait
+    if (rank != 0 && threadIdx.x < p.n_q)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n\tfence.mbarrier_init.release.cluster;" :: "r"(smem_u32(s_mbar + threadIdx.x)) : "memory");
+    __syncthreads();
+    cluster_arrive();
     if (rank == 0) {
-        stage_one<SPT, IPT, true>(p, ti, p.n_launch, smem, smem_u32(s_count));
+        stage_one<SPT, IPT, true>(p, ti, p.n_launch, smem, smem_u32(s_mbar));
+        if (p.out.n_slots) cluster_arrive();                           // the outputs are written
         return;
     }
-    const uint32_t cpr = p.row_bytes >> 4;
-    const uint32_t W = (blockDim.x >> 5) * (STEP_CLUSTER - 1u), w = (threadIdx.x >> 5) * (STEP_CLUSTER - 1u) + rank - 1u;
-    const int2* list = p.miss_list + (size_t)ti * p.list_stride;
+    const uint32_t cpr = p.row_bytes >> 4, W = blockDim.x >> 5, warp = threadIdx.x >> 5;
     const uint64_t src = p.kv_base[ti], stride = p.kv_stride[ti];
     const uint64_t dst = reinterpret_cast<uint64_t>(p.buffer + (size_t)p.table_id[ti] * p.S * p.row_bytes);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     cluster_wait();
-    cluster_arrive();
-    uint32_t from = 0, off = 0;                                        // the warp that is next; list entries copied
+    if (p.out.n_slots) cluster_arrive();
+    uint32_t from = 0;                                                 // the warp that is next
     for (uint32_t g = 0; g < p.n_q; ++g) {
-        cluster_wait();                                                // Stage One has announced
-        const uint32_t count = *reinterpret_cast<volatile uint32_t*>(&s_count[g & 1u]);
-        if (g + 1u < p.n_q) cluster_arrive();
-        else if (p.out.n_slots) put_outputs_of(p.out, ti, p.n_q * p.K, p.n_q, w, W, lane);
-        for (uint32_t k = w >= from ? w - from : w + W - from; k < count; k += W) {
-            const int2 e = off + k < p.list_stride ? __ldcg(list + off + k) : make_int2(-1, -1);
+        const int2* got = reinterpret_cast<const int2*>(smem) + g * step_rows(p.K);
+        const uint32_t mbar = smem_u32(s_mbar + g);
+        uint32_t spin = 0;
+        while (!mbar_done(mbar) && ++spin < STEP_SPIN_LIMIT) {}
+        if (spin == STEP_SPIN_LIMIT) {                                 // (Stage One's loops are bounded, far below this)
+            if (lane == 0) atomicOr(p.status, ST_WAIT_TIMEOUT);
+            break;
+        }
+        __syncwarp();
+        const uint32_t count = (uint32_t)got[0].x;
+        for (uint32_t k = warp >= from ? warp - from : warp + W - from; k < count; k += W) {
+            const int2 e = got[1u + k];
             if (e.x < 0 || e.y < 0 || (uint32_t)e.y >= p.S) {
                 if (lane == 0) atomicOr(p.status, ST_BAD_SLOT);
                 continue;
             }
             copy_row(src + (uint64_t)(uint32_t)e.x * stride, dst + (uint64_t)(uint32_t)e.y * p.row_bytes, cpr, lane);
         }
-        off += count;
         from = (from + count) % W;
+    }
+    if (p.out.n_slots) {
+        cluster_wait();
+        put_outputs_of(p.out, ti, p.n_q * p.K, p.n_q, warp * STEP_COPYING + rank - 1u, W * STEP_COPYING, lane);
     }
 }
 
@@ -953,7 +980,7 @@ cudaError_t launch_step(const StepParams& p, cudaStream_t stream)
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     const uint32_t nt = step_threads(p.S, p.K);
-    step_config(cfg, attr, p.n_launch, nt, s1_layout(p.S, p.K, p.n_q, nt).total);
+    step_config(cfg, attr, p.n_launch, nt, s1_layout(p.S, p.K, p.n_q, nt).total);      // (holds step_rows() n_q times)
     cfg.stream = stream;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;

@@ -30,6 +30,24 @@ __device__ __forceinline__ void addc_u32(uint32_t a, uint32_t v)
 {
     asm volatile("red.shared::cluster.add.u32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
 }
+// Eight bytes into another block's shared memory, counted there by an mbarrier: no fence on either side.
+__device__ __forceinline__ void send_async(uint32_t a, int32_t x, int32_t y, uint32_t mbar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
+                 :: "r"(a), "r"(x), "r"(y), "r"(mbar) : "memory");
+}
+// Another block's mbarrier: its one arrival, with the bytes that are sent to it.
+__device__ __forceinline__ void arrive_expect(uint32_t mbar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" :: "r"(mbar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool mbar_done(uint32_t mbar)
+{
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0, %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(done) : "r"(mbar), "r"(1000u) : "memory");     // (suspended 1 us at most)
+    return done != 0;
+}
 // All threads of all blocks of the cluster; earlier (distributed) shared-memory and global writes of the cluster
 // are visible to every thread of the cluster afterwards.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
