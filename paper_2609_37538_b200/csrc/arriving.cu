@@ -42,11 +42,11 @@ __global__ void __launch_bounds__(512) avsg_arriving_kernel(const __grid_constan
                     uint32_t v = 0, spin = 0;
                     for (; spin < OVERLAP_SPIN_LIMIT; ++spin) {
                         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
-                        if (v) break;
+                        if (v >= p.announcers * ANNOUNCED) break;
                         __nanosleep(64);
                     }
                     if (spin == OVERLAP_SPIN_LIMIT) { s_ok = 0; atomicOr(p.status, ST_WAIT_TIMEOUT); }
-                    count += v - (v ? 1u : 0u);
+                    count += v & (ANNOUNCED - 1u);
                 }
                 s_count = count;
             } else {

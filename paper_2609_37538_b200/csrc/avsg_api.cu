@@ -200,7 +200,7 @@ template <typename X>
 void overlap_params(avsg_ctx* c, X& x, uint32_t n, uint32_t n_q, uint32_t round_size)
 {
     x.miss_list = c->d_list; x.status = c->d_status; x.buffer = c->d_buffer;
-    x.flags = c->d_flags;
+    x.flags = c->d_flags; x.announcers = c->s1_cluster;
     x.n = n; x.n_q = n_q; x.list_stride = c->list_stride; x.row_bytes = c->cfg.row_bytes; x.S = c->cfg.buffer_slots;
     x.round_size = round_size; x.t_range = nullptr;
 }
@@ -329,7 +329,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
                                       : (a->arriving ? nullptr : reinterpret_cast<unsigned long long*>(a->stage_one_done));
         p.done_ctr = reinterpret_cast<uint32_t*>(c->d_sync + 3);
         p.host_seq = wait_on_sequence ? c->host_seq + 1 : a->stage_one_done_value;
-        p.expect = n;
+        p.expect = n * c->s1_cluster;
         for (uint32_t i = 0; i < cnt; ++i) {
             p.table_id[i] = a->table_ids[first + i];
             p.verified_len[i] = a->verified_len ? a->verified_len[first + i] : 0;
@@ -381,7 +381,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
         q.value = a->stage_one_done_value;
         q.n = n; q.per_table = n_q * K; q.S = c->cfg.buffer_slots; q.list_stride = c->list_stride;
         q.flags = overlap ? c->d_flags : nullptr;
-        q.n_q = n_q; q.status = c->d_status;
+        q.announcers = c->s1_cluster; q.n_q = n_q; q.status = c->d_status;
         CU(launch_arriving(q, (uint32_t)c->sm_count, stream));
     }
     // (no event between the two grids in overlap mode: it would serialise them; ev[1] is recorded with ev[2])

@@ -110,15 +110,15 @@ struct S1ParamsT {
     uint32_t* qword;             // paper-literal mode: packed metadata words [num_tables][S], else null
     uint32_t probe_retries, hash_a1, hash_a2;   // paper-literal mode: R, a1, a2
     unsigned long long* t_range = nullptr;      // timing on: [0] earliest block start, [1] latest block end (ns)
-    // overlapped Stage Two (null otherwise): flags[ti * n_q + g] = 1 + misses of token g of the ti-th table of the call,
-    // written when that token is placed; zero until then (see take_flags_down())
+    // overlapped Stage Two (null otherwise): flags[ti * n_q + g], for token g of the ti-th table of the call: every block
+    // of the table adds ANNOUNCED + the misses it has placed; zero until then (see take_flags_down())
     uint32_t* flags = nullptr;
     // calls with host buffers in that mode (null otherwise): the table that places the call's last token last
     // writes the call's sequence number to *done_seq, which the output download waits for
     unsigned long long* done_seq = nullptr;
     uint32_t*           done_ctr = nullptr;     // arrivals after the call's last token; wraps to zero at `expect`
     unsigned long long  host_seq = 0;
-    uint32_t            expect = 0;             // tables of the call
+    uint32_t            expect = 0;             // Stage One blocks that place tables of the call
     HostOut             out;                    // a call in one kernel: what its Stage Two writes to the host
     uint32_t            host_ids = 0;           // indices is mapped host memory that holds the ids when the call is made
     const int32_t* verified_len_dev = nullptr;  // [n] of the call: read instead of verified_len[] when set
@@ -145,6 +145,7 @@ struct XferParams {
 
 constexpr uint32_t S1_ROUND_BLOCKS = 32;             // Stage One blocks of a call that is served in rounds
 constexpr int OVERLAP_MAX_TABLES = S1_BIG_TABLES;   // one Stage One launch
+constexpr uint32_t ANNOUNCED = 1u << 16;            // in a hand-over flag: one block's announcement (a count needs 16 bits)
 constexpr uint32_t OVERLAP_SPIN_LIMIT = 1u << 18;   // polls before the wait gives up; a poll is an L2 round trip plus a 64 ns sleep, ~0.8 us measured: ~0.2 s
 
 // Stage Two that is resident while Stage One runs and starts on misses as they are announced (see the kernel).
@@ -153,7 +154,8 @@ template <int CAP>
 struct XferOverlapParamsT {
     const int2*    miss_list;
     uint32_t*      status;
-    const uint32_t* flags;       // [n][n_q] 1 + miss count, written by Stage One
+    const uint32_t* flags;       // [n][n_q] written by Stage One (see S1ParamsT)
+    uint32_t announcers;         // Stage One blocks per table
     uint8_t*       buffer;       // [num_tables][S * row_bytes]
     uint32_t n, n_q, list_stride, row_bytes, S;
     uint32_t round_size;         // tables per round (n: one round)
@@ -239,6 +241,7 @@ struct ArrivingParams {
     uint32_t n, per_table, S, list_stride;
     // overlapped Stage Two: Stage One's hand-over flags (see S1ParamsT), else null
     const uint32_t* flags;
+    uint32_t announcers;             // Stage One blocks per table
     uint32_t n_q;
     uint32_t* status;
 };

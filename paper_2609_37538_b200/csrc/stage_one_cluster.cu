@@ -17,7 +17,9 @@
 // So every block computes for itself how many slots have to be taken and which of the misses are its own: the k-th dead
 // slot in slot order (block order, then the block's) takes the k-th miss in position order, and the block that owns the
 // slot selects that miss from the bits and installs it.  A decay adds a barrier per four candidate values of d and one
-// for the new dead counts; an overlapped Stage Two one more per token, behind which block 0 announces it.
+// for the new dead counts.  For an overlapped Stage Two every block announces its own misses of a token, on one flag that
+// they add to: where block 0 announced them all behind one more barrier of the cluster, Stage One took 25.4 us beside the
+// transfer grid and not 23.6 (16 tables, four tokens), and the call 108.7 us and not 108.2.
 // Measured inside the kernel, 16 tables, K = 2048, four tokens: S = 16384 (C = 2) 22.3 us, S = 32768 (C = 4) 21.8 us.  With
 // positions split over the blocks: 85 and 70 us with a distributed open-addressing index, 40 and 42 with an entry per
 // context position in device memory.  S = 32768, K = 8192, three tokens, four tables: 35 us against 133.
@@ -375,12 +377,8 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_cluster_kernel(const _
         }
         list_off += n_take;
         sum_decay += d;
-        if (p.flags || (p.done_seq && last)) {
-            cluster_sync();                                            // every block has installed its misses
-            if (rank == 0) announce_token(p, ti, g, n_take);
-        } else {
-            __syncthreads();
-        }
+        __syncthreads();
+        announce_token<true>(p, ti, g, mine);
     }
 
     // ---- write back: lifetimes; resident ids that are no longer verified become empty (Alg. 4) ----

@@ -205,9 +205,9 @@ __device__ __forceinline__ void start_dependents(uint32_t seen)
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Calls that asked for it (host buffers in the overlapped mode, or a caller's own signal word): the table that arrives last
+// Calls that asked for it (host buffers in the overlapped mode, or a caller's own signal word): the block that arrives last
 // after the call's last token announces that every table of the call has written its slot table, hit mask and miss counts.
-// The arrivals are counted in a word of their own that wraps to zero by itself (atomicInc).  One thread per table.
+// The arrivals are counted in a word of their own that wraps to zero by itself (atomicInc).  One thread per block.
 template <typename P>
 __device__ __forceinline__ void announce_call(const P& p, bool announce)
 {
@@ -220,14 +220,17 @@ __device__ __forceinline__ void announce_call(const P& p, bool announce)
 // Tells the overlapped transfer kernel, which is already resident (p.flags set), that token g of this table is placed:
 // `count` more entries of the table's miss list are final.  Called by every thread of the block after a barrier behind
 // the list writes; one thread then fences (the barrier makes the fence cover the whole block's earlier writes, as in a
-// grid-wide barrier) and raises the table's flag.
-template <typename P>
+// grid-wide barrier) and raises the table's flag.  SHARED: one of several blocks that place the table, each for itself.
+template <bool SHARED = false, typename P>
 __device__ __forceinline__ void announce_token(const P& p, uint32_t ti, uint32_t g, uint32_t count)
 {
     const bool announce = p.done_seq && g + 1 == p.n_q;
     if ((!p.flags && !announce) || threadIdx.x != 0) return;
     __threadfence();
-    if (p.flags) *reinterpret_cast<volatile uint32_t*>(p.flags + (size_t)ti * p.n_q + g) = 1u + count;
+    if (p.flags) {
+        if constexpr (SHARED) atomicAdd(p.flags + (size_t)ti * p.n_q + g, ANNOUNCED + count);
+        else *reinterpret_cast<volatile uint32_t*>(p.flags + (size_t)ti * p.n_q + g) = ANNOUNCED + count;
+    }
     announce_call(p, announce);
 }
 

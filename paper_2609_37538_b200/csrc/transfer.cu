@@ -124,7 +124,9 @@ __global__ void __launch_bounds__(1024, 1) avsg_transfer_overlap_kernel(const __
     const bool copied = follow_stage_one(p, p.n, p.n_q, p.round_size, blockIdx.x, gridDim.x, p.t_range, s_phase,
         [&](uint32_t t, uint32_t g, uint32_t& count) {                 // the flag of table t and token g
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(count) : "l"(p.flags + (size_t)t * p.n_q + g) : "memory");
-            return count-- != 0;
+            const bool raised = count >= p.announcers * ANNOUNCED;
+            count &= ANNOUNCED - 1u;
+            return raised;
         });
     const unsigned long long t_copied = p.t_range ? global_ns() : 0ull;
     asm volatile("griddepcontrol.wait;" ::: "memory");
