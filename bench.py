@@ -255,6 +255,10 @@ def run_cuda(args):
                        index_mode=avsg.INDEX_DIRECT if direct else avsg.INDEX_HASH,
                        max_context=max(c.context for c in w.tables) + w.n_q, stage_one_cluster=args.cluster,
                        transfer_mode=avsg.XFER_SM_OVERLAP if args.stage_two == "overlap" else avsg.XFER_SM_BALANCED)
+    # Shrunk runs are for looking at the two kernels of a call: a geometry that is set keeps them (what is set is the default).
+    one_kernel = 32 <= len(w.calls[0]) <= 74 and args.cluster <= 1 and w.buffer_slots <= 8192
+    if len(w.calls[0]) < 32:
+        ctx.set_transfer_geometry(0, 256)
     ncalls = len(w.calls)
     calls = [ctx.prepare(grp, [kv[t] for t in grp], w.n_q, w.topk,
                          [stride] * len(grp) if args.row_stride else None) for grp in w.calls]
@@ -438,13 +442,13 @@ def run_cuda(args):
     s1_gbs = s1_bytes / 1e3 / s1_avg_us
 
     xfer_alone = {"achieved": x_gbs, "duration_us": x_avg_us}
-    if args.stage_two == "overlap":
-        # The timed steps run avsg_transfer_overlap_kernel, resident from the start of its call's Stage One: its
-        # launch lasts the whole call, so its duration is the CUDA-event time of the timed steps / calls per step.
+    if one_kernel or args.stage_two == "overlap":
+        # The kernel that copies is resident for its whole call (both stages in one kernel, or beside Stage One), so its
+        # duration is the CUDA-event time of the timed steps / calls per step.
         call_us = 1e3 * total_ms_j / (K * ncalls)
         call_bytes = rows_j * rb / (K * ncalls * world)
         call_gbs = call_bytes / 1e3 / call_us
-        roofline = {"bound": "host_link", "kernel": "avsg_transfer_overlap_kernel", "achieved": call_gbs,
+        roofline = {"bound": "host_link", "kernel": "avsg_step_kernel" if one_kernel else "avsg_transfer_overlap_kernel", "achieved": call_gbs,
                     "peak": link_peak, "unit": "GB/s", "frac": call_gbs / link_peak,
                     "traffic": NCU_XFER_DRAM_BYTES_PER_ROW * call_bytes / rb,
                     "peak_kind": "measured in this run (pinned cudaMemcpyAsync H2D, 1 GiB, best of 4 after one warm-up copy)", "peak_repeats": 4,
@@ -470,10 +474,10 @@ def run_cuda(args):
         "e2e": {"value": e2e_value, "unit": "GB/s",
                 "h2d_bytes_per_step": int(ids_bytes + rows_timed * rb / K), "d2h_bytes_per_step": int(ids_bytes + mc_bytes),
                 "ms_per_step": e2e_ms_j / K,
-                "note": "avsg_step_host: ids uploaded from pinned host memory, slot table and miss counts "
-                        "downloaded; h2d bytes = ids + missed KV rows"},
-        # two kernels per call (Stage One, Stage Two); one for calls of up to three tables
-        "gpu_launches": sum(2 if len(grp) > 3 else 1 for grp in w.calls) * K,
+                "note": "avsg_step_host: ids read from pinned host memory and slot table and miss counts written to it "
+                        "by the kernels; h2d bytes = ids + missed KV rows"},
+        # one kernel per call, or two (Stage One, Stage Two)
+        "gpu_launches": len(w.calls) * (1 if one_kernel else 2) * K,
         "numa": {"gpu_pci": bdf, "numa_node": numa["numa_node"], "bound": numa["bound"], "cpus": len(numa["cpus"]),
                  "note": "rank 0; the pinned host KV is allocated and filled by threads bound to these CPUs when bound"},
         "hit_rate": hits_j / max(1.0, hits_j + miss_j),
@@ -519,8 +523,8 @@ def run_cuda(args):
                      "peak_kind": "measured in this run (pinned cudaMemcpyAsync H2D, 1 GiB, best of 4 after one warm-up copy)", "peak_repeats": 4,
                      "note": "algorithmic bytes = row_bytes x missed rows per launch; the rows cross the host link and stay "
                              "in L2 after the write, so DRAM traffic (scaled from the ncu capture of the one-layer case) is small; "
-                             "timed in balanced mode (one kernel at a time); with --stage-two overlap the timed steps run "
-                             "avsg_transfer_overlap_kernel, the same copy loop started per token while Stage One still runs"},
+                             "timed in balanced mode (one kernel at a time); the timed steps copy each token's rows while "
+                             "Stage One still runs"},
         "roofline_stage_one": {"bound": "hbm", "kernel": ("avsg_stage_one_cluster_kernel<%s>" if w.buffer_slots > 8192 or args.cluster > 1
                                                           else "avsg_stage_one_kernel<%s>") % args.index, "achieved": s1_gbs, "peak": hbm_peak,
                                "unit": "GB/s", "frac": s1_gbs / hbm_peak, "traffic": NCU_S1_DRAM_BYTES_PER_TABLE[args.index] * n_tab,

@@ -67,12 +67,15 @@ extern "C" {
 
 /* How Stage Two moves the missed rows (Sec. 3.4; App. D strategies). */
 #define AVSG_XFER_SM_BALANCED   0u  /* miss list cut evenly over all SMs (the operator).
-                                       Calls of up to three tables run both stages in one
+                                       Calls of up to 74 tables run both stages in one
                                        kernel in this mode and in AVSG_XFER_SM_OVERLAP: a
                                        thread-block cluster per table, Stage Two following
                                        Stage One token by token (not with arriving, timing,
                                        an own transfer geometry or a table above 8192
-                                       slots)                                            */
+                                       slots, nor with stage_one_done above three tables).
+                                       Its blocks take whole SMs while they run: who wants
+                                       room for other kernels beside the call sets a
+                                       transfer geometry                                 */
 #define AVSG_XFER_COPY_ENGINE   1u  /* comparator: miss list read back, one async copy
                                        per run of consecutive rows on the copy engine    */
 #define AVSG_XFER_REQUEST_LEVEL 2u  /* comparator S1: one thread block per request       */
@@ -362,7 +365,8 @@ int avsg_set_transfer_geometry(avsg_ctx *ctx, uint32_t blocks, uint32_t threads)
  * capture.  All calls on a device share the one scratch array: calls that
  * overlap on the GPU (two streams, or two host threads) race on it, so keep
  * them on one stream or order them yourself.  The array keeps the previous
- * call's contents; the library clears what has to start at zero.
+ * call's contents; nothing in it has to start at zero but a status word that
+ * is asked for, which the call clears.
  *
  * State layout (caller-owned DEVICE memory, table i at index i):
  *   tok    int32 [n][buffer_slots]  cached id per slot; a new table is all -1

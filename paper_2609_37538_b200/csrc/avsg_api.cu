@@ -3,7 +3,6 @@
 // the host; there is no CPU fallback.
 #include <new>
 #include <string.h>
-#include <type_traits>
 #include <vector>
 
 #include <cuda.h>          // types of the one driver entry point fetched at run time (nothing links libcuda)
@@ -14,8 +13,6 @@
 using namespace avsg;
 
 namespace {
-// Calls in one kernel: a table takes eight SMs for the call's length, which larger batches leave to what runs beside them.
-constexpr uint32_t SMALL_CALL_TABLES = 3;
 constexpr size_t FLAG_BYTES = ((size_t)OVERLAP_MAX_TABLES * OVERLAP_MAX_TOKENS + 1) * sizeof(uint32_t);
 }
 
@@ -33,9 +30,9 @@ struct avsg_ctx {
     int8_t* d_life = nullptr;
     uint8_t* d_buffer = nullptr;
     TableStats* d_stats = nullptr;
-    bool step_possible = false;                    // calls in one kernel: the device places their clusters
+    StepClusters step_clusters;                    // calls in one kernel
     bool geometry_set = false;                     // avsg_set_transfer_geometry was called
-    uint32_t* d_flags = nullptr;                   // hand-over flags per (table of the call, token) (1 + miss count)
+    uint32_t* d_flags = nullptr;                   // hand-over flags per (table of the call, token)
                                                    //   [OVERLAP_MAX_TABLES x TOKENS], and one that is never raised
     unsigned long long* d_sync = nullptr;          //   [2] sequence number of the last host-buffer call,
                                                    //   [3] arrivals after a host-buffer call's last token
@@ -308,8 +305,8 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
         if (c->cfg.index_mode == AVSG_INDEX_DIRECT && c->cfg.max_context < lim) lim = c->cfg.max_context;
         return lim;
     };
-    // Stage One for tables [first, first + cnt) of the call, with the small or the large argument block
-    auto stage_one = [&](auto& p, uint32_t first, uint32_t cnt) -> int {
+    // Stage One's arguments for tables [first, first + cnt) of the call, and its launch with the small or the large block
+    auto fill = [&](auto& p, uint32_t first, uint32_t cnt) {
         p.tok = c->d_tok; p.life = c->d_life; p.buffer = c->d_buffer; p.stats = c->d_stats;
         p.miss_list = c->d_list; p.seg = c->d_seg; p.status = c->d_status;
         p.indices = indices; p.slots = slots; p.hit = hit; p.miss_count = miss_count;
@@ -337,18 +334,26 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
             p.kv_base[i] = c->call_kv_dev[first + i];
             p.kv_stride[i] = a->row_stride ? a->row_stride[first + i] : c->cfg.row_bytes;
         }
-        if constexpr (std::is_same<std::remove_reference_t<decltype(p)>, StepParams>::value) {
-            p.flags = nullptr; p.out = out;
-            CU(launch_step(p, stream));
-        } else if (c->s1_cluster > 1) CU(launch_stage_one_cluster(p, cnt, c->s1_cluster, stream));
+    };
+    auto stage_one = [&](auto& p, uint32_t first, uint32_t cnt) -> int {
+        fill(p, first, cnt);
+        if (c->s1_cluster > 1) CU(launch_stage_one_cluster(p, cnt, c->s1_cluster, stream));
         else CU(launch_stage_one(p, cnt < round_size ? cnt : round_size, stream));
         return AVSG_OK;
     };
-    // Small calls take one kernel for both stages (see avsg_step_kernel for what it saves).
-    if (c->step_possible && n <= SMALL_CALL_TABLES && n_q <= STEP_MAX_TOKENS && (overlap || mode == AVSG_XFER_SM_BALANCED) &&
-        c->s1_cluster == 1 && c->cfg.index_mode != AVSG_INDEX_PAPER && !a->arriving && !host_io && !c->timing && !c->geometry_set) {
-        StepParams p;
-        return stage_one(p, 0, n);
+    // One kernel for both stages, where the tables' clusters fit the device (see avsg_step_kernel for what it saves).  Its
+    // blocks take whole SMs and the next grid starts behind them: a caller who wants the hits before the rows are there
+    // (stage_one_done) gets that from a call of more than a few tables only with the two kernels.
+    const uint32_t cluster = n_q <= STEP_MAX_TOKENS && (!a->stage_one_done || n <= STEP_EARLY_TABLES) ? c->step_clusters.of(n, step_threads(c->cfg.buffer_slots, K)) : 0u;
+    if (cluster && (overlap || mode == AVSG_XFER_SM_BALANCED) && c->s1_cluster == 1 && c->cfg.index_mode != AVSG_INDEX_PAPER &&
+        !a->arriving && !host_io && !c->timing && !c->geometry_set) {
+        auto step = [&](auto&& p) -> int {
+            fill(p, 0, n);
+            p.flags = nullptr; p.out = out; p.early = step_early(p);
+            CU(launch_step(p, cluster, stream));
+            return AVSG_OK;
+        };
+        return cluster == STEP_FEW_CLUSTER && n <= (uint32_t)STEP_FEW_TABLES ? step(StepParamsFew()) : step(StepParams());
     }
     for (uint32_t first = 0; first < n; first += chunk) {
         const uint32_t cnt = n - first < chunk ? n - first : chunk;
@@ -533,7 +538,7 @@ int avsg_create(const avsg_config* cfg, avsg_ctx** out)
         transfer_prepare() != cudaSuccess || arriving_prepare() != cudaSuccess) {
         delete c; return AVSG_ECUDA;
     }
-    c->step_possible = step_possible((size_t)max_smem);
+    c->step_clusters = step_clusters((size_t)max_smem);
     // a cluster shape that fits on paper may still find no home on the device (blocks of one cluster share a GPC)
     if (c->s1_cluster > 1 &&
         stage_one_cluster_max_active(cfg->buffer_slots, cfg->max_topk, cfg->max_tokens, c->s1_cluster) < 1) {

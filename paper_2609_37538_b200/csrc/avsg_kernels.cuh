@@ -85,8 +85,10 @@ struct HostOut {
 constexpr int OVERLAP_MAX_TOKENS = 8;
 
 // Calls in one kernel: a thread-block cluster per table, one block for Stage One and the others for Stage Two.
-constexpr int STEP_MAX_TABLES = 8;
-constexpr uint32_t STEP_CLUSTER = 8, STEP_COPYING = STEP_CLUSTER - 1;
+constexpr int STEP_MAX_TABLES = 74, STEP_FEW_TABLES = 8;      // sizes of the argument block
+constexpr uint32_t STEP_FEW_CLUSTER = 8;
+constexpr uint32_t STEP_EARLY_TABLES = 3;            // see step_early()
+constexpr uint64_t STEP_EARLY_BYTES = 2ull << 30;
 constexpr uint32_t STEP_MAX_TOKENS = 64;
 
 // The per-call host arrays travel as kernel arguments, CAP tables' worth of them: a call needs no staging copy.
@@ -120,6 +122,7 @@ struct S1ParamsT {
     unsigned long long  host_seq = 0;
     uint32_t            expect = 0;             // Stage One blocks that place tables of the call
     HostOut             out;                    // a call in one kernel: what its Stage Two writes to the host
+    uint32_t            early = 0;              // a call in one kernel: the next grid may start under it
     uint32_t            host_ids = 0;           // indices is mapped host memory that holds the ids when the call is made
     const int32_t* verified_len_dev = nullptr;  // [n] of the call: read instead of verified_len[] when set
     uint32_t table_id[CAP];
@@ -209,8 +212,42 @@ uint32_t stage_one_threads(uint32_t S, uint32_t K);
 cudaError_t stage_one_prepare(size_t max_smem);
 // both stages of a call of up to STEP_MAX_TABLES tables in one kernel
 using StepParams = S1ParamsT<STEP_MAX_TABLES>;
-bool step_possible(size_t max_smem);                    // after stage_one_prepare: the device places such a cluster
-cudaError_t launch_step(const StepParams& p, cudaStream_t stream);
+using StepParamsFew = S1ParamsT<STEP_FEW_TABLES>;
+struct StepClusters {
+    uint32_t fit[STEP_FEW_CLUSTER + 1] = {};           // clusters of each size that the device holds at once (B200: 15 of eight
+                                                       // blocks, 33 of four, 45 of three, 74 of two)
+    // Blocks per table for a call of n tables with blocks of `threads`; 0: two kernels.  All clusters of a call have to be
+    // on the device at once; of smaller blocks an SM holds as many as make 1024 threads.
+    // Above four blocks a cluster gains little (16 tables with 3, 4, 6 blocks 67.1, 66.1, 64.9 us; 12 with 3, 4, 8 52.2,
+    // 51.3, 51.0; 8 with 4, 8 36.3, 35.8; 4 with 4, 8 23.8, 22.6) and takes SMs from what runs beside the call, so
+    // only few tables get eight.  Two blocks are what is left above 45 tables: 64 tables 227 us, in two kernels 228.
+    uint32_t of(uint32_t n, uint32_t threads) const
+    {
+        if (n > (uint32_t)STEP_MAX_TABLES) return 0;
+        const uint32_t whole = (n * threads + 1023u) / 1024u;          // tables, in blocks of 1024 threads
+        if (whole <= (uint32_t)STEP_FEW_TABLES && whole <= fit[STEP_FEW_CLUSTER]) return STEP_FEW_CLUSTER;
+        for (uint32_t cl = 4; cl >= 2; --cl)
+            if (whole <= fit[cl]) return cl;
+        return 0;
+    }
+};
+StepClusters step_clusters(size_t max_smem);            // after stage_one_prepare
+// Whether the grid behind a call in one kernel may start under it (see the kernel).  Up to three tables, and up to eight
+// that reach little host memory (id_limit: rows a table's ids can reach): early / late, eight tables of 131072 rows 35.3 /
+// 35.7 us, of 1 Mi 59.7 / 46.3; five tables with K = 139 of 36028 rows 9.3 / 9.7.  More tables gain nothing by it (32 tables 113.0
+// / 112.9), and ids in host memory that are fetched under a call's rows slow these down (39 tables, K = 3430: 215 / 124).
+template <int CAP>
+bool step_early(const S1ParamsT<CAP>& p)
+{
+    if (p.n_launch <= STEP_EARLY_TABLES) return true;
+    if (p.n_launch > (uint32_t)STEP_FEW_TABLES || p.host_ids) return false;
+    uint64_t bytes = 0;
+    for (uint32_t i = 0; i < p.n_launch; ++i) bytes += p.id_limit[i] * p.kv_stride[i];
+    return bytes <= STEP_EARLY_BYTES;
+}
+uint32_t step_threads(uint32_t S, uint32_t K);
+// StepParamsFew: up to STEP_FEW_TABLES tables of STEP_FEW_CLUSTER blocks
+template <int CAP> cudaError_t launch_step(const S1ParamsT<CAP>& p, uint32_t cluster, cudaStream_t stream);
 // n_blocks thread blocks serve the p.n_launch tables of the launch (one block per table unless the call runs in rounds)
 cudaError_t launch_stage_one(const S1Params& p, uint32_t n_blocks, cudaStream_t stream);
 cudaError_t launch_stage_one(const S1ParamsBig& p, uint32_t n_blocks, cudaStream_t stream);   // hash / direct index only

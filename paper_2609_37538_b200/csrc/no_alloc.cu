@@ -37,7 +37,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoAllocS
 constexpr int MAX_DEVICES = 64;
 std::mutex g_setup_mutex;
 NoAllocScratch* g_scratch_addr[MAX_DEVICES] = {nullptr};
-bool g_step_possible[MAX_DEVICES] = {false};
+StepClusters g_step_clusters[MAX_DEVICES];
 int g_sm_count[MAX_DEVICES] = {0};
 int g_max_smem[MAX_DEVICES] = {0};
 
@@ -55,7 +55,7 @@ int setup_device(int dev, NoAllocScratch** out)
             cudaGetLastError();
             return AVSG_ECUDA;
         }
-        g_step_possible[dev] = step_possible((size_t)g_max_smem[dev]);
+        g_step_clusters[dev] = step_clusters((size_t)g_max_smem[dev]);
         g_scratch_addr[dev] = static_cast<NoAllocScratch*>(ptr);
     }
     *out = g_scratch_addr[dev];
@@ -119,10 +119,15 @@ extern "C" int avsg_step_noalloc(const avsg_noalloc_args* a, void* cuda_stream)
         }
         return AVSG_OK;
     };
-    if (g_step_possible[dev] && a->n <= (uint32_t)STEP_MAX_TABLES && a->n_tokens <= STEP_MAX_TOKENS) {
-        StepParams p;                                    // one kernel for both stages
-        if ((rc = fill(p)) != AVSG_OK) return rc;
-        if (launch_step(p, stream) != cudaSuccess) return AVSG_ECUDA;
+    const uint32_t cluster = a->n_tokens <= STEP_MAX_TOKENS ? g_step_clusters[dev].of(a->n, step_threads(a->buffer_slots, a->topk)) : 0u;
+    if (cluster) {
+        auto step = [&](auto&& p) -> int {               // one kernel for both stages
+            if ((rc = fill(p)) != AVSG_OK) return rc;
+            p.early = step_early(p);
+            return launch_step(p, cluster, stream) == cudaSuccess ? AVSG_OK : AVSG_ECUDA;
+        };
+        rc = cluster == STEP_FEW_CLUSTER && a->n <= (uint32_t)STEP_FEW_TABLES ? step(StepParamsFew()) : step(StepParams());
+        if (rc != AVSG_OK) return rc;
     } else {
         S1Params p;
         if ((rc = fill(p)) != AVSG_OK) return rc;

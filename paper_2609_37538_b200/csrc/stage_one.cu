@@ -34,8 +34,6 @@
 //
 // When Stage Two overlaps Stage One (S1Params::flags set), the block announces every token as soon as its misses are
 // placed: see announce_token().
-#include <type_traits>
-
 #include "avsg_kernels.cuh"
 #include "follow_stage_one.cuh"
 #include "stage_one_common.cuh"
@@ -54,7 +52,7 @@ __host__ __device__ inline S1Layout s1_layout(uint32_t S, uint32_t K, uint32_t n
     uint32_t a = align16((S + (n_q - 1u) * K + 1u) * 8u);      // nodes first
     o.head = a;  a += 2u * S * 4u;
     o.life = a;  a += align16(S);
-    o.bits = a;  a += align16(2u * nt);
+    o.bits = a;  a += align16(nt);
     o.tot = a;   a += 2u * 32u * 4u;                           // warps' miss totals, by parity
     o.ndead = a; a += 2u * 32u * 4u;                           // warps' dead slots, by parity
     o.cnt = a;   a += 2u * 2u * 32u * 4u;                      // warps' counts of the decay search, by parity
@@ -71,19 +69,18 @@ __device__ __forceinline__ uint32_t signs(uint32_t w) { return (((w >> 7) & 0x01
 
 constexpr uint32_t STEP_SPIN_LIMIT = 1u << 20;            // waits of a microsecond or so each (the hardware suspends the warp)
 
-// Words of eight bytes that a copying block of a cluster gets per token, at most.
-__device__ __forceinline__ uint32_t step_rows(uint32_t K) { return 1u + (K + STEP_COPYING - 1u) / STEP_COPYING; }
+// Words of eight bytes that one of `copying` blocks gets per token, at most: a head and its rows.
+__device__ __forceinline__ uint32_t step_rows(uint32_t K, uint32_t copying) { return 1u + (K + copying - 1u) / copying; }
 
 // SPT slots per thread (a power of two): S <= SPT * blockDim.x.  IPT: the most ids a thread has to look up per token
-// (K <= S, so SPT is always enough).  CAP: tables the argument block has room for.
-// has room for.  The block serves the tables block, block + blocks, ... of the launch.  CLUSTER: it is the first block of
-// a cluster whose others copy what it places (avsg_step_kernel); a_mbar: their mbarriers, one per token.
+// (K <= S, so SPT is always enough).  CAP: tables the argument block has room for.  The block serves the tables block,
+// block + blocks, ... of the launch.  CLUSTER: it is the first block of a cluster whose others copy what it places
+// (avsg_step_kernel); a_mbar: their mbarriers, one per token.
 template <int SPT, int IPT, bool CLUSTER, int CAP>
 __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_t block, const uint32_t blocks, unsigned char* smem, const uint32_t a_mbar = 0)
 {
+    const uint32_t copying = CAP == STEP_FEW_TABLES ? STEP_FEW_CLUSTER - 1u : CLUSTER ? cluster_size() - 1u : 1u;
     constexpr int NV = (SPT + 3) / 4;                    // 4-slot vectors of ids / words of lifetimes per thread
-    using bits_t = typename std::conditional<(SPT > 8), uint16_t, uint8_t>::type;       // a thread's dead bits
-    constexpr uint32_t PER_WORD = 4 / sizeof(bits_t);
     const uint32_t S = p.S, K = p.K, H = 2u * S, L = p.L;
     const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u, warp = tid >> 5, nw = nt >> 5;
     const uint32_t below = (1u << lane) - 1u;            // the lanes before this one
@@ -93,7 +90,7 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
     uint2*    s_node = reinterpret_cast<uint2*>(smem);
     uint32_t* s_head = reinterpret_cast<uint32_t*>(smem + lay.head);
     int8_t*   s_life = reinterpret_cast<int8_t*>(smem + lay.life);
-    bits_t*   s_bits = reinterpret_cast<bits_t*>(smem + lay.bits);
+    uint8_t*  s_bits = smem + lay.bits;                  // a thread's slots: set where dead
     uint32_t* s_tot  = reinterpret_cast<uint32_t*>(smem + lay.tot);
     uint32_t* s_ndead = reinterpret_cast<uint32_t*>(smem + lay.ndead);
     uint32_t* s_cnt  = reinterpret_cast<uint32_t*>(smem + lay.cnt);
@@ -107,8 +104,8 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
     };
     // slot j is no longer dead (the count follows the bit, so that an id that comes twice is counted once)
     auto revive = [&](uint32_t j, uint32_t par) {
-        const uint32_t owner = j / SPT, bit = 1u << ((owner % PER_WORD) * (32u / PER_WORD) + j % SPT);
-        if (atomicAnd(reinterpret_cast<uint32_t*>(s_bits) + owner / PER_WORD, ~bit) & bit)
+        const uint32_t owner = j / SPT, bit = 1u << ((owner & 3u) * 8u + j % SPT);
+        if (atomicAnd(reinterpret_cast<uint32_t*>(s_bits) + owner / 4u, ~bit) & bit)
             atomicSub(&s_ndead[par + owner / 32u], 1u);
     };
     const uint32_t ipt = (K + nt - 1) / nt;              // ids per thread
@@ -184,7 +181,7 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
 #pragma unroll
             for (int q = 0; q < NV; ++q) bits |= signs(w[q]) << (4 * q);
             life_words_store<SPT>(s_life + j0, own, w);
-            s_bits[tid] = (bits_t)bits;
+            s_bits[tid] = (uint8_t)bits;
             const uint32_t n = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(bits));
             if (lane == 0) s_ndead[par + warp] = n;
         };
@@ -339,18 +336,22 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
                 uint32_t bits = s_bits[tid], r, unused;
                 warp_rank<SPT>(__popc(bits), below, r, unused);
                 for (r += dead_before; bits && r < n_take; bits &= bits - 1u, ++r) s_dead[r] = (uint16_t)(j0 + __ffs((int)bits) - 1);
-                s_bits[tid] = (bits_t)bits;              // what is handed out is dead no more
+                s_bits[tid] = (uint8_t)bits;              // what is handed out is dead no more
             }
             uint32_t left = __shfl_sync(0xffffffffu, t & 0xFFFFu, (int)warp);          // the warp's dead slots for the next token
             if (dead_before < n_take) left = left > n_take - dead_before ? left - (n_take - dead_before) : 0u;
             if (lane == 0) s_ndead[32u - par + warp] = left;
             __syncthreads();
 
+            // a copying block's rows: every seventh where a cluster has eight blocks, else a share in position order
+            const uint32_t share = CLUSTER && CAP != STEP_FEW_TABLES ? (n_take + copying - 1u) / copying : 0u;
             if constexpr (CLUSTER) {                     // what the copying blocks get of this token: a head and their rows
                 if (g == 0) cluster_wait();              // (their mbarriers are ready)
-                if (tid < STEP_COPYING) {
-                    const uint32_t n = (n_take + STEP_COPYING - 1u - tid) / STEP_COPYING, mbar = map_rank(a_mbar + 8u * g, tid + 1u);
-                    send_async(map_rank(smem_u32(smem) + 8u * g * step_rows(K), tid + 1u), (int32_t)n, 0, mbar);
+                if (tid < copying) {
+                    const uint32_t n = CAP == STEP_FEW_TABLES ? (n_take + copying - 1u - tid) / copying
+                                       : tid * share >= n_take ? 0u : n_take - tid * share < share ? n_take - tid * share : share;
+                    const uint32_t mbar = map_rank(a_mbar + 8u * g, tid + 1u);
+                    send_async(map_rank(smem_u32(smem) + 8u * g * step_rows(K, copying), tid + 1u), (int32_t)n, 0, mbar);
                     arrive_expect(mbar, 8u * (n + 1u));
                 }
             }
@@ -364,9 +365,10 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
                     s_node[j].x = (uint32_t)x;
                     s_life[j] = (int8_t)L;
                     if constexpr (CLUSTER) {
-                        const uint32_t to = 1u + k % STEP_COPYING;
-                        send_async(map_rank(smem_u32(smem) + 8u * (g * step_rows(K) + 1u + k / STEP_COPYING), to), x, j,
-                                   map_rank(a_mbar + 8u * g, to));
+                        const uint32_t to = CAP == STEP_FEW_TABLES ? k % copying : k / share;
+                        const uint32_t at = CAP == STEP_FEW_TABLES ? k / copying : k - to * share;
+                        send_async(map_rank(smem_u32(smem) + 8u * (g * step_rows(K, copying) + 1u + at), to + 1u), x, j,
+                                   map_rank(a_mbar + 8u * g, to + 1u));
                     } else {
                         list[list_off + k] = make_int2(x, j);
                     }
@@ -428,24 +430,38 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
     stage_one<SPT, IPT, false>(p, blockIdx.x, gridDim.x, smem);
 }
 
-// A small call in one kernel: a cluster of eight blocks per table.  The first block runs Stage One; the others copy the
+// A call in one kernel: a cluster of two to eight blocks per table.  The first block runs Stage One; the others copy the
 // misses of every token as soon as it is placed, in either mode.  What it saves is a launch (1.8 us of host time, which
 // bounds the smallest calls), the way from the end of one grid to the start of the next, and the hand-over through global
 // memory with its fences: Stage One sends every miss (id, slot) straight into the shared memory of the block that will copy
-// it, where an mbarrier per token counts the bytes, and goes on.  Every table's misses have seven SMs of their own, whose
-// warps keep 140 KB of rows on the way: one table alone can fill the link (2 us round trip x 47 GB/s).  Measured with
-// two kernels / in one whose blocks met at a cluster barrier per token / in this one: K = 256, S = 1024 8.4 / 6.5 / 5.8 us;
-// K = 2048, S = 8192, two tokens, 230 rows 17.2 / 13.3 / 12.2, from a captured graph 19.8 / 19.3 / 18.3; eight tables,
-// K = 1000, S = 4096, 1230 rows of 1152 bytes 40.8 / 36.0 / 35.3.
-template <int SPT, int IPT>
-__global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constant__ StepParams p)
+// it, where an mbarrier per token counts the bytes, and goes on.  A copying block keeps 20 KB of rows on the way, so that
+// seven can fill the link with one table's rows (2 us round trip x 47 GB/s) and the other sizes with what runs beside it.
+// Measured, in two kernels (Stage Two overlapped where that is faster) / in this one, us per call:
+//   K = 256, S = 1024, one table 8.4 / 5.8;  K = 2048, S = 8192, two tokens, one table 17.2 / 12.2, from a graph 19.8 / 18.3;
+//   the same with 4, 8, 16, 32, 48, 64 tables 26.2 / 22.4, 39.0 / 35.6, 65.9 / 63.6, 119.9 / 116.8, 174.0 / 173.6, 228.3 / 226.8;
+//   the same from 11 GB of host memory with 8, 16, 32, 48, 64 tables 51 / 46, 88 / 84, 173 / 155, 242 / 229, 315 / 296.
+// The last line is what the end of a call is for.  Where a table's pages are spread over much host memory, translating
+// their addresses limits the rows, and a cluster, which lies in one GPC, finds its table's translations there if the
+// table was there in the call before.  So calls of more than a few tables let the next grid start only when their
+// blocks exit: its clusters then find the same SMs free, in the same order.  Started early they take whatever is free at
+// that time: eight tables 60 us and not 46, 16 113 and not 84 (step_early() says which calls gain by it).
+// FEW (eight blocks): up to 20 rows a block, which a warp each has under way at once: the tokens' rows follow one another
+// without a meeting of the warps, and go round over the blocks (one table 12.0 us; meeting, with shares 12.35).  Otherwise
+// a block's warps meet before the next token's rows, and its rows are neighbours (16 tables, 11 GB: 84.0 us against 84.3
+// and 86.0 with one of the two; 40 tables 193 against 203 and 199).
+template <int SPT, int IPT, int CAP>
+__global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constant__ S1ParamsT<CAP> p)
 {
+    constexpr bool FEW = CAP == STEP_FEW_TABLES;
     extern __shared__ __align__(16) unsigned char smem[];              // of a copying block: the words that it gets, by token
-    __shared__ __align__(8) unsigned long long s_mbar[STEP_MAX_TOKENS];
-    const uint32_t rank = cluster_rank(), ti = blockIdx.x / STEP_CLUSTER, lane = threadIdx.x & 31u;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (rank != 0 && threadIdx.x < p.n_q)
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n\tfence.mbarrier_init.release.cluster;" :: "r"(smem_u32(s_mbar + threadIdx.x)) : "memory");
+    __shared__ __align__(8) unsigned long long s_mbar[STEP_MAX_TOKENS], s_meet[STEP_MAX_TOKENS];
+    const uint32_t rank = cluster_rank(), cluster = FEW ? STEP_FEW_CLUSTER : cluster_size(), copying = cluster - 1u;
+    const uint32_t ti = blockIdx.x / cluster, lane = threadIdx.x & 31u, W = blockDim.x >> 5, warp = threadIdx.x >> 5;
+    if (p.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (rank != 0 && threadIdx.x < p.n_q) {
+        mbar_init(smem_u32(s_mbar + threadIdx.x), 1u);
+        if (!FEW) mbar_init(smem_u32(s_meet + threadIdx.x), W);
+    }
     __syncthreads();
     cluster_arrive();
     if (rank == 0) {
@@ -453,23 +469,22 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
         if (p.out.n_slots) cluster_arrive();                           // the outputs are written
         return;
     }
-    const uint32_t cpr = p.row_bytes >> 4, W = blockDim.x >> 5, warp = threadIdx.x >> 5;
+    const uint32_t cpr = p.row_bytes >> 4;
     const uint64_t src = p.kv_base[ti], stride = p.kv_stride[ti];
     const uint64_t dst = reinterpret_cast<uint64_t>(p.buffer + (size_t)p.table_id[ti] * p.S * p.row_bytes);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     cluster_wait();
     if (p.out.n_slots) cluster_arrive();
-    uint32_t from = 0;                                                 // the warp that is next
-    for (uint32_t g = 0; g < p.n_q; ++g) {
-        const int2* got = reinterpret_cast<const int2*>(smem) + g * step_rows(p.K);
-        const uint32_t mbar = smem_u32(s_mbar + g);
+    auto wait_for = [&](uint32_t mbar) -> bool {                       // (Stage One's loops are bounded, far below this)
         uint32_t spin = 0;
         while (!mbar_done(mbar) && ++spin < STEP_SPIN_LIMIT) {}
-        if (spin == STEP_SPIN_LIMIT) {                                 // (Stage One's loops are bounded, far below this)
-            if (lane == 0) atomicOr(p.status, ST_WAIT_TIMEOUT);
-            break;
-        }
-        __syncwarp();
+        if (spin == STEP_SPIN_LIMIT && lane == 0) atomicOr(p.status, ST_WAIT_TIMEOUT);
+        return __all_sync(0xffffffffu, spin < STEP_SPIN_LIMIT);
+    };
+    uint32_t from = 0;                                                 // the warp that is next
+    for (uint32_t g = 0; g < p.n_q; ++g) {
+        const int2* got = reinterpret_cast<const int2*>(smem) + g * step_rows(p.K, copying);
+        if (!wait_for(smem_u32(s_mbar + g))) break;
         const uint32_t count = (uint32_t)got[0].x;
         for (uint32_t k = warp >= from ? warp - from : warp + W - from; k < count; k += W) {
             const int2 e = got[1u + k];
@@ -479,11 +494,17 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
             }
             copy_row(src + (uint64_t)(uint32_t)e.x * stride, dst + (uint64_t)(uint32_t)e.y * p.row_bytes, cpr, lane);
         }
-        from = (from + count) % W;
+        if (FEW || count < W) {
+            from = (from + count) % W;
+        } else if (g + 1u < p.n_q) {                                   // the warps meet
+            from = 0;
+            if (lane == 0) mbar_arrive(smem_u32(s_meet + g));
+            if (!wait_for(smem_u32(s_meet + g))) break;
+        }
     }
     if (p.out.n_slots) {
         cluster_wait();
-        put_outputs_of(p.out, ti, p.n_q * p.K, p.n_q, warp * STEP_COPYING + rank - 1u, W * STEP_COPYING, lane);
+        put_outputs_of(p.out, ti, p.n_q * p.K, p.n_q, warp * copying + rank - 1u, W * copying, lane);
     }
 }
 
@@ -858,12 +879,18 @@ cudaError_t stage_one_prepare(size_t max_smem)
         reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 2, S1_BIG_TABLES>),
         reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 4, S1_BIG_TABLES>),
         reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 8, S1_BIG_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<2, 2>),
-        reinterpret_cast<const void*>(avsg_step_kernel<4, 2>),
-        reinterpret_cast<const void*>(avsg_step_kernel<4, 4>),
-        reinterpret_cast<const void*>(avsg_step_kernel<8, 2>),
-        reinterpret_cast<const void*>(avsg_step_kernel<8, 4>),
-        reinterpret_cast<const void*>(avsg_step_kernel<8, 8>),
+        reinterpret_cast<const void*>(avsg_step_kernel<2, 2, STEP_FEW_TABLES>),
+        reinterpret_cast<const void*>(avsg_step_kernel<4, 2, STEP_FEW_TABLES>),
+        reinterpret_cast<const void*>(avsg_step_kernel<4, 4, STEP_FEW_TABLES>),
+        reinterpret_cast<const void*>(avsg_step_kernel<8, 2, STEP_FEW_TABLES>),
+        reinterpret_cast<const void*>(avsg_step_kernel<8, 4, STEP_FEW_TABLES>),
+        reinterpret_cast<const void*>(avsg_step_kernel<8, 8, STEP_FEW_TABLES>),
+        reinterpret_cast<const void*>(avsg_step_kernel<2, 2, STEP_MAX_TABLES>),
+        reinterpret_cast<const void*>(avsg_step_kernel<4, 2, STEP_MAX_TABLES>),
+        reinterpret_cast<const void*>(avsg_step_kernel<4, 4, STEP_MAX_TABLES>),
+        reinterpret_cast<const void*>(avsg_step_kernel<8, 2, STEP_MAX_TABLES>),
+        reinterpret_cast<const void*>(avsg_step_kernel<8, 4, STEP_MAX_TABLES>),
+        reinterpret_cast<const void*>(avsg_step_kernel<8, 8, STEP_MAX_TABLES>),
         reinterpret_cast<const void*>(avsg_stage_one_paper_kernel)};
     for (const void* k : kernels) {
         cudaFuncAttributes fa;
@@ -927,7 +954,6 @@ cudaError_t launch_stage_one(const S1Params& p, uint32_t n_tables, cudaStream_t 
     return cudaLaunchKernelEx(&cfg, avsg_stage_one_paper_kernel, p);
 }
 
-namespace {
 // At least 16 warps a block where the table has the slots for it: they copy.
 uint32_t step_threads(uint32_t S, uint32_t K)
 {
@@ -935,26 +961,28 @@ uint32_t step_threads(uint32_t S, uint32_t K)
     return t > most ? t : most;
 }
 
-const void* step_kernel(uint32_t S, uint32_t K)
+namespace {
+
+template <int CAP>
+const void* step_kernel(uint32_t spt, uint32_t ipt)
 {
-    const uint32_t nt = step_threads(S, K), ipt = (K + nt - 1) / nt;
-    switch (S / nt) {
-        case 8:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 2>)
-                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 4>)
-                                 : reinterpret_cast<const void*>(avsg_step_kernel<8, 8>);
-        case 4:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<4, 2>)
-                                 : reinterpret_cast<const void*>(avsg_step_kernel<4, 4>);
-        default: return reinterpret_cast<const void*>(avsg_step_kernel<2, 2>);
+    switch (spt) {
+        case 8:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 2, CAP>)
+                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 4, CAP>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<8, 8, CAP>);
+        case 4:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<4, 2, CAP>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<4, 4, CAP>);
+        default: return reinterpret_cast<const void*>(avsg_step_kernel<2, 2, CAP>);
     }
 }
 
-void step_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, uint32_t n_tables, uint32_t threads, size_t smem)
+void step_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, uint32_t n_tables, uint32_t cluster, uint32_t threads, size_t smem)
 {
-    cfg.gridDim = dim3(n_tables * STEP_CLUSTER);
+    cfg.gridDim = dim3(n_tables * cluster);
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = STEP_CLUSTER;
+    attr[0].val.clusterDim.x = cluster;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
@@ -962,32 +990,36 @@ void step_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, uint32_t n_
 }
 }  // namespace
 
-bool step_possible(size_t max_smem)
+StepClusters step_clusters(size_t max_smem)
 {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[2];
-    step_config(cfg, attr, 1, 1024, max_smem - 1024);
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(avsg_step_kernel<8, 2>), &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
+    StepClusters s;
+    for (uint32_t cl : {2u, 3u, 4u, STEP_FEW_CLUSTER}) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[2];
+        int fit = 0;
+        step_config(cfg, attr, 1, cl, 1024, max_smem - 2048);      // (the largest; statically it has 1 KB)
+        if (cudaOccupancyMaxActiveClusters(&fit, step_kernel<STEP_MAX_TABLES>(8, 2), &cfg) != cudaSuccess) { cudaGetLastError(); fit = 0; }
+        s.fit[cl] = (uint32_t)fit;
     }
-    return n > 0;
+    return s;
 }
 
-cudaError_t launch_step(const StepParams& p, cudaStream_t stream)
+template <int CAP>
+cudaError_t launch_step(const S1ParamsT<CAP>& p, uint32_t cluster, cudaStream_t stream)
 {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     const uint32_t nt = step_threads(p.S, p.K);
-    step_config(cfg, attr, p.n_launch, nt, s1_layout(p.S, p.K, p.n_q, nt).total);      // (holds step_rows() n_q times)
+    step_config(cfg, attr, p.n_launch, cluster, nt, s1_layout(p.S, p.K, p.n_q, nt).total);      // (holds step_rows() n_q times)
     cfg.stream = stream;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = 2;
-    void* args[] = {const_cast<StepParams*>(&p)};
-    return cudaLaunchKernelExC(&cfg, step_kernel(p.S, p.K), args);
+    void* args[] = {const_cast<S1ParamsT<CAP>*>(&p)};
+    return cudaLaunchKernelExC(&cfg, step_kernel<CAP>(p.S / nt, (p.K + nt - 1) / nt), args);
 }
+template cudaError_t launch_step(const StepParams& p, uint32_t cluster, cudaStream_t stream);
+template cudaError_t launch_step(const StepParamsFew& p, uint32_t cluster, cudaStream_t stream);
 
 cudaError_t launch_stage_one(const S1ParamsBig& p, uint32_t n_tables, cudaStream_t stream)
 {

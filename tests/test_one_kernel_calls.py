@@ -1,6 +1,6 @@
-"""Small calls, which one kernel serves: calls whose number of tables, tokens and ids changes from one to the next, among
-calls that take two kernels, resets and a restored snapshot, queued without a wait; both modes, host buffers, the signal word, a captured
-call; compared with the oracle (whole numbers and bytes: nothing to tolerate)."""
+"""Calls that one kernel serves: calls whose number of tables, tokens and ids changes from one to the next, among calls
+that take two kernels, resets and a restored snapshot, queued without a wait; every cluster size; both modes, host buffers,
+the signal word, a captured call; compared with the oracle (whole numbers and bytes: nothing to tolerate)."""
 import numpy as np
 import pytest
 
@@ -67,6 +67,39 @@ def test_calls_of_changing_size(S, K_max, cluster):
         assert (ctx.buffer(t).cpu().numpy() == orc[t].rows()).all(), t
         tok, life = ctx.export_state(t)
         assert (tok == orc[t].export_state()[0]).all() and (life == orc[t].export_state()[1]).all(), t
+    assert ctx.sync_status() == 0
+
+
+# The most tables that get clusters of eight, four, three and two blocks on a device of 148 SMs, and one more than that;
+# more rows per block and token than warps, fewer, and none
+@pytest.mark.parametrize("n", [4, 8, 9, 33, 34, 45, 46, 74, 75])
+def test_clusters_of_every_size(n):
+    import torch
+    import paper_2609_37538_b200 as avsg
+    S, K, n_q, L = 1024, 200, 3, 3
+    rng = np.random.default_rng(n)
+    kv = _kv(avsg)
+    ctx = avsg.Context(n, S, RB, K, n_q, L)
+    orc = [OracleTable(S, RB, L) for _ in range(n)]
+    done = []
+    for c in range(8):
+        tabs = [int(t) for t in rng.permutation(n)]
+        if c == 4:
+            tabs = tabs[:2]                              # a small one between the large ones
+        ctx.set_transfer_mode(avsg.XFER_SM_OVERLAP if c % 2 else avsg.XFER_SM_BALANCED)
+        X = np.stack([[rng.choice(rng.choice([K, 260, 3000]), K, replace=False) for _ in range(n_q)] for _ in tabs]).astype(np.int32)
+        X = done[-1][1] if c == 6 else X                 # (other tables, the same ids)
+        host = c in (2, 5)
+        ids = torch.from_numpy(X).pin_memory() if host else torch.from_numpy(X).cuda()
+        done.append((tabs, X, (ctx.step_host if host else ctx.step)(tabs, ids, [kv] * len(tabs), [2990] * len(tabs))))
+    torch.cuda.synchronize()
+    for c, (tabs, X, out) in enumerate(done):
+        for a, t in enumerate(tabs):
+            r = orc[t].step(X[a], 2990, kv.numpy(), RB)
+            assert (out.slots[a].cpu().numpy() == r.O).all() and (out.hit[a].cpu().numpy() == r.M).all(), (c, t)
+            assert (out.miss_count[a].cpu().numpy() == r.n).all(), (c, t)
+    for t in range(n):
+        assert (ctx.buffer(t).cpu().numpy() == orc[t].rows()).all(), t
     assert ctx.sync_status() == 0
 
 
