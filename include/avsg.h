@@ -75,7 +75,9 @@ extern "C" {
                                        slots, nor with stage_one_done above three tables).
                                        Its blocks take whole SMs while they run: who wants
                                        room for other kernels beside the call sets a
-                                       transfer geometry                                 */
+                                       transfer geometry.  Calls whose Stage One takes
+                                       more than half of the SMs are served as in
+                                       AVSG_XFER_SM_OVERLAP                              */
 #define AVSG_XFER_COPY_ENGINE   1u  /* comparator: miss list read back, one async copy
                                        per run of consecutive rows on the copy engine    */
 #define AVSG_XFER_REQUEST_LEVEL 2u  /* comparator S1: one thread block per request       */

@@ -265,6 +265,13 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     // that one), else the large one
     const uint32_t chunk = (n <= (uint32_t)S1_MAX_TABLES || mode == AVSG_XFER_ALL_K || c->cfg.index_mode == AVSG_INDEX_PAPER)
                                ? (uint32_t)S1_MAX_TABLES : (uint32_t)S1_BIG_TABLES;
+    // With a Stage One block per table on most of the SMs, the blocks of a transfer kernel behind it crowd onto the rest: a
+    // balanced call of that many tables is served like an overlapped one, in rounds (below).  128 tables with 2.8, 5.5, 11
+    // GB of host memory 414, 575, 743 us behind Stage One, 393, 426, 443 in rounds; 80 tables 251 and 250; from and to
+    // host memory 80, 96, 128 tables 316, 375, 537 and 305, 365, 487.
+    if (mode == AVSG_XFER_SM_BALANCED && n > (uint32_t)c->sm_count / 2 && c->s1_cluster == 1 && c->cfg.index_mode != AVSG_INDEX_PAPER &&
+        !host_io && !c->timing && !c->geometry_set)
+        mode = AVSG_XFER_SM_OVERLAP;
     if (mode == AVSG_XFER_SM_OVERLAP && (n > chunk || n_q > (uint32_t)OVERLAP_MAX_TOKENS))
         mode = AVSG_XFER_SM_BALANCED;                  // the overlapped kernel pairs with ONE Stage One launch
     // The overlapped transfer grid shares the GPU with the Stage One grid it waits for.  When Stage One's blocks
