@@ -230,10 +230,12 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     // Host buffers.  Page-locked ones are used by the kernels themselves: Stage One reads the ids in place and Stage Two
     // writes the outputs back, so that the calls of a stream follow one another as launches do, without an event between
     // them (measured with 32 tables: see put_outputs()).  Pageable ones, the paper-literal kernel and the comparators
-    // go through copies on a side stream.
+    // go through copies on a side stream, and so do tables of several Stage One blocks, each of which would read all ids
+    // from the host (S = 16384 with 38, 50, 64 tables 168, 210, 263 us by copies, 219, 285, 372 in place; S = 32768, four
+    // tokens, 16 tables 146 and 306; only one to four tables were quicker in place).
     HostOut out;
     bool host_ids = false;
-    if (host_io && c->cfg.index_mode != AVSG_INDEX_PAPER &&
+    if (host_io && c->cfg.index_mode != AVSG_INDEX_PAPER && c->s1_cluster == 1 &&
         (c->cfg.transfer_mode == AVSG_XFER_SM_BALANCED || c->cfg.transfer_mode == AVSG_XFER_SM_OVERLAP)) {
         const int32_t* ids = mapped(a->indices);
         out.host_slots = mapped(a->slots);
@@ -322,6 +324,10 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
         p.K = K; p.n_q = n_q; p.L = (uint32_t)c->cfg.max_lifetime;
         p.first = first; p.list_stride = c->list_stride;
         p.n_launch = cnt;
+        // A transfer grid that is placed while Stage One holds nearly all SMs crowds onto the others: it has to wait then
+        // (S = 16384, two blocks a table, not overlapped, 64 and 72 tables: 334, 311 us and 233, 259 where it waits; with 50
+        // tables 186 and 185).
+        p.early = cnt * c->s1_cluster <= (uint32_t)c->sm_count * 3u / 4u;
         p.qword = c->d_q; p.probe_retries = c->cfg.probe_retries; p.hash_a1 = c->cfg.hash_a1; p.hash_a2 = c->cfg.hash_a2;
         p.t_range = c->timing ? c->d_trange : nullptr;
         p.verified_len_dev = a->verified_len_dev;

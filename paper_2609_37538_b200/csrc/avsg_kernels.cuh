@@ -122,7 +122,7 @@ struct S1ParamsT {
     unsigned long long  host_seq = 0;
     uint32_t            expect = 0;             // Stage One blocks that place tables of the call
     HostOut             out;                    // a call in one kernel: what its Stage Two writes to the host
-    uint32_t            early = 0;              // a call in one kernel: the next grid may start under it
+    uint32_t            early = 1;              // the next grid may start under this one (with flags it has to)
     uint32_t            host_ids = 0;           // indices is mapped host memory that holds the ids when the call is made
     const int32_t* verified_len_dev = nullptr;  // [n] of the call: read instead of verified_len[] when set
     uint32_t table_id[CAP];

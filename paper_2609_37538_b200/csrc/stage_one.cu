@@ -267,7 +267,7 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
                 if (lane == 0 && valid) atomicAdd(s_sum, valid);
             }
             if (lane == 0) s_tot[par + warp] = wmiss;
-            if (!CLUSTER && g == 0 && bt == block) start_dependents(seen);
+            if (!CLUSTER && g == 0 && bt == block && (p.flags || p.early)) start_dependents(seen);
             __syncthreads();
 
             // ---- CollectDead and the misses, each in order; the prefix over the warps: lane l looks at warp l ----

@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_cluster_kernel(const _
 #pragma unroll
         for (int k = 0; k < IPT; ++k) {
             const uint32_t i = (w0 + warp * IPT + k) * 32u + lane;
-            xs[k] = i < K ? (p.host_ids ? __ldcv(ids + (size_t)g * K + i) : __ldcg(ids + (size_t)g * K + i)) : -1;
+            xs[k] = i < K ? __ldcg(ids + (size_t)g * K + i) : -1;
         }
     };
     auto revive = [&](uint32_t j, uint32_t par) -> bool {        // the slot is no longer dead; false: it was not
@@ -123,7 +123,6 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_cluster_kernel(const _
     if (tid < 2u * MAX_CL) s_rev[tid] = 0;
     if (tid < 3u * (2u + MAX_CL)) s_cnt[tid] = 0;
     cluster_arrive();                                            // what the other blocks write to is ready (waited for below)
-    if (p.host_ids) load_ids(0, 0);                              // (see the single-block kernel)
 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (p.t_range && tid == 0) atomicMin(p.t_range, global_ns());
@@ -135,7 +134,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_cluster_kernel(const _
     for (int q = 0; q < NV; ++q)
         if (tid + q * nt < Sc / 4) t4[q] = __ldcg(reinterpret_cast<const int4*>(g_tok) + tid + q * nt);
     life_words<SPT, true>(g_life + j0, own, w);
-    if (!p.host_ids) load_ids(0, 0);
+    load_ids(0, 0);
     if (p.verified_len_dev) N = __ldg(p.verified_len_dev + ti);
     const uint32_t seen = take_flags_down(p, bt, gridDim.x, rank == 0 ? p.n_launch : 0u);      // (a cluster serves one table)
     cluster_wait();                                              // (the index is empty, too)
@@ -249,7 +248,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_cluster_kernel(const _
             if (lane == 0 && valid) atomicAdd(s_sum, valid);
         }
         if (!last) load_ids(g + 1, 0);                                 // arrives while this token's misses are placed
-        if (g == 0) start_dependents(seen);
+        if (g == 0 && (p.flags || p.early)) start_dependents(seen);
         cluster_sync();
 
         // ---- the token's misses, and the dead slots of the blocks ----
@@ -359,7 +358,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_cluster_kernel(const _
             if (m == 0 || i >= K) { atomicOr(p.status, ST_BAD_SLOT); continue; }
             int32_t j = -1;
             if (k < mine) {
-                const int32_t x = p.host_ids ? __ldcv(ids + (size_t)g * K + i) : __ldcg(ids + (size_t)g * K + i);
+                const int32_t x = __ldcg(ids + (size_t)g * K + i);
                 const uint32_t jl = s_dead[k];
                 j = (int32_t)(j_base + jl);
                 s_node[jl].x = (uint32_t)x;
