@@ -35,8 +35,7 @@ METRIC = "miss-only H2D gather GB/s (% of link peak); match+reserve us per decod
 # DRAM traffic per unit from the ncu capture summarised under profiles/ (dram__bytes_read + dram__bytes_write
 # per launch of the one-layer case, divided by the units of that launch); scaled by the units of a launch here.
 NCU_XFER_DRAM_BYTES_PER_ROW = 91.0          # 0.94 MB per launch of 10.3 k rows: the written rows stay in L2
-NCU_S1_DRAM_BYTES_PER_TABLE = {"hash": 59400.0,     # 1.90 MB per launch of 32 tables
-                               "direct": 174000.0}  # 5.57 MB: the 2-byte index entries arrive as 32-byte sectors
+NCU_S1_DRAM_BYTES_PER_TABLE = 59400.0       # 1.90 MB per launch of 32 tables (state and ids in; the writes stay in L2)
 PAPER_CONTEXT = {
     "hardware": "Ascend 910B NPU (paper), not comparable",
     "hash_vs_dual_pointer_speedup": 2.80, "stage_one_us_K2048_S2048": 53.7,
@@ -436,8 +435,6 @@ def run_cuda(args):
     # Stage One algorithmic bytes per call: state read + write, ids in, slots out, miss counts, miss list
     n_tab = len(w.calls[0])
     s1_bytes = n_tab * (2 * w.buffer_slots * 5 + 2 * w.n_q * w.topk * 4 + w.n_q * 4 + 32) + 8 * sum(x_rows) / n_launch
-    if direct:      # direct index: one 2-byte entry read per id, one written per miss
-        s1_bytes += n_tab * w.n_q * w.topk * 2 + 2 * sum(x_rows) / n_launch
     s1_avg_us = sum(s1_us) / len(s1_us)
     s1_gbs = s1_bytes / 1e3 / s1_avg_us
 
@@ -525,9 +522,9 @@ def run_cuda(args):
                              "in L2 after the write, so DRAM traffic (scaled from the ncu capture of the one-layer case) is small; "
                              "timed in balanced mode (one kernel at a time); the timed steps copy each token's rows while "
                              "Stage One still runs"},
-        "roofline_stage_one": {"bound": "hbm", "kernel": ("avsg_stage_one_cluster_kernel<%s>" if w.buffer_slots > 8192 or args.cluster > 1
-                                                          else "avsg_stage_one_kernel<%s>") % args.index, "achieved": s1_gbs, "peak": hbm_peak,
-                               "unit": "GB/s", "frac": s1_gbs / hbm_peak, "traffic": NCU_S1_DRAM_BYTES_PER_TABLE[args.index] * n_tab,
+        "roofline_stage_one": {"bound": "hbm", "kernel": "avsg_stage_one_cluster_kernel" if w.buffer_slots > 8192 or args.cluster > 1
+                                                         else "avsg_stage_one_kernel", "achieved": s1_gbs, "peak": hbm_peak,
+                               "unit": "GB/s", "frac": s1_gbs / hbm_peak, "traffic": NCU_S1_DRAM_BYTES_PER_TABLE * n_tab,
                                "peak_kind": peak_kind,
                                "bytes_per_launch": s1_bytes},
         "paper_context": PAPER_CONTEXT,
@@ -1215,7 +1212,7 @@ def main():
                          "cluster per table, e.g. --buffer-slots 16384 --n-tokens 4 for an MTP-3 deployment")
     ap.add_argument("--n-tokens", type=int, default=0, help="query tokens per iteration (0 = the configuration's 2)")
     ap.add_argument("--index", default="direct", choices=["hash", "direct"],
-                    help="Stage One index: direct-address table in device memory (default) or shared-memory hash table")
+                    help="Stage One index mode (the same index in shared memory; direct, the default, bounds the ids)")
     ap.add_argument("--stage-two", default="overlap", choices=["balanced", "overlap"],
                     help="overlap: Stage Two starts on token g's misses while Stage One places token g+1; balanced: it "
                          "starts when Stage One is complete (the per-kernel figures are always taken in balanced mode, "
