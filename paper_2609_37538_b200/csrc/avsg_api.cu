@@ -232,10 +232,15 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     // them (measured with 32 tables: see put_outputs()).  Pageable ones, the paper-literal kernel and the comparators
     // go through copies on a side stream, and so do tables of several Stage One blocks, each of which would read all ids
     // from the host (S = 16384 with 38, 50, 64 tables 168, 210, 263 us by copies, 219, 285, 372 in place; S = 32768, four
-    // tokens, 16 tables 146 and 306; only one to four tables were quicker in place).
+    // tokens, 16 tables 146 and 306; only one to four tables were quicker in place).  So do calls of more than a few
+    // tables and several tokens whose ids do not begin on 64-byte boundaries: the link moves them in parts of lines, and
+    // the tokens wait for one another's.  32 tables in place / by copies: K = 256, 272 (four tokens) 42, 44 / 62, 65; K =
+    // 257, 260 92, 70 / 63, 63; K = 500, 1001 (two tokens) 62, 108 / 57, 78; K = 257 (one token) 27.6 / 27.8; eight
+    // tables, K = 257, four tokens 34.7 / 41.7.
     HostOut out;
     bool host_ids = false;
-    if (host_io && c->cfg.index_mode != AVSG_INDEX_PAPER && c->s1_cluster == 1 &&
+    const bool whole_lines = K % 16u == 0 || n_q == 1 || n <= (uint32_t)STEP_FEW_TABLES;
+    if (host_io && c->cfg.index_mode != AVSG_INDEX_PAPER && c->s1_cluster == 1 && whole_lines &&
         (c->cfg.transfer_mode == AVSG_XFER_SM_BALANCED || c->cfg.transfer_mode == AVSG_XFER_SM_OVERLAP)) {
         const int32_t* ids = mapped(a->indices);
         out.host_slots = mapped(a->slots);

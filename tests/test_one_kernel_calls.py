@@ -72,11 +72,12 @@ def test_calls_of_changing_size(S, K_max, cluster):
 
 # The most tables that get clusters of eight, four, three and two blocks on a device of 148 SMs, and one more than that;
 # more rows per block and token than warps, fewer, and none
-@pytest.mark.parametrize("n", [4, 8, 9, 33, 34, 45, 46, 74, 75])
-def test_clusters_of_every_size(n):
+# (the host's ids and outputs are used in place where K is a multiple of 16 or the tables are few)
+@pytest.mark.parametrize("n,K", [(4, 200), (8, 201), (9, 200), (9, 208), (33, 208), (34, 200), (45, 208), (46, 208), (74, 208), (75, 208)])
+def test_clusters_of_every_size(n, K):
     import torch
     import paper_2609_37538_b200 as avsg
-    S, K, n_q, L = 1024, 200, 3, 3
+    S, n_q, L = 1024, 3, 3
     rng = np.random.default_rng(n)
     kv = _kv(avsg)
     ctx = avsg.Context(n, S, RB, K, n_q, L)
