@@ -374,6 +374,9 @@ int avsg_set_transfer_geometry(avsg_ctx *ctx, uint32_t blocks, uint32_t threads)
  *   tok    int32 [n][buffer_slots]  cached id per slot; a new table is all -1
  *   life   int8  [n][buffer_slots]  lifetime per slot;  a new table is all -1
  *   buffer bytes [n][buffer_slots * row_bytes]  the KV rows attention reads
+ * buffer begins on a 16-byte boundary; every other array wherever its element
+ * type may (state on 16-byte (tok) and 8-byte (life) boundaries is read in
+ * wider pieces).
  * Results are the same, bit for bit, as avsg_step on a context in the same
  * state.
  */

@@ -246,9 +246,18 @@ bool step_early(const S1ParamsT<CAP>& p)
     return bytes <= STEP_EARLY_BYTES;
 }
 uint32_t step_threads(uint32_t S, uint32_t K);
+// State that Stage One can read in pieces of 16 (ids) and 8 bytes (lifetimes).  A context's is; a caller's own may begin at
+// any id and any lifetime (S is a multiple of 32, so that what holds for the first table holds for all).  Such a call takes
+// two kernels, whose Stage One reads element by element: a test of the alignment inside the kernels made every call slower
+// (one table 12.1 us, with it 12.6).
+inline bool state_is_aligned(const int32_t* tok, const int8_t* life)
+{
+    return reinterpret_cast<uint64_t>(tok) % 16u == 0 && reinterpret_cast<uint64_t>(life) % 8u == 0;
+}
 // StepParamsFew: up to STEP_FEW_TABLES tables of STEP_FEW_CLUSTER blocks
 template <int CAP> cudaError_t launch_step(const S1ParamsT<CAP>& p, uint32_t cluster, cudaStream_t stream);
-// n_blocks thread blocks serve the p.n_launch tables of the launch (one block per table unless the call runs in rounds)
+// n_blocks thread blocks serve the p.n_launch tables of the launch (one block per table unless the call runs in rounds);
+// state that is not aligned: with the small argument block only
 cudaError_t launch_stage_one(const S1Params& p, uint32_t n_blocks, cudaStream_t stream);
 cudaError_t launch_stage_one(const S1ParamsBig& p, uint32_t n_blocks, cudaStream_t stream);   // hash / direct index only
 // Stage One with one table per thread-block cluster of C blocks (C = 2, 4 or 8; hash / direct index only)

@@ -119,7 +119,7 @@ extern "C" int avsg_step_noalloc(const avsg_noalloc_args* a, void* cuda_stream)
         }
         return AVSG_OK;
     };
-    const uint32_t cluster = a->n_tokens <= STEP_MAX_TOKENS ? g_step_clusters[dev].of(a->n, step_threads(a->buffer_slots, a->topk)) : 0u;
+    const uint32_t cluster = a->n_tokens <= STEP_MAX_TOKENS && state_is_aligned(a->tok, a->life) ? g_step_clusters[dev].of(a->n, step_threads(a->buffer_slots, a->topk)) : 0u;
     if (cluster) {
         auto step = [&](auto&& p) -> int {               // one kernel for both stages
             if ((rc = fill(p)) != AVSG_OK) return rc;

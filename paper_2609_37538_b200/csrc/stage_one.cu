@@ -75,8 +75,8 @@ __device__ __forceinline__ uint32_t step_rows(uint32_t K, uint32_t copying) { re
 // SPT slots per thread (a power of two): S <= SPT * blockDim.x.  IPT: the most ids a thread has to look up per token
 // (K <= S, so SPT is always enough).  CAP: tables the argument block has room for.  The block serves the tables block,
 // block + blocks, ... of the launch.  CLUSTER: it is the first block of a cluster whose others copy what it places
-// (avsg_step_kernel); a_mbar: their mbarriers, one per token.
-template <int SPT, int IPT, bool CLUSTER, int CAP>
+// (avsg_step_kernel); a_mbar: their mbarriers, one per token.  WIDE: the state is aligned (state_is_aligned()).
+template <int SPT, int IPT, bool CLUSTER, bool WIDE, int CAP>
 __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_t block, const uint32_t blocks, unsigned char* smem, const uint32_t a_mbar = 0)
 {
     const uint32_t copying = CAP == STEP_FEW_TABLES ? STEP_FEW_CLUSTER - 1u : CLUSTER ? cluster_size() - 1u : 1u;
@@ -149,8 +149,12 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
         uint32_t w[NV];
 #pragma unroll
         for (int q = 0; q < NV; ++q)
-            if (tid + q * nt < S / 4) t4[q] = __ldcg(reinterpret_cast<const int4*>(g_tok) + tid + q * nt);
-        life_words<SPT, true>(g_life + j0, own, w);
+            if (tid + q * nt < S / 4) {
+                const int32_t* at = g_tok + 4u * (tid + q * nt);
+                if constexpr (WIDE) t4[q] = __ldcg(reinterpret_cast<const int4*>(at));
+                else t4[q] = make_int4(__ldcg(at), __ldcg(at + 1), __ldcg(at + 2), __ldcg(at + 3));
+            }
+        life_words<SPT, true, WIDE>(g_life + j0, own, w);
         if (!p.host_ids || bt != block) load_token(ti, 0);
         if (p.verified_len_dev) N = __ldg(p.verified_len_dev + ti);
         const uint32_t seen = !CLUSTER && bt == block ? take_flags_down(p, bt, blocks, p.n_launch) : 0u;
@@ -389,7 +393,7 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
 
         // ---- write back: lifetimes; resident ids that are no longer verified become empty (Alg. 4) ----
         life_words<SPT>(s_life + j0, own, w);
-        life_words_store<SPT>(g_life + j0, own, w);
+        life_words_store<SPT, WIDE>(g_life + j0, own, w);
         if (stale_ids) {
             for (uint32_t q = 0; q < NV; ++q)
                 for (uint32_t j = 4u * (tid + q * nt); j < 4u * (tid + q * nt) + 4u && j < S; ++j)
@@ -423,11 +427,11 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
     }
 }
 
-template <int SPT, int IPT, int CAP>
+template <int SPT, int IPT, int CAP, bool WIDE = true>
 __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_constant__ S1ParamsT<CAP> p)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    stage_one<SPT, IPT, false>(p, blockIdx.x, gridDim.x, smem);
+    stage_one<SPT, IPT, false, WIDE>(p, blockIdx.x, gridDim.x, smem);
 }
 
 // A call in one kernel: a cluster of two to eight blocks per table.  The first block runs Stage One; the others copy the
@@ -465,7 +469,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
     __syncthreads();
     cluster_arrive();
     if (rank == 0) {
-        stage_one<SPT, IPT, true>(p, ti, p.n_launch, smem, smem_u32(s_mbar));
+        stage_one<SPT, IPT, true, true>(p, ti, p.n_launch, smem, smem_u32(s_mbar));
         if (p.out.n_slots) cluster_arrive();                           // the outputs are written
         return;
     }
@@ -873,6 +877,9 @@ cudaError_t stage_one_prepare(size_t max_smem)
         reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 2, S1_MAX_TABLES>),
         reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 4, S1_MAX_TABLES>),
         reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 8, S1_MAX_TABLES>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<2, 2, S1_MAX_TABLES, false>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<4, 4, S1_MAX_TABLES, false>),
+        reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 8, S1_MAX_TABLES, false>),
         reinterpret_cast<const void*>(avsg_stage_one_kernel<2, 2, S1_BIG_TABLES>),
         reinterpret_cast<const void*>(avsg_stage_one_kernel<4, 2, S1_BIG_TABLES>),
         reinterpret_cast<const void*>(avsg_stage_one_kernel<4, 4, S1_BIG_TABLES>),
@@ -927,6 +934,13 @@ cudaError_t launch_stage_one_t(const S1ParamsT<CAP>& p, uint32_t n_blocks, cudaS
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const uint32_t ipt = (p.K + cfg.blockDim.x - 1) / cfg.blockDim.x;      // ids per thread
+    if constexpr (CAP == S1_MAX_TABLES)
+        if (!state_is_aligned(p.tok, p.life))
+            switch (p.S / cfg.blockDim.x) {
+                case 8:  return cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<8, 8, CAP, false>, p);
+                case 4:  return cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<4, 4, CAP, false>, p);
+                default: return cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<2, 2, CAP, false>, p);
+            }
     switch (p.S / cfg.blockDim.x) {
         case 8:  return ipt <= 2 ? cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<8, 2, CAP>, p)
                       : ipt <= 4 ? cudaLaunchKernelEx(&cfg, avsg_stage_one_kernel<8, 4, CAP>, p)

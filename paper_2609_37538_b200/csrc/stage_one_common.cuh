@@ -74,14 +74,20 @@ __device__ __forceinline__ uint32_t decay4(uint32_t w, uint32_t d)
 }
 
 // The lifetimes of a thread's SPT consecutive slots (2, 4 or 8), packed one signed byte each, four to a word; unused
-// bytes carry 0x7F (never counted, never dead).  GLOBAL: from global memory, past L1.
-template <int SPT, bool GLOBAL = false>
+// bytes carry 0x7F (never counted, never dead).  GLOBAL: from global memory, past L1; WIDE: `at` is a multiple of SPT.
+template <int SPT, bool GLOBAL = false, bool WIDE = true>
 __device__ __forceinline__ void life_words(const int8_t* at, bool own, uint32_t (&w)[(SPT + 3) / 4])
 {
 #pragma unroll
     for (int q = 0; q < (SPT + 3) / 4; ++q) w[q] = 0x7F7F7F7Fu;
     if (!own) return;
-    if constexpr (SPT == 8) {
+    if constexpr (!WIDE) {
+#pragma unroll
+        for (int k = 0; k < SPT; ++k) {
+            const uint32_t v = (uint8_t)__ldcg(reinterpret_cast<const signed char*>(at) + k);
+            w[k / 4] = (w[k / 4] & ~(0xFFu << (8 * (k & 3)))) | v << (8 * (k & 3));
+        }
+    } else if constexpr (SPT == 8) {
         const uint2 v = GLOBAL ? __ldcg(reinterpret_cast<const uint2*>(at)) : *reinterpret_cast<const uint2*>(at);
         w[0] = v.x; w[1] = v.y;
     } else if constexpr (SPT == 4) {
@@ -91,11 +97,15 @@ __device__ __forceinline__ void life_words(const int8_t* at, bool own, uint32_t 
     }
 }
 
-template <int SPT>
+template <int SPT, bool WIDE = true>
 __device__ __forceinline__ void life_words_store(int8_t* at, bool own, const uint32_t (&w)[(SPT + 3) / 4])
 {
     if (!own) return;
-    if constexpr (SPT == 8) *reinterpret_cast<uint2*>(at) = make_uint2(w[0], w[1]);
+    if constexpr (!WIDE) {
+#pragma unroll
+        for (int k = 0; k < SPT; ++k) at[k] = (int8_t)(w[k / 4] >> (8 * (k & 3)));
+    }
+    else if constexpr (SPT == 8) *reinterpret_cast<uint2*>(at) = make_uint2(w[0], w[1]);
     else if constexpr (SPT == 4) *reinterpret_cast<uint32_t*>(at) = w[0];
     else *reinterpret_cast<uint16_t*>(at) = (uint16_t)w[0];
 }

@@ -111,3 +111,39 @@ def test_lifetimes_above_the_maximum():
         assert (slots[0].cpu().numpy() == r.O).all() and (hit[0].cpu().numpy() == r.M).all(), t
         assert (tok_d[0].cpu().numpy() == c).all() and (life_d[0].cpu().numpy() == l).all(), t
         assert int(status.item()) == 0
+
+
+# slots per thread of two, four and eight; the last one takes two kernels
+@pytest.mark.parametrize("S,K,n_q", [(32, 8, 2), (256, 31, 3), (1024, 300, 2), (2048, 500, 2), (4096, 1000, 3), (8192, 2048, 2),
+                                     (256, 2, 70)])
+@pytest.mark.parametrize("tok_at,life_at", [(1, 0), (0, 1), (2, 2), (3, 4), (1, 7)])
+def test_caller_owned_state_at_any_place(S, K, n_q, tok_at, life_at):
+    """State that begins at any id and any lifetime of a larger allocation (a pool that packs tables); what lies before and
+    behind it stays as it is."""
+    import torch
+    import paper_2609_37538_b200 as avsg
+    n, L = 2, 3
+    rng = np.random.default_rng([S, K, n_q])
+    kv = avsg.pinned_empty(CTX * RB)
+    tr.fill_kv(kv.data_ptr(), 1, 0, CTX, RB)
+    orc = [OracleTable(S, RB, L) for _ in range(n)]
+    d = dict(device="cuda")
+    toks, lifes = torch.full((n * S + 8,), -77, dtype=torch.int32, **d), torch.full((n * S + 16,), 77, dtype=torch.int8, **d)
+    tok, life = toks[tok_at : tok_at + n * S].view(n, S), lifes[life_at : life_at + n * S].view(n, S)
+    tok.fill_(-1); life.fill_(-1)
+    buf, status = torch.zeros((n, S, RB), dtype=torch.uint8, **d), torch.zeros(1, dtype=torch.int32, **d)
+    slots, hit = torch.empty((n, n_q, K), dtype=torch.int32, **d), torch.empty((n, n_q, K), dtype=torch.uint8, **d)
+    for t in range(4):
+        X = np.stack([[rng.choice(3 * S // 2 + K, K, replace=False) for _ in range(n_q)] for _ in range(n)]).astype(np.int32)
+        N = 3 * S // 2 - 7 * t
+        avsg.step_noalloc(tok, life, buf, torch.from_numpy(X).cuda(), [kv] * n, [N] * n, max_lifetime=L, slots=slots, hit=hit,
+                          status=status)
+        assert int(status.item()) == 0
+        for i in range(n):
+            r = orc[i].step(X[i], N, kv.numpy(), RB)
+            c, l = orc[i].export_state()
+            assert (slots[i].cpu().numpy() == r.O).all() and (hit[i].cpu().numpy() == r.M).all(), (t, i)
+            assert (tok[i].cpu().numpy() == c).all() and (life[i].cpu().numpy() == l).all(), (t, i)
+            assert (buf[i].cpu().numpy() == orc[i].rows()).all(), (t, i)
+    assert (toks[:tok_at] == -77).all() and (toks[tok_at + n * S :] == -77).all()
+    assert (lifes[:life_at] == 77).all() and (lifes[life_at + n * S :] == 77).all()
