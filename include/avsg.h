@@ -58,7 +58,7 @@ extern "C" {
 #define AVSG_STATUS_BAD_SEGMENT     0x08u /* Stage Two could not resolve a miss-list entry      */
 #define AVSG_STATUS_BAD_ID          0x10u /* an id >= kv_rows of its table, or >= max_context
                                              with the direct index (taken as padding)          */
-#define AVSG_STATUS_WAIT_TIMEOUT    0x20u /* overlapped Stage Two gave up waiting for Stage One:
+#define AVSG_STATUS_WAIT_TIMEOUT    0x20u /* Stage Two gave up waiting for the Stage One that it follows:
                                              rows of THAT call were not copied.  Later calls are
                                              not affected (each takes the hand-over flags down
                                              before its transfer kernel can start)              */

@@ -67,7 +67,10 @@ __host__ __device__ inline S1Layout s1_layout(uint32_t S, uint32_t K, uint32_t n
 // Bits 0 .. 3: the sign bits of a word's four bytes.
 __device__ __forceinline__ uint32_t signs(uint32_t w) { return (((w >> 7) & 0x01010101u) * 0x10204080u) >> 28; }
 
-constexpr uint32_t STEP_SPIN_LIMIT = 1u << 20;            // waits of a microsecond or so each (the hardware suspends the warp)
+constexpr uint32_t STEP_SPIN_LIMIT = 1u << 18;            // tries; the hardware suspends the warp for 4 us in each: 1 s
+#ifndef AVSG_STEP_GIVE_UP                                 // (a test builds the library with waits that run out)
+#define AVSG_STEP_GIVE_UP STEP_SPIN_LIMIT
+#endif
 
 // Words of eight bytes that one of `copying` blocks gets per token, at most: a head and its rows.
 __device__ __forceinline__ uint32_t step_rows(uint32_t K, uint32_t copying) { return 1u + (K + copying - 1u) / copying; }
@@ -470,7 +473,8 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
     cluster_arrive();
     if (rank == 0) {
         stage_one<SPT, IPT, true, true>(p, ti, p.n_launch, smem, smem_u32(s_mbar));
-        if (p.out.n_slots) cluster_arrive();                           // the outputs are written
+        __syncwarp();
+        cluster_arrive();                                              // the outputs are written, everything is sent
         return;
     }
     const uint32_t cpr = p.row_bytes >> 4;
@@ -478,17 +482,16 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
     const uint64_t dst = reinterpret_cast<uint64_t>(p.buffer + (size_t)p.table_id[ti] * p.S * p.row_bytes);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     cluster_wait();
-    if (p.out.n_slots) cluster_arrive();
-    auto wait_for = [&](uint32_t mbar) -> bool {                       // (Stage One's loops are bounded, far below this)
+    cluster_arrive();
+    auto wait_for = [&](uint32_t mbar, uint32_t limit) -> bool {       // (Stage One's loops are bounded, far below this)
         uint32_t spin = 0;
-        while (!mbar_done(mbar) && ++spin < STEP_SPIN_LIMIT) {}
-        if (spin == STEP_SPIN_LIMIT && lane == 0) atomicOr(p.status, ST_WAIT_TIMEOUT);
-        return __all_sync(0xffffffffu, spin < STEP_SPIN_LIMIT);
+        while (spin < limit && !mbar_done(mbar)) ++spin;
+        return __all_sync(0xffffffffu, spin < limit);
     };
-    uint32_t from = 0;                                                 // the warp that is next
-    for (uint32_t g = 0; g < p.n_q; ++g) {
+    uint32_t from = 0, g = 0;                                          // the warp that is next; the token
+    for (; g < p.n_q; ++g) {
         const int2* got = reinterpret_cast<const int2*>(smem) + g * step_rows(p.K, copying);
-        if (!wait_for(smem_u32(s_mbar + g))) break;
+        if (!wait_for(smem_u32(s_mbar + g), AVSG_STEP_GIVE_UP)) break;
         const uint32_t count = (uint32_t)got[0].x;
         for (uint32_t k = warp >= from ? warp - from : warp + W - from; k < count; k += W) {
             const int2 e = got[1u + k];
@@ -503,13 +506,17 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
         } else if (g + 1u < p.n_q) {                                   // the warps meet
             from = 0;
             if (lane == 0) mbar_arrive(smem_u32(s_meet + g));
-            if (!wait_for(smem_u32(s_meet + g))) break;
+            if (!wait_for(smem_u32(s_meet + g), AVSG_STEP_GIVE_UP)) break;
         }
     }
-    if (p.out.n_slots) {
-        cluster_wait();
-        put_outputs_of(p.out, ti, p.n_q * p.K, p.n_q, warp * copying + rank - 1u, W * copying, lane);
+    // Stage One does not know who has given up, and nothing may be sent to a block that is gone: every block stays until
+    // Stage One is through, and one that gave up until what was sent has arrived.
+    cluster_wait();
+    if (g < p.n_q) {
+        if (lane == 0) atomicOr(p.status, ST_WAIT_TIMEOUT);
+        for (g = 0; g < p.n_q && wait_for(smem_u32(s_mbar + g), STEP_SPIN_LIMIT); ++g) {}
     }
+    if (p.out.n_slots) put_outputs_of(p.out, ti, p.n_q * p.K, p.n_q, warp * copying + rank - 1u, W * copying, lane);
 }
 
 // A request ended: its tables become empty (id -1) and dead (lifetime -1) again, their counters and rows zero;

@@ -53,7 +53,7 @@ __device__ __forceinline__ bool mbar_done(uint32_t mbar)
 {
     uint32_t done;
     asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0, %2;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(done) : "r"(mbar), "r"(1000u) : "memory");     // (suspended 1 us at most)
+                 "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(done) : "r"(mbar), "r"(1000u) : "memory");     // (asked for 1 us, suspended 4)
     return done != 0;
 }
 // All threads of all blocks of the cluster; earlier (distributed) shared-memory and global writes of the cluster

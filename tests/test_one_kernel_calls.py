@@ -163,3 +163,48 @@ def test_noalloc_with_and_without_a_status_word():
         for i in range(2):
             r = orc[i].step(np.where(X[i] >= 700, -1, X[i]), CTX, kv.numpy(), RB)
             assert (slots[i].cpu().numpy() == r.O).all() and (buf[i].cpu().numpy() == orc[i].rows()).all(), (t, i)
+
+
+_GIVES_UP = """
+import sys
+sys.path[:0] = [%(root)r, %(root)r + "/tests"]
+import numpy as np, torch
+from paper_2609_37538_b200 import build
+build.LIB = %(lib)r
+import paper_2609_37538_b200 as avsg
+from oracle import OracleTable
+from test_one_kernel_calls import RB, _kv
+S, K, n_q, L = 8192, 600, 3, 3
+kv = _kv(avsg)
+rng = np.random.default_rng(8)
+for n in (1, 20, 40, 74, 80):                            # clusters of eight, four, three, two blocks; two kernels
+    ctx = avsg.Context(n, S, RB, K, n_q, L)
+    orc = [OracleTable(S, RB, L) for _ in range(n)]
+    for host in (False, True, False):
+        X = np.stack([[rng.choice(900, K, replace=False) for _ in range(n_q)] for _ in range(n)]).astype(np.int32)
+        ids = torch.from_numpy(X).pin_memory() if host else torch.from_numpy(X).cuda()
+        out = (ctx.step_host if host else ctx.step)(list(range(n)), ids, [kv] * n, [890] * n)
+        assert ctx.sync_status() == (avsg.STATUS_WAIT_TIMEOUT if n <= 74 else 0), n
+        for i in range(n):
+            r = orc[i].step(X[i], 890, kv.numpy(), RB)
+            assert (out.slots[i].cpu().numpy() == r.O).all() and (out.hit[i].cpu().numpy() == r.M).all(), (n, i)
+    ctx.clear_status()
+    for i in range(n):
+        assert (ctx.export_state(i)[0] == orc[i].export_state()[0]).all(), (n, i)
+print("gave up")
+"""
+
+
+def test_blocks_that_give_up_waiting(tmp_path):
+    """A build whose copying blocks do not wait for what Stage One sends them: they say so, the rows do not
+    come, everything that Stage One writes does, and the context stays usable."""
+    import os
+    import subprocess
+    import sys
+    from paper_2609_37538_b200 import build
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    lib = str(tmp_path / "libavsg.so")
+    subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")] + build.NVCC_FLAGS + ["-DAVSG_STEP_GIVE_UP=0u", "-I",
+                          build.INCLUDE, "-I", build.CSRC, "-o", lib] + build.sources())
+    run = subprocess.run([sys.executable, "-c", _GIVES_UP % dict(root=root, lib=lib)], capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0 and "gave up" in run.stdout, run.stdout + run.stderr
