@@ -236,13 +236,13 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     // tables and several tokens whose ids do not begin on 64-byte boundaries: the link moves them in parts of lines, and
     // the tokens wait for one another's.  32 tables in place / by copies: K = 256, 272 (four tokens) 42, 44 / 62, 65; K =
     // 257, 260 92, 70 / 63, 63; K = 500, 1001 (two tokens) 62, 108 / 57, 78; K = 257 (one token) 27.6 / 27.8; eight
-    // tables, K = 257, four tokens 34.7 / 41.7.
+    // tables, K = 257, four tokens 34.7 / 41.7.  And ids that do not begin on a word's boundary, which the copies take.
     HostOut out;
     bool host_ids = false;
     const bool whole_lines = K % 16u == 0 || n_q == 1 || n <= (uint32_t)STEP_FEW_TABLES;
     if (host_io && c->cfg.index_mode != AVSG_INDEX_PAPER && c->s1_cluster == 1 && whole_lines &&
         (c->cfg.transfer_mode == AVSG_XFER_SM_BALANCED || c->cfg.transfer_mode == AVSG_XFER_SM_OVERLAP)) {
-        const int32_t* ids = mapped(a->indices);
+        const int32_t* ids = reinterpret_cast<uint64_t>(a->indices) % 4u == 0 ? mapped(a->indices) : nullptr;
         out.host_slots = mapped(a->slots);
         out.host_hit = a->hit ? mapped(a->hit) : nullptr;
         out.host_count = a->miss_count ? mapped(a->miss_count) : nullptr;

@@ -88,3 +88,36 @@ def test_calls_that_queue_behind_one_another(mode, cluster):
     for i in range(n):
         assert (ctx.buffer(i).cpu().numpy() == orc[i].rows()).all(), i
     assert ctx.sync_status() == 0
+
+
+@pytest.mark.parametrize("mode", ["XFER_SM_BALANCED", "XFER_SM_OVERLAP"])
+@pytest.mark.parametrize("n", [2, 76])
+@pytest.mark.parametrize("ids_at,slots_at,hit_at,count_at", [(1, 0, 0, 0), (2, 6, 1, 2), (3, 4, 3, 1), (0, 1, 5, 3), (4, 3, 2, 0)])
+def test_buffers_off_the_boundary_of_a_word(mode, n, ids_at, slots_at, hit_at, count_at):
+    """Pinned buffers that begin at any byte of a message, as host-side packing may leave them."""
+    import torch
+    import paper_2609_37538_b200 as avsg
+    T, S, rb, ctxlen, n_q, K = 4, 256, 48, 4000, 2, 32
+    traces, kv, ctx, orc = _setup(avsg, n, n_q, K, S, rb, ctxlen, mode, T)
+    call = ctx.prepare(list(range(n)), [kv] * n, n_q, K)
+
+    def place(at, dtype, *shape):
+        whole = torch.full((at + int(np.prod(shape)) * np.dtype(dtype).itemsize + 8,), 0x5A, dtype=torch.uint8, pin_memory=True)
+        return whole, np.ndarray(shape, dtype, buffer=whole.numpy(), offset=at)
+
+    bufs = [place(ids_at, np.int32, n, n_q, K), place(slots_at, np.int32, n, n_q, K), place(hit_at, np.uint8, n, n_q, K),
+            place(count_at, np.int32, n, n_q)]
+    ids, slots, hit, count = [view for _, view in bufs]
+    for t in range(T):
+        X = np.stack([traces[i][0][t] for i in range(n)])
+        N = [int(traces[i][1][t]) for i in range(n)]
+        ids[:] = X
+        call.run(*[x if isinstance(x, list) else x.ctypes.data for x in (ids, N, slots, hit, count)], host=True)
+        torch.cuda.synchronize()
+        for i in range(n):
+            r = orc[i].step(X[i], N[i], kv.numpy(), rb)
+            assert (slots[i] == r.O).all() and (hit[i] == r.M).all() and (count[i] == r.n).all(), (t, i)
+    for whole, view in bufs:                             # nothing beside them was written
+        at = view.ctypes.data - whole.data_ptr()
+        assert (whole[:at] == 0x5A).all() and (whole[at + view.nbytes :] == 0x5A).all()
+    assert ctx.sync_status() == 0
