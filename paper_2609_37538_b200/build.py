@@ -21,7 +21,7 @@ def sources():
 def _stale(srcs) -> bool:
     if not os.path.exists(LIB):
         return True
-    deps = srcs + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    deps = srcs + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(INCLUDE, "*.h"))
     return any(os.path.getmtime(d) > os.path.getmtime(LIB) for d in deps)
 
 

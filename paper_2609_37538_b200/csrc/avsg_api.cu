@@ -9,6 +9,7 @@
 
 #include "avsg.h"
 #include "avsg_kernels.cuh"
+#include "host_buffers.h"
 
 using namespace avsg;
 
@@ -202,15 +203,6 @@ void overlap_params(avsg_ctx* c, X& x, uint32_t n, uint32_t n_q, uint32_t round_
     x.round_size = round_size; x.t_range = nullptr;
 }
 
-// Device-visible address of a caller's host buffer (page-locked and mapped), or null.
-template <typename T>
-T* mapped(T* p)
-{
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    return at.type == cudaMemoryTypeHost ? static_cast<T*>(at.devicePointer) : nullptr;
-}
-
 int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool host_io)
 {
     int rc = check_args(c, a);
@@ -242,10 +234,10 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     const bool whole_lines = K % 16u == 0 || n_q == 1 || n <= (uint32_t)STEP_FEW_TABLES;
     if (host_io && c->cfg.index_mode != AVSG_INDEX_PAPER && c->s1_cluster == 1 && whole_lines &&
         (c->cfg.transfer_mode == AVSG_XFER_SM_BALANCED || c->cfg.transfer_mode == AVSG_XFER_SM_OVERLAP)) {
-        const int32_t* ids = reinterpret_cast<uint64_t>(a->indices) % 4u == 0 ? mapped(a->indices) : nullptr;
-        out.host_slots = mapped(a->slots);
-        out.host_hit = a->hit ? mapped(a->hit) : nullptr;
-        out.host_count = a->miss_count ? mapped(a->miss_count) : nullptr;
+        const int32_t* ids = reinterpret_cast<uint64_t>(a->indices) % 4u == 0 ? mapped(a->indices, n_ids) : nullptr;
+        out.host_slots = mapped(a->slots, n_ids);
+        out.host_hit = a->hit ? mapped(a->hit, n_ids) : nullptr;
+        out.host_count = a->miss_count ? mapped(a->miss_count, (size_t)n * n_q) : nullptr;
         if (ids && out.host_slots && !a->hit == !out.host_hit && !a->miss_count == !out.host_count) {
             host_ids = true;
             host_io = false;

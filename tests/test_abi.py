@@ -80,3 +80,13 @@ def test_product_sources_do_not_touch_the_oracle():
             if f.endswith((".py", ".cu", ".cuh", ".h")):
                 text = open(os.path.join(dirpath, f)).read()
                 assert "oracle" not in text.lower().replace("no cpu fallback", ""), f
+
+
+def test_host_buffers_are_used_in_place_only_where_all_of_them_is_mapped(tmp_path):
+    import subprocess
+    from paper_2609_37538_b200 import build
+    exe = str(tmp_path / "mapped_range")
+    subprocess.check_call(["g++", "-std=c++17", "-Wall", "-Wextra", "-I", "/usr/local/cuda/include", "-I", build.CSRC, "-o", exe,
+                           os.path.join(ROOT, "tests", "abi", "mapped_range.cpp")])
+    run = subprocess.run([exe], capture_output=True, text=True)
+    assert run.returncode == 0, run.stdout
