@@ -264,6 +264,8 @@ class PreparedCall:
             a.verified_len_dev = verified_len.data_ptr()
         else:
             a.verified_len_dev = None
+            if not isinstance(verified_len, (list, tuple)):
+                verified_len = list(verified_len)        # (an iterator can be read once only)
             try:
                 self._pack_vlen(self._vlen, 0, *verified_len)
             except struct.error:                         # not n integers that fit: as the element type converts them
@@ -433,6 +435,8 @@ def _c_array(kind: str, values, n: int):
     a ctypes array's cost; what it does not take (other numbers, another count, values that wrap) goes that way."""
     if values is None:
         return None, None
+    if not isinstance(values, (list, tuple)):
+        values = list(values)                            # (an iterator can be read once only)
     try:
         out = array.array(kind, values)
         if len(out) == n:

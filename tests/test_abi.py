@@ -90,3 +90,22 @@ def test_host_buffers_are_used_in_place_only_where_all_of_them_is_mapped(tmp_pat
                            os.path.join(ROOT, "tests", "abi", "mapped_range.cpp")])
     run = subprocess.run([exe], capture_output=True, text=True)
     assert run.returncode == 0, run.stdout
+
+
+def test_lengths_are_taken_from_any_iterable():
+    """Lists, arrays and one-shot iterators of integers, of other numbers and of values that wrap give the same lengths."""
+    import types
+    import numpy as np
+    from paper_2609_37538_b200.binding import PreparedCall, _c_array
+    got = []
+    lib = types.SimpleNamespace(avsg_step=lambda h, ref, stream: got.append(list(call._vlen)) or 0)
+    call = PreparedCall(types.SimpleNamespace(_lib=lib, _h=None), [0, 1, 2], [16, 16, 16], 1, 1)
+    want = [5, -1, 7]
+    kinds = [want, tuple(want), np.array(want), np.array(want, np.float64), [5.0, -1, 7.9], [5, 2**32 - 1, 7]]
+    for values in kinds + [iter(k) for k in kinds] + [(v for v in k) for k in kinds]:
+        call.run(16, values, 16, stream=0)
+        assert got[-1] == want
+    for values in kinds + [iter(k) for k in kinds]:
+        owner, at = _c_array("i", values, 3)
+        assert list((ctypes.c_int32 * 3).from_address(at)) == want
+    assert _c_array("I", None, 3) == (None, None)
