@@ -70,7 +70,10 @@ extern "C" {
                                        Calls of up to 74 tables run both stages in one
                                        kernel in this mode and in AVSG_XFER_SM_OVERLAP: a
                                        thread-block cluster per table, Stage Two following
-                                       Stage One token by token (not with arriving, timing,
+                                       Stage One token by token; the split over SMs is then
+                                       even within a table, and from 34 tables on rows of a
+                                       table that misses more than 512 ids of a token are
+                                       taken over by blocks of others that are through (not with arriving, timing,
                                        an own transfer geometry or a table above 8192
                                        slots, nor with stage_one_done above three tables).
                                        Its blocks take whole SMs while they run: who wants
@@ -90,7 +93,8 @@ extern "C" {
 #define AVSG_XFER_SM_OVERLAP    5u  /* the operator with Stage Two overlapping Stage One
                                        (App. G, latency hiding): the transfer kernel is
                                        resident while Stage One runs and starts on token
-                                       g's misses, cut evenly over all SMs per token,
+                                       g's misses, cut evenly over all SMs per token (but see
+                                       AVSG_XFER_SM_BALANCED for calls of up to 74 tables),
                                        while token g+1 is being placed.  Same results.
                                        A call whose Stage One, with a block per table,
                                        would take more than half of the SMs is served in

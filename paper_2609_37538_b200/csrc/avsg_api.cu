@@ -33,6 +33,7 @@ struct avsg_ctx {
     TableStats* d_stats = nullptr;
     StepClusters step_clusters;                    // calls in one kernel
     bool geometry_set = false;                     // avsg_set_transfer_geometry was called
+    SharedRows* d_shared = nullptr;                // calls in one kernel [STEP_MAX_TABLES]
     uint32_t* d_flags = nullptr;                   // hand-over flags per (table of the call, token)
                                                    //   [OVERLAP_MAX_TABLES x TOKENS], and one that is never raised
     unsigned long long* d_sync = nullptr;          //   [2] sequence number of the last host-buffer call,
@@ -95,7 +96,7 @@ uint32_t ilog2(uint32_t v) { uint32_t l = 0; while ((1u << l) < v) ++l; return l
 void free_all(avsg_ctx* c)
 {
     cudaFree(c->d_tok); cudaFree(c->d_life); cudaFree(c->d_buffer); cudaFree(c->d_stats); cudaFree(c->d_trange);
-    cudaFree(c->d_flags); cudaFree(c->d_sync);
+    cudaFree(c->d_shared); cudaFree(c->d_flags); cudaFree(c->d_sync);
     delete c->big_args;
     delete c->big_xfer_args;
     cudaFree(c->d_list); cudaFree(c->d_seg); cudaFree(c->d_status); cudaFree(c->d_q); cudaFree(c->d_q_snap);
@@ -359,7 +360,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
         !a->arriving && !host_io && !c->timing && !c->geometry_set) {
         auto step = [&](auto&& p) -> int {
             fill(p, 0, n);
-            p.flags = nullptr; p.out = out; p.early = step_early(p);
+            p.flags = nullptr; p.out = out; p.early = step_early(p); p.shared = c->d_shared;
             CU(launch_step(p, cluster, stream));
             return AVSG_OK;
         };
@@ -562,6 +563,7 @@ int avsg_create(const avsg_config* cfg, avsg_ctx** out)
     ok = ok && cudaMalloc(&c->d_buffer, T * S * cfg->row_bytes) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_stats, T * sizeof(TableStats)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_trange, 16 * sizeof(unsigned long long)) == cudaSuccess;
+    ok = ok && cudaMalloc(&c->d_shared, STEP_MAX_TABLES * sizeof(SharedRows)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_flags, FLAG_BYTES) == cudaSuccess;
     ok = ok && cudaMalloc(&c->d_sync, 8 * sizeof(unsigned long long)) == cudaSuccess;
     c->big_args = new (std::nothrow) S1ParamsBig();
@@ -608,6 +610,7 @@ int avsg_create(const avsg_config* cfg, avsg_ctx** out)
         const unsigned long long init[16] = {never, 0, never, 0, never, never, never, 0, never, 0, never, 0, never, never, never, 0};
         c->d_trange_init = c->d_trange + 8;
         if (cudaMemcpy(c->d_trange, init, sizeof(init), cudaMemcpyHostToDevice) != cudaSuccess ||
+            cudaMemset(c->d_shared, 0, STEP_MAX_TABLES * sizeof(SharedRows)) != cudaSuccess ||
             cudaMemset(c->d_flags, 0, FLAG_BYTES) != cudaSuccess ||
             cudaMemset(c->d_sync, 0, 8 * sizeof(unsigned long long)) != cudaSuccess) {
             free_all(c); delete c; return AVSG_ECUDA;
@@ -752,9 +755,10 @@ int avsg_clear_status(avsg_ctx* c)
     if (!guard.ok) return AVSG_ECUDA;
     CU(cudaDeviceSynchronize());
     CU(cudaMemset(c->d_status, 0, sizeof(uint32_t)));
-    // (every call takes its hand-over flags down itself; the arrival counter wraps to zero by itself unless a grid was
-    // lost half way)
+    // (every call takes its hand-over flags down itself; the arrival counter wraps to zero by itself, and a
+    // table closes the rows that it shares, unless a grid was lost half way)
     CU(cudaMemset(c->d_sync + 3, 0, sizeof(unsigned long long)));
+    CU(cudaMemset(c->d_shared, 0, STEP_MAX_TABLES * sizeof(SharedRows)));
     c->host_status = 0;
     return AVSG_OK;
 }

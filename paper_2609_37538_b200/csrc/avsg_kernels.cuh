@@ -90,6 +90,15 @@ constexpr uint32_t STEP_FEW_CLUSTER = 8;
 constexpr uint32_t STEP_EARLY_TABLES = 3;            // see step_early()
 constexpr uint64_t STEP_EARLY_BYTES = 2ull << 30;
 constexpr uint32_t STEP_MAX_TOKENS = 64;
+// What a table that misses far more than its cluster's blocks can have under way shares with the other blocks of the call:
+// see avsg_step_kernel.
+struct __align__(16) SharedRows {
+    uint32_t rows;      // how many there are, with SHARED_OPEN while others may begin to take some; SHARED_COMING until that is known
+    uint32_t pad;
+    uint32_t taken;     // by others, from the last one backwards
+    uint32_t begun;     // by the table's own blocks, about
+};
+constexpr uint32_t SHARED_COMING = 1u << 31, SHARED_OPEN = 1u << 30;
 
 // The per-call host arrays travel as kernel arguments, CAP tables' worth of them: a call needs no staging copy.
 template <int CAP>
@@ -122,6 +131,7 @@ struct S1ParamsT {
     unsigned long long  host_seq = 0;
     uint32_t            expect = 0;             // Stage One blocks that place tables of the call
     HostOut             out;                    // a call in one kernel: what its Stage Two writes to the host
+    SharedRows*         shared = nullptr;       // a call in one kernel: [STEP_MAX_TABLES], neither coming nor open between calls
     uint32_t            early = 1;              // the next grid may start under this one (with flags it has to)
     uint32_t            host_ids = 0;           // indices is mapped host memory that holds the ids when the call is made
     const int32_t* verified_len_dev = nullptr;  // [n] of the call: read instead of verified_len[] when set

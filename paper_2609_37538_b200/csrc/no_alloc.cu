@@ -25,6 +25,7 @@ namespace {
 
 struct NoAllocScratch {
     uint32_t   status[64];                                   // word 0: device status, word 1: that of calls that ask for none
+    SharedRows shared[AVSG_NOALLOC_MAX_TABLES];              // closed between calls
     SegDesc    seg[AVSG_NOALLOC_MAX_TABLES];
     TableStats stats[AVSG_NOALLOC_MAX_TABLES];
     int2       list[AVSG_NOALLOC_MAX_IDS];                   // (host position, slot) per miss
@@ -124,6 +125,7 @@ extern "C" int avsg_step_noalloc(const avsg_noalloc_args* a, void* cuda_stream)
         auto step = [&](auto&& p) -> int {               // one kernel for both stages
             if ((rc = fill(p)) != AVSG_OK) return rc;
             p.early = step_early(p);
+            p.shared = sc->shared;
             return launch_step(p, cluster, stream) == cudaSuccess ? AVSG_OK : AVSG_ECUDA;
         };
         rc = cluster == STEP_FEW_CLUSTER && a->n <= (uint32_t)STEP_FEW_TABLES ? step(StepParamsFew()) : step(StepParams());

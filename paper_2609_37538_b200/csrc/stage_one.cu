@@ -75,14 +75,22 @@ constexpr uint32_t STEP_SPIN_LIMIT = 1u << 18;            // tries; the hardware
 // Words of eight bytes that one of `copying` blocks gets per token, at most: a head and its rows.
 __device__ __forceinline__ uint32_t step_rows(uint32_t K, uint32_t copying) { return 1u + (K + copying - 1u) / copying; }
 
+// Rows that blocks of other tables may take (see avsg_step_kernel): from how many misses of a token on, how many of a
+// table's rows stay for its own blocks (other blocks' caches of translations do not know the table: with 256 left 64 unequal
+// requests take 326 us, with 128 330, without any sharing 324), how many warps of the call take some at most (of 144 rows
+// under way the link is full; more only copy the last rows twice).
+constexpr uint32_t SHARED_FROM = 512, SHARED_LEFT = 256, SHARED_WARPS = 144, SHARED_CLUSTER = 4;
+
 // SPT slots per thread (a power of two): S <= SPT * blockDim.x.  IPT: the most ids a thread has to look up per token
 // (K <= S, so SPT is always enough).  CAP: tables the argument block has room for.  The block serves the tables block,
 // block + blocks, ... of the launch.  CLUSTER: it is the first block of a cluster whose others copy what it places
 // (avsg_step_kernel); a_mbar: their mbarriers, one per token.  WIDE: the state is aligned (state_is_aligned()).
-template <int SPT, int IPT, bool CLUSTER, bool WIDE, int CAP>
+// SHARE: rows of a table with very many misses may be copied by other tables' blocks.
+template <int SPT, int IPT, bool CLUSTER, bool WIDE, bool SHARE, int CAP>
 __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_t block, const uint32_t blocks, unsigned char* smem, const uint32_t a_mbar = 0)
 {
     const uint32_t copying = CAP == STEP_FEW_TABLES ? STEP_FEW_CLUSTER - 1u : CLUSTER ? cluster_size() - 1u : 1u;
+    constexpr bool SHARES = CLUSTER && CAP != STEP_FEW_TABLES;         // a copying block's rows are a share in position order
     constexpr int NV = (SPT + 3) / 4;                    // 4-slot vectors of ids / words of lifetimes per thread
     const uint32_t S = p.S, K = p.K, H = 2u * S, L = p.L;
     const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u, warp = tid >> 5, nw = nt >> 5;
@@ -202,6 +210,7 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
         const bool unusual = __syncthreads_or(high != 0);
 
         uint32_t list_off = 0, sum_miss = 0, sum_decay = 0, valid = 0;
+        uint32_t shared = 0;                             // SHARE: rows that other blocks may take (bit 31: there will be some)
         int2* list = p.miss_list + (size_t)ti * p.list_stride;
 
         for (uint32_t g = 0; g < p.n_q; ++g) {
@@ -285,6 +294,16 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
             uint32_t dtotal = all & 0xFFFFu, dead_before = before & 0xFFFFu, d = 0;
             sum_miss += n_g;
             if (tid == 0 && p.miss_count) p.miss_count[(size_t)ti * p.n_q + g] = (int32_t)n_g;
+            const bool share_it = SHARE && n_g > SHARED_FROM;
+            if (share_it && !shared) {
+                shared = SHARED_COMING;
+                if (tid == 0) {                          // (in place before the table's own blocks hear of the rows)
+                    p.shared[ti].taken = p.shared[ti].begun = 0;
+                    __threadfence();
+                    *reinterpret_cast<volatile uint32_t*>(&p.shared[ti].rows) = SHARED_COMING;
+                    __threadfence();
+                }
+            }
             if (missing) {
 #pragma unroll
                 for (int k = 0; k < IPT; ++k) {
@@ -350,15 +369,18 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
             if (lane == 0) s_ndead[32u - par + warp] = left;
             __syncthreads();
 
-            // a copying block's rows: every seventh where a cluster has eight blocks, else a share in position order
-            const uint32_t share = CLUSTER && CAP != STEP_FEW_TABLES ? (n_take + copying - 1u) / copying : 0u;
+            // a copying block's rows: in turn where few tables have eight blocks each, and where other blocks may take some
+            // (so that what is left is at the end), else a share in position order
+            const bool in_turn = CAP == STEP_FEW_TABLES || share_it;
+            const uint32_t share = SHARES ? (n_take + copying - 1u) / copying : 0u;
             if constexpr (CLUSTER) {                     // what the copying blocks get of this token: a head and their rows
                 if (g == 0) cluster_wait();              // (their mbarriers are ready)
                 if (tid < copying) {
-                    const uint32_t n = CAP == STEP_FEW_TABLES ? (n_take + copying - 1u - tid) / copying
+                    const uint32_t n = in_turn ? (n_take + copying - 1u - tid) / copying
                                        : tid * share >= n_take ? 0u : n_take - tid * share < share ? n_take - tid * share : share;
                     const uint32_t mbar = map_rank(a_mbar + 8u * g, tid + 1u);
-                    send_async(map_rank(smem_u32(smem) + 8u * g * step_rows(K, copying), tid + 1u), (int32_t)n, 0, mbar);
+                    send_async(map_rank(smem_u32(smem) + 8u * g * step_rows(K, copying), tid + 1u), (int32_t)n,
+                               share_it ? (int32_t)((shared & ~SHARED_COMING) + tid) : -1, mbar);
                     arrive_expect(mbar, 8u * (n + 1u));
                 }
             }
@@ -372,8 +394,9 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
                     s_node[j].x = (uint32_t)x;
                     s_life[j] = (int8_t)L;
                     if constexpr (CLUSTER) {
-                        const uint32_t to = CAP == STEP_FEW_TABLES ? k % copying : k / share;
-                        const uint32_t at = CAP == STEP_FEW_TABLES ? k / copying : k - to * share;
+                        const uint32_t to = in_turn ? k % copying : k / share;
+                        const uint32_t at = in_turn ? k / copying : k - to * share;
+                        if (share_it) list[(shared & ~SHARED_COMING) + k] = make_int2(x, j);
                         send_async(map_rank(smem_u32(smem) + 8u * (g * step_rows(K, copying) + 1u + at), to + 1u), x, j,
                                    map_rank(a_mbar + 8u * g, to + 1u));
                     } else {
@@ -389,9 +412,14 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
                 if (Hm) Hm[i] = 0;
             }
             list_off += n_take;
+            if (share_it) shared += n_take;
             sum_decay += d;
             __syncthreads();
             announce_token(p, ti, g, n_take);
+        }
+        if (SHARE && shared && tid == 0) {
+            __threadfence();
+            *reinterpret_cast<volatile uint32_t*>(&p.shared[ti].rows) = shared == SHARED_COMING ? 0u : shared ^ (SHARED_COMING | SHARED_OPEN);
         }
 
         // ---- write back: lifetimes; resident ids that are no longer verified become empty (Alg. 4) ----
@@ -434,7 +462,54 @@ template <int SPT, int IPT, int CAP, bool WIDE = true>
 __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_constant__ S1ParamsT<CAP> p)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    stage_one<SPT, IPT, false, WIDE>(p, blockIdx.x, gridDim.x, smem);
+    stage_one<SPT, IPT, false, WIDE, false>(p, blockIdx.x, gridDim.x, smem);
+}
+
+__device__ __forceinline__ SharedRows read_shared(const SharedRows* at)
+{
+    SharedRows s;
+    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(s.rows), "=r"(s.pad), "=r"(s.taken), "=r"(s.begun) : "l"(at) : "memory");
+    return s;
+}
+
+// A warp that is through with its own table's rows copies rows that other tables share.
+template <int CAP>
+__device__ __forceinline__ void take_shared_rows(const S1ParamsT<CAP>& p, const uint32_t ti, const uint32_t group)
+{
+    const uint32_t lane = threadIdx.x & 31u, cpr = p.row_bytes >> 4;
+    // all tables at a time: one after the other they had held up the end of a call with many
+    SharedRows now = {0u, 0u, 0u, 0u};
+    if (group + lane < p.n_launch && group + lane != ti) now = read_shared(p.shared + group + lane);
+    const bool some = (now.rows & SHARED_COMING) ||
+                      ((now.rows & SHARED_OPEN) && now.taken + now.begun + SHARED_LEFT < (now.rows & ~SHARED_OPEN));
+    for (uint32_t which = __ballot_sync(0xffffffffu, some); which; which &= which - 1u) {
+        const uint32_t t = group + __ffs((int)which) - 1u;
+        SharedRows s = read_shared(p.shared + t);
+        for (uint32_t spin = 0; (s.rows & SHARED_COMING) && spin < OVERLAP_SPIN_LIMIT; ++spin) {     // (that Stage One runs, and waits for nobody)
+            __nanosleep(64);
+            s = read_shared(p.shared + t);
+        }
+        __threadfence();
+        const uint32_t rows = __shfl_sync(0xffffffffu, s.rows, 0) ^ SHARED_OPEN;
+        if (rows >= SHARED_OPEN) continue;                             // closed meanwhile
+        const uint64_t src = p.kv_base[t], stride = p.kv_stride[t];
+        const uint64_t dst = reinterpret_cast<uint64_t>(p.buffer + (size_t)p.table_id[t] * p.S * p.row_bytes);
+        const int2* list = p.miss_list + (size_t)t * p.list_stride;
+        for (;;) {
+            uint32_t at = 0xFFFFFFFFu;
+            if (lane == 0 && s.taken + s.begun + SHARED_LEFT < rows) at = atomicAdd(&p.shared[t].taken, 1u);
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (at >= rows) break;
+            const int2 e = __ldcg(list + (rows - 1u - at));            // what is taken is copied
+            s = read_shared(p.shared + t);                             // (comes with the row)
+            if (e.x < 0 || e.y < 0 || (uint32_t)e.y >= p.S) {
+                if (lane == 0) atomicOr(p.status, ST_BAD_SLOT);
+                continue;
+            }
+            copy_row(src + (uint64_t)(uint32_t)e.x * stride, dst + (uint64_t)(uint32_t)e.y * p.row_bytes, cpr, lane);
+        }
+    }
 }
 
 // A call in one kernel: a cluster of two to eight blocks per table.  The first block runs Stage One; the others copy the
@@ -456,15 +531,31 @@ __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_co
 // without a meeting of the warps, and go round over the blocks (one table 12.0 us; meeting, with shares 12.35).  Otherwise
 // a block's warps meet before the next token's rows, and its rows are neighbours (16 tables, 11 GB: 84.0 us against 84.3
 // and 86.0 with one of the two; 40 tables 193 against 203 and 199).
-template <int SPT, int IPT, int CAP>
+// SHARE (two and three blocks).  A cluster alone cannot fill the link with one table's rows where it has few copying blocks (an
+// SM gets 20 of them a us, the link carries 72), so a new request among steady ones would be left behind: 64 tables, one of
+// them cold, 332 us against 277 in two kernels, whose rows are cut evenly over all SMs (Eq. 6).  So a table that misses more
+// than SHARED_FROM ids in a token writes these misses to its list in global memory too, and says so.  Its own blocks copy them
+// from the front; a few warps of other tables that are through take single rows from the back, counted in SharedRows::taken,
+// until few are left; the own blocks stop where the others have begun.  Both may copy a row in the middle, to the same effect.
+// Every row is copied: what the own blocks leave out is counted in `taken`, and what is counted there is copied by who counted it.
+// Nobody waits, but for a Stage One that has announced rows and runs.  One cold table of 45, 64: 229, 332 us without, 215, 283
+// with it, 211, 277 in two kernels; the others with hits only 70, 124, 50, 57, 46, 46; all steady 169, 239.5, 170, 240.5, 172, 241.
+// With four blocks it costs every call more (16 tables 64.7 us, 65.5 with it) than it gives one with a new request (16, 32
+// tables, one cold: 115, 172 without, 113, 170 with it, 110, 167 in two kernels).  With all rows of such a table claimed one by
+// one, its own blocks' too, the cold calls were quicker still (45 tables 214), but a call where most tables had many misses
+// lost 5 to 20 %: the requests for claims and list entries wait behind the rows'.  Several rows of a warp at once bring an SM
+// from 20 rows a us to 28 at most.
+template <int SPT, int IPT, int CAP, bool SHARE = false>
 __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constant__ S1ParamsT<CAP> p)
 {
     constexpr bool FEW = CAP == STEP_FEW_TABLES;
     extern __shared__ __align__(16) unsigned char smem[];              // of a copying block: the words that it gets, by token
     __shared__ __align__(8) unsigned long long s_mbar[STEP_MAX_TOKENS], s_meet[STEP_MAX_TOKENS];
+    __shared__ volatile uint32_t s_mine;                               // rows that are shared: the first that others have taken
     const uint32_t rank = cluster_rank(), cluster = FEW ? STEP_FEW_CLUSTER : cluster_size(), copying = cluster - 1u;
     const uint32_t ti = blockIdx.x / cluster, lane = threadIdx.x & 31u, W = blockDim.x >> 5, warp = threadIdx.x >> 5;
     if (p.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (SHARE && threadIdx.x == 0) s_mine = 0xFFFFFFFFu;
     if (rank != 0 && threadIdx.x < p.n_q) {
         mbar_init(smem_u32(s_mbar + threadIdx.x), 1u);
         if (!FEW) mbar_init(smem_u32(s_meet + threadIdx.x), W);
@@ -472,7 +563,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
     __syncthreads();
     cluster_arrive();
     if (rank == 0) {
-        stage_one<SPT, IPT, true, true>(p, ti, p.n_launch, smem, smem_u32(s_mbar));
+        stage_one<SPT, IPT, true, true, SHARE>(p, ti, p.n_launch, smem, smem_u32(s_mbar));
         __syncwarp();
         cluster_arrive();                                              // the outputs are written, everything is sent
         return;
@@ -493,7 +584,17 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
         const int2* got = reinterpret_cast<const int2*>(smem) + g * step_rows(p.K, copying);
         if (!wait_for(smem_u32(s_mbar + g), AVSG_STEP_GIVE_UP)) break;
         const uint32_t count = (uint32_t)got[0].x;
+        const int32_t at = got[0].y;                                   // of the first row among those that are shared; -1
+        SharedRows s = {SHARED_COMING, 0u, 0u, 0u};
         for (uint32_t k = warp >= from ? warp - from : warp + W - from; k < count; k += W) {
+            if (SHARE && at >= 0) {
+                if (warp == 0) {                                       // for all warps: requests wait behind the rows' where the link is full
+                    if (!(s.rows & SHARED_COMING)) s_mine = (s.rows & ~SHARED_OPEN) > s.taken ? (s.rows & ~SHARED_OPEN) - s.taken : 0u;
+                    s = read_shared(p.shared + ti);                    // (comes with the row)
+                    if (lane == 0) atomicAdd(&p.shared[ti].begun, W);
+                }
+                if (at + k * copying >= s_mine) break;                 // others have the rest
+            }
             const int2 e = got[1u + k];
             if (e.x < 0 || e.y < 0 || (uint32_t)e.y >= p.S) {
                 if (lane == 0) atomicOr(p.status, ST_BAD_SLOT);
@@ -501,7 +602,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
             }
             copy_row(src + (uint64_t)(uint32_t)e.x * stride, dst + (uint64_t)(uint32_t)e.y * p.row_bytes, cpr, lane);
         }
-        if (FEW || count < W) {
+        if (FEW || count < W || (SHARE && g + 1u == p.n_q)) {
             from = (from + count) % W;
         } else if (g + 1u < p.n_q) {                                   // the warps meet
             from = 0;
@@ -509,6 +610,11 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
             if (!wait_for(smem_u32(s_meet + g), AVSG_STEP_GIVE_UP)) break;
         }
     }
+    // Warps that take other tables' rows: those that had the fewest of the last token, a few of each block
+    uint32_t others = 0;                                               // what 32 of the tables share, one a lane
+    const uint32_t turn = warp >= from ? warp - from : warp + W - from, group = (ti + turn) % ((p.n_launch + 31u) / 32u) * 32u;
+    const bool takes = SHARE && turn * (p.n_launch - 1u) * copying < SHARED_WARPS * ((p.n_launch + 31u) / 32u);
+    if (takes && group + lane < p.n_launch) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(others) : "l"(&p.shared[group + lane].rows) : "memory");
     // Stage One does not know who has given up, and nothing may be sent to a block that is gone: every block stays until
     // Stage One is through, and one that gave up until what was sent has arrived.
     cluster_wait();
@@ -517,6 +623,11 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
         for (g = 0; g < p.n_q && wait_for(smem_u32(s_mbar + g), STEP_SPIN_LIMIT); ++g) {}
     }
     if (p.out.n_slots) put_outputs_of(p.out, ti, p.n_q * p.K, p.n_q, warp * copying + rank - 1u, W * copying, lane);
+    if constexpr (SHARE) {
+        // Closed for who has not begun yet, and so closed between calls (Stage One is through and writes it no more).
+        if (threadIdx.x == 0) atomicAnd(&p.shared[ti].rows, SHARED_OPEN - 1u);
+        if (takes && __any_sync(0xffffffffu, (others & (SHARED_COMING | SHARED_OPEN)) != 0)) take_shared_rows(p, ti, group);
+    }
 }
 
 // A request ended: its tables become empty (id -1) and dead (lifetime -1) again, their counters and rows zero;
@@ -905,6 +1016,12 @@ cudaError_t stage_one_prepare(size_t max_smem)
         reinterpret_cast<const void*>(avsg_step_kernel<8, 2, STEP_MAX_TABLES>),
         reinterpret_cast<const void*>(avsg_step_kernel<8, 4, STEP_MAX_TABLES>),
         reinterpret_cast<const void*>(avsg_step_kernel<8, 8, STEP_MAX_TABLES>),
+        reinterpret_cast<const void*>(avsg_step_kernel<2, 2, STEP_MAX_TABLES, true>),
+        reinterpret_cast<const void*>(avsg_step_kernel<4, 2, STEP_MAX_TABLES, true>),
+        reinterpret_cast<const void*>(avsg_step_kernel<4, 4, STEP_MAX_TABLES, true>),
+        reinterpret_cast<const void*>(avsg_step_kernel<8, 2, STEP_MAX_TABLES, true>),
+        reinterpret_cast<const void*>(avsg_step_kernel<8, 4, STEP_MAX_TABLES, true>),
+        reinterpret_cast<const void*>(avsg_step_kernel<8, 8, STEP_MAX_TABLES, true>),
         reinterpret_cast<const void*>(avsg_stage_one_paper_kernel)};
     for (const void* k : kernels) {
         cudaFuncAttributes fa;
@@ -984,16 +1101,16 @@ uint32_t step_threads(uint32_t S, uint32_t K)
 
 namespace {
 
-template <int CAP>
+template <int CAP, bool SHARE = false>
 const void* step_kernel(uint32_t spt, uint32_t ipt)
 {
     switch (spt) {
-        case 8:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 2, CAP>)
-                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 4, CAP>)
-                                 : reinterpret_cast<const void*>(avsg_step_kernel<8, 8, CAP>);
-        case 4:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<4, 2, CAP>)
-                                 : reinterpret_cast<const void*>(avsg_step_kernel<4, 4, CAP>);
-        default: return reinterpret_cast<const void*>(avsg_step_kernel<2, 2, CAP>);
+        case 8:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 2, CAP, SHARE>)
+                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 4, CAP, SHARE>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<8, 8, CAP, SHARE>);
+        case 4:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<4, 2, CAP, SHARE>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<4, 4, CAP, SHARE>);
+        default: return reinterpret_cast<const void*>(avsg_step_kernel<2, 2, CAP, SHARE>);
     }
 }
 
@@ -1037,7 +1154,10 @@ cudaError_t launch_step(const S1ParamsT<CAP>& p, uint32_t cluster, cudaStream_t 
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = 2;
     void* args[] = {const_cast<S1ParamsT<CAP>*>(&p)};
-    return cudaLaunchKernelExC(&cfg, step_kernel<CAP>(p.S / nt, (p.K + nt - 1) / nt), args);
+    const uint32_t spt = p.S / nt, ipt = (p.K + nt - 1) / nt;
+    if constexpr (CAP == STEP_MAX_TABLES)
+        if (cluster < SHARED_CLUSTER) return cudaLaunchKernelExC(&cfg, step_kernel<CAP, true>(spt, ipt), args);
+    return cudaLaunchKernelExC(&cfg, step_kernel<CAP>(spt, ipt), args);
 }
 template cudaError_t launch_step(const StepParams& p, uint32_t cluster, cudaStream_t stream);
 template cudaError_t launch_step(const StepParamsFew& p, uint32_t cluster, cudaStream_t stream);

@@ -208,3 +208,79 @@ def test_blocks_that_give_up_waiting(tmp_path):
                           build.INCLUDE, "-I", build.CSRC, "-o", lib] + build.sources())
     run = subprocess.run([sys.executable, "-c", _GIVES_UP % dict(root=root, lib=lib)], capture_output=True, text=True, timeout=300)
     assert run.returncode == 0 and "gave up" in run.stdout, run.stdout + run.stderr
+
+
+# clusters of eight (of small blocks), four, three and two blocks; rows of one and of two parts
+@pytest.mark.parametrize("n,S,K,n_q,rb", [(12, 2048, 600, 3, 48), (9, 8192, 2048, 2, 1040), (33, 8192, 800, 1, 48), (45, 8192, 1100, 2, 48),
+                                          (46, 8192, 513, 3, 48), (74, 8192, 1000, 2, 48)])
+def test_rows_that_tables_share(n, S, K, n_q, rb):
+    """Tables that miss far more than the others: all of them, one, several, with host buffers, with tables whose place in the
+    call changes; queued without a wait, so that the blocks of one call start on what the call before has left behind."""
+    import torch
+    import paper_2609_37538_b200 as avsg
+    L, context = 3, 9000
+    rng = np.random.default_rng([n, K])
+    kv = avsg.pinned_empty(context * rb)
+    tr.fill_kv(kv.data_ptr(), 1, 0, context, rb)
+    ctx = avsg.Context(n, S, rb, K, n_q, L)
+    orc = [OracleTable(S, rb, L) for _ in range(n)]
+    last = [rng.choice(context, K, replace=False) for _ in range(n)]
+    done = []
+    for c in range(10):
+        tabs = [int(t) for t in rng.permutation(n)]
+        cold = [int(t) for t in rng.permutation(n)[: [n, 0, 1, 1, 3, 0, n // 2, 1, 1, 2][c]]]
+        if cold:
+            ctx.reset_async(cold)
+        X = np.empty((n, n_q, K), np.int32)
+        for a, t in enumerate(tabs):
+            for g in range(n_q):                         # a few new ids, or none, in a new order
+                keep = rng.choice(last[t], K - (0 if c == 7 else 5), replace=False)
+                new = np.setdiff1d(rng.integers(0, context, 60), keep)
+                last[t] = rng.permutation(np.concatenate([keep, new[: K - len(keep)]]))
+                X[a, g] = last[t]
+        host = c in (3, 6)
+        ids = torch.from_numpy(X).pin_memory() if host else torch.from_numpy(X).cuda()
+        done.append((tabs, cold, X, (ctx.step_host if host else ctx.step)(tabs, ids, [kv] * n, [context] * n)))
+    torch.cuda.synchronize()
+    for c, (tabs, cold, X, out) in enumerate(done):
+        for t in cold:
+            orc[t].reset()
+        for a, t in enumerate(tabs):
+            r = orc[t].step(X[a], context, kv.numpy(), rb)
+            assert (out.slots[a].cpu().numpy() == r.O).all() and (out.hit[a].cpu().numpy() == r.M).all(), (c, t)
+    for t in range(n):
+        assert (ctx.buffer(t).cpu().numpy() == orc[t].rows()).all(), t
+    assert ctx.sync_status() == 0
+
+
+def test_rows_that_tables_share_in_a_captured_call_and_without_a_context():
+    import torch
+    import paper_2609_37538_b200 as avsg
+    n, S, K, n_q, L, context = 20, 8192, 1500, 2, 3, 6000
+    rng = np.random.default_rng(2)
+    kv = avsg.pinned_empty(context * RB)
+    tr.fill_kv(kv.data_ptr(), 1, 0, context, RB)
+    ctx = avsg.Context(n, S, RB, K, n_q, L)
+    call = ctx.prepare(list(range(n)), [kv] * n, n_q, K)
+    d = dict(device="cuda")
+    X, N = torch.empty((n, n_q, K), dtype=torch.int32, **d), torch.full((n,), context, dtype=torch.int32, **d)
+    slots, slots2 = torch.empty_like(X), torch.empty_like(X)
+    tok, life = torch.full((n, S), -1, dtype=torch.int32, **d), torch.full((n, S), -1, dtype=torch.int8, **d)
+    buf = torch.zeros((n, S, RB), dtype=torch.uint8, **d)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call.run(X, N, slots)
+    orc = [OracleTable(S, RB, L) for _ in range(n)]
+    ids = np.stack([[rng.choice(context, K, replace=False)] * n_q for _ in range(n)]).astype(np.int32)
+    for c in range(5):
+        for t in rng.permutation(n)[:2]:                 # two tables turn to other ids
+            ids[t] = rng.choice(context, K, replace=False)
+        X.copy_(torch.from_numpy(ids))
+        graph.replay()
+        avsg.step_noalloc(tok, life, buf, X, [kv] * n, [context] * n, max_lifetime=L, slots=slots2)
+        torch.cuda.synchronize()
+        for t in range(n):
+            r = orc[t].step(ids[t], context, kv.numpy(), RB)
+            assert (slots[t].cpu().numpy() == r.O).all() and (slots2[t].cpu().numpy() == r.O).all(), (c, t)
+            assert (ctx.buffer(t).cpu().numpy() == orc[t].rows()).all() and (buf[t].cpu().numpy() == orc[t].rows()).all(), (c, t)
+    assert ctx.sync_status() == 0
