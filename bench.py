@@ -254,10 +254,11 @@ def run_cuda(args):
                        index_mode=avsg.INDEX_DIRECT if direct else avsg.INDEX_HASH,
                        max_context=max(c.context for c in w.tables) + w.n_q, stage_one_cluster=args.cluster,
                        transfer_mode=avsg.XFER_SM_OVERLAP if args.stage_two == "overlap" else avsg.XFER_SM_BALANCED)
-    # Shrunk runs are for looking at the two kernels of a call: a geometry that is set keeps them (what is set is the default).
-    one_kernel = 32 <= len(w.calls[0]) <= 74 and args.cluster <= 1 and w.buffer_slots <= 8192
-    if len(w.calls[0]) < 32:
-        ctx.set_transfer_geometry(0, 256)
+    # Which path the library takes (on a B200); --tiny lines look at the two kernels of a call, which a geometry of the
+    # caller's own keeps (one block per SM is what the default comes to).
+    one_kernel = not args.tiny and len(w.calls[0]) <= 74 and args.cluster <= 1 and w.buffer_slots <= 8192
+    if args.tiny:
+        ctx.set_transfer_geometry(torch.cuda.get_device_properties(local).multi_processor_count, 256)
     ncalls = len(w.calls)
     calls = [ctx.prepare(grp, [kv[t] for t in grp], w.n_q, w.topk,
                          [stride] * len(grp) if args.row_stride else None) for grp in w.calls]
@@ -466,7 +467,8 @@ def run_cuda(args):
         "scaling": args.scaling if world > 1 else "weak", "vs_baseline": None,
         "dtype": "int32/u8", "data": "synthetic", "config": _config(w),
         "variant": {"host_row_stride": stride, "stage_one_index": args.index, "stage_two": args.stage_two,
-                    "stage_one_cluster": args.cluster, "host_kv": args.host_kv},
+                    "stage_one_cluster": args.cluster, "host_kv": args.host_kv,
+                    "kernels_per_call": "1" if one_kernel else "2 (a transfer geometry is set)" if args.tiny else "2"},
         "clocks": clocks,
         "e2e": {"value": e2e_value, "unit": "GB/s",
                 "h2d_bytes_per_step": int(ids_bytes + rows_timed * rb / K), "d2h_bytes_per_step": int(ids_bytes + mc_bytes),
@@ -520,8 +522,9 @@ def run_cuda(args):
                      "peak_kind": "measured in this run (pinned cudaMemcpyAsync H2D, 1 GiB, best of 4 after one warm-up copy)", "peak_repeats": 4,
                      "note": "algorithmic bytes = row_bytes x missed rows per launch; the rows cross the host link and stay "
                              "in L2 after the write, so DRAM traffic (scaled from the ncu capture of the one-layer case) is small; "
-                             "timed in balanced mode (one kernel at a time); the timed steps copy each token's rows while "
-                             "Stage One still runs"},
+                             "timed in balanced mode with the library's own timing on, which keeps two kernels, one at a "
+                             "time; the timed steps copy each token's rows while Stage One still runs, in one kernel "
+                             "where variant.kernels_per_call says so"},
         "roofline_stage_one": {"bound": "hbm", "kernel": "avsg_stage_one_cluster_kernel" if w.buffer_slots > 8192 or args.cluster > 1
                                                          else "avsg_stage_one_kernel", "achieved": s1_gbs, "peak": hbm_peak,
                                "unit": "GB/s", "frac": s1_gbs / hbm_peak, "traffic": NCU_S1_DRAM_BYTES_PER_TABLE * n_tab,

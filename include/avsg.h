@@ -344,7 +344,10 @@ int avsg_set_transfer_mode(avsg_ctx *ctx, uint32_t mode);
 int avsg_set_timing(avsg_ctx *ctx, int enable);
 
 /* Eq. 6 cuts the miss list over C cores: C = thread blocks (0 = one per SM);
- * threads per block is this build's own knob. */
+ * threads per block is this build's own knob.  With a geometry of its own a
+ * context's calls keep Stage One and Stage Two in two kernels, and balanced
+ * ones of many tables do not run in rounds (see AVSG_XFER_SM_BALANCED); blocks
+ * = 0 with threads = 256 is the default again. */
 int avsg_set_transfer_geometry(avsg_ctx *ctx, uint32_t blocks, uint32_t threads);
 
 /*

@@ -14,6 +14,7 @@
 using namespace avsg;
 
 namespace {
+constexpr uint32_t XFER_THREADS = 256;             // per block of a transfer grid, unless the caller sets a geometry
 constexpr size_t FLAG_BYTES = ((size_t)OVERLAP_MAX_TABLES * OVERLAP_MAX_TOKENS + 1) * sizeof(uint32_t);
 }
 
@@ -24,7 +25,7 @@ struct avsg_ctx {
     uint32_t host_status = 0;          // status bits raised on the host side (sticky like the device word)
     uint32_t list_stride = 0;          // entries per miss-list segment
     int sm_count = 0;
-    uint32_t xfer_blocks = 0, xfer_threads = 256;
+    uint32_t xfer_blocks = 0, xfer_threads = XFER_THREADS;
     bool timing = false, events_recorded = false;
 
     int32_t* d_tok = nullptr;
@@ -32,7 +33,7 @@ struct avsg_ctx {
     uint8_t* d_buffer = nullptr;
     TableStats* d_stats = nullptr;
     StepClusters step_clusters;                    // calls in one kernel
-    bool geometry_set = false;                     // avsg_set_transfer_geometry was called
+    bool geometry_set = false;                     // another geometry than the default one
     SharedRows* d_shared = nullptr;                // calls in one kernel [STEP_MAX_TABLES]
     uint32_t* d_flags = nullptr;                   // hand-over flags per (table of the call, token)
                                                    //   [OVERLAP_MAX_TABLES x TOKENS], and one that is never raised
@@ -884,7 +885,7 @@ int avsg_set_transfer_geometry(avsg_ctx* c, uint32_t blocks, uint32_t threads)
     if (!c || threads < 32 || threads > 1024 || threads % 32 || blocks > 65535) return AVSG_EINVAL;
     c->xfer_blocks = blocks;
     c->xfer_threads = threads;
-    c->geometry_set = true;
+    c->geometry_set = blocks != 0 || threads != XFER_THREADS;
     return AVSG_OK;
 }
 

@@ -284,3 +284,32 @@ def test_rows_that_tables_share_in_a_captured_call_and_without_a_context():
             assert (slots[t].cpu().numpy() == r.O).all() and (slots2[t].cpu().numpy() == r.O).all(), (c, t)
             assert (ctx.buffer(t).cpu().numpy() == orc[t].rows()).all() and (buf[t].cpu().numpy() == orc[t].rows()).all(), (c, t)
     assert ctx.sync_status() == 0
+
+
+def test_the_default_geometry_brings_the_one_kernel_back():
+    import ctypes
+    import torch
+    import paper_2609_37538_b200 as avsg
+    kv = _kv(avsg)
+    ctx = avsg.Context(100, 256, RB, 16, 2, 4)
+    cudart = ctypes.CDLL("libcudart.so.12")
+    stream = torch.cuda.Stream()
+
+    def kernels(n):                                      # of a call that is captured
+        X = torch.zeros((n, 2, 16), dtype=torch.int32, device="cuda")
+        slots = torch.empty_like(X)
+        torch.cuda.synchronize()
+        s, graph, nodes = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
+        assert cudart.cudaStreamBeginCapture(s, 2) == 0
+        ctx.prepare(list(range(n)), [kv] * n, 2, 16).run(X, [CTX] * n, slots, stream=stream)
+        assert cudart.cudaStreamEndCapture(s, ctypes.byref(graph)) == 0
+        assert cudart.cudaGraphGetNodes(graph, None, ctypes.byref(nodes)) == 0
+        assert cudart.cudaGraphDestroy(graph) == 0
+        return nodes.value
+
+    assert kernels(3) == 1 and kernels(74) == 1 and kernels(100) == 2
+    for geometry in ((148, 256), (0, 128), (37, 64)):
+        ctx.set_transfer_geometry(*geometry)
+        assert kernels(3) == 2, geometry
+        ctx.set_transfer_geometry(0, 256)
+        assert kernels(3) == 1 and kernels(74) == 1
