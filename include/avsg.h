@@ -193,9 +193,9 @@ typedef struct {
                                       are resident by then): it polls the word, works on
                                       the hits, and executes griddepcontrol.wait before it
                                       touches a missed row.  avsg_step only:
-                                      avsg_step_host (which returns its outputs that early
-                                      by itself) and AVSG_XFER_ALL_K (no hits) refuse it
-                                      with AVSG_EINVAL                                   */
+                                      avsg_step_host (whose caller waits for the whole call)
+                                      and AVSG_XFER_ALL_K (no hits) refuse it with
+                                      AVSG_EINVAL                                        */
     uint64_t        stage_one_done_value; /* what is stored; the caller chooses values that
                                       let it tell calls apart (e.g. a running count).  A
                                       call captured in a CUDA graph stores the value it was
@@ -279,10 +279,12 @@ int avsg_reset_async(avsg_ctx *ctx, const uint32_t *table_ids, uint32_t n, void 
 int avsg_step(avsg_ctx *ctx, const avsg_step_args *args, void *cuda_stream);
 
 /* Same operation (Algorithm 4), but indices / slots / hit / miss_count are HOST pointers (pinned for
- * asynchrony), and the ids are in place when the call is made.  Pinned buffers are read and
- * written by the kernels themselves (AVSG_XFER_SM_BALANCED or _OVERLAP, not AVSG_INDEX_PAPER);
- * otherwise the library stages them through its own device buffers: one upload of the ids, one
- * download per requested output. */
+ * asynchrony), and the ids are in place when the call is made.  The outputs are there when the
+ * call has finished.  Pinned buffers are read and
+ * written by the kernels themselves (AVSG_XFER_SM_BALANCED or _OVERLAP, not AVSG_INDEX_PAPER nor
+ * tables of several Stage One blocks); otherwise, and for more than 16384 ids that do not begin on a
+ * 32-byte boundary with a K that is a multiple of 8, the library stages them through its own device
+ * buffers: one upload of the ids, one download per requested output. */
 int avsg_step_host(avsg_ctx *ctx, const avsg_step_args *args, void *cuda_stream);
 
 /* Sec. 3.1: the S-slot device buffer that sparse attention reads through the

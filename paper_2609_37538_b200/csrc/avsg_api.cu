@@ -14,6 +14,7 @@
 using namespace avsg;
 
 namespace {
+constexpr size_t HOST_ODD_IDS = 16384;             // see step_impl()
 constexpr uint32_t XFER_THREADS = 256;             // per block of a transfer grid, unless the caller sets a geometry
 constexpr size_t FLAG_BYTES = ((size_t)OVERLAP_MAX_TABLES * OVERLAP_MAX_TOKENS + 1) * sizeof(uint32_t);
 }
@@ -226,15 +227,16 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     // them (measured with 32 tables: see put_outputs()).  Pageable ones, the paper-literal kernel and the comparators
     // go through copies on a side stream, and so do tables of several Stage One blocks, each of which would read all ids
     // from the host (S = 16384 with 38, 50, 64 tables 168, 210, 263 us by copies, 219, 285, 372 in place; S = 32768, four
-    // tokens, 16 tables 146 and 306; only one to four tables were quicker in place).  So do calls of more than a few
-    // tables and several tokens whose ids do not begin on 64-byte boundaries: the link moves them in parts of lines, and
-    // the tokens wait for one another's.  32 tables in place / by copies: K = 256, 272 (four tokens) 42, 44 / 62, 65; K =
-    // 257, 260 92, 70 / 63, 63; K = 500, 1001 (two tokens) 62, 108 / 57, 78; K = 257 (one token) 27.6 / 27.8; eight
-    // tables, K = 257, four tokens 34.7 / 41.7.  And ids that do not begin on a word's boundary, which the copies take.
+    // tokens, 16 tables 146 and 306; only one to four tables were quicker in place).  So do calls of more than
+    // HOST_ODD_IDS ids whose tokens do not all begin on 32-byte boundaries, which the link moves in parts of its units, while
+    // a copy costs its event.  In place, begun 0, 32 and 4 bytes behind a line / by copies: 32 tables with K = 264 (four
+    // tokens) 51, 44, - / 71; 520 (two) 44, 34, 60 / 62; 2048 (two) 139, 130, 222 / 153; 100 tables, one token, K = 168 31, 30,
+    // 61 / 51; 328 41, 34, 84 / 58; six tables, K = 1000, four tokens 37, 34, 69 / 57; 16384 ids: eight tables, two tokens 26,
+    // 21, 42 / 45; 32 tables, one token 22, 18, 32 / 41.  And ids that do not begin on a word's boundary, which the copies take.
     HostOut out;
     bool host_ids = false;
-    const bool whole_lines = K % 16u == 0 || n_q == 1 || n <= (uint32_t)STEP_FEW_TABLES;
-    if (host_io && c->cfg.index_mode != AVSG_INDEX_PAPER && c->s1_cluster == 1 && whole_lines &&
+    const bool in_place = (K % 8u == 0 && reinterpret_cast<uint64_t>(a->indices) % 32u == 0) || n_ids <= HOST_ODD_IDS;
+    if (host_io && c->cfg.index_mode != AVSG_INDEX_PAPER && c->s1_cluster == 1 && in_place &&
         (c->cfg.transfer_mode == AVSG_XFER_SM_BALANCED || c->cfg.transfer_mode == AVSG_XFER_SM_OVERLAP)) {
         const int32_t* ids = reinterpret_cast<uint64_t>(a->indices) % 4u == 0 ? mapped(a->indices, n_ids) : nullptr;
         out.host_slots = mapped(a->slots, n_ids);

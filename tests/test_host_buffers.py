@@ -121,3 +121,27 @@ def test_buffers_off_the_boundary_of_a_word(mode, n, ids_at, slots_at, hit_at, c
         at = view.ctypes.data - whole.data_ptr()
         assert (whole[:at] == 0x5A).all() and (whole[at + view.nbytes :] == 0x5A).all()
     assert ctx.sync_status() == 0
+
+
+def test_many_ids_off_the_link_s_units_go_by_copy():
+    """Where more than 16384 ids begin decides the route."""
+    import torch
+    import paper_2609_37538_b200 as avsg
+    n, n_q, ctxlen, rb = 12, 2, 4000, 48
+    for K, offsets in ((704, (0, 1, 8, 4, 24, 7)), (700, (0, 8)), (682, (0, 1))):          # (in ids; the last has 16368)
+        traces, kv, ctx, orc = _setup(avsg, n, n_q, K, 2048, rb, ctxlen, "XFER_SM_BALANCED", len(offsets))
+        whole = torch.full((n * n_q * K + 32,), -1, dtype=torch.int32, pin_memory=True)
+        base = -whole.data_ptr() % 64 // 4
+        slots = torch.empty((n, n_q, K), dtype=torch.int32, pin_memory=True)
+        for t, off in enumerate(offsets):
+            ids = whole[base + off : base + off + n * n_q * K].view(n, n_q, K)
+            ids.copy_(torch.from_numpy(np.stack([traces[i][0][t] for i in range(n)])))
+            N = [int(traces[i][1][t]) for i in range(n)]
+            with torch.autograd.profiler.profile(use_device="cuda") as seen:
+                ctx.prepare(list(range(n)), [kv] * n, n_q, K).run(ids, N, slots, host=True)
+                torch.cuda.synchronize()
+            copies = sum("Memcpy" in e.name for e in seen.function_events)
+            for i in range(n):
+                assert (slots[i].numpy() == orc[i].step(traces[i][0][t], N[i], kv.numpy(), rb).O).all(), (K, t, i)
+            assert (copies > 0) == (K == 700 or (K == 704 and off % 8 != 0)), (K, off, copies)
+        assert ctx.sync_status() == 0

@@ -72,7 +72,7 @@ def test_calls_of_changing_size(S, K_max, cluster):
 
 # The most tables that get clusters of eight, four, three and two blocks on a device of 148 SMs, and one more than that;
 # more rows per block and token than warps, fewer, and none
-# (the host's ids and outputs are used in place where K is a multiple of 16 or the tables are few)
+# (the host's ids are used in place where there are few or K is a multiple of 8, else they go by copy)
 @pytest.mark.parametrize("n,K", [(4, 200), (8, 201), (9, 200), (9, 208), (33, 208), (34, 200), (45, 208), (46, 208), (74, 208), (75, 208)])
 def test_clusters_of_every_size(n, K):
     import torch
