@@ -88,9 +88,16 @@ SHAPES = [
 ]
 
 
+# Calls of up to 74 tables run both stages in one kernel unless the context has a transfer geometry of its own; this one is
+# what the default comes to on a B200.
+TWO_KERNELS = (148, 256)
+both_paths = pytest.mark.parametrize("geometry", [None, TWO_KERNELS], ids=["default", "two-kernels"])
+
+
+@both_paths
 @pytest.mark.parametrize("name,kw", SHAPES)
-def test_shapes(avsg, name, kw):
-    _parity(tr.workload(name, **kw))
+def test_shapes(avsg, name, kw, geometry):
+    _parity(tr.workload(name, **kw), xfer_geometry=geometry)
 
 
 def test_more_tables_than_one_launch_takes(avsg):
@@ -226,18 +233,22 @@ def test_cluster_full_c2_c3_and_unsorted(avsg):
 
 
 # ---- Stage Two overlapping Stage One (latency hiding, App. G) ---------------------------------------------------
-@pytest.mark.parametrize("name,kw,index", [
-    ("C1", {}, "INDEX_HASH"), ("C2", {}, "INDEX_HASH"), ("C2", {}, "INDEX_DIRECT"), ("C3", {}, "INDEX_DIRECT"),
-    ("C3", dict(requests=16, layers=2, n_iters=32), "INDEX_HASH"), ("C4", {}, "INDEX_DIRECT"), ("C5", {}, "INDEX_HASH"),
+@pytest.mark.parametrize("name,kw,index,geometry", [
+    ("C1", {}, "INDEX_HASH", None), ("C2", {}, "INDEX_HASH", None), ("C2", {}, "INDEX_DIRECT", None), ("C3", {}, "INDEX_DIRECT", None),
+    ("C3", dict(requests=16, layers=2, n_iters=32), "INDEX_HASH", None), ("C4", {}, "INDEX_DIRECT", None), ("C5", {}, "INDEX_HASH", None),
+    ("C1", {}, "INDEX_HASH", TWO_KERNELS), ("C2", {}, "INDEX_HASH", TWO_KERNELS),
+    ("C3", dict(requests=16, layers=2, n_iters=32), "INDEX_DIRECT", TWO_KERNELS),
 ])
-def test_overlap_mode_full(avsg, name, kw, index):
-    r = _parity(tr.workload(name, **kw), mode=avsg.XFER_SM_OVERLAP, index_mode=getattr(avsg, index), buffer_every=8)
+def test_overlap_mode_full(avsg, name, kw, index, geometry):
+    r = _parity(tr.workload(name, **kw), mode=avsg.XFER_SM_OVERLAP, index_mode=getattr(avsg, index), buffer_every=8,
+                xfer_geometry=geometry)
     assert r["gpu"]["rows_copied"] == r["oracle"]["rows_copied"] > 0
 
 
+@both_paths
 @pytest.mark.parametrize("name,kw", SHAPES)
-def test_overlap_mode_shapes(avsg, name, kw):
-    _parity(tr.workload(name, **kw), mode=avsg.XFER_SM_OVERLAP)
+def test_overlap_mode_shapes(avsg, name, kw, geometry):
+    _parity(tr.workload(name, **kw), mode=avsg.XFER_SM_OVERLAP, xfer_geometry=geometry)
 
 
 def test_overlap_mode_host_io_strides_geometries_and_fallbacks(avsg):
@@ -252,9 +263,10 @@ def test_overlap_mode_host_io_strides_geometries_and_fallbacks(avsg):
     _parity(many, mode=avsg.XFER_SM_OVERLAP, buffer_every=3)
 
 
-def test_overlap_mode_four_tokens_and_mode_switches(avsg):
+@both_paths
+def test_overlap_mode_four_tokens_and_mode_switches(avsg, geometry):
     """MTP-3: four tokens per iteration, i.e. four publish / wait rounds per call; the transfer mode is switched
-    between calls, so calls with and without the per-token counters alternate on one context."""
+    between calls, so that, in two kernels, calls with and without the hand-over flags alternate on one context."""
     import torch
     S, K, n_q, T, rb, n = 2048, 384, 4, 12, 656, 3
     w = tr.workload("C5", topk=K, buffer_slots=S, n_iters=n_q * T, requests=n, ctx_lo=20000, ctx_hi=20001, row_bytes=rb)
@@ -265,6 +277,8 @@ def test_overlap_mode_four_tokens_and_mode_switches(avsg):
         tr.fill_kv(b.data_ptr(), w.seed, ti, cfg.context, rb)
         kv.append(b); kvn.append(b.numpy())
     ctx = avsg.Context(n, S, rb, K, n_q, 16, transfer_mode=avsg.XFER_SM_OVERLAP)
+    if geometry:
+        ctx.set_transfer_geometry(*geometry)
     orc = [OracleTable(S, rb, 16) for _ in range(n)]
     for t in range(T):
         ctx.set_transfer_mode(avsg.XFER_SM_BALANCED if t % 4 == 3 else avsg.XFER_SM_OVERLAP)
@@ -638,9 +652,11 @@ def test_stream_ordered_reset(avsg, mode_name, index_name):
     assert ctx.sync_status() == 0
 
 
-def test_overlap_wait_gives_up_and_the_context_stays_usable(avsg):
+@both_paths
+def test_overlap_wait_gives_up_and_the_context_stays_usable(avsg, geometry):
     """The overlapped transfer kernel launched without its Stage One: every block polls up to its limit, raises
-    the status bit, copies nothing and returns; after clearing the status word the context works as before."""
+    the status bit, copies nothing and returns; after clearing the status word the context works as before, whether its
+    calls use the hand-over flags (two kernels) or not."""
     import time
     import torch
     w = tr.workload("C2", topk=256, buffer_slots=1024, n_iters=8, context=16384, recent_window=1024)
@@ -648,6 +664,8 @@ def test_overlap_wait_gives_up_and_the_context_stays_usable(avsg):
     kv = avsg.pinned_empty(w.tables[0].context * w.row_bytes)
     tr.fill_kv(kv.data_ptr(), w.seed, 0, w.tables[0].context, w.row_bytes)
     ctx = avsg.Context(1, w.buffer_slots, w.row_bytes, w.topk, w.n_q, 16, transfer_mode=avsg.XFER_SM_OVERLAP)
+    if geometry:
+        ctx.set_transfer_geometry(*geometry)
     orc = OracleTable(w.buffer_slots, w.row_bytes, 16)
 
     def step(t):
@@ -667,8 +685,8 @@ def test_overlap_wait_gives_up_and_the_context_stays_usable(avsg):
     assert time.time() - t0 < 10.0
     assert word == avsg.STATUS_WAIT_TIMEOUT, word
     assert (ctx.buffer(0).cpu().numpy() == before).all()
-    # the flags of the overlapped mode carry the number of their call, which the kernel that gave up advanced all
-    # the same: the next calls run correctly even BEFORE the status word is cleared (it stays set: it is sticky)
+    # every call takes its hand-over flags down itself before its transfer kernel can start: the next calls run correctly
+    # even BEFORE the status word is cleared (it stays set: it is sticky)
     for t in range(4, 6):
         step(t)
     assert ctx.sync_status() == avsg.STATUS_WAIT_TIMEOUT
@@ -681,12 +699,14 @@ def test_overlap_wait_gives_up_and_the_context_stays_usable(avsg):
     assert ctx.sync_status() == 0
 
 
-@pytest.mark.parametrize("index,cluster", [("INDEX_HASH", 0), ("INDEX_DIRECT", 0), ("INDEX_DIRECT", 2)])
-def test_soak_random_subsets_modes_and_token_counts(avsg, index, cluster):
+@pytest.mark.parametrize("index,cluster,geometry", [("INDEX_HASH", 0, None), ("INDEX_DIRECT", 0, TWO_KERNELS),
+                                                    ("INDEX_DIRECT", 2, None), ("INDEX_HASH", 0, "both")])
+def test_soak_random_subsets_modes_and_token_counts(avsg, index, cluster, geometry):
     """300 calls on one context: every call takes a random subset of the tables in a random order, a random number
     of tokens, a random Stage Two mode and either device or host buffers; every table is compared with its own
-    oracle after every call it took part in.  Exercises the hand-over flags of the overlapped mode across calls of
-    different shapes (a table's flag of an earlier call must never be taken for a current one)."""
+    oracle after every call it took part in.  With a geometry or clusters it exercises the hand-over flags of the
+    overlapped mode across calls of different shapes (a table's flag of an earlier call must never be taken for a current
+    one), without both the calls in one kernel, and in the last case the two in turn."""
     import torch
     rng = np.random.default_rng(77)
     n, S, K, n_q_max, rb, ctxlen, L = 7, 512, 48, 4, 48, 4000, 5
@@ -701,7 +721,11 @@ def test_soak_random_subsets_modes_and_token_counts(avsg, index, cluster):
     prev = [rng.choice(ctxlen, K, replace=False) for _ in range(n)]
     modes = [avsg.XFER_SM_OVERLAP, avsg.XFER_SM_OVERLAP, avsg.XFER_SM_BALANCED, avsg.XFER_REQUEST_LEVEL,
              avsg.XFER_POSITION_LEVEL]
+    if geometry == TWO_KERNELS:
+        ctx.set_transfer_geometry(*geometry)
     for call in range(300):
+        if geometry == "both":
+            ctx.set_transfer_geometry(*((0, 256) if rng.random() < 0.5 else TWO_KERNELS))
         tabs = [int(t) for t in rng.permutation(n)[: int(rng.integers(1, n + 1))]]
         n_q = int(rng.integers(1, n_q_max + 1))
         ctx.set_transfer_mode(int(rng.choice(modes)))
@@ -732,10 +756,12 @@ def test_soak_random_subsets_modes_and_token_counts(avsg, index, cluster):
     assert ctx.sync_status() == 0
 
 
-@pytest.mark.parametrize("n,mode_name", [(6, "XFER_SM_OVERLAP"), (90, "XFER_SM_OVERLAP"), (40, "XFER_SM_BALANCED")])
-def test_two_contexts_on_two_streams_at_once(avsg, n, mode_name):
+@pytest.mark.parametrize("n,mode_name,geometry", [(6, "XFER_SM_OVERLAP", None), (90, "XFER_SM_OVERLAP", None), (40, "XFER_SM_BALANCED", None),
+                                                  (6, "XFER_SM_OVERLAP", TWO_KERNELS), (40, "XFER_SM_OVERLAP", TWO_KERNELS),
+                                                  (40, "XFER_SM_BALANCED", TWO_KERNELS)])
+def test_two_contexts_on_two_streams_at_once(avsg, n, mode_name, geometry):
     """Two contexts, each on a stream of its own, issue their calls without waiting for one another: the kernels of
-    both share the GPU.  In the overlapped mode the waiting transfer grid of one context must never keep the other's
+    both share the GPU.  In the overlapped mode, in two kernels, the waiting transfer grid of one context must never keep the other's
     Stage One off the SMs (a transfer grid only starts once every block of its own Stage One has started; 90 tables
     take the round-by-round path).  Both are compared with their oracles after every iteration."""
     import torch
@@ -747,6 +773,8 @@ def test_two_contexts_on_two_streams_at_once(avsg, n, mode_name):
     for c in range(2):
         ctxs.append(avsg.Context(n, S, rb, K, n_q, 16, transfer_mode=getattr(avsg, mode_name),
                                  index_mode=avsg.INDEX_DIRECT if c == 0 else avsg.INDEX_HASH, max_context=ctxlen + n_q))
+        if geometry:
+            ctxs[c].set_transfer_geometry(*geometry)
         orcs.append([OracleTable(S, rb, 16) for _ in range(n)])
         traces.append([tr.generate(tr.TraceConfig(seed=60 + c, table=i, topk=K, n_q=n_q, n_iters=T, context=ctxlen,
                                                   ctx_growth=True, beta=(9, 1), p_recent=0.5, recent_window=512))

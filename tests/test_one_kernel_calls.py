@@ -70,14 +70,17 @@ def test_calls_of_changing_size(S, K_max, cluster):
     assert ctx.sync_status() == 0
 
 
-# The most tables that get clusters of eight, four, three and two blocks on a device of 148 SMs, and one more than that;
-# more rows per block and token than warps, fewer, and none
+# The most tables that get clusters of eight, four, three and two blocks on a device of 148 SMs, and one more than that: with
+# 8192 slots 8, 33, 45 and 74 tables, with 1024 slots (blocks of half the size) 16, 66 and 74 of the first three; more rows
+# per block and token than warps, fewer, and none
 # (the host's ids are used in place where there are few or K is a multiple of 8, else they go by copy)
-@pytest.mark.parametrize("n,K", [(4, 200), (8, 201), (9, 200), (9, 208), (33, 208), (34, 200), (45, 208), (46, 208), (74, 208), (75, 208)])
-def test_clusters_of_every_size(n, K):
+@pytest.mark.parametrize("n,K,S", [(n, K, 1024) for n, K in ((4, 200), (8, 201), (9, 200), (9, 208), (33, 208), (34, 200), (45, 208),
+                                                             (46, 208), (74, 208), (75, 208), (16, 200), (17, 200), (66, 200), (67, 200))] +
+                                  [(n, K, 8192) for n, K in ((8, 600), (9, 601), (33, 400), (34, 400), (45, 300), (46, 601), (74, 300))])
+def test_clusters_of_every_size(n, K, S):
     import torch
     import paper_2609_37538_b200 as avsg
-    S, n_q, L = 1024, 3, 3
+    n_q, L = 3, 3
     rng = np.random.default_rng(n)
     kv = _kv(avsg)
     ctx = avsg.Context(n, S, RB, K, n_q, L)
@@ -88,7 +91,7 @@ def test_clusters_of_every_size(n, K):
         if c == 4:
             tabs = tabs[:2]                              # a small one between the large ones
         ctx.set_transfer_mode(avsg.XFER_SM_OVERLAP if c % 2 else avsg.XFER_SM_BALANCED)
-        X = np.stack([[rng.choice(rng.choice([K, 260, 3000]), K, replace=False) for _ in range(n_q)] for _ in tabs]).astype(np.int32)
+        X = np.stack([[rng.choice(rng.choice([K, max(K, 260), 3000]), K, replace=False) for _ in range(n_q)] for _ in tabs]).astype(np.int32)
         X = done[-1][1] if c == 6 else X                 # (other tables, the same ids)
         host = c in (2, 5)
         ids = torch.from_numpy(X).pin_memory() if host else torch.from_numpy(X).cuda()
