@@ -35,7 +35,7 @@ METRIC = "miss-only H2D gather GB/s (% of link peak); match+reserve us per decod
 # DRAM traffic per unit from the ncu capture summarised under profiles/ (dram__bytes_read + dram__bytes_write
 # per launch of the one-layer case, divided by the units of that launch); scaled by the units of a launch here.
 NCU_XFER_DRAM_BYTES_PER_ROW = 91.0          # 0.94 MB per launch of 10.3 k rows: the written rows stay in L2
-NCU_S1_DRAM_BYTES_PER_TABLE = 59400.0       # 1.90 MB per launch of 32 tables (state and ids in; the writes stay in L2)
+NCU_S1_DRAM_BYTES_PER_TABLE = 58400.0       # 1.87 MB per launch of 32 tables (state and ids in; the writes stay in L2)
 PAPER_CONTEXT = {
     "hardware": "Ascend 910B NPU (paper), not comparable",
     "hash_vs_dual_pointer_speedup": 2.80, "stage_one_us_K2048_S2048": 53.7,
@@ -448,7 +448,7 @@ def run_cuda(args):
         call_gbs = call_bytes / 1e3 / call_us
         roofline = {"bound": "host_link", "kernel": "avsg_step_kernel" if one_kernel else "avsg_transfer_overlap_kernel", "achieved": call_gbs,
                     "peak": link_peak, "unit": "GB/s", "frac": call_gbs / link_peak,
-                    "traffic": NCU_XFER_DRAM_BYTES_PER_ROW * call_bytes / rb,
+                    "traffic": NCU_XFER_DRAM_BYTES_PER_ROW * call_bytes / rb + (NCU_S1_DRAM_BYTES_PER_TABLE * n_tab if one_kernel else 0.0),
                     "peak_kind": "measured in this run (pinned cudaMemcpyAsync H2D, 1 GiB, best of 4 after one warm-up copy)", "peak_repeats": 4,
                     "duration_us": call_us,
                     "note": "algorithmic bytes = row_bytes x missed rows per launch; duration = CUDA events around the "
