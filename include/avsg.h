@@ -78,7 +78,11 @@ extern "C" {
                                        slots, nor with stage_one_done above three tables).
                                        Its blocks take whole SMs while they run: who wants
                                        room for other kernels beside the call sets a
-                                       transfer geometry.  Calls whose Stage One takes
+                                       transfer geometry (100 calls of 8, 32, 64 tables
+                                       beside 100 GEMMs of 9.8 ms on another stream: both
+                                       through after 10.8, 17.1, 25.1 ms, with a geometry
+                                       9.6, 14.0, 25.5; alone the calls take 3.8, 12.5, 24.5
+                                       and 4.4, 12.8, 24.6).  Calls whose Stage One takes
                                        more than half of the SMs are served as in
                                        AVSG_XFER_SM_OVERLAP                              */
 #define AVSG_XFER_COPY_ENGINE   1u  /* comparator: miss list read back, one async copy

@@ -243,9 +243,12 @@ struct StepClusters {
 };
 StepClusters step_clusters(size_t max_smem);            // after stage_one_prepare
 // Whether the grid behind a call in one kernel may start under it (see the kernel).  Up to three tables, and up to eight
-// that reach little host memory (id_limit: rows a table's ids can reach): early / late, eight tables of 131072 rows 35.3 /
-// 35.7 us, of 1 Mi 59.7 / 46.3; five tables with K = 139 of 36028 rows 9.3 / 9.7.  More tables gain nothing by it (32 tables 113.0
-// / 112.9), and ids in host memory that are fetched under a call's rows slow these down (39 tables, K = 3430: 215 / 124).
+// that reach little host memory (id_limit: rows a table's ids can reach).  Early / late, calls of K = 2048: one table 13.2 / 13.4
+// us (0.08 GB) and 13.7 / 13.9 (0.6 GB); two 17.1 / 17.1, 18.0 / 18.0 (1.3 GB); three 21.4 / 21.3, 23.3 / 23.7 (1.9 GB); four 25.8 /
+// 25.8 (0.3 GB), 27.8 / 27.3 (1.3 GB), 28.9 / 28.2 (2.6 GB); six 34.4 / 34.4 (0.5 GB), 36.7 / 36.0 (1.9 GB), 39.1 / 37.2 (3.8 GB); eight 42.8 /
+// 42.8 (0.6 GB), 44.2 / 44.3 (1.3 GB), 45.2 / 44.9 (1.9 GB), 46.5 / 45.3 (2.6 GB), 58.3 / 46.7 (5.1 GB); five tables with K = 139 9.3 / 9.7.
+// More tables gain nothing by it (32 tables 113.0 / 112.9), and ids in host memory that are fetched under a call's rows slow these
+// down (39 tables, K = 3430: 215 / 124).
 template <int CAP>
 bool step_early(const S1ParamsT<CAP>& p)
 {

@@ -86,9 +86,9 @@ __device__ __forceinline__ void put_outputs_of(HostOut o, uint32_t ti, uint32_t 
 // blocks, and a block's over its warps).  With few rows no barrier ties the warps together and phases go round over the
 // blocks and warps: a row is a round trip of 2 us, and a warp without one in this phase is already at work on the next
 // (230 rows in two tokens: 17.3 us a call where the block met after every phase and found its last block with a counter,
-// 15.8 now).  With more rows per block than warps the copying warps do meet: rows of a
-// later phase that mix with this one's cost 1 % where the link is the limit (128 tables in one call: 392 us against
-// 394), and 5 % where translations on the way to 11 GB of host memory are.
+// 15.8 now).  With more rows per block than warps
+// the copying warps do meet: rows of a later phase that mix with this one's cost 5 % where translations on the way to 11 GB of
+// host memory are the limit (where the link is, no difference was found).
 constexpr uint32_t READY_SPIN_LIMIT = 1u << 28;              // over 10 s: the polling warp ends the wait long before
 
 // Words of shared memory that the phases of a call take: prefix sums [round_size + 1] and first list entries [round_size].

@@ -1,5 +1,5 @@
-// Device helpers shared by the Stage One kernels (single-block and cluster): packed lifetime arithmetic, the
-// lifetime histogram, id loads, and the per-token publication of the overlapped Stage Two.
+// Device helpers of the Stage One kernels: thread-block clusters, packed lifetimes, warp ranks and the hand-over to the
+// overlapped Stage Two, shared by all of them; id loads, the range check and the lifetime histogram of the paper-literal one.
 #pragma once
 #include "avsg_kernels.cuh"
 
