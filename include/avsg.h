@@ -71,7 +71,7 @@ extern "C" {
                                        kernel in this mode and in AVSG_XFER_SM_OVERLAP: a
                                        thread-block cluster per table, Stage Two following
                                        Stage One token by token; the split over SMs is then
-                                       even within a table, and from 34 tables on rows of a
+                                       by position within a table, and from 34 tables on rows of a
                                        table that misses more than 512 ids of a token are
                                        taken over by blocks of others that are through (not with arriving, timing,
                                        an own transfer geometry or a table above 8192

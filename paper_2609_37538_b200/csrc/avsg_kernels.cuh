@@ -241,7 +241,8 @@ struct StepClusters {
         return 0;
     }
 };
-StepClusters step_clusters(size_t max_smem);            // after stage_one_prepare
+cudaError_t step_prepare(size_t max_smem);
+StepClusters step_clusters(size_t max_smem);            // after step_prepare
 // Whether the grid behind a call in one kernel may start under it (see the kernel).  Up to three tables, and up to eight
 // that reach little host memory (id_limit: rows a table's ids can reach).  Early / late, calls of K = 2048: one table 13.2 / 13.4
 // us (0.08 GB) and 13.7 / 13.9 (0.6 GB); two 17.1 / 17.1, 18.0 / 18.0 (1.3 GB); three 21.4 / 21.3, 23.3 / 23.7 (1.9 GB); four 25.8 /

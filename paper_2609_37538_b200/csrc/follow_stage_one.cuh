@@ -19,6 +19,25 @@ __device__ __forceinline__ void st16(uint64_t addr, const int4& v)
     asm volatile("st.global.v4.s32 [%0], {%1, %2, %3, %4};" :: "l"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
+// A row of up to ROW_CHUNKS 16-byte pieces in a warp's registers, for a kernel that asks for it before it knows where it goes.
+// (By cp.async into shared memory, which would need no registers, 32 tables take 245 us past L1 and 125 through it, and not 117:
+// those requests are smaller.)
+constexpr uint32_t ROW_CHUNKS = 96;
+struct Row { int4 v[ROW_CHUNKS / 32]; };
+__device__ __forceinline__ void load_row(Row& r, uint64_t src, uint32_t cpr, uint32_t lane)
+{
+#pragma unroll
+    for (uint32_t k = 0; k < ROW_CHUNKS / 32; ++k)
+        if (lane + 32u * k < cpr) r.v[k] = ld16(src + 16ull * (lane + 32u * k));
+    __syncwarp();                      // (the compiler may move plain loads behind a wait, but not behind this)
+}
+__device__ __forceinline__ void store_row(const Row& r, uint64_t dst, uint32_t cpr, uint32_t lane)
+{
+#pragma unroll
+    for (uint32_t k = 0; k < ROW_CHUNKS / 32; ++k)
+        if (lane + 32u * k < cpr) st16(dst + 16ull * (lane + 32u * k), r.v[k]);
+}
+
 // One warp moves one row: 16-byte loads from the (host) source, all issued before the 16-byte stores into the slot.
 // Rows of up to 1 KiB (two loads per lane) take the short path, whose instruction order is fixed by hand: both
 // loads of a lane are in flight together.

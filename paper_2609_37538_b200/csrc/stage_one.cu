@@ -45,7 +45,6 @@ namespace {
 struct S1Layout {
     uint32_t head, life, bits, tot, ndead, cnt, sum, miss, pos, dead, total;
 };
-__host__ __device__ inline uint32_t align16(uint32_t n) { return (n + 15u) & ~15u; }
 __host__ __device__ inline S1Layout s1_layout(uint32_t S, uint32_t K, uint32_t n_q, uint32_t nt)
 {
     S1Layout o;
@@ -64,33 +63,12 @@ __host__ __device__ inline S1Layout s1_layout(uint32_t S, uint32_t K, uint32_t n
     return o;
 }
 
-// Bits 0 .. 3: the sign bits of a word's four bytes.
-__device__ __forceinline__ uint32_t signs(uint32_t w) { return (((w >> 7) & 0x01010101u) * 0x10204080u) >> 28; }
-
-constexpr uint32_t STEP_SPIN_LIMIT = 1u << 18;            // tries; the hardware suspends the warp for 4 us in each: 1 s
-#ifndef AVSG_STEP_GIVE_UP                                 // (a test builds the library with waits that run out)
-#define AVSG_STEP_GIVE_UP STEP_SPIN_LIMIT
-#endif
-
-// Words of eight bytes that one of `copying` blocks gets per token, at most: a head and its rows.
-__device__ __forceinline__ uint32_t step_rows(uint32_t K, uint32_t copying) { return 1u + (K + copying - 1u) / copying; }
-
-// Rows that blocks of other tables may take (see avsg_step_kernel): from how many misses of a token on, how many of a
-// table's rows stay for its own blocks (other blocks' caches of translations do not know the table: with 256 left 64 unequal
-// requests take 326 us, with 128 330, without any sharing 324), how many warps of the call take some at most (of 144 rows
-// under way the link is full; more only copy the last rows twice).
-constexpr uint32_t SHARED_FROM = 512, SHARED_LEFT = 256, SHARED_WARPS = 144, SHARED_CLUSTER = 4;
-
 // SPT slots per thread (a power of two): S <= SPT * blockDim.x.  IPT: the most ids a thread has to look up per token
 // (K <= S, so SPT is always enough).  CAP: tables the argument block has room for.  The block serves the tables block,
-// block + blocks, ... of the launch.  CLUSTER: it is the first block of a cluster whose others copy what it places
-// (avsg_step_kernel); a_mbar: their mbarriers, one per token.  WIDE: the state is aligned (state_is_aligned()).
-// SHARE: rows of a table with very many misses may be copied by other tables' blocks.
-template <int SPT, int IPT, bool CLUSTER, bool WIDE, bool SHARE, int CAP>
-__device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_t block, const uint32_t blocks, unsigned char* smem, const uint32_t a_mbar = 0)
+// block + blocks, ... of the launch.  WIDE: the state is aligned (state_is_aligned()).
+template <int SPT, int IPT, bool WIDE, int CAP>
+__device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_t block, const uint32_t blocks, unsigned char* smem)
 {
-    const uint32_t copying = CAP == STEP_FEW_TABLES ? STEP_FEW_CLUSTER - 1u : CLUSTER ? cluster_size() - 1u : 1u;
-    constexpr bool SHARES = CLUSTER && CAP != STEP_FEW_TABLES;         // a copying block's rows are a share in position order
     constexpr int NV = (SPT + 3) / 4;                    // 4-slot vectors of ids / words of lifetimes per thread
     const uint32_t S = p.S, K = p.K, H = 2u * S, L = p.L;
     const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u, warp = tid >> 5, nw = nt >> 5;
@@ -168,49 +146,26 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
         life_words<SPT, true, WIDE>(g_life + j0, own, w);
         if (!p.host_ids || bt != block) load_token(ti, 0);
         if (p.verified_len_dev) N = __ldg(p.verified_len_dev + ti);
-        const uint32_t seen = !CLUSTER && bt == block ? take_flags_down(p, bt, blocks, p.n_launch) : 0u;
+        const uint32_t seen = bt == block ? take_flags_down(p, bt, blocks, p.n_launch) : 0u;
         if (tid == 0) s_sum[0] = 0;
         __syncthreads();                                 // the index is empty
 
         // ---- ids to shared memory and into the index; global pre-decay of the lifetimes (Alg. 1 Pass 1) ----
         bool stale_ids = false;                          // ids that are no longer verified (the caller took tokens back)
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            if (tid + q * nt < S / 4) {
-                const uint32_t j = 4u * (tid + q * nt);
-                const int32_t x[4] = {t4[q].x, t4[q].y, t4[q].z, t4[q].w};
-                uint32_t next[4];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    next[c] = x[c] >= 0 ? atomicExch(&s_head[hash_id(x[c], p.logH)], j + c) : NIL;
-                    stale_ids = stale_ids || x[c] >= N;
-                }
-#pragma unroll
-                for (int c = 0; c < 4; c += 2)
-                    reinterpret_cast<uint4*>(s_node)[(j + c) / 2] = make_uint4((uint32_t)x[c], (j + c) << 16 | next[c],
-                                                                               (uint32_t)x[c + 1], (j + c + 1) << 16 | next[c + 1]);
-            }
-        }
-        auto store_life = [&](uint32_t par) {            // the thread's lifetimes and dead bits, the warp's dead slots
-            uint32_t bits = 0;
-#pragma unroll
-            for (int q = 0; q < NV; ++q) bits |= signs(w[q]) << (4 * q);
-            life_words_store<SPT>(s_life + j0, own, w);
-            s_bits[tid] = (uint8_t)bits;
-            const uint32_t n = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(bits));
-            if (lane == 0) s_ndead[par + warp] = n;
-        };
+        for (int q = 0; q < NV; ++q)
+            if (tid + q * nt < S / 4) stale_ids = stale_ids || t4[q].x >= N || t4[q].y >= N || t4[q].z >= N || t4[q].w >= N;
+        index_slots(t4, s_node, s_head, S, p.logH, NIL);
         uint32_t high = 0;                               // lifetimes above L (only a caller's own state can have them)
 #pragma unroll
         for (int q = 0; q < NV; ++q) {
             if (own) high |= __vcmpgts4(w[q], L * 0x01010101u) & (SPT == 2 ? 0xFFFFu : 0xFFFFFFFFu);
             w[q] = decay4(w[q], 1);
         }
-        store_life(0);
+        store_lifetimes<SPT>(s_life, s_bits, s_ndead, own, w);
         const bool unusual = __syncthreads_or(high != 0);
 
         uint32_t list_off = 0, sum_miss = 0, sum_decay = 0, valid = 0;
-        uint32_t shared = 0;                             // SHARE: rows that other blocks may take (bit 31: there will be some)
         int2* list = p.miss_list + (size_t)ti * p.list_stride;
 
         for (uint32_t g = 0; g < p.n_q; ++g) {
@@ -222,7 +177,7 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
 
             // ---- lookups; hits: lifetime <- L, slot and flag out (Pass 1 + Pass 2) ----
             // (pass after pass over the thread's ids, so that their reads are in flight together)
-            uint32_t node[IPT], rank[IPT], missing = 0, wmiss = 0;
+            uint32_t rank[IPT], missing = 0, wmiss = 0;
             int32_t slot[IPT], was[IPT];
             bool bad = false;
 #pragma unroll
@@ -231,27 +186,9 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
                 bad = bad || (!ok && xs[k] >= 0);
                 xs[k] = ok ? xs[k] : -1;
                 valid += ok;
-                slot[k] = -1;
-                node[k] = NIL;
-                if (ok) node[k] = s_head[hash_id(xs[k], p.logH)];
             }
             if (bad) atomicOr(p.status, ST_BAD_ID);                    // not fetched: reported and taken as padding
-            uint32_t open = 1;
-            for (uint32_t it = 0; open && it <= NIL; ++it) {           // all chains of the warp side by side
-                uint2 v[IPT];
-#pragma unroll
-                for (int k = 0; k < IPT; ++k) v[k] = s_node[node[k]];
-                open = 0;
-#pragma unroll
-                for (int k = 0; k < IPT; ++k) {
-                    const bool found = (int32_t)v[k].x == xs[k];
-                    slot[k] = found ? (int32_t)(v[k].y >> 16) : slot[k];
-                    node[k] = found ? NIL : v[k].y & 0xFFFFu;
-                    open |= node[k] ^ NIL;
-                }
-                open = __any_sync(0xffffffffu, open);
-            }
-            if (open) atomicOr(p.status, ST_PROBE_EXHAUSTED);
+            find_slots(xs, s_node, s_head, p.logH, NIL, p.status, slot);
             // with lifetimes above L on entry a slot reserved in this step may go to yet another id: its first node is stale
             if (unusual) {
 #pragma unroll
@@ -283,7 +220,7 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
                 if (lane == 0 && valid) atomicAdd(s_sum, valid);
             }
             if (lane == 0) s_tot[par + warp] = wmiss;
-            if (!CLUSTER && g == 0 && bt == block && (p.flags || p.early)) start_dependents(seen);
+            if (g == 0 && bt == block && (p.flags || p.early)) start_dependents(seen);
             __syncthreads();
 
             // ---- CollectDead and the misses, each in order; the prefix over the warps: lane l looks at warp l ----
@@ -294,16 +231,6 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
             uint32_t dtotal = all & 0xFFFFu, dead_before = before & 0xFFFFu, d = 0;
             sum_miss += n_g;
             if (tid == 0 && p.miss_count) p.miss_count[(size_t)ti * p.n_q + g] = (int32_t)n_g;
-            const bool share_it = SHARE && n_g > SHARED_FROM;
-            if (share_it && !shared) {
-                shared = SHARED_COMING;
-                if (tid == 0) {                          // (in place before the table's own blocks hear of the rows)
-                    p.shared[ti].taken = p.shared[ti].begun = 0;
-                    __threadfence();
-                    *reinterpret_cast<volatile uint32_t*>(&p.shared[ti].rows) = SHARED_COMING;
-                    __threadfence();
-                }
-            }
             if (missing) {
 #pragma unroll
                 for (int k = 0; k < IPT; ++k) {
@@ -318,39 +245,10 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
             // Pass 3, the while-loop of Alg. 1: decay until n_g slots are dead
             if (dtotal < n_g) {
                 life_words<SPT>(s_life + j0, own, w);
-                uint32_t lo = 0, hi = L + 1u, buf = 0;   // lo decays are too few, hi are enough (lifetimes are <= L)
-                while (hi - lo > 1u) {                   // (L >= 1: at least once, so every warp has read the old counts)
-                    uint32_t c[4];                       // candidates in (lo, hi), ascending; small ones first
-#pragma unroll
-                    for (uint32_t i = 0; i < 4; ++i) {
-                        c[i] = lo == 0 ? 1u << i : lo + ((i + 1u) * (hi - lo)) / 5u;
-                        c[i] = c[i] <= lo ? lo + 1u : (c[i] >= hi ? hi - 1u : c[i]);
-                    }
-                    uint32_t n01 = 0, n23 = 0;
-#pragma unroll
-                    for (int q = 0; q < NV; ++q) {
-                        n01 += __popc(__vsubss4(w[q], c[0] * 0x01010101u) & 0x80808080u) |
-                               (__popc(__vsubss4(w[q], c[1] * 0x01010101u) & 0x80808080u) << 16);
-                        n23 += __popc(__vsubss4(w[q], c[2] * 0x01010101u) & 0x80808080u) |
-                               (__popc(__vsubss4(w[q], c[3] * 0x01010101u) & 0x80808080u) << 16);
-                    }
-                    n01 = __reduce_add_sync(0xffffffffu, n01);
-                    n23 = __reduce_add_sync(0xffffffffu, n23);
-                    if (lane == 0) { s_cnt[buf + warp] = n01; s_cnt[buf + 32u + warp] = n23; }
-                    __syncthreads();
-                    n01 = __reduce_add_sync(0xffffffffu, lane < nw ? s_cnt[buf + lane] : 0u);
-                    n23 = __reduce_add_sync(0xffffffffu, lane < nw ? s_cnt[buf + 32u + lane] : 0u);
-                    const uint32_t n[4] = {n01 & 0xFFFFu, n01 >> 16, n23 & 0xFFFFu, n23 >> 16};
-#pragma unroll
-                    for (int i = 3; i >= 0; --i) if (n[i] >= n_g) hi = c[i];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) if (n[i] < n_g) lo = c[i];
-                    buf ^= 64u;
-                }
-                d = hi;
+                d = decays_until(w, n_g, L, s_cnt);
 #pragma unroll
                 for (int q = 0; q < NV; ++q) w[q] = decay4(w[q], d);
-                store_life(par);
+                store_lifetimes<SPT>(s_life, s_bits, s_ndead + par, own, w);
                 __syncthreads();
                 t = lane < nw ? s_ndead[par + lane] : 0u;
                 dead_before = __reduce_add_sync(0xffffffffu, lane < warp ? t : 0u);
@@ -369,22 +267,6 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
             if (lane == 0) s_ndead[32u - par + warp] = left;
             __syncthreads();
 
-            // a copying block's rows: in turn where few tables have eight blocks each, and where other blocks may take some
-            // (so that what is left is at the end), else a share in position order
-            const bool in_turn = CAP == STEP_FEW_TABLES || share_it;
-            const uint32_t share = SHARES ? (n_take + copying - 1u) / copying : 0u;
-            if constexpr (CLUSTER) {                     // what the copying blocks get of this token: a head and their rows
-                if (g == 0) cluster_wait();              // (their mbarriers are ready)
-                if (tid < copying) {
-                    const uint32_t n = in_turn ? (n_take + copying - 1u - tid) / copying
-                                       : tid * share >= n_take ? 0u : n_take - tid * share < share ? n_take - tid * share : share;
-                    const uint32_t mbar = map_rank(a_mbar + 8u * g, tid + 1u);
-                    send_async(map_rank(smem_u32(smem) + 8u * g * step_rows(K, copying), tid + 1u), (int32_t)n,
-                               share_it ? (int32_t)((shared & ~SHARED_COMING) + tid) : -1, mbar);
-                    arrive_expect(mbar, 8u * (n + 1u));
-                }
-            }
-
             // ---- install: the k-th miss in position order takes the k-th dead slot ----
             for (uint32_t k = tid; k < n_g; k += nt) {
                 const uint32_t i = s_pos[k];
@@ -393,15 +275,7 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
                 if (k < n_take) {
                     s_node[j].x = (uint32_t)x;
                     s_life[j] = (int8_t)L;
-                    if constexpr (CLUSTER) {
-                        const uint32_t to = in_turn ? k % copying : k / share;
-                        const uint32_t at = in_turn ? k / copying : k - to * share;
-                        if (share_it) list[(shared & ~SHARED_COMING) + k] = make_int2(x, j);
-                        send_async(map_rank(smem_u32(smem) + 8u * (g * step_rows(K, copying) + 1u + at), to + 1u), x, j,
-                                   map_rank(a_mbar + 8u * g, to + 1u));
-                    } else {
-                        list[list_off + k] = make_int2(x, j);
-                    }
+                    list[list_off + k] = make_int2(x, j);
                     g_tok[j] = x >= N ? -1 : x;                        // speculative ids are forgotten (end of Alg. 4)
                     if (!last) {
                         const uint32_t n = S + list_off + k;
@@ -412,14 +286,9 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
                 if (Hm) Hm[i] = 0;
             }
             list_off += n_take;
-            if (share_it) shared += n_take;
             sum_decay += d;
             __syncthreads();
             announce_token(p, ti, g, n_take);
-        }
-        if (SHARE && shared && tid == 0) {
-            __threadfence();
-            *reinterpret_cast<volatile uint32_t*>(&p.shared[ti].rows) = shared == SHARED_COMING ? 0u : shared ^ (SHARED_COMING | SHARED_OPEN);
         }
 
         // ---- write back: lifetimes; resident ids that are no longer verified become empty (Alg. 4) ----
@@ -462,172 +331,7 @@ template <int SPT, int IPT, int CAP, bool WIDE = true>
 __global__ void __launch_bounds__(1024, 1) avsg_stage_one_kernel(const __grid_constant__ S1ParamsT<CAP> p)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    stage_one<SPT, IPT, false, WIDE, false>(p, blockIdx.x, gridDim.x, smem);
-}
-
-__device__ __forceinline__ SharedRows read_shared(const SharedRows* at)
-{
-    SharedRows s;
-    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(s.rows), "=r"(s.pad), "=r"(s.taken), "=r"(s.begun) : "l"(at) : "memory");
-    return s;
-}
-
-// A warp that is through with its own table's rows copies rows that other tables share.
-template <int CAP>
-__device__ __forceinline__ void take_shared_rows(const S1ParamsT<CAP>& p, const uint32_t ti, const uint32_t group)
-{
-    const uint32_t lane = threadIdx.x & 31u, cpr = p.row_bytes >> 4;
-    // all tables at a time: one after the other they had held up the end of a call with many
-    SharedRows now = {0u, 0u, 0u, 0u};
-    if (group + lane < p.n_launch && group + lane != ti) now = read_shared(p.shared + group + lane);
-    const bool some = (now.rows & SHARED_COMING) ||
-                      ((now.rows & SHARED_OPEN) && now.taken + now.begun + SHARED_LEFT < (now.rows & ~SHARED_OPEN));
-    for (uint32_t which = __ballot_sync(0xffffffffu, some); which; which &= which - 1u) {
-        const uint32_t t = group + __ffs((int)which) - 1u;
-        SharedRows s = read_shared(p.shared + t);
-        for (uint32_t spin = 0; (s.rows & SHARED_COMING) && spin < OVERLAP_SPIN_LIMIT; ++spin) {     // (that Stage One runs, and waits for nobody)
-            __nanosleep(64);
-            s = read_shared(p.shared + t);
-        }
-        __threadfence();
-        const uint32_t rows = __shfl_sync(0xffffffffu, s.rows, 0) ^ SHARED_OPEN;
-        if (rows >= SHARED_OPEN) continue;                             // closed meanwhile
-        const uint64_t src = p.kv_base[t], stride = p.kv_stride[t];
-        const uint64_t dst = reinterpret_cast<uint64_t>(p.buffer + (size_t)p.table_id[t] * p.S * p.row_bytes);
-        const int2* list = p.miss_list + (size_t)t * p.list_stride;
-        for (;;) {
-            uint32_t at = 0xFFFFFFFFu;
-            if (lane == 0 && s.taken + s.begun + SHARED_LEFT < rows) at = atomicAdd(&p.shared[t].taken, 1u);
-            at = __shfl_sync(0xffffffffu, at, 0);
-            if (at >= rows) break;
-            const int2 e = __ldcg(list + (rows - 1u - at));            // what is taken is copied
-            s = read_shared(p.shared + t);                             // (comes with the row)
-            if (e.x < 0 || e.y < 0 || (uint32_t)e.y >= p.S) {
-                if (lane == 0) atomicOr(p.status, ST_BAD_SLOT);
-                continue;
-            }
-            copy_row(src + (uint64_t)(uint32_t)e.x * stride, dst + (uint64_t)(uint32_t)e.y * p.row_bytes, cpr, lane);
-        }
-    }
-}
-
-// A call in one kernel: a cluster of two to eight blocks per table.  The first block runs Stage One; the others copy the
-// misses of every token as soon as it is placed, in either mode.  What it saves is a launch (1.8 us of host time, which
-// bounds the smallest calls), the way from the end of one grid to the start of the next, and the hand-over through global
-// memory with its fences: Stage One sends every miss (id, slot) straight into the shared memory of the block that will copy
-// it, where an mbarrier per token counts the bytes, and goes on.  A copying block keeps 20 KB of rows on the way, so that
-// seven can fill the link with one table's rows (2 us round trip x 47 GB/s) and the other sizes with what runs beside it.
-// Measured, in two kernels (Stage Two overlapped where that is faster) / in this one, us per call:
-//   K = 256, S = 1024, one table 8.4 / 5.8;  K = 2048, S = 8192, two tokens, one table 17.2 / 12.2, from a graph 19.8 / 18.3;
-//   the same with 4, 8, 16, 32, 48, 64 tables 26.2 / 22.4, 39.0 / 35.6, 65.9 / 63.6, 119.9 / 116.8, 174.0 / 173.6, 228.3 / 226.8;
-//   the same from 11 GB of host memory with 8, 16, 32, 48, 64 tables 51 / 46, 88 / 84, 173 / 155, 242 / 229, 315 / 296.
-// The last line is what the end of a call is for.  Where a table's pages are spread over much host memory, translating
-// their addresses limits the rows, and a cluster, which lies in one GPC, finds its table's translations there if the
-// table was there in the call before.  So calls of more than a few tables let the next grid start only when their
-// blocks exit: its clusters then find the same SMs free, in the same order.  Started early they take whatever is free at
-// that time: eight tables 60 us and not 46, 16 113 and not 84 (step_early() says which calls gain by it).
-// FEW (eight blocks): up to 20 rows a block, which a warp each has under way at once: the tokens' rows follow one another
-// without a meeting of the warps, and go round over the blocks (one table 12.0 us; meeting, with shares 12.35).  Otherwise
-// a block's warps meet before the next token's rows, and its rows are neighbours (16 tables, 11 GB: 84.0 us against 84.3
-// and 86.0 with one of the two; 40 tables 193 against 203 and 199).
-// SHARE (two and three blocks).  A cluster alone cannot fill the link with one table's rows where it has few copying blocks (an
-// SM gets 20 of them a us, the link carries 72), so a new request among steady ones would be left behind: 64 tables, one of
-// them cold, 332 us against 277 in two kernels, whose rows are cut evenly over all SMs (Eq. 6).  So a table that misses more
-// than SHARED_FROM ids in a token writes these misses to its list in global memory too, and says so.  Its own blocks copy them
-// from the front; a few warps of other tables that are through take single rows from the back, counted in SharedRows::taken,
-// until few are left; the own blocks stop where the others have begun.  Both may copy a row in the middle, to the same effect.
-// Every row is copied: what the own blocks leave out is counted in `taken`, and what is counted there is copied by who counted it.
-// Nobody waits, but for a Stage One that has announced rows and runs.  One cold table of 45, 64: 229, 332 us without, 215, 283
-// with it, 211, 277 in two kernels; the others with hits only 70, 124, 50, 57, 46, 46; all steady 169, 239.5, 170, 240.5, 172, 241.
-// With four blocks it costs every call more (16 tables 64.7 us, 65.5 with it) than it gives one with a new request (16, 32
-// tables, one cold: 115, 172 without, 113, 170 with it, 110, 167 in two kernels).  With all rows of such a table claimed one by
-// one, its own blocks' too, the cold calls were quicker still (45 tables 214), but a call where most tables had many misses
-// lost 5 to 20 %: the requests for claims and list entries wait behind the rows'.  Several rows of a warp at once bring an SM
-// from 20 rows a us to 28 at most.
-template <int SPT, int IPT, int CAP, bool SHARE = false>
-__global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constant__ S1ParamsT<CAP> p)
-{
-    constexpr bool FEW = CAP == STEP_FEW_TABLES;
-    extern __shared__ __align__(16) unsigned char smem[];              // of a copying block: the words that it gets, by token
-    __shared__ __align__(8) unsigned long long s_mbar[STEP_MAX_TOKENS], s_meet[STEP_MAX_TOKENS];
-    __shared__ volatile uint32_t s_mine;                               // rows that are shared: the first that others have taken
-    const uint32_t rank = cluster_rank(), cluster = FEW ? STEP_FEW_CLUSTER : cluster_size(), copying = cluster - 1u;
-    const uint32_t ti = blockIdx.x / cluster, lane = threadIdx.x & 31u, W = blockDim.x >> 5, warp = threadIdx.x >> 5;
-    if (p.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (SHARE && threadIdx.x == 0) s_mine = 0xFFFFFFFFu;
-    if (rank != 0 && threadIdx.x < p.n_q) {
-        mbar_init(smem_u32(s_mbar + threadIdx.x), 1u);
-        if (!FEW) mbar_init(smem_u32(s_meet + threadIdx.x), W);
-    }
-    __syncthreads();
-    cluster_arrive();
-    if (rank == 0) {
-        stage_one<SPT, IPT, true, true, SHARE>(p, ti, p.n_launch, smem, smem_u32(s_mbar));
-        __syncwarp();
-        cluster_arrive();                                              // the outputs are written, everything is sent
-        return;
-    }
-    const uint32_t cpr = p.row_bytes >> 4;
-    const uint64_t src = p.kv_base[ti], stride = p.kv_stride[ti];
-    const uint64_t dst = reinterpret_cast<uint64_t>(p.buffer + (size_t)p.table_id[ti] * p.S * p.row_bytes);
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    cluster_wait();
-    cluster_arrive();
-    auto wait_for = [&](uint32_t mbar, uint32_t limit) -> bool {       // (Stage One's loops are bounded, far below this)
-        uint32_t spin = 0;
-        while (spin < limit && !mbar_done(mbar)) ++spin;
-        return __all_sync(0xffffffffu, spin < limit);
-    };
-    uint32_t from = 0, g = 0;                                          // the warp that is next; the token
-    for (; g < p.n_q; ++g) {
-        const int2* got = reinterpret_cast<const int2*>(smem) + g * step_rows(p.K, copying);
-        if (!wait_for(smem_u32(s_mbar + g), AVSG_STEP_GIVE_UP)) break;
-        const uint32_t count = (uint32_t)got[0].x;
-        const int32_t at = got[0].y;                                   // of the first row among those that are shared; -1
-        SharedRows s = {SHARED_COMING, 0u, 0u, 0u};
-        for (uint32_t k = warp >= from ? warp - from : warp + W - from; k < count; k += W) {
-            if (SHARE && at >= 0) {
-                if (warp == 0) {                                       // for all warps: requests wait behind the rows' where the link is full
-                    if (!(s.rows & SHARED_COMING)) s_mine = (s.rows & ~SHARED_OPEN) > s.taken ? (s.rows & ~SHARED_OPEN) - s.taken : 0u;
-                    s = read_shared(p.shared + ti);                    // (comes with the row)
-                    if (lane == 0) atomicAdd(&p.shared[ti].begun, W);
-                }
-                if (at + k * copying >= s_mine) break;                 // others have the rest
-            }
-            const int2 e = got[1u + k];
-            if (e.x < 0 || e.y < 0 || (uint32_t)e.y >= p.S) {
-                if (lane == 0) atomicOr(p.status, ST_BAD_SLOT);
-                continue;
-            }
-            copy_row(src + (uint64_t)(uint32_t)e.x * stride, dst + (uint64_t)(uint32_t)e.y * p.row_bytes, cpr, lane);
-        }
-        if (FEW || count < W || (SHARE && g + 1u == p.n_q)) {
-            from = (from + count) % W;
-        } else if (g + 1u < p.n_q) {                                   // the warps meet
-            from = 0;
-            if (lane == 0) mbar_arrive(smem_u32(s_meet + g));
-            if (!wait_for(smem_u32(s_meet + g), AVSG_STEP_GIVE_UP)) break;
-        }
-    }
-    // Warps that take other tables' rows: those that had the fewest of the last token, a few of each block
-    uint32_t others = 0;                                               // what 32 of the tables share, one a lane
-    const uint32_t turn = warp >= from ? warp - from : warp + W - from, group = (ti + turn) % ((p.n_launch + 31u) / 32u) * 32u;
-    const bool takes = SHARE && turn * (p.n_launch - 1u) * copying < SHARED_WARPS * ((p.n_launch + 31u) / 32u);
-    if (takes && group + lane < p.n_launch) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(others) : "l"(&p.shared[group + lane].rows) : "memory");
-    // Stage One does not know who has given up, and nothing may be sent to a block that is gone: every block stays until
-    // Stage One is through, and one that gave up until what was sent has arrived.
-    cluster_wait();
-    if (g < p.n_q) {
-        if (lane == 0) atomicOr(p.status, ST_WAIT_TIMEOUT);
-        for (g = 0; g < p.n_q && wait_for(smem_u32(s_mbar + g), STEP_SPIN_LIMIT); ++g) {}
-    }
-    if (p.out.n_slots) put_outputs_of(p.out, ti, p.n_q * p.K, p.n_q, warp * copying + rank - 1u, W * copying, lane);
-    if constexpr (SHARE) {
-        // Closed for who has not begun yet, and so closed between calls (Stage One is through and writes it no more).
-        if (threadIdx.x == 0) atomicAnd(&p.shared[ti].rows, SHARED_OPEN - 1u);
-        if (takes && __any_sync(0xffffffffu, (others & (SHARED_COMING | SHARED_OPEN)) != 0)) take_shared_rows(p, ti, group);
-    }
+    stage_one<SPT, IPT, WIDE>(p, blockIdx.x, gridDim.x, smem);
 }
 
 // A request ended: its tables become empty (id -1) and dead (lifetime -1) again, their counters and rows zero;
@@ -1004,24 +708,6 @@ cudaError_t stage_one_prepare(size_t max_smem)
         reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 2, S1_BIG_TABLES>),
         reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 4, S1_BIG_TABLES>),
         reinterpret_cast<const void*>(avsg_stage_one_kernel<8, 8, S1_BIG_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<2, 2, STEP_FEW_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<4, 2, STEP_FEW_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<4, 4, STEP_FEW_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<8, 2, STEP_FEW_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<8, 4, STEP_FEW_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<8, 8, STEP_FEW_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<2, 2, STEP_MAX_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<4, 2, STEP_MAX_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<4, 4, STEP_MAX_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<8, 2, STEP_MAX_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<8, 4, STEP_MAX_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<8, 8, STEP_MAX_TABLES>),
-        reinterpret_cast<const void*>(avsg_step_kernel<2, 2, STEP_MAX_TABLES, true>),
-        reinterpret_cast<const void*>(avsg_step_kernel<4, 2, STEP_MAX_TABLES, true>),
-        reinterpret_cast<const void*>(avsg_step_kernel<4, 4, STEP_MAX_TABLES, true>),
-        reinterpret_cast<const void*>(avsg_step_kernel<8, 2, STEP_MAX_TABLES, true>),
-        reinterpret_cast<const void*>(avsg_step_kernel<8, 4, STEP_MAX_TABLES, true>),
-        reinterpret_cast<const void*>(avsg_step_kernel<8, 8, STEP_MAX_TABLES, true>),
         reinterpret_cast<const void*>(avsg_stage_one_paper_kernel)};
     for (const void* k : kernels) {
         cudaFuncAttributes fa;
@@ -1091,76 +777,6 @@ cudaError_t launch_stage_one(const S1Params& p, uint32_t n_tables, cudaStream_t 
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, avsg_stage_one_paper_kernel, p);
 }
-
-// At least 16 warps a block where the table has the slots for it: they copy.
-uint32_t step_threads(uint32_t S, uint32_t K)
-{
-    const uint32_t t = stage_one_threads(S, K), most = S / 2 < 512u ? S / 2 : 512u;
-    return t > most ? t : most;
-}
-
-namespace {
-
-template <int CAP, bool SHARE = false>
-const void* step_kernel(uint32_t spt, uint32_t ipt)
-{
-    switch (spt) {
-        case 8:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 2, CAP, SHARE>)
-                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 4, CAP, SHARE>)
-                                 : reinterpret_cast<const void*>(avsg_step_kernel<8, 8, CAP, SHARE>);
-        case 4:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<4, 2, CAP, SHARE>)
-                                 : reinterpret_cast<const void*>(avsg_step_kernel<4, 4, CAP, SHARE>);
-        default: return reinterpret_cast<const void*>(avsg_step_kernel<2, 2, CAP, SHARE>);
-    }
-}
-
-void step_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, uint32_t n_tables, uint32_t cluster, uint32_t threads, size_t smem)
-{
-    cfg.gridDim = dim3(n_tables * cluster);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cluster;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-}
-}  // namespace
-
-StepClusters step_clusters(size_t max_smem)
-{
-    StepClusters s;
-    for (uint32_t cl : {2u, 3u, 4u, STEP_FEW_CLUSTER}) {
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[2];
-        int fit = 0;
-        step_config(cfg, attr, 1, cl, 1024, max_smem - 2048);      // (the largest; statically it has 1 KB)
-        if (cudaOccupancyMaxActiveClusters(&fit, step_kernel<STEP_MAX_TABLES>(8, 2), &cfg) != cudaSuccess) { cudaGetLastError(); fit = 0; }
-        s.fit[cl] = (uint32_t)fit;
-    }
-    return s;
-}
-
-template <int CAP>
-cudaError_t launch_step(const S1ParamsT<CAP>& p, uint32_t cluster, cudaStream_t stream)
-{
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[2];
-    const uint32_t nt = step_threads(p.S, p.K);
-    step_config(cfg, attr, p.n_launch, cluster, nt, s1_layout(p.S, p.K, p.n_q, nt).total);      // (holds step_rows() n_q times)
-    cfg.stream = stream;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = 2;
-    void* args[] = {const_cast<S1ParamsT<CAP>*>(&p)};
-    const uint32_t spt = p.S / nt, ipt = (p.K + nt - 1) / nt;
-    if constexpr (CAP == STEP_MAX_TABLES)
-        if (cluster < SHARED_CLUSTER) return cudaLaunchKernelExC(&cfg, step_kernel<CAP, true>(spt, ipt), args);
-    return cudaLaunchKernelExC(&cfg, step_kernel<CAP>(spt, ipt), args);
-}
-template cudaError_t launch_step(const StepParams& p, uint32_t cluster, cudaStream_t stream);
-template cudaError_t launch_step(const StepParamsFew& p, uint32_t cluster, cudaStream_t stream);
 
 cudaError_t launch_stage_one(const S1ParamsBig& p, uint32_t n_tables, cudaStream_t stream)
 {

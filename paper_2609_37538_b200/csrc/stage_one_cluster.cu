@@ -38,7 +38,6 @@ struct Layout {
     uint32_t heads, nil;                                        // numbers, not offsets: chains, the closing node
     uint32_t head, life, bits, ndead, dead, pref, mask, rev, cnt, sum, total;
 };
-__host__ __device__ inline uint32_t align16(uint32_t n) { return (n + 15u) & ~15u; }
 __host__ __device__ inline Layout make_layout(uint32_t S, uint32_t K, uint32_t n_q, uint32_t C, uint32_t nt)
 {
     const uint32_t Sc = S / C, W = (K + 31u) / 32u, extra = (n_q - 1u) * K < Sc ? (n_q - 1u) * K : Sc;
@@ -62,9 +61,6 @@ __host__ __device__ inline Layout make_layout(uint32_t S, uint32_t K, uint32_t n
         o.heads = Sc;                                           // (longer chains where the rest needs the room)
     }
 }
-
-// Bits 0 .. 3: the sign bits of a word's four bytes.
-__device__ __forceinline__ uint32_t signs(uint32_t w) { return (((w >> 7) & 0x01010101u) * 0x10204080u) >> 28; }
 
 constexpr int IPT = 2;                  // words of 32 positions that a warp looks up at a time
 

@@ -5,6 +5,8 @@
 
 namespace avsg {
 
+__host__ __device__ inline uint32_t align16(uint32_t n) { return (n + 15u) & ~15u; }
+
 constexpr int32_t PRIV_HIST_MAX_L = 30;   // private byte-counter histogram up to this L (32 rows)
 
 // ---- thread-block clusters ----
@@ -30,11 +32,15 @@ __device__ __forceinline__ void addc_u32(uint32_t a, uint32_t v)
 {
     asm volatile("red.shared::cluster.add.u32 [%0], %1;" :: "r"(a), "r"(v) : "memory");
 }
-// Eight bytes into another block's shared memory, counted there by an mbarrier: no fence on either side.
+// Four or eight bytes into another block's shared memory, counted there by an mbarrier: no fence on either side.
 __device__ __forceinline__ void send_async(uint32_t a, int32_t x, int32_t y, uint32_t mbar)
 {
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
                  :: "r"(a), "r"(x), "r"(y), "r"(mbar) : "memory");
+}
+__device__ __forceinline__ void send_async(uint32_t a, uint32_t v, uint32_t mbar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" :: "r"(a), "r"(v), "r"(mbar) : "memory");
 }
 // Another block's mbarrier: its one arrival, with the bytes that are sent to it.
 __device__ __forceinline__ void arrive_expect(uint32_t mbar, uint32_t bytes)
@@ -44,10 +50,6 @@ __device__ __forceinline__ void arrive_expect(uint32_t mbar, uint32_t bytes)
 __device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t arrivals)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n\tfence.mbarrier_init.release.cluster;" :: "r"(mbar), "r"(arrivals) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t mbar)              // the block's own
-{
-    asm volatile("{\n\t.reg .b64 s;\n\tmbarrier.arrive.release.cta.shared::cta.b64 s, [%0];\n\t}" :: "r"(mbar) : "memory");
 }
 __device__ __forceinline__ bool mbar_done(uint32_t mbar)
 {
@@ -59,6 +61,7 @@ __device__ __forceinline__ bool mbar_done(uint32_t mbar)
 // All threads of all blocks of the cluster; earlier (distributed) shared-memory and global writes of the cluster
 // are visible to every thread of the cluster afterwards.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
 
@@ -108,6 +111,112 @@ __device__ __forceinline__ void life_words_store(int8_t* at, bool own, const uin
     else if constexpr (SPT == 8) *reinterpret_cast<uint2*>(at) = make_uint2(w[0], w[1]);
     else if constexpr (SPT == 4) *reinterpret_cast<uint32_t*>(at) = w[0];
     else *reinterpret_cast<uint16_t*>(at) = (uint16_t)w[0];
+}
+
+// ---- the chained index id -> slot (see stage_one.cu): nodes {id, slot << 16 | next node}, chains' first nodes ----
+// The thread's q-th vector of ids is that of the slots from 4 (tid + q blockDim.x) on; node n < S is slot n.
+template <int NV>
+__device__ __forceinline__ void index_slots(const int4 (&t4)[NV], uint2* s_node, uint32_t* s_head, uint32_t S, uint32_t log_heads, uint32_t nil)
+{
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        if (threadIdx.x + q * blockDim.x < S / 4) {
+            const uint32_t j = 4u * (threadIdx.x + q * blockDim.x);
+            const int32_t x[4] = {t4[q].x, t4[q].y, t4[q].z, t4[q].w};
+            uint32_t next[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) next[c] = x[c] >= 0 ? atomicExch(&s_head[hash_id(x[c], log_heads)], j + c) : nil;
+#pragma unroll
+            for (int c = 0; c < 4; c += 2)
+                reinterpret_cast<uint4*>(s_node)[(j + c) / 2] = make_uint4((uint32_t)x[c], (j + c) << 16 | next[c],
+                                                                           (uint32_t)x[c + 1], (j + c + 1) << 16 | next[c + 1]);
+        }
+    }
+}
+
+// The slots of M ids (-1: none; an id of -1 is not looked for).
+template <int M>
+__device__ __forceinline__ void find_slots(const int32_t (&x)[M], const uint2* s_node, const uint32_t* s_head,
+                                           uint32_t log_heads, uint32_t nil, uint32_t* status, int32_t (&slot)[M])
+{
+    uint32_t node[M];
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+        slot[k] = -1;
+        node[k] = nil;
+        if (x[k] >= 0) node[k] = s_head[hash_id(x[k], log_heads)];
+    }
+    uint32_t open = 1;
+    for (uint32_t it = 0; open && it <= nil; ++it) {                   // all chains of the warp side by side
+        uint2 v[M];
+#pragma unroll
+        for (int k = 0; k < M; ++k) v[k] = s_node[node[k]];
+        open = 0;
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            const bool found = (int32_t)v[k].x == x[k];
+            slot[k] = found ? (int32_t)(v[k].y >> 16) : slot[k];
+            node[k] = found ? nil : v[k].y & 0xFFFFu;
+            open |= node[k] ^ nil;
+        }
+        open = __any_sync(0xffffffffu, open);
+    }
+    if (open) atomicOr(status, ST_PROBE_EXHAUSTED);
+}
+
+// Bits 0 .. 3: the sign bits of a word's four bytes.
+__device__ __forceinline__ uint32_t signs(uint32_t w) { return (((w >> 7) & 0x01010101u) * 0x10204080u) >> 28; }
+
+// The thread's lifetimes to shared memory, its dead slots as bits (a byte per thread), the warp's number of them.
+template <int SPT>
+__device__ __forceinline__ void store_lifetimes(int8_t* s_life, uint8_t* s_bits, uint32_t* s_ndead, bool own,
+                                                const uint32_t (&w)[(SPT + 3) / 4])
+{
+    uint32_t bits = 0;
+#pragma unroll
+    for (int q = 0; q < (SPT + 3) / 4; ++q) bits |= signs(w[q]) << (4 * q);
+    life_words_store<SPT>(s_life + threadIdx.x * SPT, own, w);
+    s_bits[threadIdx.x] = (uint8_t)bits;
+    const uint32_t n = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(bits));
+    if ((threadIdx.x & 31u) == 0) s_ndead[threadIdx.x >> 5] = n;
+}
+
+// The while-loop of Alg. 1 in closed form: the fewest unit decays after which n_g of the block's lifetimes are negative
+// (L + 1 where even those are too few; lifetimes are <= L).  All threads of the block; s_cnt: 4 x 32 words.
+template <int NV>
+__device__ __forceinline__ uint32_t decays_until(const uint32_t (&w)[NV], uint32_t n_g, uint32_t L, uint32_t* s_cnt)
+{
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    uint32_t lo = 0, hi = L + 1u, buf = 0;               // lo decays are too few, hi are enough
+    while (hi - lo > 1u) {                               // (L >= 1: at least once, so every warp has read the old counts)
+        uint32_t c[4];                                   // candidates in (lo, hi), ascending; small ones first
+#pragma unroll
+        for (uint32_t i = 0; i < 4; ++i) {
+            c[i] = lo == 0 ? 1u << i : lo + ((i + 1u) * (hi - lo)) / 5u;
+            c[i] = c[i] <= lo ? lo + 1u : (c[i] >= hi ? hi - 1u : c[i]);
+        }
+        uint32_t n01 = 0, n23 = 0;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            n01 += __popc(__vsubss4(w[q], c[0] * 0x01010101u) & 0x80808080u) |
+                   (__popc(__vsubss4(w[q], c[1] * 0x01010101u) & 0x80808080u) << 16);
+            n23 += __popc(__vsubss4(w[q], c[2] * 0x01010101u) & 0x80808080u) |
+                   (__popc(__vsubss4(w[q], c[3] * 0x01010101u) & 0x80808080u) << 16);
+        }
+        n01 = __reduce_add_sync(0xffffffffu, n01);
+        n23 = __reduce_add_sync(0xffffffffu, n23);
+        if (lane == 0) { s_cnt[buf + warp] = n01; s_cnt[buf + 32u + warp] = n23; }
+        __syncthreads();
+        n01 = __reduce_add_sync(0xffffffffu, lane < nw ? s_cnt[buf + lane] : 0u);
+        n23 = __reduce_add_sync(0xffffffffu, lane < nw ? s_cnt[buf + 32u + lane] : 0u);
+        const uint32_t n[4] = {n01 & 0xFFFFu, n01 >> 16, n23 & 0xFFFFu, n23 >> 16};
+#pragma unroll
+        for (int i = 3; i >= 0; --i) if (n[i] >= n_g) hi = c[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) if (n[i] < n_g) lo = c[i];
+        buf ^= 64u;
+    }
+    return hi;
 }
 
 // Exclusive prefix over the lanes and total of a count 0 .. MAX that every lane of the warp has: one ballot per bit.

@@ -1,0 +1,842 @@
+// Both stages of a call in one kernel: a thread-block cluster per table.
+//
+// The first block of a cluster runs Stage One (match + reserve: Algorithm 1 with the lifetime operations of Algorithm 3,
+// the tokens of an iteration in order as in Algorithm 4, the end-of-step invalidation); the others copy the rows of the
+// misses.  Which block copies a position's row follows from the position alone: groups of neighbours go round over the
+// copying blocks.  So a copying block need not be told what to fetch.  It puts the table's cached ids into a set of its own
+// (bits by hash), and an id of its positions that is not in there, nor in those of the earlier tokens, is missed for certain,
+// whatever the tokens before it take away: its row is asked for at once, and is on its way (2 us, over the host link) while
+// Stage One still finds out which slot it goes to.  The slot arrives by st.async in a place that again follows from the
+// position, counted by an mbarrier per token.  Misses that the block could not know of (an id that seems to be in a set, or
+// that loses its slot to an earlier token of the call) it finds in the list of its misses that comes with the slots.
+#include "avsg_kernels.cuh"
+#include "follow_stage_one.cuh"
+#include "stage_one_common.cuh"
+
+namespace avsg {
+namespace {
+
+constexpr uint32_t STEP_SPIN_LIMIT = 1u << 18;            // tries; the hardware suspends the warp for 4 us in each: 1 s
+#ifndef AVSG_STEP_GIVE_UP                                 // (a test builds the library with waits that run out)
+#define AVSG_STEP_GIVE_UP STEP_SPIN_LIMIT
+#endif
+
+// Rows that blocks of other tables may take (see avsg_step_kernel): from how many misses of a token on, how many of a
+// table's rows stay for its own blocks (other blocks' caches of translations do not know the table: with 256 left 64 unequal
+// requests take 326 us, with 128 330, without any sharing 324), how many warps of the call take some at most (of 144 rows
+// under way the link is full; more only copy the last rows twice).
+constexpr uint32_t SHARED_FROM = 512, SHARED_LEFT = 256, SHARED_WARPS = 144, SHARED_CLUSTER = 4;
+
+// Shared memory of a call's blocks, in bytes from the start (every part on a 16-byte boundary), and what else follows from
+// the sizes.  A token's positions are counted by groups of 1 << log_group neighbours: group n_q * groups, token after token,
+// belongs to copying block group % copying, whose (group / copying)-th it is; the block counts its own positions through.
+struct StepLayout {
+    uint32_t log_group, groups;          // groups of a token
+    uint32_t local;                      // positions that a copying block has room for
+    uint32_t by_copying, by_groups;      // n / copying == n * by_copying >> 18 for every group; the same for groups
+    uint32_t per_lane, per_token;        // words of 32 local positions to a lane; of a token's positions, a block's at most
+    uint32_t log_heads, nil;             // chains of the index; its closing node
+    uint32_t log_seen, log_asked;        // words of the copying blocks' sets: cached ids; ids of an earlier token, each
+    uint32_t early;                      // the copying blocks have them
+    uint32_t node, head, life, bits, tot, ndead, cnt, sum, votes, miss, pos, dead, ids;    // first block
+    uint32_t seen, asked, slots, id, mask, rest, list, their_ids;              // copying blocks
+    uint32_t total;
+};
+StepLayout step_layout(uint32_t S, uint32_t K, uint32_t n_q, uint32_t nt, uint32_t copying, uint32_t row_bytes, bool host_ids)
+{
+    StepLayout o;
+    // At least 32 groups a token, so that seven blocks have about the same to do: 9 tables with K = 256 30.8 us with groups of
+    // 32 positions, 27.5 with rows handed out in turn.  Larger ones are loaded in longer pieces.
+    o.log_group = 5u;
+    while (o.log_group && K >> o.log_group < 32u) --o.log_group;
+    o.groups = (K + (1u << o.log_group) - 1u) >> o.log_group;
+    o.local = (((n_q * o.groups + copying - 1u) / copying << o.log_group) + 31u) & ~31u;
+    o.by_copying = (1u << 18) / copying + 1u;
+    o.by_groups = (1u << 18) / o.groups + 1u;
+    o.per_lane = (o.local / 32u + 31u) / 32u;
+    o.per_token = (o.groups + copying - 1u) / copying << o.log_group;
+    o.nil = S + (n_q - 1u) * K;
+    o.log_heads = 1u;
+    while ((1u << o.log_heads) < 2u * S) ++o.log_heads;
+    o.log_seen = o.log_heads;                              // 64 bits an id
+    o.log_asked = 2u;
+    while ((1u << o.log_asked) < 2u * K) ++o.log_asked;
+    o.early = row_bytes <= 16u * ROW_CHUNKS;
+    const uint32_t ids = host_ids ? align16(n_q * K * 4u) : 0u, room = (228u << 10) / (1024u / nt) - 2560u;
+    for (;;) {
+        uint32_t a = 0;
+        o.node = a;    a += align16((o.nil + 1u) * 8u);
+        o.head = a;    a += 4u << o.log_heads;
+        o.life = a;    a += align16(S);                    // lifetime per slot, one signed byte
+        o.bits = a;    a += align16(nt);                   // one bit per slot, set where it is dead (lifetime < 0)
+        o.tot = a;     a += 2u * 32u * 4u;                 // warps' miss totals, by parity
+        o.ndead = a;   a += 2u * 32u * 4u;                 // warps' dead slots, by parity
+        o.cnt = a;     a += 2u * 2u * 32u * 4u;            // warps' counts of the decay search, by parity
+        o.sum = a;     a += 16u;                           // valid ids of the call
+        o.votes = a;   a += align16((K + 31u) / 32u * 4u);  // the token's misses, a bit per position
+        o.miss = a;    a += align16(K * 4u);               // misses in position order: ids,
+        o.pos = a;     a += align16(K * 2u);               //   positions
+        o.dead = a;    a += align16(K * 2u);               // dead slots in slot order
+        o.ids = a;     a += ids;                           // received: the ids of a call with host buffers
+        const uint32_t first = a;
+        a = 0;
+        o.seen = a;    a += o.early ? 4u << o.log_seen : 0u;
+        o.asked = a;   a += o.early ? (n_q - 1u) * 4u << o.log_asked : 0u;
+        o.slots = a;   a += o.local * 4u;                  // received: what has become of a position
+        o.id = a;      a += o.local * 4u;                  // its id
+        o.mask = a;    a += align16(o.local / 32u * 4u);   // positions whose rows are asked for early
+        o.rest = a;    a += align16(o.local / 32u * 4u);   //   but not by the warp that has found them
+        o.list = a;    a += align16(n_q * o.per_token * 8u);   // received: a token's misses in the block's positions {position, slot}
+        o.their_ids = a; a += ids;                         // received: the ids of a call with host buffers, but others' last token's
+        o.total = first > a ? first : a;
+        if (o.total <= room) return o;
+        if (o.early && a > room) o.early = 0;              // no rows early, longer chains where the rest needs the room
+        else if ((1u << o.log_heads) > S) --o.log_heads;
+        else return o;
+    }
+}
+constexpr uint32_t NO_ITEM = 0xFFFFFFFFu;
+constexpr uint32_t NOT_MISSED = 0xFFFFFFFFu, NO_SLOT = 0xFFFFu;        // of a position; else its slot, and << 16 its rank among the token's misses
+
+__device__ __forceinline__ bool wait_for(uint32_t mbar, uint32_t limit)
+{
+    uint32_t spin = 0;
+    while (spin < limit && !mbar_done(mbar)) ++spin;
+    return __all_sync(0xffffffffu, spin < limit);
+}
+
+// The first block of a cluster: Stage One.  SPT slots per thread (a power of two): S <= SPT * blockDim.x.  IPT: the most
+// ids a thread has of a token (K <= S, so SPT is always enough).  a_mbar: the copying blocks' mbarriers, one per token.
+// The passes are those of avsg_stage_one_kernel, which says what they are and why.  SHARE: rows of a table with very many
+// misses may be copied by other tables' blocks; a_first: where the copying blocks hear of the token's first row among them.
+template <int SPT, int IPT, bool SHARE, int CAP>
+__device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const StepLayout& lay, const uint32_t ti, const uint32_t copying,
+                                             unsigned char* smem, const uint32_t a_mbar, const uint32_t a_sent, const uint32_t a_first, uint32_t* s_own)
+{
+    constexpr int NV = (SPT + 3) / 4;                    // 4-slot vectors of ids / words of lifetimes per thread
+    const uint32_t S = p.S, K = p.K, L = p.L, NIL = lay.nil;
+    const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u, warp = tid >> 5, nw = nt >> 5;
+    const uint32_t below = (1u << lane) - 1u;            // the lanes before this one
+
+    uint2*    s_node = reinterpret_cast<uint2*>(smem + lay.node);
+    uint32_t* s_head = reinterpret_cast<uint32_t*>(smem + lay.head);
+    int8_t*   s_life = reinterpret_cast<int8_t*>(smem + lay.life);
+    uint8_t*  s_bits = smem + lay.bits;                  // a thread's slots: set where dead
+    uint32_t* s_tot  = reinterpret_cast<uint32_t*>(smem + lay.tot);
+    uint32_t* s_ndead = reinterpret_cast<uint32_t*>(smem + lay.ndead);
+    uint32_t* s_cnt  = reinterpret_cast<uint32_t*>(smem + lay.cnt);
+    uint32_t* s_sum  = reinterpret_cast<uint32_t*>(smem + lay.sum);
+    uint32_t* s_votes = reinterpret_cast<uint32_t*>(smem + lay.votes);
+    int32_t*  s_miss = reinterpret_cast<int32_t*>(smem + lay.miss);
+    uint16_t* s_pos  = reinterpret_cast<uint16_t*>(smem + lay.pos);
+    uint16_t* s_dead = reinterpret_cast<uint16_t*>(smem + lay.dead);
+    const int32_t* s_ids = reinterpret_cast<const int32_t*>(smem + lay.ids);
+
+    // slot j is no longer dead (the count follows the bit, so that an id that comes twice is counted once)
+    auto revive = [&](uint32_t j, uint32_t par) {
+        const uint32_t owner = j / SPT, bit = 1u << ((owner & 3u) * 8u + j % SPT);
+        if (atomicAnd(reinterpret_cast<uint32_t*>(s_bits) + owner / 4u, ~bit) & bit)
+            atomicSub(&s_ndead[par + owner / 32u], 1u);
+    };
+    const uint32_t ipt = (K + nt - 1) / nt;              // ids per thread
+    const uint32_t i0 = warp * ipt * 32u + lane;         // position of the thread's k-th id: i0 + 32 k, below i1
+    const uint32_t i1 = (warp + 1u) * ipt * 32u < K ? (warp + 1u) * ipt * 32u : K;
+    int32_t xs[IPT];
+    auto load_token = [&](uint32_t g) {
+        const int32_t* ids = p.indices + ((size_t)ti * p.n_q + g) * K;
+#pragma unroll
+        for (int k = 0; k < IPT; ++k)
+            xs[k] = i0 + 32u * k < i1 ? (p.host_ids ? s_ids[g * K + i0 + 32u * k] : __ldcg(ids + i0 + 32u * k)) : -1;
+    };
+    // the clearing comes before the wait: under the previous kernel's tail
+    const uint32_t table = p.table_id[ti], id_limit = p.id_limit[ti];
+    int32_t N = p.verified_len[ti];
+    for (uint32_t i = tid; i < (1u << lay.log_heads) / 4; i += nt) reinterpret_cast<uint4*>(s_head)[i] = make_uint4(NIL, NIL, NIL, NIL);
+    if (tid == 0) s_node[NIL] = make_uint2(0xFFFFFFFEu, NIL);          // an id that nobody looks for
+    if (tid == 0) s_sum[0] = 0;
+    if (tid < 2u * STEP_FEW_CLUSTER) s_own[tid] = 0;
+
+    // Programmatic dependent launch: this grid may have been started while the previous kernel of the stream
+    // was still running; nothing that the device writes is read before that kernel has completed.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    const uint32_t j0 = tid * SPT;                       // first of the thread's slots
+    const bool own = j0 < S;
+    int32_t* g_tok = p.tok + (size_t)table * S;
+    int8_t*  g_life = p.life + (size_t)table * S;
+    int4 t4[NV];
+    uint32_t w[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q)
+        if (tid + q * nt < S / 4) t4[q] = __ldcg(reinterpret_cast<const int4*>(g_tok) + tid + q * nt);
+    life_words<SPT, true>(g_life + j0, own, w);
+    if (!p.host_ids) load_token(0);
+    if (p.verified_len_dev) N = __ldg(p.verified_len_dev + ti);
+    cluster_wait();                                      // (the copying blocks' mbarriers are ready)
+    __syncthreads();                                     // the index is empty
+
+    // ---- ids to shared memory and into the index; global pre-decay of the lifetimes (Alg. 1 Pass 1) ----
+    bool stale_ids = false;                              // ids that are no longer verified (the caller took tokens back)
+#pragma unroll
+    for (int q = 0; q < NV; ++q)
+        if (tid + q * nt < S / 4) stale_ids = stale_ids || t4[q].x >= N || t4[q].y >= N || t4[q].z >= N || t4[q].w >= N;
+    index_slots(t4, s_node, s_head, S, lay.log_heads, NIL);
+    uint32_t high = 0;                                   // lifetimes above L (only a caller's own state can have them)
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        if (own) high |= __vcmpgts4(w[q], L * 0x01010101u) & (SPT == 2 ? 0xFFFFu : 0xFFFFFFFFu);
+        w[q] = decay4(w[q], 1);
+    }
+    store_lifetimes<SPT>(s_life, s_bits, s_ndead, own, w);
+    if (p.host_ids) {
+        cluster_sync();                                  // (the copying blocks have sent the ids)
+        load_token(0);
+    }
+    const bool unusual = __syncthreads_or(high != 0);
+
+    uint32_t list_off = 0, sum_miss = 0, sum_decay = 0, valid = 0;
+    uint32_t shared = 0;                                 // SHARE: rows that other blocks may take (bit 31: there will be some)
+    int2* list = p.miss_list + (size_t)ti * p.list_stride;
+
+    for (uint32_t g = 0; g < p.n_q; ++g) {
+        const bool last = g + 1 == p.n_q;
+        const uint32_t par = 32u * (g & 1u);
+        const size_t row = ((size_t)ti * p.n_q + g) * K;
+        int32_t* O = p.slots + row;
+        uint8_t* Hm = p.hit ? p.hit + row : nullptr;
+
+        // ---- lookups; hits: lifetime <- L, slot and flag out (Pass 1 + Pass 2) ----
+        // (pass after pass over the thread's ids, so that their reads are in flight together)
+        uint32_t rank[IPT], missing = 0, wmiss = 0;
+        int32_t slot[IPT], was[IPT];
+        bool bad = false;
+#pragma unroll
+        for (int k = 0; k < IPT; ++k) {
+            const bool ok = (uint32_t)xs[k] < id_limit;
+            bad = bad || (!ok && xs[k] >= 0);
+            xs[k] = ok ? xs[k] : -1;
+            valid += ok;
+        }
+        if (bad) atomicOr(p.status, ST_BAD_ID);                        // not fetched: reported and taken as padding
+        find_slots(xs, s_node, s_head, lay.log_heads, NIL, p.status, slot);
+        // with lifetimes above L on entry a slot reserved in this step may go to yet another id: its first node is stale
+        if (unusual) {
+#pragma unroll
+            for (int k = 0; k < IPT; ++k)
+                if (slot[k] >= 0 && (int32_t)s_node[slot[k]].x != xs[k]) slot[k] = -1;
+        }
+#pragma unroll
+        for (int k = 0; k < IPT; ++k) was[k] = slot[k] >= 0 ? s_life[slot[k]] : 0;
+        bool revived = false;
+#pragma unroll
+        for (int k = 0; k < IPT; ++k) {
+            const bool miss = xs[k] >= 0 && slot[k] < 0, store = !miss && i0 + 32u * k < i1;
+            const uint32_t votes = __ballot_sync(0xffffffffu, miss);
+            rank[k] = wmiss + __popc(votes & below);                   // within the warp, in position order
+            wmiss += __popc(votes);
+            if (lane == 0 && i0 + 32u * k < i1) s_votes[warp * ipt + k] = votes;
+            missing |= miss ? 1u << k : 0u;
+            if (slot[k] >= 0) s_life[slot[k]] = (int8_t)L;
+            if (store) O[i0 + 32u * k] = slot[k];
+            if (store && Hm) Hm[i0 + 32u * k] = slot[k] >= 0;
+            revived = revived || was[k] < 0;
+        }
+        if (revived) {
+#pragma unroll
+            for (int k = 0; k < IPT; ++k)
+                if (was[k] < 0) revive((uint32_t)slot[k], par);
+        }
+        if (last) {
+            valid = __reduce_add_sync(0xffffffffu, valid);
+            if (lane == 0 && valid) atomicAdd(s_sum, valid);
+        }
+        if (lane == 0) s_tot[par + warp] = wmiss;
+        __syncthreads();
+
+        // ---- CollectDead and the misses, each in order; the prefix over the warps: lane l looks at warp l ----
+        uint32_t t = lane < nw ? s_ndead[par + lane] | s_tot[par + lane] << 16 : 0u;
+        const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? t : 0u);
+        const uint32_t all = __reduce_add_sync(0xffffffffu, t);
+        const uint32_t n_g = all >> 16;
+        uint32_t dtotal = all & 0xFFFFu, dead_before = before & 0xFFFFu, d = 0;
+        sum_miss += n_g;
+        if (tid == 0 && p.miss_count) p.miss_count[(size_t)ti * p.n_q + g] = (int32_t)n_g;
+        const bool share_it = SHARE && n_g > SHARED_FROM;
+        if (share_it && !shared) {
+            shared = SHARED_COMING;
+            if (tid == 0) {                              // (in place before the table's own blocks hear of the rows)
+                p.shared[ti].taken = p.shared[ti].begun = 0;
+                __threadfence();
+                *reinterpret_cast<volatile uint32_t*>(&p.shared[ti].rows) = SHARED_COMING;
+                __threadfence();
+            }
+        }
+        if (missing) {
+#pragma unroll
+            for (int k = 0; k < IPT; ++k) {
+                if (missing & (1u << k)) {
+                    s_miss[(before >> 16) + rank[k]] = xs[k];
+                    s_pos[(before >> 16) + rank[k]] = (uint16_t)(i0 + 32u * k);
+                }
+            }
+        }
+        if (!last) load_token(g + 1);                                      // arrives while this token's misses are placed
+        const uint32_t group0 = g * lay.groups, in_group = (1u << lay.log_group) - 1u;
+        // Pass 3, the while-loop of Alg. 1: decay until n_g slots are dead
+        if (dtotal < n_g) {
+            life_words<SPT>(s_life + j0, own, w);
+            d = decays_until(w, n_g, L, s_cnt);
+#pragma unroll
+            for (int q = 0; q < NV; ++q) w[q] = decay4(w[q], d);
+            store_lifetimes<SPT>(s_life, s_bits, s_ndead + par, own, w);
+            __syncthreads();
+            t = lane < nw ? s_ndead[par + lane] : 0u;
+            dead_before = __reduce_add_sync(0xffffffffu, lane < warp ? t : 0u);
+            dtotal = __reduce_add_sync(0xffffffffu, t);
+            if (dtotal < n_g && tid == 0) atomicOr(p.status, ST_NO_DEAD_SLOTS);
+        }
+        if (tid < STEP_FEW_CLUSTER) s_own[(~g & 1u) * STEP_FEW_CLUSTER + tid] = 0;         // for the next token
+        const uint32_t n_take = n_g < dtotal ? n_g : dtotal;
+        if (dead_before < n_take) {                      // some of the first n_g dead slots are this warp's
+            uint32_t bits = s_bits[tid], r, unused;
+            warp_rank<SPT>(__popc(bits), below, r, unused);
+            for (r += dead_before; bits && r < n_take; bits &= bits - 1u, ++r) s_dead[r] = (uint16_t)(j0 + __ffs((int)bits) - 1);
+            s_bits[tid] = (uint8_t)bits;                  // what is handed out is dead no more
+        }
+        uint32_t left = __shfl_sync(0xffffffffu, t & 0xFFFFu, (int)warp);          // the warp's dead slots for the next token
+        if (dead_before < n_take) left = left > n_take - dead_before ? left - (n_take - dead_before) : 0u;
+        if (lane == 0) s_ndead[32u - par + warp] = left;
+        __syncthreads();
+
+        for (uint32_t to = nw - 1u - warp; to < copying; to += nw) {       // what a copying block gets of this token (the first warps install)
+            // (its first group is the first one that is `to` modulo copying)
+            uint32_t group = (group0 * lay.by_copying >> 18) * copying + to, n = 0;
+            if (group < group0) group += copying;
+            for (uint32_t q = group - group0 + lane * copying; n_g && q < lay.groups; q += 32u * copying) {
+                const uint32_t i = q << lay.log_group;
+                n += __popc(s_votes[i / 32u] >> i % 32u & ~(~1u << in_group));
+            }
+            n = __reduce_add_sync(0xffffffffu, n);
+            if (lane == 0) {
+                const uint32_t mbar = map_rank(a_mbar + 8u * g, to + 1u);
+                send_async(map_rank(a_sent + 4u * g, to + 1u), n, mbar);
+                if (SHARE) send_async(map_rank(a_first + 4u * g, to + 1u), share_it ? shared & ~SHARED_COMING : ~0u, mbar);
+                arrive_expect(mbar, 12u * n + (SHARE ? 8u : 4u));
+            }
+        }
+
+        // ---- install: the k-th miss in position order takes the k-th dead slot ----
+        for (uint32_t k = tid; k < n_g; k += nt) {
+            const uint32_t i = s_pos[k];
+            const int32_t x = s_miss[k];
+            const int32_t j = k < n_take ? s_dead[k] : -1;
+            // to the block that the position belongs to: the slot where the position's place is, and an entry of its list
+            const uint32_t group = group0 + (i >> lay.log_group), at = group * lay.by_copying >> 18, to = group - at * copying;
+            const uint32_t n = (at << lay.log_group) + (i & in_group), what = ((uint32_t)j & 0xFFFFu) | k << 16, mbar = map_rank(a_mbar + 8u * g, to + 1u);
+            send_async(map_rank(smem_u32(smem) + lay.slots + 4u * n, to + 1u), what, mbar);
+            const uint32_t e = atomicAdd(s_own + (g & 1u) * STEP_FEW_CLUSTER + to, 1u);
+            send_async(map_rank(smem_u32(smem) + lay.list + 8u * (g * lay.per_token + e), to + 1u), (int32_t)n, (int32_t)what, mbar);
+            if (k < n_take) {
+                s_node[j].x = (uint32_t)x;
+                s_life[j] = (int8_t)L;
+                if (share_it) list[(shared & ~SHARED_COMING) + k] = make_int2(x, j);
+                g_tok[j] = x >= N ? -1 : x;                            // speculative ids are forgotten (end of Alg. 4)
+                if (!last) {
+                    const uint32_t n = S + list_off + k;
+                    s_node[n] = make_uint2((uint32_t)x, (uint32_t)j << 16 | atomicExch(&s_head[hash_id(x, lay.log_heads)], n));
+                }
+            }
+            O[i] = j;
+            if (Hm) Hm[i] = 0;
+        }
+        list_off += n_take;
+        if (share_it) shared += n_take;
+        sum_decay += d;
+        __syncthreads();
+        announce_token(p, ti, g, n_take);
+    }
+    if (SHARE && shared && tid == 0) {
+        __threadfence();
+        *reinterpret_cast<volatile uint32_t*>(&p.shared[ti].rows) = shared == SHARED_COMING ? 0u : shared ^ (SHARED_COMING | SHARED_OPEN);
+    }
+
+    // ---- write back: lifetimes; resident ids that are no longer verified become empty (Alg. 4) ----
+    life_words<SPT>(s_life + j0, own, w);
+    life_words_store<SPT>(g_life + j0, own, w);
+    if (stale_ids) {
+        for (uint32_t q = 0; q < NV; ++q)
+            for (uint32_t j = 4u * (tid + q * nt); j < 4u * (tid + q * nt) + 4u && j < S; ++j)
+                if ((int32_t)s_node[j].x >= N) g_tok[j] = -1;
+    }
+    if (tid == 0) {
+        TableStats* st = p.stats + table;                // (reductions: nothing waits for the old values)
+        atomicAdd(&st->steps, 1ull);
+        atomicAdd(&st->tokens, (unsigned long long)p.n_q);
+        atomicAdd(&st->hits, (unsigned long long)(s_sum[0] - sum_miss));
+        atomicAdd(&st->misses, (unsigned long long)sum_miss);
+        atomicAdd(&st->rows, (unsigned long long)list_off);
+        atomicAdd(&st->extra_decays, (unsigned long long)sum_decay);
+    }
+}
+
+// The positions of a copying block (block `rank` of its cluster) in the call's first n groups.
+__device__ __forceinline__ uint32_t positions_of(const StepLayout& lay, uint32_t rank, uint32_t n)
+{
+    return n >= rank ? (((n - rank) * lay.by_copying >> 18) + 1u) << lay.log_group : 0u;
+}
+// The token and the position in it (K or more: none) of a block's n-th.
+struct Place { uint32_t g, i; };
+__device__ __forceinline__ Place place(const StepLayout& lay, uint32_t rank, uint32_t copying, uint32_t n)
+{
+    const uint32_t group = rank - 1u + copying * (n >> lay.log_group), g = group * lay.by_groups >> 18;
+    return {g, (group - g * lay.groups << lay.log_group) + (n & ~(~0u << lay.log_group))};
+}
+
+// A set of ids: three bits, by hash, of a word, by hash.  An id that is in it is found; of those that are not, 0.1 % are found
+// too at 64 bits an id (1.6 % with one bit: a small call then often waits for the row that it has asked for late).
+__device__ __forceinline__ uint32_t set_bits(int32_t x)
+{
+    const uint32_t h = (uint32_t)x * 0x85EBCA6Bu;
+    return __funnelshift_l(0u, 1u, h >> 27) | __funnelshift_l(0u, 1u, h >> 22) | __funnelshift_l(0u, 1u, h >> 17);
+}
+__device__ __forceinline__ void set_add(uint32_t* set, uint32_t log_words, int32_t x)
+{
+    atomicOr(set + hash_id(x, log_words), set_bits(x));
+}
+__device__ __forceinline__ bool set_has(const uint32_t* set, uint32_t log_words, int32_t x)
+{
+    return (~set[hash_id(x, log_words)] & set_bits(x)) == 0;
+}
+
+// A row that a copying block owes: the position in the block's own count, and the token.
+struct Item { uint32_t n, g; };
+
+// A copying block finds out which of its positions are missed for certain: their ids are in no slot and in no earlier token
+// of the call.  What it does not find so (an id that seems to be in a set; a resident one that loses its slot to an earlier
+// token) is news from the first block.  The first row that a warp finds is on its way when this returns (`item`, `row`), the
+// others are left in lay.rest, in position order, token after token.
+// What takes the time is instruction issue and bank conflicts for 32 warps.  From the call's start, 32 tables of 8192 slots,
+// K = 2048, two tokens, three copying blocks: ids and cached ids are loaded after 2.9 us, the sets are there after 3.9, the first
+// rows are asked for after 4.7, where rows that wait for their slots are asked for after 6.5.  Other ways to know: a chained index
+// like Stage One's 5.9 us; the block's positions in a chained index, and the cached ids looked up in that, 7.1 to 8.
+template <int SPT, int IPT, int CAP>
+__device__ __forceinline__ void match(const S1ParamsT<CAP>& p, const StepLayout& lay, const uint32_t ti, const uint32_t rank,
+                                          const uint32_t copying, unsigned char* smem, const uint64_t src, const uint64_t stride,
+                                          Row& row, Item& item)
+{
+    constexpr int NV = (SPT + 3) / 4, OWN = 4;           // of its positions a warp takes OWN times 32 at a time
+    const uint32_t S = p.S, K = p.K, id_limit = p.id_limit[ti], cpr = p.row_bytes >> 4;
+    const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u, warp = tid >> 5, W = nt >> 5;
+    uint32_t* s_seen = reinterpret_cast<uint32_t*>(smem + lay.seen);
+    uint32_t* s_asked = reinterpret_cast<uint32_t*>(smem + lay.asked);
+    int32_t*  s_id   = reinterpret_cast<int32_t*>(smem + lay.id);
+    uint32_t* s_mask = reinterpret_cast<uint32_t*>(smem + lay.mask);
+    uint32_t* s_rest = reinterpret_cast<uint32_t*>(smem + lay.rest);
+    int32_t*  s_ids  = reinterpret_cast<int32_t*>(smem + lay.their_ids);
+    const uint32_t mine = positions_of(lay, rank, p.n_q * lay.groups), asked_words = 1u << lay.log_asked;
+    const int32_t* g_ids = p.indices + (size_t)ti * p.n_q * K;
+
+    auto id_at = [&](uint32_t i) -> int32_t { return p.host_ids ? s_ids[i] : __ldcg(g_ids + i); };
+
+    if (lay.early)
+        for (uint32_t i = tid; i < (lay.slots - lay.seen) / 16u; i += nt) reinterpret_cast<uint4*>(s_seen)[i] = make_uint4(0, 0, 0, 0);
+    if (p.host_ids) {
+        // Ids in host memory are there when the call is made, and nothing on the device writes them: a call that queues
+        // behind another fetches its first ones while that one's rows travel.  The copying blocks share the reading, and
+        // send what they have read to all blocks.
+        const uint32_t all = p.n_q * K, step = copying * nt;
+        int32_t x[OWN];
+        for (uint32_t from = (rank - 1u) * nt + tid, first = 1;; from += OWN * step) {
+#pragma unroll
+            for (int m = 0; m < OWN; ++m) x[m] = from + m * step < all ? __ldcv(g_ids + from + m * step) : -1;
+            if (first) {
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+                cluster_wait();
+                first = 0;
+            }
+#pragma unroll
+            for (int m = 0; m < OWN; ++m) {
+                const uint32_t i = from + m * step;
+                if (i >= all) break;
+                for (uint32_t r = 0; r <= copying; ++r)
+                    stc_u32(map_rank(smem_u32(smem) + (r ? lay.their_ids : lay.ids) + 4u * i, r), (uint32_t)x[m]);
+            }
+            if (from - tid + OWN * step >= all) break;
+        }
+        cluster_sync();
+    } else {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        cluster_wait();
+    }
+    cluster_arrive_relaxed();                            // (what this block sends is sent)
+
+    // ---- every global load is issued first: cached ids, the first token's, the block's own ids ----
+    int4 t4[NV];
+    int32_t xo[OWN], xe[IPT];
+    const int4* g_tok = reinterpret_cast<const int4*>(p.tok + (size_t)p.table_id[ti] * S);
+#pragma unroll
+    for (int q = 0; q < NV; ++q)
+        if (lay.early && tid + q * nt < S / 4) t4[q] = __ldcg(g_tok + tid + q * nt);
+    auto load_own = [&](uint32_t from) {
+#pragma unroll
+        for (int m = 0; m < OWN; ++m) {
+            const uint32_t n = (from + warp + W * m) * 32u + lane;
+            xo[m] = -1;
+            if (n < mine) {
+                const Place q = place(lay, rank, copying, n);
+                if (q.i < K) xo[m] = id_at(q.g * K + q.i);
+            }
+        }
+    };
+    auto load_earlier = [&](uint32_t g) {
+#pragma unroll
+        for (int k = 0; k < IPT; ++k)
+            if (tid + k * nt < K) xe[k] = id_at(g * K + tid + k * nt);
+    };
+    if (lay.early && p.n_q > 1u) load_earlier(0);
+    load_own(0);
+    if (lay.early) {
+        __syncthreads();                                 // the sets are empty
+#pragma unroll
+        for (int q = 0; q < NV; ++q)
+            if (tid + q * nt < S / 4) {                  // (not those of empty slots: a word that all add to takes 4 us)
+                if (t4[q].x >= 0) set_add(s_seen, lay.log_seen, t4[q].x);
+                if (t4[q].y >= 0) set_add(s_seen, lay.log_seen, t4[q].y);
+                if (t4[q].z >= 0) set_add(s_seen, lay.log_seen, t4[q].z);
+                if (t4[q].w >= 0) set_add(s_seen, lay.log_seen, t4[q].w);
+            }
+        for (uint32_t g = 0; g + 1u < p.n_q; ++g) {
+#pragma unroll
+            for (int k = 0; k < IPT; ++k)
+                if (tid + k * nt < K && xe[k] >= 0) set_add(s_asked + g * asked_words, lay.log_asked, xe[k]);
+            if (g + 2u < p.n_q) load_earlier(g + 1u);
+        }
+        __syncthreads();
+    }
+    item.n = NO_ITEM;
+    uint32_t first = 0;
+    for (uint32_t from = 0; from * 32u < mine; from += OWN * W) {
+        if (from) load_own(from);
+#pragma unroll
+        for (int m = 0; m < OWN; ++m) {
+            const uint32_t word = from + warp + W * m, n = word * 32u + lane;
+            if (word * 32u >= mine) break;
+            const uint32_t g = place(lay, rank, copying, n).g;
+            const int32_t x = xo[m];
+            bool certain = lay.early && (uint32_t)x < id_limit && !set_has(s_seen, lay.log_seen, x);
+            for (uint32_t e = 0; e < g && certain; ++e) certain = !set_has(s_asked + e * asked_words, lay.log_asked, x);
+            const uint32_t votes = __ballot_sync(0xffffffffu, certain);
+            s_id[n] = x;
+            uint32_t rest = votes;
+            if (votes && item.n == NO_ITEM) {
+                const uint32_t l = __ffs((int)votes) - 1u;
+                item = {word * 32u + l, __shfl_sync(0xffffffffu, g, (int)l)};
+                first = (uint32_t)__shfl_sync(0xffffffffu, x, (int)l);
+                rest &= rest - 1u;
+            }
+            if (lane == 0) { s_mask[word] = votes; s_rest[word] = rest; }
+        }
+    }
+    if (item.n != NO_ITEM) load_row(row, src + (uint64_t)first * stride, cpr, lane);
+    __syncthreads();
+}
+
+__device__ __forceinline__ SharedRows read_shared(const SharedRows* at)
+{
+    SharedRows s;
+    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(s.rows), "=r"(s.pad), "=r"(s.taken), "=r"(s.begun) : "l"(at) : "memory");
+    return s;
+}
+
+// A warp that is through with its own table's rows copies rows that other tables share.
+template <int CAP>
+__device__ __forceinline__ void take_shared_rows(const S1ParamsT<CAP>& p, const uint32_t ti, const uint32_t group)
+{
+    const uint32_t lane = threadIdx.x & 31u, cpr = p.row_bytes >> 4;
+    // all tables at a time: one after the other they had held up the end of a call with many
+    SharedRows now = {0u, 0u, 0u, 0u};
+    if (group + lane < p.n_launch && group + lane != ti) now = read_shared(p.shared + group + lane);
+    const bool some = (now.rows & SHARED_COMING) ||
+                      ((now.rows & SHARED_OPEN) && now.taken + now.begun + SHARED_LEFT < (now.rows & ~SHARED_OPEN));
+    for (uint32_t which = __ballot_sync(0xffffffffu, some); which; which &= which - 1u) {
+        const uint32_t t = group + __ffs((int)which) - 1u;
+        SharedRows s = read_shared(p.shared + t);
+        for (uint32_t spin = 0; (s.rows & SHARED_COMING) && spin < OVERLAP_SPIN_LIMIT; ++spin) {     // (that Stage One runs, and waits for nobody)
+            __nanosleep(64);
+            s = read_shared(p.shared + t);
+        }
+        __threadfence();
+        const uint32_t rows = __shfl_sync(0xffffffffu, s.rows, 0) ^ SHARED_OPEN;
+        if (rows >= SHARED_OPEN) continue;                             // closed meanwhile
+        const uint64_t src = p.kv_base[t], stride = p.kv_stride[t];
+        const uint64_t dst = reinterpret_cast<uint64_t>(p.buffer + (size_t)p.table_id[t] * p.S * p.row_bytes);
+        const int2* list = p.miss_list + (size_t)t * p.list_stride;
+        for (;;) {
+            uint32_t at = 0xFFFFFFFFu;
+            if (lane == 0 && s.taken + s.begun + SHARED_LEFT < rows) at = atomicAdd(&p.shared[t].taken, 1u);
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (at >= rows) break;
+            const int2 e = __ldcg(list + (rows - 1u - at));            // what is taken is copied
+            s = read_shared(p.shared + t);                             // (comes with the row)
+            if (e.x < 0 || e.y < 0 || (uint32_t)e.y >= p.S) {
+                if (lane == 0) atomicOr(p.status, ST_BAD_SLOT);
+                continue;
+            }
+            copy_row(src + (uint64_t)(uint32_t)e.x * stride, dst + (uint64_t)(uint32_t)e.y * p.row_bytes, cpr, lane);
+        }
+    }
+}
+
+// A call in one kernel: a cluster of two to eight blocks per table, in either mode.  What it saves is a launch (1.8 us of host
+// time, which bounds the smallest calls), the way from the end of one grid to the start of the next, and the hand-over
+// through global memory with its fences.  A copying block keeps 20 KB of rows on the way, a row per warp, so that
+// seven can fill the link with one table's rows (2 us round trip x 47 GB/s) and the other sizes with what runs beside it.
+// Measured, in two kernels (Stage Two overlapped where that is faster) / in one whose rows are asked for when their slots are
+// known, us per call:
+//   K = 256, S = 1024, one table 8.4 / 5.8;  K = 2048, S = 8192, two tokens, one table 17.2 / 12.2, from a graph 19.8 / 18.3;
+//   the same with 4, 8, 16, 32, 48, 64 tables 26.2 / 22.4, 39.0 / 35.6, 65.9 / 63.6, 119.9 / 116.8, 174.0 / 173.6, 228.3 / 226.8;
+//   the same from 11 GB of host memory with 8, 16, 32, 48, 64 tables 51 / 46, 88 / 84, 173 / 155, 242 / 229, 315 / 296.
+// Asked for at once, before / now: one table 12.4 / 11.1, 8 tables with K = 1000 and 1152-byte rows 35.3 / 33.7, 32 tables 119.1 /
+// 116.9, 16 from 11 GB 84.4 / 82.5.  A call that keeps selecting what it has just lost gains nothing (S = 1024, three tokens of K = 196: 12.6 / 13.8).
+// The line of 11 GB is what the end of a call is for.  Where a table's pages are spread over much host memory, translating
+// their addresses limits the rows, and a cluster, which lies in one GPC, finds its table's translations there if the
+// table was there in the call before.  So calls of more than a few tables let the next grid start only when their
+// blocks exit: its clusters then find the same SMs free, in the same order.  Started early they take whatever is free at
+// that time: eight tables 60 us and not 46, 16 113 and not 84 (step_early() says which calls gain by it).
+// The warps of a block take its rows from a counter, in position order, so that neighbours in host memory go together.
+// SHARE (two and three blocks).  A cluster alone cannot fill the link with one table's rows where it has few copying blocks (an
+// SM gets 20 of them a us, the link carries 72), so a new request among steady ones would be left behind: 64 tables, one of
+// them cold, 332 us against 277 in two kernels, whose rows are cut evenly over all SMs (Eq. 6).  So a table that misses more
+// than SHARED_FROM ids in a token writes these misses to its list in global memory too, and says so.  Its own blocks copy them
+// from the front; a few warps of other tables that are through take single rows from the back, counted in SharedRows::taken,
+// until few are left; the own blocks stop where the others have begun.  Both may copy a row in the middle, to the same effect.
+// Every row is copied: what the own blocks leave out is counted in `taken`, and what is counted there is copied by who counted it.
+// Nobody waits, but for a Stage One that has announced rows and runs.  One cold table of 45, 64: 229, 332 us without, 215, 283
+// with it, 211, 277 in two kernels; the others with hits only 70, 124, 50, 57, 46, 46; all steady 169, 239.5, 170, 240.5, 172, 241.
+// With four blocks it costs every call more (16 tables 64.7 us, 65.5 with it) than it gives one with a new request (16, 32
+// tables, one cold: 115, 172 without, 113, 170 with it, 110, 167 in two kernels).  With all rows of such a table claimed one by
+// one, its own blocks' too, the cold calls were quicker still (45 tables 214), but a call where most tables had many misses
+// lost 5 to 20 %: the requests for claims and list entries wait behind the rows'.  Several rows of a warp at once bring an SM
+// from 20 rows a us to 28 at most.
+template <int SPT, int IPT, int CAP, bool SHARE = false>
+__global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constant__ S1ParamsT<CAP> p, const __grid_constant__ StepLayout lay)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ __align__(8) unsigned long long s_mbar[STEP_MAX_TOKENS];
+    __shared__ uint32_t s_sent[STEP_MAX_TOKENS];                       // received: a token's misses in the block's positions
+    __shared__ uint32_t s_own[2 * STEP_FEW_CLUSTER];                   // first block: of those, how many it has sent, by parity of the token
+    __shared__ uint32_t s_first[SHARE ? STEP_MAX_TOKENS : 1];          // received: the token's first row among those that are shared; -1
+    __shared__ uint32_t s_next;                                        // of the listed rows, the first that no warp has taken
+    __shared__ volatile uint32_t s_mine;                               // rows that are shared: the first that others have taken
+    const uint32_t rank = cluster_rank(), cluster = cluster_size(), copying = cluster - 1u;
+    const uint32_t ti = blockIdx.x / cluster, lane = threadIdx.x & 31u, W = blockDim.x >> 5, warp = threadIdx.x >> 5;
+    uint32_t* s_slots = reinterpret_cast<uint32_t*>(smem + lay.slots);
+    if (p.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (SHARE && threadIdx.x == 0) s_mine = 0xFFFFFFFFu;
+    if (rank != 0) {
+        if (threadIdx.x == 0) s_next = 0;
+        if (threadIdx.x < p.n_q) mbar_init(smem_u32(s_mbar + threadIdx.x), 1u);
+        for (uint32_t i = threadIdx.x; i < lay.local; i += blockDim.x) s_slots[i] = NOT_MISSED;
+        for (uint32_t i = threadIdx.x; i < lay.local / 32u; i += blockDim.x) reinterpret_cast<uint32_t*>(smem + lay.rest)[i] = 0;
+    }
+    __syncthreads();
+    cluster_arrive();
+    if (rank == 0) {
+        place_tokens<SPT, IPT, SHARE>(p, lay, ti, copying, smem, smem_u32(s_mbar), smem_u32(s_sent), smem_u32(s_first), s_own);
+        __syncwarp();
+        cluster_arrive();                                              // the outputs are written, everything is sent
+        return;
+    }
+    const uint32_t cpr = p.row_bytes >> 4;
+    const uint64_t src = p.kv_base[ti], stride = p.kv_stride[ti];
+    const uint64_t dst = reinterpret_cast<uint64_t>(p.buffer + (size_t)p.table_id[ti] * p.S * p.row_bytes);
+    Row row;
+    Item item;
+    match<SPT, IPT>(p, lay, ti, rank, copying, smem, src, stride, row, item);
+    const int32_t* s_id = reinterpret_cast<const int32_t*>(smem + lay.id);
+    const uint32_t* s_mask = reinterpret_cast<const uint32_t*>(smem + lay.mask);
+    const uint32_t* s_rest = reinterpret_cast<const uint32_t*>(smem + lay.rest);
+    uint32_t placed = 0;                                               // tokens
+    auto wait_until = [&](uint32_t g) -> bool {                        // (Stage One's loops are bounded, far below this)
+        while (placed <= g && wait_for(smem_u32(s_mbar + placed), AVSG_STEP_GIVE_UP)) ++placed;
+        return placed > g;
+    };
+    auto slot_of = [&](uint32_t what) -> uint32_t {                    // what a position has received; NO_SLOT: there were not enough
+        const uint32_t j = what & 0xFFFFu;
+        if (j < p.S) return j;
+        if (j != NO_SLOT && lane == 0) atomicOr(p.status, ST_BAD_SLOT);
+        return NO_SLOT;
+    };
+    bool there = true;
+    SharedRows s = {SHARED_COMING, 0u, 0u, 0u};
+    // The rows that no warp has asked for yet: a lane counts those of a few neighbouring words, and those before them
+    uint32_t upto = 0;
+    if (lay.early)
+        for (uint32_t a = lane * lay.per_lane; a < lay.local / 32u && a < (lane + 1u) * lay.per_lane; ++a) upto += __popc(s_rest[a]);
+    upto = warp_incl_scan(upto, lane);
+    auto next = [&] {                                                  // the warp's next row, on its way before its slot is known
+        for (;;) {
+            uint32_t k = 0;
+            if (lane == 0) k = atomicAdd(&s_next, 1u);
+            k = __shfl_sync(0xffffffffu, k, 0);
+            item.n = NO_ITEM;
+            const uint32_t behind = __ballot_sync(0xffffffffu, upto > k);
+            if (behind == 0) return;
+            const uint32_t l = __ffs((int)behind) - 1u;
+            if (l) k -= __shfl_sync(0xffffffffu, upto, (int)l - 1);
+            uint32_t a = l * lay.per_lane, m = s_rest[a];
+            for (; k >= __popc(m); m = s_rest[++a]) k -= __popc(m);
+            const uint32_t n = a * 32u + __ffs((int)__ballot_sync(0xffffffffu, (m >> lane & 1u) && __popc(m & ((1u << lane) - 1u)) == k)) - 1u;
+            const uint32_t g = place(lay, rank, copying, n).g;
+            if (SHARE) {
+                if (!(there = wait_until(g))) return;
+                if (s_first[g] != ~0u) {
+                    if (warp == 0) {                                   // for all warps: requests wait behind the rows' where the link is full
+                        if (!(s.rows & SHARED_COMING)) s_mine = (s.rows & ~SHARED_OPEN) > s.taken ? (s.rows & ~SHARED_OPEN) - s.taken : 0u;
+                        s = read_shared(p.shared + ti);                // (comes with the row)
+                        if (lane == 0) atomicAdd(&p.shared[ti].begun, W);
+                    }
+                    if (s_first[g] + (s_slots[n] >> 16) >= s_mine) continue;           // others have it
+                }
+            }
+            item.n = n;
+            item.g = g;
+            load_row(row, src + (uint64_t)(uint32_t)s_id[n] * stride, cpr, lane);
+            return;
+        }
+    };
+    auto put = [&] {
+        const uint32_t j = slot_of(s_slots[item.n]);
+        if (j != NO_SLOT) store_row(row, dst + (uint64_t)j * p.row_bytes, cpr, lane);
+    };
+    if (item.n == NO_ITEM) next();
+    const int2* s_list = reinterpret_cast<const int2*>(smem + lay.list);
+    for (uint32_t g = 0; there && g < p.n_q; ++g) {
+        if (!(there = wait_until(g))) break;
+        bool placed_one = item.n != NO_ITEM && item.g <= g;
+        if (placed_one) put();
+        // the token's other misses (all of them where nothing is asked for early), in turn
+        for (uint32_t e = W - 1u - warp; e < s_sent[g]; e += W) {
+            const int2 what = s_list[g * lay.per_token + e];
+            const uint32_t n = (uint32_t)what.x;
+            if (s_mask[n / 32u] >> n % 32u & 1u) continue;
+            const uint32_t j = slot_of((uint32_t)what.y);
+            if (j != NO_SLOT) copy_row(src + (uint64_t)(uint32_t)s_id[n] * stride, dst + (uint64_t)j * p.row_bytes, cpr, lane);
+        }
+        while (placed_one && there) {
+            next();
+            placed_one = item.n != NO_ITEM && item.g <= g;
+            if (placed_one && there) put();
+        }
+    }
+    // Warps that take other tables' rows: a few of each block
+    uint32_t others = 0;                                               // what 32 of the tables share, one a lane
+    const uint32_t group = (ti + warp) % ((p.n_launch + 31u) / 32u) * 32u;
+    const bool takes = SHARE && warp * (p.n_launch - 1u) * copying < SHARED_WARPS * ((p.n_launch + 31u) / 32u);
+    if (takes && group + lane < p.n_launch) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(others) : "l"(&p.shared[group + lane].rows) : "memory");
+    // Stage One does not know who has given up, and nothing may be sent to a block that is gone: every block stays until
+    // Stage One is through, and one that gave up until what was sent has arrived.
+    cluster_wait();
+    if (!there) {
+        if (lane == 0) atomicOr(p.status, ST_WAIT_TIMEOUT);
+        for (uint32_t g = 0; g < p.n_q && wait_for(smem_u32(s_mbar + g), STEP_SPIN_LIMIT); ++g) {}
+    }
+    if (p.out.n_slots) put_outputs_of(p.out, ti, p.n_q * p.K, p.n_q, warp * copying + rank - 1u, W * copying, lane);
+    if constexpr (SHARE) {
+        // Closed for who has not begun yet, and so closed between calls (Stage One is through and writes it no more).
+        if (threadIdx.x == 0) atomicAnd(&p.shared[ti].rows, SHARED_OPEN - 1u);
+        if (takes && __any_sync(0xffffffffu, (others & (SHARED_COMING | SHARED_OPEN)) != 0)) take_shared_rows(p, ti, group);
+    }
+}
+
+}  // namespace
+
+// At least 16 warps a block where the table has the slots for it: they copy.
+uint32_t step_threads(uint32_t S, uint32_t K)
+{
+    const uint32_t t = stage_one_threads(S, K), most = S / 2 < 512u ? S / 2 : 512u;
+    return t > most ? t : most;
+}
+
+namespace {
+
+template <int CAP, bool SHARE = false>
+const void* step_kernel(uint32_t spt, uint32_t ipt)
+{
+    switch (spt) {
+        case 8:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 2, CAP, SHARE>)
+                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 4, CAP, SHARE>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<8, 8, CAP, SHARE>);
+        case 4:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<4, 2, CAP, SHARE>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<4, 4, CAP, SHARE>);
+        default: return reinterpret_cast<const void*>(avsg_step_kernel<2, 2, CAP, SHARE>);
+    }
+}
+
+void step_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, uint32_t n_tables, uint32_t cluster, uint32_t threads, size_t smem)
+{
+    cfg.gridDim = dim3(n_tables * cluster);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+}
+}  // namespace
+
+// Loads this file's kernels and raises their limit of dynamic shared memory to the device's (see stage_one_prepare() on why
+// that is not left to their first launch).
+cudaError_t step_prepare(size_t max_smem)
+{
+    for (uint32_t spt : {2u, 4u, 8u})
+        for (uint32_t ipt = 2u; ipt <= spt; ipt *= 2u)                 // (K <= S)
+            for (const void* k : {step_kernel<STEP_FEW_TABLES>(spt, ipt), step_kernel<STEP_MAX_TABLES>(spt, ipt), step_kernel<STEP_MAX_TABLES, true>(spt, ipt)}) {
+                cudaFuncAttributes fa;
+                cudaError_t e = cudaFuncGetAttributes(&fa, k);
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(max_smem - fa.sharedSizeBytes));
+                if (e != cudaSuccess) return e;
+            }
+    return cudaSuccess;
+}
+
+StepClusters step_clusters(size_t max_smem)
+{
+    StepClusters s;
+    for (uint32_t cl : {2u, 3u, 4u, STEP_FEW_CLUSTER}) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[2];
+        int fit = 0;
+        step_config(cfg, attr, 1, cl, 1024, max_smem - 2048);      // (the largest; statically it has 1 KB)
+        if (cudaOccupancyMaxActiveClusters(&fit, step_kernel<STEP_MAX_TABLES>(8, 2), &cfg) != cudaSuccess) { cudaGetLastError(); fit = 0; }
+        s.fit[cl] = (uint32_t)fit;
+    }
+    return s;
+}
+
+template <int CAP>
+cudaError_t launch_step(const S1ParamsT<CAP>& p, uint32_t cluster, cudaStream_t stream)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    const uint32_t nt = step_threads(p.S, p.K);
+    StepLayout lay = step_layout(p.S, p.K, p.n_q, nt, cluster - 1u, p.row_bytes, p.host_ids != 0);
+    step_config(cfg, attr, p.n_launch, cluster, nt, lay.total);
+    cfg.stream = stream;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+    void* args[] = {const_cast<S1ParamsT<CAP>*>(&p), &lay};
+    const uint32_t spt = p.S / nt, ipt = (p.K + nt - 1) / nt;
+    if constexpr (CAP == STEP_MAX_TABLES)
+        if (cluster < SHARED_CLUSTER) return cudaLaunchKernelExC(&cfg, step_kernel<CAP, true>(spt, ipt), args);
+    return cudaLaunchKernelExC(&cfg, step_kernel<CAP>(spt, ipt), args);
+}
+template cudaError_t launch_step(const StepParams& p, uint32_t cluster, cudaStream_t stream);
+template cudaError_t launch_step(const StepParamsFew& p, uint32_t cluster, cudaStream_t stream);
+
+}  // namespace avsg
