@@ -291,6 +291,8 @@ __device__ __forceinline__ void stage_one(const S1ParamsT<CAP>& p, const uint32_
             announce_token(p, ti, g, n_take);
         }
 
+        if (unusual) drop_lost_rows(list, list_off, s_node);
+
         // ---- write back: lifetimes; resident ids that are no longer verified become empty (Alg. 4) ----
         life_words<SPT>(s_life + j0, own, w);
         life_words_store<SPT, WIDE>(g_life + j0, own, w);

@@ -164,6 +164,20 @@ __device__ __forceinline__ void find_slots(const int32_t (&x)[M], const uint2* s
     if (open) atomicOr(status, ST_PROBE_EXHAUSTED);
 }
 
+// With lifetimes above L on entry a slot that one token of a call reserves may be reserved again by a later one.  Nothing orders
+// the copies of a call's rows, so only the last reservation's row may be copied: the entries {id, slot (and more, from bit
+// LIST_SLOT_BITS on)} of a table's list whose slots hold another id by now become padding.  All threads of the block, behind a
+// barrier; thread t has the entries t, t + blockDim.x, ...  Lifetimes above L come with a caller's own state only, so with no
+// Stage Two that already follows the list.
+constexpr uint32_t LIST_SLOT_BITS = 13;                  // S <= 8192 here
+__device__ __forceinline__ void drop_lost_rows(int2* list, uint32_t count, const uint2* s_node)
+{
+    for (uint32_t e = threadIdx.x; e < count; e += blockDim.x) {
+        const int2 v = list[e];
+        if ((int32_t)s_node[(uint32_t)v.y & ((1u << LIST_SLOT_BITS) - 1u)].x != v.x) list[e].x = -1;
+    }
+}
+
 // Bits 0 .. 3: the sign bits of a word's four bytes.
 __device__ __forceinline__ uint32_t signs(uint32_t w) { return (((w >> 7) & 0x01010101u) * 0x10204080u) >> 28; }
 

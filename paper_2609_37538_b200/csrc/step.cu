@@ -105,6 +105,54 @@ __device__ __forceinline__ bool wait_for(uint32_t mbar, uint32_t limit)
     return __all_sync(0xffffffffu, spin < limit);
 }
 
+// What the copying blocks are told of a token: `to` of them that it has n misses in the block's positions, and from which row on
+// they are shared (SHARE); of a miss, the block that the position i belongs to the slot, where the position's place is and in
+// the next entry of its list.
+struct Tell {
+    const StepLayout& lay;
+    uint32_t copying, smem, mbar, sent, first;           // of the first block's own: the same places as in the others
+
+    template <bool SHARE>
+    __device__ __forceinline__ void token(uint32_t g, uint32_t to, uint32_t n, uint32_t first_shared) const
+    {
+        const uint32_t bar = map_rank(mbar + 8u * g, to + 1u);
+        send_async(map_rank(sent + 4u * g, to + 1u), n, bar);
+        if (SHARE) send_async(map_rank(first + 4u * g, to + 1u), first_shared, bar);
+        arrive_expect(bar, 12u * n + (SHARE ? 8u : 4u));
+    }
+    // own: the misses of the token that the blocks have been told of
+    __device__ __forceinline__ void miss(uint32_t g, uint32_t i, uint32_t what, uint32_t* own) const
+    {
+        const uint32_t group = g * lay.groups + (i >> lay.log_group), at = group * lay.by_copying >> 18, to = group - at * copying;
+        const uint32_t n = (at << lay.log_group) + (i & ((1u << lay.log_group) - 1u)), bar = map_rank(mbar + 8u * g, to + 1u);
+        send_async(map_rank(smem + lay.slots + 4u * n, to + 1u), what, bar);
+        const uint32_t e = atomicAdd(own + to, 1u);
+        send_async(map_rank(smem + lay.list + 8u * (g * lay.per_token + e), to + 1u), (int32_t)n, (int32_t)what, bar);
+    }
+};
+
+// A call with lifetimes above L on entry: the copying blocks hear of all tokens when the last one is placed, and only of
+// rows that their slots still wait for.  list: {id, slot | position << 13 | token << 26}.  (Inline: a function call in the kernel
+// brings every call's row loads late; 8 new requests 265 us and not 257.)
+template <bool SHARE>
+__device__ __forceinline__ void tell_at_last(const Tell tell, uint32_t n_q, int2* list, uint32_t count, const uint2* s_node, uint32_t* s_own)
+{
+    static_assert(STEP_MAX_TOKENS <= 1u << (32u - 2u * LIST_SLOT_BITS), "a token does not fit an entry");
+    drop_lost_rows(list, count, s_node);
+    for (uint32_t g = 0; g < n_q; ++g) {
+        if (threadIdx.x < STEP_FEW_CLUSTER) s_own[threadIdx.x] = 0;
+        __syncthreads();
+        for (uint32_t e = threadIdx.x; e < count; e += blockDim.x) {
+            const int2 v = list[e];
+            const uint32_t what = (uint32_t)v.y, mask = (1u << LIST_SLOT_BITS) - 1u;
+            if (v.x >= 0 && what >> (2u * LIST_SLOT_BITS) == g) tell.miss(g, what >> LIST_SLOT_BITS & mask, what & mask, s_own);
+        }
+        __syncthreads();
+        if (threadIdx.x < tell.copying) tell.token<SHARE>(g, threadIdx.x, s_own[threadIdx.x], ~0u);
+        __syncthreads();
+    }
+}
+
 // The first block of a cluster: Stage One.  SPT slots per thread (a power of two): S <= SPT * blockDim.x.  IPT: the most
 // ids a thread has of a token (K <= S, so SPT is always enough).  a_mbar: the copying blocks' mbarriers, one per token.
 // The passes are those of avsg_stage_one_kernel, which says what they are and why.  SHARE: rows of a table with very many
@@ -197,6 +245,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
     uint32_t list_off = 0, sum_miss = 0, sum_decay = 0, valid = 0;
     uint32_t shared = 0;                                 // SHARE: rows that other blocks may take (bit 31: there will be some)
     int2* list = p.miss_list + (size_t)ti * p.list_stride;
+    const Tell tell = {lay, copying, smem_u32(smem), a_mbar, a_sent, a_first};
 
     for (uint32_t g = 0; g < p.n_q; ++g) {
         const bool last = g + 1 == p.n_q;
@@ -261,7 +310,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
         uint32_t dtotal = all & 0xFFFFu, dead_before = before & 0xFFFFu, d = 0;
         sum_miss += n_g;
         if (tid == 0 && p.miss_count) p.miss_count[(size_t)ti * p.n_q + g] = (int32_t)n_g;
-        const bool share_it = SHARE && n_g > SHARED_FROM;
+        const bool share_it = SHARE && n_g > SHARED_FROM && !unusual;
         if (share_it && !shared) {
             shared = SHARED_COMING;
             if (tid == 0) {                              // (in place before the table's own blocks hear of the rows)
@@ -308,7 +357,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
         if (lane == 0) s_ndead[32u - par + warp] = left;
         __syncthreads();
 
-        for (uint32_t to = nw - 1u - warp; to < copying; to += nw) {       // what a copying block gets of this token (the first warps install)
+        for (uint32_t to = nw - 1u - warp; to < copying && !unusual; to += nw) {       // what a copying block gets of this token (the first warps install)
             // (its first group is the first one that is `to` modulo copying)
             uint32_t group = (group0 * lay.by_copying >> 18) * copying + to, n = 0;
             if (group < group0) group += copying;
@@ -317,12 +366,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
                 n += __popc(s_votes[i / 32u] >> i % 32u & ~(~1u << in_group));
             }
             n = __reduce_add_sync(0xffffffffu, n);
-            if (lane == 0) {
-                const uint32_t mbar = map_rank(a_mbar + 8u * g, to + 1u);
-                send_async(map_rank(a_sent + 4u * g, to + 1u), n, mbar);
-                if (SHARE) send_async(map_rank(a_first + 4u * g, to + 1u), share_it ? shared & ~SHARED_COMING : ~0u, mbar);
-                arrive_expect(mbar, 12u * n + (SHARE ? 8u : 4u));
-            }
+            if (lane == 0) tell.token<SHARE>(g, to, n, share_it ? shared & ~SHARED_COMING : ~0u);
         }
 
         // ---- install: the k-th miss in position order takes the k-th dead slot ----
@@ -330,12 +374,11 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
             const uint32_t i = s_pos[k];
             const int32_t x = s_miss[k];
             const int32_t j = k < n_take ? s_dead[k] : -1;
-            // to the block that the position belongs to: the slot where the position's place is, and an entry of its list
-            const uint32_t group = group0 + (i >> lay.log_group), at = group * lay.by_copying >> 18, to = group - at * copying;
-            const uint32_t n = (at << lay.log_group) + (i & in_group), what = ((uint32_t)j & 0xFFFFu) | k << 16, mbar = map_rank(a_mbar + 8u * g, to + 1u);
-            send_async(map_rank(smem_u32(smem) + lay.slots + 4u * n, to + 1u), what, mbar);
-            const uint32_t e = atomicAdd(s_own + (g & 1u) * STEP_FEW_CLUSTER + to, 1u);
-            send_async(map_rank(smem_u32(smem) + lay.list + 8u * (g * lay.per_token + e), to + 1u), (int32_t)n, (int32_t)what, mbar);
+            if (!unusual) {
+                tell.miss(g, i, ((uint32_t)j & 0xFFFFu) | k << 16, s_own + (g & 1u) * STEP_FEW_CLUSTER);
+            } else if (k < n_take) {
+                list[list_off + k] = make_int2(x, (int32_t)((uint32_t)j | i << LIST_SLOT_BITS | g << (2u * LIST_SLOT_BITS)));
+            }
             if (k < n_take) {
                 s_node[j].x = (uint32_t)x;
                 s_life[j] = (int8_t)L;
@@ -355,6 +398,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
         __syncthreads();
         announce_token(p, ti, g, n_take);
     }
+    if (unusual) tell_at_last<SHARE>(tell, p.n_q, list, list_off, s_node, s_own);
     if (SHARE && shared && tid == 0) {
         __threadfence();
         *reinterpret_cast<volatile uint32_t*>(&p.shared[ti].rows) = shared == SHARED_COMING ? 0u : shared ^ (SHARED_COMING | SHARED_OPEN);

@@ -113,6 +113,46 @@ def test_lifetimes_above_the_maximum():
         assert int(status.item()) == 0
 
 
+# clusters of eight, four and three blocks, and two kernels (state off its alignment); the small sizes of the test above too
+@pytest.mark.parametrize("n,S,K,n_q", [(2, 64, 16, 4), (1, 4096, 2048, 2), (9, 4096, 2048, 2), (32, 4096, 2048, 2), (3, 8192, 1000, 8)])
+@pytest.mark.parametrize("aligned", [True, False])
+def test_the_last_reservation_of_a_slot_has_its_row(n, S, K, n_q, aligned):
+    """Lifetimes above the maximum: a slot that two tokens of a call reserve holds the row of the later one."""
+    import torch
+    import paper_2609_37538_b200 as avsg
+    L, context, calls, rb = 3, 40000, 3, 64
+    kv = avsg.pinned_empty(context * rb)
+    tr.fill_kv(kv.data_ptr(), 3, 0, context, rb)
+    rng = np.random.default_rng([n, S, K])
+    d = dict(device="cuda")
+    tok_d, life_d = (torch.empty(n * S + 1, dtype=t, **d)[0 if aligned else 1 :][: n * S].view(n, S) for t in (torch.int32, torch.int8))
+    buf, status = torch.zeros((n, S, rb), dtype=torch.uint8, **d), torch.zeros(1, dtype=torch.int32, **d)
+    slots, hit = torch.empty((n, n_q, K), dtype=torch.int32, **d), torch.empty((n, n_q, K), dtype=torch.uint8, **d)
+    orc = [OracleTable(S, rb, L) for _ in range(n)]
+    twice = 0
+    for c in range(calls):
+        tok, life = np.full(S, -1, np.int32), np.full(S, -1, np.int8)
+        tok[::2], life[::2] = context - 1 - np.arange(S // 2), 90        # half of the table outlives the call
+        for o in orc:
+            o.import_state(tok, life)
+        tok_d.copy_(torch.from_numpy(tok).expand(n, S)); life_d.copy_(torch.from_numpy(life).expand(n, S))
+        X = np.stack([rng.permutation(context - S)[: n_q * K].reshape(n_q, K) for _ in range(n)]).astype(np.int32)
+        X[:, 1, 0] = -1                                                   # what is reserved again moves by a row
+        avsg.step_noalloc(tok_d, life_d, buf, torch.from_numpy(X).cuda(), [kv] * n, [context] * n, max_lifetime=L, slots=slots,
+                          hit=hit, status=status)
+        assert int(status.item()) == 0
+        for i in range(n):
+            r = orc[i].step(X[i], context, kv.numpy(), rb)
+            o, l = orc[i].export_state()
+            assert (slots[i].cpu().numpy() == r.O).all() and (hit[i].cpu().numpy() == r.M).all(), (c, i)
+            assert (tok_d[i].cpu().numpy() == o).all() and (life_d[i].cpu().numpy() == l).all(), (c, i)
+            got, want = buf[i].cpu().numpy(), orc[i].rows()
+            assert (got == want).all(), (c, i, int((got != want).any(axis=1).sum()))
+            taken = r.O[r.O >= 0]
+            twice += len(taken) - len(np.unique(taken))
+    assert twice > 0
+
+
 # slots per thread of two, four and eight; the last one takes two kernels
 @pytest.mark.parametrize("S,K,n_q", [(32, 8, 2), (256, 31, 3), (1024, 300, 2), (2048, 500, 2), (4096, 1000, 3), (8192, 2048, 2),
                                      (256, 2, 70)])
