@@ -71,10 +71,11 @@ extern "C" {
                                        kernel in this mode and in AVSG_XFER_SM_OVERLAP: a
                                        thread-block cluster per table, Stage Two following
                                        Stage One token by token; the split over SMs is then
-                                       by position within a table, and from 34 tables on rows of a
-                                       table that misses more than 512 ids of a token are
-                                       taken over by blocks of others that are through (not with arriving, timing,
-                                       an own transfer geometry or a table above 8192
+                                       within a table: by position, or even from 34 tables
+                                       (of 8192 slots) on, where rows of a table that misses
+                                       more than 512 ids of a token are also taken over by
+                                       blocks of others that are through (not with arriving,
+                                       timing, an own transfer geometry or a table above 8192
                                        slots, nor with stage_one_done above three tables).
                                        Its blocks take whole SMs while they run: who wants
                                        room for other kernels beside the call sets a

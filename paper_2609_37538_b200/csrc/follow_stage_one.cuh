@@ -24,11 +24,19 @@ __device__ __forceinline__ void st16(uint64_t addr, const int4& v)
 // those requests are smaller.)
 constexpr uint32_t ROW_CHUNKS = 96;
 struct Row { int4 v[ROW_CHUNKS / 32]; };
-__device__ __forceinline__ void load_row(Row& r, uint64_t src, uint32_t cpr, uint32_t lane)
+__device__ __forceinline__ void load_row(Row& r, uint64_t src, uint32_t chunks, uint32_t lane)
 {
-#pragma unroll
-    for (uint32_t k = 0; k < ROW_CHUNKS / 32; ++k)
-        if (lane + 32u * k < cpr) r.v[k] = ld16(src + 16ull * (lane + 32u * k));
+    // (One statement, predicated inside: with a branch around it a piece would have an old and a new value, and a copy from register
+    // to register where these meet would wait for the load.  The pieces' loads follow one another without anything in between.)
+    static_assert(ROW_CHUNKS == 96, "three loads");
+    asm volatile("{\n\t.reg .pred p, q, r;\n\t"
+                 "setp.gt.u32 p, %14, %13;\n\tsetp.gt.u32 q, %15, %13;\n\tsetp.gt.u32 r, %16, %13;\n\t"
+                 "@p ld.global.v4.s32 {%0, %1, %2, %3}, [%12];\n\t"
+                 "@q ld.global.v4.s32 {%4, %5, %6, %7}, [%12 + 512];\n\t"
+                 "@r ld.global.v4.s32 {%8, %9, %10, %11}, [%12 + 1024];\n\t}"
+                 : "=r"(r.v[0].x), "=r"(r.v[0].y), "=r"(r.v[0].z), "=r"(r.v[0].w), "=r"(r.v[1].x), "=r"(r.v[1].y), "=r"(r.v[1].z), "=r"(r.v[1].w),
+                   "=r"(r.v[2].x), "=r"(r.v[2].y), "=r"(r.v[2].z), "=r"(r.v[2].w)
+                 : "l"(src + 16ull * lane), "r"(lane), "r"(chunks), "r"(chunks > 32u ? chunks - 32u : 0u), "r"(chunks > 64u ? chunks - 64u : 0u));
     __syncwarp();                      // (the compiler may move plain loads behind a wait, but not behind this)
 }
 __device__ __forceinline__ void store_row(const Row& r, uint64_t dst, uint32_t cpr, uint32_t lane)

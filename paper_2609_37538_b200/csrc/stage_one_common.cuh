@@ -51,6 +51,10 @@ __device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t arrivals)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n\tfence.mbarrier_init.release.cluster;" :: "r"(mbar), "r"(arrivals) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(uint32_t mbar)              // the block's own
+{
+    asm volatile("{\n\t.reg .b64 s;\n\tmbarrier.arrive.release.cta.shared::cta.b64 s, [%0];\n\t}" :: "r"(mbar) : "memory");
+}
 __device__ __forceinline__ bool mbar_done(uint32_t mbar)
 {
     uint32_t done;

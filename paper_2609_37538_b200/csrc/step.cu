@@ -2,13 +2,21 @@
 //
 // The first block of a cluster runs Stage One (match + reserve: Algorithm 1 with the lifetime operations of Algorithm 3,
 // the tokens of an iteration in order as in Algorithm 4, the end-of-step invalidation); the others copy the rows of the
-// misses.  Which block copies a position's row follows from the position alone: groups of neighbours go round over the
-// copying blocks.  So a copying block need not be told what to fetch.  It puts the table's cached ids into a set of its own
+// misses, in one of two ways.
+//
+// Rows asked for early (clusters of four blocks and more, rows that fit a warp's registers, sets that fit beside one another).
+// Which block copies a position's row follows from the position alone: groups of neighbours go round over the copying blocks.
+// So a copying block need not be told what to fetch.  It puts the table's cached ids into a set of its own
 // (bits by hash), and an id of its positions that is not in there, nor in those of the earlier tokens, is missed for certain,
 // whatever the tokens before it take away: its row is asked for at once, and is on its way (2 us, over the host link) while
 // Stage One still finds out which slot it goes to.  The slot arrives by st.async in a place that again follows from the
 // position, counted by an mbarrier per token.  Misses that the block could not know of (an id that seems to be in a set, or
 // that loses its slot to an earlier token of the call) it finds in the list of its misses that comes with the slots.
+//
+// Rows in the order of the misses.  Stage One deals the misses out, the k-th to block k % copying or in shares of neighbours, and
+// sends {id, slot}.  Clusters of two and three blocks share rows with other tables' blocks (see the kernel), which takes rows
+// from the end of a table's misses: so their own blocks have to take them from the front.  Rows of 1552 bytes and more: one table
+// 15.5 us, with misses listed by position but not asked for early 16.0; 4096 bytes 25.4, 25.9.
 #include "avsg_kernels.cuh"
 #include "follow_stage_one.cuh"
 #include "stage_one_common.cuh"
@@ -28,41 +36,40 @@ constexpr uint32_t STEP_SPIN_LIMIT = 1u << 18;            // tries; the hardware
 constexpr uint32_t SHARED_FROM = 512, SHARED_LEFT = 256, SHARED_WARPS = 144, SHARED_CLUSTER = 4;
 
 // Shared memory of a call's blocks, in bytes from the start (every part on a 16-byte boundary), and what else follows from
-// the sizes.  A token's positions are counted by groups of 1 << log_group neighbours: group n_q * groups, token after token,
-// belongs to copying block group % copying, whose (group / copying)-th it is; the block counts its own positions through.
+// the sizes.  Rows that are asked for early: a token's positions are counted by groups of 1 << log_group neighbours: group
+// n_q * groups, token after token, belongs to copying block group % copying, whose (group / copying)-th it is; the block counts
+// its own positions through.
 struct StepLayout {
     uint32_t log_group, groups;          // groups of a token
     uint32_t local;                      // positions that a copying block has room for
-    uint32_t by_copying, by_groups;      // n / copying == n * by_copying >> 18 for every group; the same for groups
-    uint32_t per_lane, per_token;        // words of 32 local positions to a lane; of a token's positions, a block's at most
+    uint32_t by_copying, by_groups;      // n / copying == n * by_copying >> 18 for every group and position; the same for groups
+    uint32_t per_lane, per_token;        // words of 32 local positions to a lane; entries of a token in a block's list, at most
     uint32_t log_heads, nil;             // chains of the index; its closing node
     uint32_t log_seen, log_asked;        // words of the copying blocks' sets: cached ids; ids of an earlier token, each
-    uint32_t early;                      // the copying blocks have them
     uint32_t node, head, life, bits, tot, ndead, cnt, sum, votes, miss, pos, dead, ids;    // first block
     uint32_t seen, asked, slots, id, mask, rest, list, their_ids;              // copying blocks
     uint32_t total;
 };
-StepLayout step_layout(uint32_t S, uint32_t K, uint32_t n_q, uint32_t nt, uint32_t copying, uint32_t row_bytes, bool host_ids)
+// ask: rows are asked for early.  False if there is no room for that (without it there always is).
+bool step_layout(StepLayout& o, uint32_t S, uint32_t K, uint32_t n_q, uint32_t nt, uint32_t copying, bool host_ids, bool ask)
 {
-    StepLayout o;
     // At least 32 groups a token, so that seven blocks have about the same to do: 9 tables with K = 256 30.8 us with groups of
     // 32 positions, 27.5 with rows handed out in turn.  Larger ones are loaded in longer pieces.
     o.log_group = 5u;
     while (o.log_group && K >> o.log_group < 32u) --o.log_group;
     o.groups = (K + (1u << o.log_group) - 1u) >> o.log_group;
-    o.local = (((n_q * o.groups + copying - 1u) / copying << o.log_group) + 31u) & ~31u;
+    o.local = ask ? (((n_q * o.groups + copying - 1u) / copying << o.log_group) + 31u) & ~31u : 0u;
     o.by_copying = (1u << 18) / copying + 1u;
     o.by_groups = (1u << 18) / o.groups + 1u;
     o.per_lane = (o.local / 32u + 31u) / 32u;
-    o.per_token = (o.groups + copying - 1u) / copying << o.log_group;
+    o.per_token = ask ? (o.groups + copying - 1u) / copying << o.log_group : 1u + (K + copying - 1u) / copying;
     o.nil = S + (n_q - 1u) * K;
     o.log_heads = 1u;
     while ((1u << o.log_heads) < 2u * S) ++o.log_heads;
     o.log_seen = o.log_heads;                              // 64 bits an id
     o.log_asked = 2u;
     while ((1u << o.log_asked) < 2u * K) ++o.log_asked;
-    o.early = row_bytes <= 16u * ROW_CHUNKS;
-    const uint32_t ids = host_ids ? align16(n_q * K * 4u) : 0u, room = (228u << 10) / (1024u / nt) - 2560u;
+    const uint32_t ids = ask && host_ids ? align16(n_q * K * 4u) : 0u, room = (228u << 10) / (1024u / nt) - 2560u;
     for (;;) {
         uint32_t a = 0;
         o.node = a;    a += align16((o.nil + 1u) * 8u);
@@ -73,30 +80,31 @@ StepLayout step_layout(uint32_t S, uint32_t K, uint32_t n_q, uint32_t nt, uint32
         o.ndead = a;   a += 2u * 32u * 4u;                 // warps' dead slots, by parity
         o.cnt = a;     a += 2u * 2u * 32u * 4u;            // warps' counts of the decay search, by parity
         o.sum = a;     a += 16u;                           // valid ids of the call
-        o.votes = a;   a += align16((K + 31u) / 32u * 4u);  // the token's misses, a bit per position
+        o.votes = a;   a += ask ? align16((K + 31u) / 32u * 4u) : 0u;      // the token's misses, a bit per position
         o.miss = a;    a += align16(K * 4u);               // misses in position order: ids,
         o.pos = a;     a += align16(K * 2u);               //   positions
         o.dead = a;    a += align16(K * 2u);               // dead slots in slot order
         o.ids = a;     a += ids;                           // received: the ids of a call with host buffers
         const uint32_t first = a;
         a = 0;
-        o.seen = a;    a += o.early ? 4u << o.log_seen : 0u;
-        o.asked = a;   a += o.early ? (n_q - 1u) * 4u << o.log_asked : 0u;
+        o.seen = a;    a += ask ? 4u << o.log_seen : 0u;
+        o.asked = a;   a += ask ? (n_q - 1u) * 4u << o.log_asked : 0u;
         o.slots = a;   a += o.local * 4u;                  // received: what has become of a position
         o.id = a;      a += o.local * 4u;                  // its id
         o.mask = a;    a += align16(o.local / 32u * 4u);   // positions whose rows are asked for early
         o.rest = a;    a += align16(o.local / 32u * 4u);   //   but not by the warp that has found them
-        o.list = a;    a += align16(n_q * o.per_token * 8u);   // received: a token's misses in the block's positions {position, slot}
-        o.their_ids = a; a += ids;                         // received: the ids of a call with host buffers, but others' last token's
+        o.list = a;    a += align16(n_q * o.per_token * 8u);   // received: a token's misses in the block's positions {place, slot}; or
+                                                           //   a head {rows, first shared} and the rows that it copies {id, slot}
+        o.their_ids = a; a += ids;                         // received: the ids of a call with host buffers
         o.total = first > a ? first : a;
-        if (o.total <= room) return o;
-        if (o.early && a > room) o.early = 0;              // no rows early, longer chains where the rest needs the room
-        else if ((1u << o.log_heads) > S) --o.log_heads;
-        else return o;
+        if (o.total <= room) return true;
+        if (ask && a > room) return false;
+        if ((1u << o.log_heads) <= S) return !ask;
+        --o.log_heads;                                     // longer chains where the rest needs the room
     }
 }
 constexpr uint32_t NO_ITEM = 0xFFFFFFFFu;
-constexpr uint32_t NOT_MISSED = 0xFFFFFFFFu, NO_SLOT = 0xFFFFu;        // of a position; else its slot, and << 16 its rank among the token's misses
+constexpr uint32_t NOT_MISSED = 0xFFFFFFFFu, NO_SLOT = 0xFFFFu;        // of a position; else its slot
 
 __device__ __forceinline__ bool wait_for(uint32_t mbar, uint32_t limit)
 {
@@ -105,61 +113,82 @@ __device__ __forceinline__ bool wait_for(uint32_t mbar, uint32_t limit)
     return __all_sync(0xffffffffu, spin < limit);
 }
 
-// What the copying blocks are told of a token: `to` of them that it has n misses in the block's positions, and from which row on
-// they are shared (SHARE); of a miss, the block that the position i belongs to the slot, where the position's place is and in
-// the next entry of its list.
+// What the copying blocks are told.  Where they ask for rows early: `token`, that block `to` has n misses in its positions; `miss`,
+// to the block that position i belongs to, the slot, where the position's place is and in the next entry of its list.  Where
+// they don't, the rows to copy, in the order of the misses: in turn, or (share) `share` neighbours to a block; `head`, how many of n
+// they are, and the first one's number among those that are shared (-1: none are); `row`, the k-th.
 struct Tell {
     const StepLayout& lay;
-    uint32_t copying, smem, mbar, sent, first;           // of the first block's own: the same places as in the others
+    uint32_t copying, smem, mbar, sent;                  // of the first block's own: the same places as in the others
 
-    template <bool SHARE>
-    __device__ __forceinline__ void token(uint32_t g, uint32_t to, uint32_t n, uint32_t first_shared) const
+    __device__ __forceinline__ void token(uint32_t g, uint32_t to, uint32_t n) const
     {
         const uint32_t bar = map_rank(mbar + 8u * g, to + 1u);
         send_async(map_rank(sent + 4u * g, to + 1u), n, bar);
-        if (SHARE) send_async(map_rank(first + 4u * g, to + 1u), first_shared, bar);
-        arrive_expect(bar, 12u * n + (SHARE ? 8u : 4u));
+        arrive_expect(bar, 12u * n + 4u);
     }
     // own: the misses of the token that the blocks have been told of
-    __device__ __forceinline__ void miss(uint32_t g, uint32_t i, uint32_t what, uint32_t* own) const
+    __device__ __forceinline__ void miss(uint32_t g, uint32_t i, uint32_t j, uint32_t* own) const
     {
         const uint32_t group = g * lay.groups + (i >> lay.log_group), at = group * lay.by_copying >> 18, to = group - at * copying;
         const uint32_t n = (at << lay.log_group) + (i & ((1u << lay.log_group) - 1u)), bar = map_rank(mbar + 8u * g, to + 1u);
-        send_async(map_rank(smem + lay.slots + 4u * n, to + 1u), what, bar);
+        send_async(map_rank(smem + lay.slots + 4u * n, to + 1u), j, bar);
         const uint32_t e = atomicAdd(own + to, 1u);
-        send_async(map_rank(smem + lay.list + 8u * (g * lay.per_token + e), to + 1u), (int32_t)n, (int32_t)what, bar);
+        send_async(map_rank(smem + lay.list + 8u * (g * lay.per_token + e), to + 1u), (int32_t)n, (int32_t)j, bar);
+    }
+    __device__ __forceinline__ void head(uint32_t g, uint32_t to, uint32_t n, uint32_t share, int32_t first) const
+    {
+        const uint32_t rows = share == 0 ? (n + copying - 1u - to) * lay.by_copying >> 18
+                              : to * share >= n ? 0u : n - to * share < share ? n - to * share : share;
+        const uint32_t bar = map_rank(mbar + 8u * g, to + 1u);
+        send_async(map_rank(smem + lay.list + 8u * g * lay.per_token, to + 1u), (int32_t)rows, first, bar);
+        arrive_expect(bar, 8u * (rows + 1u));
+    }
+    __device__ __forceinline__ void row(uint32_t g, uint32_t k, uint32_t share, int32_t x, int32_t j) const
+    {
+        const uint32_t q = share ? k / share : k * lay.by_copying >> 18, r = k - q * (share ? share : copying);
+        const uint32_t to = share ? q : r, at = share ? r : q;
+        send_async(map_rank(smem + lay.list + 8u * (g * lay.per_token + 1u + at), to + 1u), x, j, map_rank(mbar + 8u * g, to + 1u));
     }
 };
 
-// A call with lifetimes above L on entry: the copying blocks hear of all tokens when the last one is placed, and only of
-// rows that their slots still wait for.  list: {id, slot | position << 13 | token << 26}.  (Inline: a function call in the kernel
-// brings every call's row loads late; 8 new requests 265 us and not 257.)
-template <bool SHARE>
-__device__ __forceinline__ void tell_at_last(const Tell tell, uint32_t n_q, int2* list, uint32_t count, const uint2* s_node, uint32_t* s_own)
+// A call with lifetimes above L on entry: the copying blocks hear of all tokens when the last one is placed, and only of rows that
+// their slots still wait for.  list: {id, slot | position << 13 | token << 26}.  (Inline: a function call in the kernel brings every
+// call's row loads late; 8 new requests 265 us and not 257.)
+template <bool ASK>
+__device__ __forceinline__ void tell_at_last(const Tell tell, uint32_t n_q, uint32_t K, int2* list, uint32_t count, const uint2* s_node, uint32_t* s_own)
 {
+    constexpr uint32_t MASK = (1u << LIST_SLOT_BITS) - 1u;
     static_assert(STEP_MAX_TOKENS <= 1u << (32u - 2u * LIST_SLOT_BITS), "a token does not fit an entry");
     drop_lost_rows(list, count, s_node);
     for (uint32_t g = 0; g < n_q; ++g) {
-        if (threadIdx.x < STEP_FEW_CLUSTER) s_own[threadIdx.x] = 0;
-        __syncthreads();
-        for (uint32_t e = threadIdx.x; e < count; e += blockDim.x) {
-            const int2 v = list[e];
-            const uint32_t what = (uint32_t)v.y, mask = (1u << LIST_SLOT_BITS) - 1u;
-            if (v.x >= 0 && what >> (2u * LIST_SLOT_BITS) == g) tell.miss(g, what >> LIST_SLOT_BITS & mask, what & mask, s_own);
+        if constexpr (ASK) {
+            if (threadIdx.x < STEP_FEW_CLUSTER) s_own[threadIdx.x] = 0;
+            __syncthreads();
+            for (uint32_t e = threadIdx.x; e < count; e += blockDim.x) {
+                const int2 v = list[e];
+                const uint32_t what = (uint32_t)v.y;
+                if (v.x >= 0 && what >> (2u * LIST_SLOT_BITS) == g) tell.miss(g, what >> LIST_SLOT_BITS & MASK, what & MASK, s_own);
+            }
+            __syncthreads();
+            if (threadIdx.x < tell.copying) tell.token(g, threadIdx.x, s_own[threadIdx.x]);
+            __syncthreads();
+        } else {                                         // (K entries at a time, whatever token they are of)
+            const uint32_t from = g * K, n = count <= from ? 0u : count - from < K ? count - from : K;
+            if (g == 0) __syncthreads();                 // (lost rows are marked)
+            if (threadIdx.x < tell.copying) tell.head(g, threadIdx.x, n, 0u, -1);
+            for (uint32_t k = threadIdx.x; k < n; k += blockDim.x) tell.row(g, k, 0u, list[from + k].x, (int32_t)((uint32_t)list[from + k].y & MASK));
         }
-        __syncthreads();
-        if (threadIdx.x < tell.copying) tell.token<SHARE>(g, threadIdx.x, s_own[threadIdx.x], ~0u);
-        __syncthreads();
     }
 }
 
 // The first block of a cluster: Stage One.  SPT slots per thread (a power of two): S <= SPT * blockDim.x.  IPT: the most
 // ids a thread has of a token (K <= S, so SPT is always enough).  a_mbar: the copying blocks' mbarriers, one per token.
-// The passes are those of avsg_stage_one_kernel, which says what they are and why.  SHARE: rows of a table with very many
-// misses may be copied by other tables' blocks; a_first: where the copying blocks hear of the token's first row among them.
-template <int SPT, int IPT, bool SHARE, int CAP>
+// The passes are those of avsg_stage_one_kernel, which says what they are and why.  ASK: rows are asked for early.  SHARE: rows of a
+// table with very many misses may be copied by other tables' blocks.
+template <int SPT, int IPT, bool ASK, bool SHARE, int CAP>
 __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const StepLayout& lay, const uint32_t ti, const uint32_t copying,
-                                             unsigned char* smem, const uint32_t a_mbar, const uint32_t a_sent, const uint32_t a_first, uint32_t* s_own)
+                                             unsigned char* smem, const uint32_t a_mbar, const uint32_t a_sent, uint32_t* s_own)
 {
     constexpr int NV = (SPT + 3) / 4;                    // 4-slot vectors of ids / words of lifetimes per thread
     const uint32_t S = p.S, K = p.K, L = p.L, NIL = lay.nil;
@@ -194,7 +223,8 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
         const int32_t* ids = p.indices + ((size_t)ti * p.n_q + g) * K;
 #pragma unroll
         for (int k = 0; k < IPT; ++k)
-            xs[k] = i0 + 32u * k < i1 ? (p.host_ids ? s_ids[g * K + i0 + 32u * k] : __ldcg(ids + i0 + 32u * k)) : -1;
+            xs[k] = i0 + 32u * k >= i1 ? -1 : !p.host_ids ? __ldcg(ids + i0 + 32u * k)
+                    : ASK ? s_ids[g * K + i0 + 32u * k] : __ldcv(ids + i0 + 32u * k);
     };
     // the clearing comes before the wait: under the previous kernel's tail
     const uint32_t table = p.table_id[ti], id_limit = p.id_limit[ti];
@@ -202,7 +232,10 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
     for (uint32_t i = tid; i < (1u << lay.log_heads) / 4; i += nt) reinterpret_cast<uint4*>(s_head)[i] = make_uint4(NIL, NIL, NIL, NIL);
     if (tid == 0) s_node[NIL] = make_uint2(0xFFFFFFFEu, NIL);          // an id that nobody looks for
     if (tid == 0) s_sum[0] = 0;
-    if (tid < 2u * STEP_FEW_CLUSTER) s_own[tid] = 0;
+    if (ASK && tid < 2u * STEP_FEW_CLUSTER) s_own[tid] = 0;
+    // Ids in host memory are there when the call is made, and nothing on the device writes them: a call that queues behind another
+    // fetches its first ones while that one's rows travel (32 tables: 5 us of link time and a round trip).
+    if (!ASK && p.host_ids) load_token(0);
 
     // Programmatic dependent launch: this grid may have been started while the previous kernel of the stream
     // was still running; nothing that the device writes is read before that kernel has completed.
@@ -236,7 +269,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
         w[q] = decay4(w[q], 1);
     }
     store_lifetimes<SPT>(s_life, s_bits, s_ndead, own, w);
-    if (p.host_ids) {
+    if (ASK && p.host_ids) {
         cluster_sync();                                  // (the copying blocks have sent the ids)
         load_token(0);
     }
@@ -245,7 +278,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
     uint32_t list_off = 0, sum_miss = 0, sum_decay = 0, valid = 0;
     uint32_t shared = 0;                                 // SHARE: rows that other blocks may take (bit 31: there will be some)
     int2* list = p.miss_list + (size_t)ti * p.list_stride;
-    const Tell tell = {lay, copying, smem_u32(smem), a_mbar, a_sent, a_first};
+    const Tell tell = {lay, copying, smem_u32(smem), a_mbar, a_sent};
 
     for (uint32_t g = 0; g < p.n_q; ++g) {
         const bool last = g + 1 == p.n_q;
@@ -283,7 +316,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
             const uint32_t votes = __ballot_sync(0xffffffffu, miss);
             rank[k] = wmiss + __popc(votes & below);                   // within the warp, in position order
             wmiss += __popc(votes);
-            if (lane == 0 && i0 + 32u * k < i1) s_votes[warp * ipt + k] = votes;
+            if (ASK && lane == 0 && i0 + 32u * k < i1) s_votes[warp * ipt + k] = votes;
             missing |= miss ? 1u << k : 0u;
             if (slot[k] >= 0) s_life[slot[k]] = (int8_t)L;
             if (store) O[i0 + 32u * k] = slot[k];
@@ -330,7 +363,6 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
             }
         }
         if (!last) load_token(g + 1);                                      // arrives while this token's misses are placed
-        const uint32_t group0 = g * lay.groups, in_group = (1u << lay.log_group) - 1u;
         // Pass 3, the while-loop of Alg. 1: decay until n_g slots are dead
         if (dtotal < n_g) {
             life_words<SPT>(s_life + j0, own, w);
@@ -344,7 +376,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
             dtotal = __reduce_add_sync(0xffffffffu, t);
             if (dtotal < n_g && tid == 0) atomicOr(p.status, ST_NO_DEAD_SLOTS);
         }
-        if (tid < STEP_FEW_CLUSTER) s_own[(~g & 1u) * STEP_FEW_CLUSTER + tid] = 0;         // for the next token
+        if (ASK && tid < STEP_FEW_CLUSTER) s_own[(~g & 1u) * STEP_FEW_CLUSTER + tid] = 0;         // for the next token
         const uint32_t n_take = n_g < dtotal ? n_g : dtotal;
         if (dead_before < n_take) {                      // some of the first n_g dead slots are this warp's
             uint32_t bits = s_bits[tid], r, unused;
@@ -357,16 +389,24 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
         if (lane == 0) s_ndead[32u - par + warp] = left;
         __syncthreads();
 
-        for (uint32_t to = nw - 1u - warp; to < copying && !unusual; to += nw) {       // what a copying block gets of this token (the first warps install)
-            // (its first group is the first one that is `to` modulo copying)
-            uint32_t group = (group0 * lay.by_copying >> 18) * copying + to, n = 0;
-            if (group < group0) group += copying;
-            for (uint32_t q = group - group0 + lane * copying; n_g && q < lay.groups; q += 32u * copying) {
-                const uint32_t i = q << lay.log_group;
-                n += __popc(s_votes[i / 32u] >> i % 32u & ~(~1u << in_group));
+        // a copying block's rows, where none are asked for early: in turn where few tables have eight blocks each, and where other
+        // blocks may take some (so that what is left is at the end), else a share in position order
+        const uint32_t share = CAP == STEP_FEW_TABLES || share_it ? 0u : (n_take + copying - 1u) / copying;
+        if constexpr (ASK) {
+            const uint32_t group0 = g * lay.groups, in_group = (1u << lay.log_group) - 1u;
+            for (uint32_t to = nw - 1u - warp; to < copying && !unusual; to += nw) {       // what a copying block gets of this token (the first warps install)
+                // (its first group is the first one that is `to` modulo copying)
+                uint32_t group = (group0 * lay.by_copying >> 18) * copying + to, n = 0;
+                if (group < group0) group += copying;
+                for (uint32_t q = group - group0 + lane * copying; n_g && q < lay.groups; q += 32u * copying) {
+                    const uint32_t i = q << lay.log_group;
+                    n += __popc(s_votes[i / 32u] >> i % 32u & ~(~1u << in_group));
+                }
+                n = __reduce_add_sync(0xffffffffu, n);
+                if (lane == 0) tell.token(g, to, n);
             }
-            n = __reduce_add_sync(0xffffffffu, n);
-            if (lane == 0) tell.token<SHARE>(g, to, n, share_it ? shared & ~SHARED_COMING : ~0u);
+        } else if (tid < copying && !unusual) {
+            tell.head(g, tid, n_take, share, share_it ? (int32_t)((shared & ~SHARED_COMING) + tid) : -1);
         }
 
         // ---- install: the k-th miss in position order takes the k-th dead slot ----
@@ -374,10 +414,12 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
             const uint32_t i = s_pos[k];
             const int32_t x = s_miss[k];
             const int32_t j = k < n_take ? s_dead[k] : -1;
-            if (!unusual) {
-                tell.miss(g, i, ((uint32_t)j & 0xFFFFu) | k << 16, s_own + (g & 1u) * STEP_FEW_CLUSTER);
+            if (unusual) {
+                if (k < n_take) list[list_off + k] = make_int2(x, (int32_t)((uint32_t)j | i << LIST_SLOT_BITS | g << (2u * LIST_SLOT_BITS)));
+            } else if constexpr (ASK) {
+                tell.miss(g, i, (uint32_t)j & 0xFFFFu, s_own + (g & 1u) * STEP_FEW_CLUSTER);
             } else if (k < n_take) {
-                list[list_off + k] = make_int2(x, (int32_t)((uint32_t)j | i << LIST_SLOT_BITS | g << (2u * LIST_SLOT_BITS)));
+                tell.row(g, k, share, x, j);
             }
             if (k < n_take) {
                 s_node[j].x = (uint32_t)x;
@@ -398,7 +440,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
         __syncthreads();
         announce_token(p, ti, g, n_take);
     }
-    if (unusual) tell_at_last<SHARE>(tell, p.n_q, list, list_off, s_node, s_own);
+    if (unusual) tell_at_last<ASK>(tell, p.n_q, K, list, list_off, s_node, s_own);
     if (SHARE && shared && tid == 0) {
         __threadfence();
         *reinterpret_cast<volatile uint32_t*>(&p.shared[ti].rows) = shared == SHARED_COMING ? 0u : shared ^ (SHARED_COMING | SHARED_OPEN);
@@ -452,24 +494,23 @@ __device__ __forceinline__ bool set_has(const uint32_t* set, uint32_t log_words,
     return (~set[hash_id(x, log_words)] & set_bits(x)) == 0;
 }
 
-// A row that a copying block owes: the position in the block's own count, and the token.
-struct Item { uint32_t n, g; };
+// A row that a copying block owes: the position in the block's own count, the token, the id.
+struct Item { uint32_t n, g, x; };
 
 // A copying block finds out which of its positions are missed for certain: their ids are in no slot and in no earlier token
 // of the call.  What it does not find so (an id that seems to be in a set; a resident one that loses its slot to an earlier
-// token) is news from the first block.  The first row that a warp finds is on its way when this returns (`item`, `row`), the
-// others are left in lay.rest, in position order, token after token.
+// token) is news from the first block.  The first that a warp finds is its own to ask for, and returned; the others are left in
+// lay.rest, in position order, token after token (for the other warps behind a barrier).
 // What takes the time is instruction issue and bank conflicts for 32 warps.  From the call's start, 32 tables of 8192 slots,
 // K = 2048, two tokens, three copying blocks: ids and cached ids are loaded after 2.9 us, the sets are there after 3.9, the first
 // rows are asked for after 4.7, where rows that wait for their slots are asked for after 6.5.  Other ways to know: a chained index
 // like Stage One's 5.9 us; the block's positions in a chained index, and the cached ids looked up in that, 7.1 to 8.
 template <int SPT, int IPT, int CAP>
-__device__ __forceinline__ void match(const S1ParamsT<CAP>& p, const StepLayout& lay, const uint32_t ti, const uint32_t rank,
-                                          const uint32_t copying, unsigned char* smem, const uint64_t src, const uint64_t stride,
-                                          Row& row, Item& item)
+__device__ __forceinline__ Item match(const S1ParamsT<CAP>& p, const StepLayout& lay, const uint32_t ti, const uint32_t rank,
+                                      const uint32_t copying, unsigned char* smem)
 {
     constexpr int NV = (SPT + 3) / 4, OWN = 4;           // of its positions a warp takes OWN times 32 at a time
-    const uint32_t S = p.S, K = p.K, id_limit = p.id_limit[ti], cpr = p.row_bytes >> 4;
+    const uint32_t S = p.S, K = p.K, id_limit = p.id_limit[ti];
     const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u, warp = tid >> 5, W = nt >> 5;
     uint32_t* s_seen = reinterpret_cast<uint32_t*>(smem + lay.seen);
     uint32_t* s_asked = reinterpret_cast<uint32_t*>(smem + lay.asked);
@@ -482,8 +523,7 @@ __device__ __forceinline__ void match(const S1ParamsT<CAP>& p, const StepLayout&
 
     auto id_at = [&](uint32_t i) -> int32_t { return p.host_ids ? s_ids[i] : __ldcg(g_ids + i); };
 
-    if (lay.early)
-        for (uint32_t i = tid; i < (lay.slots - lay.seen) / 16u; i += nt) reinterpret_cast<uint4*>(s_seen)[i] = make_uint4(0, 0, 0, 0);
+    for (uint32_t i = tid; i < (lay.slots - lay.seen) / 16u; i += nt) reinterpret_cast<uint4*>(s_seen)[i] = make_uint4(0, 0, 0, 0);
     if (p.host_ids) {
         // Ids in host memory are there when the call is made, and nothing on the device writes them: a call that queues
         // behind another fetches its first ones while that one's rows travel.  The copying blocks share the reading, and
@@ -520,7 +560,7 @@ __device__ __forceinline__ void match(const S1ParamsT<CAP>& p, const StepLayout&
     const int4* g_tok = reinterpret_cast<const int4*>(p.tok + (size_t)p.table_id[ti] * S);
 #pragma unroll
     for (int q = 0; q < NV; ++q)
-        if (lay.early && tid + q * nt < S / 4) t4[q] = __ldcg(g_tok + tid + q * nt);
+        if (tid + q * nt < S / 4) t4[q] = __ldcg(g_tok + tid + q * nt);
     auto load_own = [&](uint32_t from) {
 #pragma unroll
         for (int m = 0; m < OWN; ++m) {
@@ -537,28 +577,25 @@ __device__ __forceinline__ void match(const S1ParamsT<CAP>& p, const StepLayout&
         for (int k = 0; k < IPT; ++k)
             if (tid + k * nt < K) xe[k] = id_at(g * K + tid + k * nt);
     };
-    if (lay.early && p.n_q > 1u) load_earlier(0);
+    if (p.n_q > 1u) load_earlier(0);
     load_own(0);
-    if (lay.early) {
-        __syncthreads();                                 // the sets are empty
+    __syncthreads();                                 // the sets are empty
 #pragma unroll
-        for (int q = 0; q < NV; ++q)
-            if (tid + q * nt < S / 4) {                  // (not those of empty slots: a word that all add to takes 4 us)
-                if (t4[q].x >= 0) set_add(s_seen, lay.log_seen, t4[q].x);
-                if (t4[q].y >= 0) set_add(s_seen, lay.log_seen, t4[q].y);
-                if (t4[q].z >= 0) set_add(s_seen, lay.log_seen, t4[q].z);
-                if (t4[q].w >= 0) set_add(s_seen, lay.log_seen, t4[q].w);
-            }
-        for (uint32_t g = 0; g + 1u < p.n_q; ++g) {
-#pragma unroll
-            for (int k = 0; k < IPT; ++k)
-                if (tid + k * nt < K && xe[k] >= 0) set_add(s_asked + g * asked_words, lay.log_asked, xe[k]);
-            if (g + 2u < p.n_q) load_earlier(g + 1u);
+    for (int q = 0; q < NV; ++q)
+        if (tid + q * nt < S / 4) {                  // (not those of empty slots: a word that all add to takes 4 us)
+            if (t4[q].x >= 0) set_add(s_seen, lay.log_seen, t4[q].x);
+            if (t4[q].y >= 0) set_add(s_seen, lay.log_seen, t4[q].y);
+            if (t4[q].z >= 0) set_add(s_seen, lay.log_seen, t4[q].z);
+            if (t4[q].w >= 0) set_add(s_seen, lay.log_seen, t4[q].w);
         }
-        __syncthreads();
+    for (uint32_t g = 0; g + 1u < p.n_q; ++g) {
+#pragma unroll
+        for (int k = 0; k < IPT; ++k)
+            if (tid + k * nt < K && xe[k] >= 0) set_add(s_asked + g * asked_words, lay.log_asked, xe[k]);
+        if (g + 2u < p.n_q) load_earlier(g + 1u);
     }
-    item.n = NO_ITEM;
-    uint32_t first = 0;
+    __syncthreads();
+    Item item = {NO_ITEM, 0u, 0u};
     for (uint32_t from = 0; from * 32u < mine; from += OWN * W) {
         if (from) load_own(from);
 #pragma unroll
@@ -567,22 +604,20 @@ __device__ __forceinline__ void match(const S1ParamsT<CAP>& p, const StepLayout&
             if (word * 32u >= mine) break;
             const uint32_t g = place(lay, rank, copying, n).g;
             const int32_t x = xo[m];
-            bool certain = lay.early && (uint32_t)x < id_limit && !set_has(s_seen, lay.log_seen, x);
+            bool certain = (uint32_t)x < id_limit && !set_has(s_seen, lay.log_seen, x);
             for (uint32_t e = 0; e < g && certain; ++e) certain = !set_has(s_asked + e * asked_words, lay.log_asked, x);
             const uint32_t votes = __ballot_sync(0xffffffffu, certain);
             s_id[n] = x;
             uint32_t rest = votes;
             if (votes && item.n == NO_ITEM) {
                 const uint32_t l = __ffs((int)votes) - 1u;
-                item = {word * 32u + l, __shfl_sync(0xffffffffu, g, (int)l)};
-                first = (uint32_t)__shfl_sync(0xffffffffu, x, (int)l);
+                item = {word * 32u + l, __shfl_sync(0xffffffffu, g, (int)l), (uint32_t)__shfl_sync(0xffffffffu, x, (int)l)};
                 rest &= rest - 1u;
             }
             if (lane == 0) { s_mask[word] = votes; s_rest[word] = rest; }
         }
     }
-    if (item.n != NO_ITEM) load_row(row, src + (uint64_t)first * stride, cpr, lane);
-    __syncthreads();
+    return item;
 }
 
 __device__ __forceinline__ SharedRows read_shared(const SharedRows* at)
@@ -641,14 +676,16 @@ __device__ __forceinline__ void take_shared_rows(const S1ParamsT<CAP>& p, const 
 //   K = 256, S = 1024, one table 8.4 / 5.8;  K = 2048, S = 8192, two tokens, one table 17.2 / 12.2, from a graph 19.8 / 18.3;
 //   the same with 4, 8, 16, 32, 48, 64 tables 26.2 / 22.4, 39.0 / 35.6, 65.9 / 63.6, 119.9 / 116.8, 174.0 / 173.6, 228.3 / 226.8;
 //   the same from 11 GB of host memory with 8, 16, 32, 48, 64 tables 51 / 46, 88 / 84, 173 / 155, 242 / 229, 315 / 296.
-// Asked for at once, before / now: one table 12.4 / 11.1, 8 tables with K = 1000 and 1152-byte rows 35.3 / 33.7, 32 tables 119.1 /
-// 116.9, 16 from 11 GB 84.4 / 82.5.  A call that keeps selecting what it has just lost gains nothing (S = 1024, three tokens of K = 196: 12.6 / 13.8).
+// Asked for at once, before / now: one table 12.9 / 11.5, 8 tables with K = 1000 and 1152-byte rows 36.9 / 34.9, 32 tables 120.5 /
+// 117.6, 16 from 11 GB 85.7 / 83.3, 8 new requests 260.4 / 257.1; 20 tables of S = 2048, K = 512 36.7 / 36.3.
 // The line of 11 GB is what the end of a call is for.  Where a table's pages are spread over much host memory, translating
 // their addresses limits the rows, and a cluster, which lies in one GPC, finds its table's translations there if the
 // table was there in the call before.  So calls of more than a few tables let the next grid start only when their
 // blocks exit: its clusters then find the same SMs free, in the same order.  Started early they take whatever is free at
 // that time: eight tables 60 us and not 46, 16 113 and not 84 (step_early() says which calls gain by it).
 // The warps of a block take its rows from a counter, in position order, so that neighbours in host memory go together.
+// (Asked for early, such clusters leave 64 unequal requests at 330 us and not 333, but rows taken by others are then spread over
+// all positions: one cold table of 64, the others with hits only, 67 us with 656-byte rows and not 62, 138 with 1552 and not 100.)
 // SHARE (two and three blocks).  A cluster alone cannot fill the link with one table's rows where it has few copying blocks (an
 // SM gets 20 of them a us, the link carries 72), so a new request among steady ones would be left behind: 64 tables, one of
 // them cold, 332 us against 277 in two kernels, whose rows are cut evenly over all SMs (Eq. 6).  So a table that misses more
@@ -663,31 +700,37 @@ __device__ __forceinline__ void take_shared_rows(const S1ParamsT<CAP>& p, const 
 // one, its own blocks' too, the cold calls were quicker still (45 tables 214), but a call where most tables had many misses
 // lost 5 to 20 %: the requests for claims and list entries wait behind the rows'.  Several rows of a warp at once bring an SM
 // from 20 rows a us to 28 at most.
-template <int SPT, int IPT, int CAP, bool SHARE = false>
+template <int SPT, int IPT, int CAP, bool ASK, bool SHARE>
 __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constant__ S1ParamsT<CAP> p, const __grid_constant__ StepLayout lay)
 {
+    static_assert(!ASK || !SHARE, "rows that are shared are copied in the order of the misses");
+    constexpr bool FEW = CAP == STEP_FEW_TABLES;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ __align__(8) unsigned long long s_mbar[STEP_MAX_TOKENS];
-    __shared__ uint32_t s_sent[STEP_MAX_TOKENS];                       // received: a token's misses in the block's positions
+    __shared__ __align__(8) unsigned long long s_mbar[STEP_MAX_TOKENS], s_meet[ASK || FEW ? 1 : STEP_MAX_TOKENS];
+    __shared__ uint32_t s_sent[ASK ? STEP_MAX_TOKENS : 1];             // received: a token's misses in the block's positions
     __shared__ uint32_t s_own[2 * STEP_FEW_CLUSTER];                   // first block: of those, how many it has sent, by parity of the token
-    __shared__ uint32_t s_first[SHARE ? STEP_MAX_TOKENS : 1];          // received: the token's first row among those that are shared; -1
-    __shared__ uint32_t s_next;                                        // of the listed rows, the first that no warp has taken
+    __shared__ uint32_t s_next;                                        // of the rows to be asked for, the first that no warp has taken
     __shared__ volatile uint32_t s_mine;                               // rows that are shared: the first that others have taken
-    const uint32_t rank = cluster_rank(), cluster = cluster_size(), copying = cluster - 1u;
+    const uint32_t rank = cluster_rank(), cluster = !ASK && FEW ? STEP_FEW_CLUSTER : cluster_size(), copying = cluster - 1u;
     const uint32_t ti = blockIdx.x / cluster, lane = threadIdx.x & 31u, W = blockDim.x >> 5, warp = threadIdx.x >> 5;
     uint32_t* s_slots = reinterpret_cast<uint32_t*>(smem + lay.slots);
     if (p.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (SHARE && threadIdx.x == 0) s_mine = 0xFFFFFFFFu;
     if (rank != 0) {
-        if (threadIdx.x == 0) s_next = 0;
-        if (threadIdx.x < p.n_q) mbar_init(smem_u32(s_mbar + threadIdx.x), 1u);
-        for (uint32_t i = threadIdx.x; i < lay.local; i += blockDim.x) s_slots[i] = NOT_MISSED;
-        for (uint32_t i = threadIdx.x; i < lay.local / 32u; i += blockDim.x) reinterpret_cast<uint32_t*>(smem + lay.rest)[i] = 0;
+        if (threadIdx.x < p.n_q) {
+            mbar_init(smem_u32(s_mbar + threadIdx.x), 1u);
+            if (!ASK && !FEW) mbar_init(smem_u32(s_meet + threadIdx.x), W);
+        }
+        if constexpr (ASK) {
+            if (threadIdx.x == 0) s_next = 0;
+            for (uint32_t i = threadIdx.x; i < lay.local; i += blockDim.x) s_slots[i] = NOT_MISSED;
+            for (uint32_t i = threadIdx.x; i < lay.local / 32u; i += blockDim.x) reinterpret_cast<uint32_t*>(smem + lay.rest)[i] = 0;
+        }
     }
     __syncthreads();
     cluster_arrive();
     if (rank == 0) {
-        place_tokens<SPT, IPT, SHARE>(p, lay, ti, copying, smem, smem_u32(s_mbar), smem_u32(s_sent), smem_u32(s_first), s_own);
+        place_tokens<SPT, IPT, ASK, SHARE>(p, lay, ti, copying, smem, smem_u32(s_mbar), smem_u32(s_sent), s_own);
         __syncwarp();
         cluster_arrive();                                              // the outputs are written, everything is sent
         return;
@@ -695,32 +738,24 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
     const uint32_t cpr = p.row_bytes >> 4;
     const uint64_t src = p.kv_base[ti], stride = p.kv_stride[ti];
     const uint64_t dst = reinterpret_cast<uint64_t>(p.buffer + (size_t)p.table_id[ti] * p.S * p.row_bytes);
-    Row row;
-    Item item;
-    match<SPT, IPT>(p, lay, ti, rank, copying, smem, src, stride, row, item);
-    const int32_t* s_id = reinterpret_cast<const int32_t*>(smem + lay.id);
-    const uint32_t* s_mask = reinterpret_cast<const uint32_t*>(smem + lay.mask);
-    const uint32_t* s_rest = reinterpret_cast<const uint32_t*>(smem + lay.rest);
-    uint32_t placed = 0;                                               // tokens
-    auto wait_until = [&](uint32_t g) -> bool {                        // (Stage One's loops are bounded, far below this)
-        while (placed <= g && wait_for(smem_u32(s_mbar + placed), AVSG_STEP_GIVE_UP)) ++placed;
-        return placed > g;
-    };
-    auto slot_of = [&](uint32_t what) -> uint32_t {                    // what a position has received; NO_SLOT: there were not enough
-        const uint32_t j = what & 0xFFFFu;
-        if (j < p.S) return j;
-        if (j != NO_SLOT && lane == 0) atomicOr(p.status, ST_BAD_SLOT);
-        return NO_SLOT;
-    };
-    bool there = true;
-    SharedRows s = {SHARED_COMING, 0u, 0u, 0u};
-    // The rows that no warp has asked for yet: a lane counts those of a few neighbouring words, and those before them
-    uint32_t upto = 0;
-    if (lay.early)
-        for (uint32_t a = lane * lay.per_lane; a < lay.local / 32u && a < (lane + 1u) * lay.per_lane; ++a) upto += __popc(s_rest[a]);
-    upto = warp_incl_scan(upto, lane);
-    auto next = [&] {                                                  // the warp's next row, on its way before its slot is known
-        for (;;) {
+    bool there = true;                                                 // nothing was waited for in vain
+    uint32_t turn = warp;                                              // SHARE: warps in the order in which they are through
+    if constexpr (ASK) {
+        Row row;
+        Item item = match<SPT, IPT>(p, lay, ti, rank, copying, smem);
+        const int32_t* s_id = reinterpret_cast<const int32_t*>(smem + lay.id);
+        const uint32_t* s_mask = reinterpret_cast<const uint32_t*>(smem + lay.mask);
+        const uint32_t* s_rest = reinterpret_cast<const uint32_t*>(smem + lay.rest);
+        const int2* s_list = reinterpret_cast<const int2*>(smem + lay.list);
+        auto slot_of = [&](uint32_t what) -> uint32_t {                // what a position has received; NO_SLOT: there were not enough
+            const uint32_t j = what & 0xFFFFu;
+            if (j < p.S) return j;
+            if (j != NO_SLOT && lane == 0) atomicOr(p.status, ST_BAD_SLOT);
+            return NO_SLOT;
+        };
+        uint32_t upto = 0;                                             // rows that no warp has found first: those of a few
+                                                                       // neighbouring words, a lane, and those before them
+        auto next = [&] {                                              // the next of these is the warp's
             uint32_t k = 0;
             if (lane == 0) k = atomicAdd(&s_next, 1u);
             k = __shfl_sync(0xffffffffu, k, 0);
@@ -731,53 +766,84 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
             if (l) k -= __shfl_sync(0xffffffffu, upto, (int)l - 1);
             uint32_t a = l * lay.per_lane, m = s_rest[a];
             for (; k >= __popc(m); m = s_rest[++a]) k -= __popc(m);
-            const uint32_t n = a * 32u + __ffs((int)__ballot_sync(0xffffffffu, (m >> lane & 1u) && __popc(m & ((1u << lane) - 1u)) == k)) - 1u;
-            const uint32_t g = place(lay, rank, copying, n).g;
-            if (SHARE) {
-                if (!(there = wait_until(g))) return;
-                if (s_first[g] != ~0u) {
+            item.n = a * 32u + __ffs((int)__ballot_sync(0xffffffffu, (m >> lane & 1u) && __popc(m & ((1u << lane) - 1u)) == k)) - 1u;
+            item.g = place(lay, rank, copying, item.n).g;
+            item.x = (uint32_t)s_id[item.n];
+        };
+        uint32_t told = 0;                                             // tokens that the block has heard of
+        for (bool first = true;; first = false) {
+            // the row is on its way before its slot is known (one place in the code, so that no copy from register to register waits for it)
+            load_row(row, src + (uint64_t)item.x * stride, item.n != NO_ITEM ? cpr : 0u, lane);
+            if (first) {
+                __syncthreads();                                       // every warp has looked at its positions
+                for (uint32_t a = lane * lay.per_lane; a < lay.local / 32u && a < (lane + 1u) * lay.per_lane; ++a) upto += __popc(s_rest[a]);
+                upto = warp_incl_scan(upto, lane);
+                if (item.n == NO_ITEM) {
+                    next();
+                    if (item.n != NO_ITEM) continue;
+                }
+            }
+            for (; told < p.n_q && (item.n == NO_ITEM || told <= item.g); ++told) {
+                there = wait_for(smem_u32(s_mbar + told), AVSG_STEP_GIVE_UP);          // (Stage One's loops are bounded, far below this)
+                if (!there) break;
+                // the token's misses that are not asked for early, in turn
+                for (uint32_t e = W - 1u - warp; e < s_sent[told]; e += W) {
+                    const int2 what = s_list[told * lay.per_token + e];
+                    const uint32_t n = (uint32_t)what.x;
+                    if (s_mask[n / 32u] >> n % 32u & 1u) continue;
+                    const uint32_t j = slot_of((uint32_t)what.y);
+                    if (j != NO_SLOT) copy_row(src + (uint64_t)(uint32_t)s_id[n] * stride, dst + (uint64_t)j * p.row_bytes, cpr, lane);
+                }
+            }
+            if (!there || item.n == NO_ITEM) break;
+            const uint32_t j = slot_of(s_slots[item.n]);
+            if (j != NO_SLOT) store_row(row, dst + (uint64_t)j * p.row_bytes, cpr, lane);
+            next();
+        }
+    } else {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        cluster_wait();
+        cluster_arrive();
+        uint32_t from = 0;                                             // the warp that is next
+        for (uint32_t g = 0; g < p.n_q; ++g) {
+            const int2* got = reinterpret_cast<const int2*>(smem + lay.list) + g * lay.per_token;
+            there = wait_for(smem_u32(s_mbar + g), AVSG_STEP_GIVE_UP);
+            if (!there) break;
+            const uint32_t count = (uint32_t)got[0].x;
+            const int32_t at = got[0].y;                               // of the first row among those that are shared; -1
+            SharedRows s = {SHARED_COMING, 0u, 0u, 0u};
+            for (uint32_t k = warp >= from ? warp - from : warp + W - from; k < count; k += W) {
+                if (SHARE && at >= 0) {
                     if (warp == 0) {                                   // for all warps: requests wait behind the rows' where the link is full
                         if (!(s.rows & SHARED_COMING)) s_mine = (s.rows & ~SHARED_OPEN) > s.taken ? (s.rows & ~SHARED_OPEN) - s.taken : 0u;
                         s = read_shared(p.shared + ti);                // (comes with the row)
                         if (lane == 0) atomicAdd(&p.shared[ti].begun, W);
                     }
-                    if (s_first[g] + (s_slots[n] >> 16) >= s_mine) continue;           // others have it
+                    if (at + k * copying >= s_mine) break;             // others have the rest
                 }
+                const int2 e = got[1u + k];
+                if (e.x < 0) continue;                                 // (its slot has gone to another id)
+                if (e.y < 0 || (uint32_t)e.y >= p.S) {
+                    if (lane == 0) atomicOr(p.status, ST_BAD_SLOT);
+                    continue;
+                }
+                copy_row(src + (uint64_t)(uint32_t)e.x * stride, dst + (uint64_t)e.y * p.row_bytes, cpr, lane);
             }
-            item.n = n;
-            item.g = g;
-            load_row(row, src + (uint64_t)(uint32_t)s_id[n] * stride, cpr, lane);
-            return;
+            if (FEW || count < W || (SHARE && g + 1u == p.n_q)) {
+                from = (from + count) % W;
+            } else if (g + 1u < p.n_q) {                               // the warps meet
+                from = 0;
+                if (lane == 0) mbar_arrive(smem_u32(s_meet + g));
+                there = wait_for(smem_u32(s_meet + g), AVSG_STEP_GIVE_UP);
+                if (!there) break;
+            }
         }
-    };
-    auto put = [&] {
-        const uint32_t j = slot_of(s_slots[item.n]);
-        if (j != NO_SLOT) store_row(row, dst + (uint64_t)j * p.row_bytes, cpr, lane);
-    };
-    if (item.n == NO_ITEM) next();
-    const int2* s_list = reinterpret_cast<const int2*>(smem + lay.list);
-    for (uint32_t g = 0; there && g < p.n_q; ++g) {
-        if (!(there = wait_until(g))) break;
-        bool placed_one = item.n != NO_ITEM && item.g <= g;
-        if (placed_one) put();
-        // the token's other misses (all of them where nothing is asked for early), in turn
-        for (uint32_t e = W - 1u - warp; e < s_sent[g]; e += W) {
-            const int2 what = s_list[g * lay.per_token + e];
-            const uint32_t n = (uint32_t)what.x;
-            if (s_mask[n / 32u] >> n % 32u & 1u) continue;
-            const uint32_t j = slot_of((uint32_t)what.y);
-            if (j != NO_SLOT) copy_row(src + (uint64_t)(uint32_t)s_id[n] * stride, dst + (uint64_t)j * p.row_bytes, cpr, lane);
-        }
-        while (placed_one && there) {
-            next();
-            placed_one = item.n != NO_ITEM && item.g <= g;
-            if (placed_one && there) put();
-        }
+        turn = warp >= from ? warp - from : warp + W - from;
     }
-    // Warps that take other tables' rows: a few of each block
+    // Warps that take other tables' rows: those that had the fewest of the last token, a few of each block
     uint32_t others = 0;                                               // what 32 of the tables share, one a lane
-    const uint32_t group = (ti + warp) % ((p.n_launch + 31u) / 32u) * 32u;
-    const bool takes = SHARE && warp * (p.n_launch - 1u) * copying < SHARED_WARPS * ((p.n_launch + 31u) / 32u);
+    const uint32_t group = (ti + turn) % ((p.n_launch + 31u) / 32u) * 32u;
+    const bool takes = SHARE && turn * (p.n_launch - 1u) * copying < SHARED_WARPS * ((p.n_launch + 31u) / 32u);
     if (takes && group + lane < p.n_launch) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(others) : "l"(&p.shared[group + lane].rows) : "memory");
     // Stage One does not know who has given up, and nothing may be sent to a block that is gone: every block stays until
     // Stage One is through, and one that gave up until what was sent has arrived.
@@ -805,16 +871,16 @@ uint32_t step_threads(uint32_t S, uint32_t K)
 
 namespace {
 
-template <int CAP, bool SHARE = false>
+template <int CAP, bool ASK, bool SHARE = false>
 const void* step_kernel(uint32_t spt, uint32_t ipt)
 {
     switch (spt) {
-        case 8:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 2, CAP, SHARE>)
-                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 4, CAP, SHARE>)
-                                 : reinterpret_cast<const void*>(avsg_step_kernel<8, 8, CAP, SHARE>);
-        case 4:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<4, 2, CAP, SHARE>)
-                                 : reinterpret_cast<const void*>(avsg_step_kernel<4, 4, CAP, SHARE>);
-        default: return reinterpret_cast<const void*>(avsg_step_kernel<2, 2, CAP, SHARE>);
+        case 8:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 2, CAP, ASK, SHARE>)
+                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 4, CAP, ASK, SHARE>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<8, 8, CAP, ASK, SHARE>);
+        case 4:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<4, 2, CAP, ASK, SHARE>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<4, 4, CAP, ASK, SHARE>);
+        default: return reinterpret_cast<const void*>(avsg_step_kernel<2, 2, CAP, ASK, SHARE>);
     }
 }
 
@@ -838,7 +904,8 @@ cudaError_t step_prepare(size_t max_smem)
 {
     for (uint32_t spt : {2u, 4u, 8u})
         for (uint32_t ipt = 2u; ipt <= spt; ipt *= 2u)                 // (K <= S)
-            for (const void* k : {step_kernel<STEP_FEW_TABLES>(spt, ipt), step_kernel<STEP_MAX_TABLES>(spt, ipt), step_kernel<STEP_MAX_TABLES, true>(spt, ipt)}) {
+            for (const void* k : {step_kernel<STEP_FEW_TABLES, true>(spt, ipt), step_kernel<STEP_FEW_TABLES, false>(spt, ipt), step_kernel<STEP_MAX_TABLES, true>(spt, ipt),
+                                  step_kernel<STEP_MAX_TABLES, false>(spt, ipt), step_kernel<STEP_MAX_TABLES, false, true>(spt, ipt)}) {
                 cudaFuncAttributes fa;
                 cudaError_t e = cudaFuncGetAttributes(&fa, k);
                 if (e == cudaSuccess)
@@ -856,7 +923,7 @@ StepClusters step_clusters(size_t max_smem)
         cudaLaunchAttribute attr[2];
         int fit = 0;
         step_config(cfg, attr, 1, cl, 1024, max_smem - 2048);      // (the largest; statically it has 1 KB)
-        if (cudaOccupancyMaxActiveClusters(&fit, step_kernel<STEP_MAX_TABLES>(8, 2), &cfg) != cudaSuccess) { cudaGetLastError(); fit = 0; }
+        if (cudaOccupancyMaxActiveClusters(&fit, step_kernel<STEP_MAX_TABLES, true>(8, 2), &cfg) != cudaSuccess) { cudaGetLastError(); fit = 0; }
         s.fit[cl] = (uint32_t)fit;
     }
     return s;
@@ -868,7 +935,10 @@ cudaError_t launch_step(const S1ParamsT<CAP>& p, uint32_t cluster, cudaStream_t 
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     const uint32_t nt = step_threads(p.S, p.K);
-    StepLayout lay = step_layout(p.S, p.K, p.n_q, nt, cluster - 1u, p.row_bytes, p.host_ids != 0);
+    const bool share = CAP == STEP_MAX_TABLES && cluster < SHARED_CLUSTER;
+    StepLayout lay;
+    const bool ask = !share && p.row_bytes <= 16u * ROW_CHUNKS && step_layout(lay, p.S, p.K, p.n_q, nt, cluster - 1u, p.host_ids != 0, true);
+    if (!ask) step_layout(lay, p.S, p.K, p.n_q, nt, cluster - 1u, p.host_ids != 0, false);
     step_config(cfg, attr, p.n_launch, cluster, nt, lay.total);
     cfg.stream = stream;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -876,9 +946,10 @@ cudaError_t launch_step(const S1ParamsT<CAP>& p, uint32_t cluster, cudaStream_t 
     cfg.numAttrs = 2;
     void* args[] = {const_cast<S1ParamsT<CAP>*>(&p), &lay};
     const uint32_t spt = p.S / nt, ipt = (p.K + nt - 1) / nt;
+    const void* kernel = ask ? step_kernel<CAP, true>(spt, ipt) : step_kernel<CAP, false>(spt, ipt);
     if constexpr (CAP == STEP_MAX_TABLES)
-        if (cluster < SHARED_CLUSTER) return cudaLaunchKernelExC(&cfg, step_kernel<CAP, true>(spt, ipt), args);
-    return cudaLaunchKernelExC(&cfg, step_kernel<CAP>(spt, ipt), args);
+        if (share) kernel = step_kernel<CAP, false, true>(spt, ipt);
+    return cudaLaunchKernelExC(&cfg, kernel, args);
 }
 template cudaError_t launch_step(const StepParams& p, uint32_t cluster, cudaStream_t stream);
 template cudaError_t launch_step(const StepParamsFew& p, uint32_t cluster, cudaStream_t stream);
