@@ -609,9 +609,10 @@ __device__ __forceinline__ Item match(const S1ParamsT<CAP>& p, const StepLayout&
             const uint32_t votes = __ballot_sync(0xffffffffu, certain);
             s_id[n] = x;
             uint32_t rest = votes;
-            if (votes && item.n == NO_ITEM) {
-                const uint32_t l = __ffs((int)votes) - 1u;
-                item = {word * 32u + l, __shfl_sync(0xffffffffu, g, (int)l), (uint32_t)__shfl_sync(0xffffffffu, x, (int)l)};
+            const uint32_t l = __ffs((int)votes) - 1u;
+            // (a row of a later token is left: the queue has the tokens in order, and who holds one copies nothing until it is placed)
+            if (votes && item.n == NO_ITEM && __shfl_sync(0xffffffffu, g, (int)l) == 0) {
+                item = {word * 32u + l, 0u, (uint32_t)__shfl_sync(0xffffffffu, x, (int)l)};
                 rest &= rest - 1u;
             }
             if (lane == 0) { s_mask[word] = votes; s_rest[word] = rest; }
