@@ -46,7 +46,7 @@ struct StepLayout {
     uint32_t per_lane, per_token;        // words of 32 local positions to a lane; entries of a token in a block's list, at most
     uint32_t log_heads, nil;             // chains of the index; its closing node
     uint32_t log_seen, log_asked;        // words of the copying blocks' sets: cached ids; ids of an earlier token, each
-    uint32_t node, head, life, bits, tot, ndead, cnt, sum, miss, pos, entry, dead, ids;    // first block
+    uint32_t node, head, life, bits, tot, ndead, cnt, sum, votes, miss, pos, dead, ids;    // first block
     uint32_t seen, asked, slots, id, mask, rest, list, their_ids;              // copying blocks
     uint32_t total;
 };
@@ -80,9 +80,9 @@ bool step_layout(StepLayout& o, uint32_t S, uint32_t K, uint32_t n_q, uint32_t n
         o.ndead = a;   a += 2u * 32u * 4u;                 // warps' dead slots, by parity
         o.cnt = a;     a += 2u * 2u * 32u * 4u;            // warps' counts of the decay search, by parity
         o.sum = a;     a += 16u;                           // valid ids of the call
+        o.votes = a;   a += ask ? align16((K + 31u) / 32u * 4u) : 0u;      // the token's misses, a bit per position
         o.miss = a;    a += align16(K * 4u);               // misses in position order: ids,
-        o.pos = a;     a += align16(K * 2u);               //   positions,
-        o.entry = a;   a += ask ? align16(K * 2u) : 0u;    //   entries in their copying blocks' lists
+        o.pos = a;     a += align16(K * 2u);               //   positions
         o.dead = a;    a += align16(K * 2u);               // dead slots in slot order
         o.ids = a;     a += ids;                           // received: the ids of a call with host buffers
         const uint32_t first = a;
@@ -127,19 +127,13 @@ struct Tell {
         send_async(map_rank(sent + 4u * g, to + 1u), n, bar);
         arrive_expect(bar, 12u * n + 4u);
     }
-    // the copying block of position i, and which of its positions it is
-    __device__ __forceinline__ uint32_t block_of(uint32_t g, uint32_t i, uint32_t& n) const
+    // own: the misses of the token that the blocks have been told of
+    __device__ __forceinline__ void miss(uint32_t g, uint32_t i, uint32_t j, uint32_t* own) const
     {
-        const uint32_t group = g * lay.groups + (i >> lay.log_group), at = group * lay.by_copying >> 18;
-        n = (at << lay.log_group) + (i & ((1u << lay.log_group) - 1u));
-        return group - at * copying;
-    }
-    // e: the entry
-    __device__ __forceinline__ void miss(uint32_t g, uint32_t i, uint32_t j, uint32_t e) const
-    {
-        uint32_t n;
-        const uint32_t to = block_of(g, i, n), bar = map_rank(mbar + 8u * g, to + 1u);
+        const uint32_t group = g * lay.groups + (i >> lay.log_group), at = group * lay.by_copying >> 18, to = group - at * copying;
+        const uint32_t n = (at << lay.log_group) + (i & ((1u << lay.log_group) - 1u)), bar = map_rank(mbar + 8u * g, to + 1u);
         send_async(map_rank(smem + lay.slots + 4u * n, to + 1u), j, bar);
+        const uint32_t e = atomicAdd(own + to, 1u);
         send_async(map_rank(smem + lay.list + 8u * (g * lay.per_token + e), to + 1u), (int32_t)n, (int32_t)j, bar);
     }
     __device__ __forceinline__ void head(uint32_t g, uint32_t to, uint32_t n, uint32_t share, int32_t first) const
@@ -174,10 +168,7 @@ __device__ __forceinline__ void tell_at_last(const Tell tell, uint32_t n_q, uint
             for (uint32_t e = threadIdx.x; e < count; e += blockDim.x) {
                 const int2 v = list[e];
                 const uint32_t what = (uint32_t)v.y;
-                if (v.x < 0 || what >> (2u * LIST_SLOT_BITS) != g) continue;
-                const uint32_t i = what >> LIST_SLOT_BITS & MASK;
-                uint32_t n;
-                tell.miss(g, i, what & MASK, atomicAdd(s_own + tell.block_of(g, i, n), 1u));
+                if (v.x >= 0 && what >> (2u * LIST_SLOT_BITS) == g) tell.miss(g, what >> LIST_SLOT_BITS & MASK, what & MASK, s_own);
             }
             __syncthreads();
             if (threadIdx.x < tell.copying) tell.token(g, threadIdx.x, s_own[threadIdx.x]);
@@ -212,9 +203,9 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
     uint32_t* s_ndead = reinterpret_cast<uint32_t*>(smem + lay.ndead);
     uint32_t* s_cnt  = reinterpret_cast<uint32_t*>(smem + lay.cnt);
     uint32_t* s_sum  = reinterpret_cast<uint32_t*>(smem + lay.sum);
+    uint32_t* s_votes = reinterpret_cast<uint32_t*>(smem + lay.votes);
     int32_t*  s_miss = reinterpret_cast<int32_t*>(smem + lay.miss);
     uint16_t* s_pos  = reinterpret_cast<uint16_t*>(smem + lay.pos);
-    uint16_t* s_entry = reinterpret_cast<uint16_t*>(smem + lay.entry);
     uint16_t* s_dead = reinterpret_cast<uint16_t*>(smem + lay.dead);
     const int32_t* s_ids = reinterpret_cast<const int32_t*>(smem + lay.ids);
 
@@ -325,6 +316,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
             const uint32_t votes = __ballot_sync(0xffffffffu, miss);
             rank[k] = wmiss + __popc(votes & below);                   // within the warp, in position order
             wmiss += __popc(votes);
+            if (ASK && lane == 0 && i0 + 32u * k < i1) s_votes[warp * ipt + k] = votes;
             missing |= miss ? 1u << k : 0u;
             if (slot[k] >= 0) s_life[slot[k]] = (int8_t)L;
             if (store) O[i0 + 32u * k] = slot[k];
@@ -349,7 +341,6 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
         const uint32_t all = __reduce_add_sync(0xffffffffu, t);
         const uint32_t n_g = all >> 16;
         uint32_t dtotal = all & 0xFFFFu, dead_before = before & 0xFFFFu, d = 0;
-        uint32_t* s_tell = s_own + (g & 1u) * STEP_FEW_CLUSTER;            // the token's misses in each copying block's positions
         sum_miss += n_g;
         if (tid == 0 && p.miss_count) p.miss_count[(size_t)ti * p.n_q + g] = (int32_t)n_g;
         const bool share_it = SHARE && n_g > SHARED_FROM && !unusual;
@@ -368,14 +359,9 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
                 if (missing & (1u << k)) {
                     s_miss[(before >> 16) + rank[k]] = xs[k];
                     s_pos[(before >> 16) + rank[k]] = (uint16_t)(i0 + 32u * k);
-                    if constexpr (ASK) {
-                        uint32_t n;
-                        s_entry[(before >> 16) + rank[k]] = (uint16_t)atomicAdd(s_tell + tell.block_of(g, i0 + 32u * k, n), 1u);
-                    }
                 }
             }
         }
-        if (ASK && tid < STEP_FEW_CLUSTER) s_own[(~g & 1u) * STEP_FEW_CLUSTER + tid] = 0;         // for the next token
         if (!last) load_token(g + 1);                                      // arrives while this token's misses are placed
         // Pass 3, the while-loop of Alg. 1: decay until n_g slots are dead
         if (dtotal < n_g) {
@@ -390,6 +376,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
             dtotal = __reduce_add_sync(0xffffffffu, t);
             if (dtotal < n_g && tid == 0) atomicOr(p.status, ST_NO_DEAD_SLOTS);
         }
+        if (ASK && tid < STEP_FEW_CLUSTER) s_own[(~g & 1u) * STEP_FEW_CLUSTER + tid] = 0;         // for the next token
         const uint32_t n_take = n_g < dtotal ? n_g : dtotal;
         if (dead_before < n_take) {                      // some of the first n_g dead slots are this warp's
             uint32_t bits = s_bits[tid], r, unused;
@@ -406,7 +393,31 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
         // blocks may take some (so that what is left is at the end), else a share in position order
         const uint32_t share = CAP == STEP_FEW_TABLES || share_it ? 0u : (n_take + copying - 1u) / copying;
         if constexpr (ASK) {
-            if (warp == nw - 1u && lane < copying && !unusual) tell.token(g, lane, s_tell[lane]);  // (the first warps install)
+            // What a copying block gets of this token: counted by a warp for each (the first warps install); in small blocks, which have
+            // down to four warps, by four lanes for each (S = 256, K = 64, two tokens: 7.5 us with a warp, 7.0).  Not both in one
+            // kernel: small calls feel its length (one table of S = 1024, K = 256: 6.3 us, 6.5 with both).
+            const uint32_t group0 = g * lay.groups, in_group = (1u << lay.log_group) - 1u;
+            auto count = [&](uint32_t to, uint32_t in, uint32_t lanes) -> uint32_t {
+                // (its first group is the first one that is `to` modulo copying)
+                uint32_t group = (group0 * lay.by_copying >> 18) * copying + to, n = 0;
+                if (group < group0) group += copying;
+                for (uint32_t q = group - group0 + in * copying; n_g && q < lay.groups; q += lanes * copying) {
+                    const uint32_t i = q << lay.log_group;
+                    n += __popc(s_votes[i / 32u] >> i % 32u & ~(~1u << in_group));
+                }
+                return n;
+            };
+            if constexpr (SPT > 2) {
+                for (uint32_t to = nw - 1u - warp; to < copying && !unusual; to += nw) {
+                    const uint32_t n = __reduce_add_sync(0xffffffffu, count(to, lane, 32u));
+                    if (lane == 0) tell.token(g, to, n);
+                }
+            } else if (warp == nw - 1u && !unusual) {
+                uint32_t n = lane / 4u < copying ? count(lane / 4u, lane & 3u, 4u) : 0u;
+                n += __shfl_xor_sync(0xffffffffu, n, 1);
+                n += __shfl_xor_sync(0xffffffffu, n, 2);
+                if ((lane & 3u) == 0 && lane / 4u < copying) tell.token(g, lane / 4u, n);
+            }
         } else if (tid < copying && !unusual) {
             tell.head(g, tid, n_take, share, share_it ? (int32_t)((shared & ~SHARED_COMING) + tid) : -1);
         }
@@ -419,7 +430,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
             if (unusual) {
                 if (k < n_take) list[list_off + k] = make_int2(x, (int32_t)((uint32_t)j | i << LIST_SLOT_BITS | g << (2u * LIST_SLOT_BITS)));
             } else if constexpr (ASK) {
-                tell.miss(g, i, (uint32_t)j & 0xFFFFu, s_entry[k]);
+                tell.miss(g, i, (uint32_t)j & 0xFFFFu, s_own + (g & 1u) * STEP_FEW_CLUSTER);
             } else if (k < n_take) {
                 tell.row(g, k, share, x, j);
             }
@@ -711,7 +722,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ __align__(8) unsigned long long s_mbar[STEP_MAX_TOKENS], s_meet[ASK || FEW ? 1 : STEP_MAX_TOKENS];
     __shared__ uint32_t s_sent[ASK ? STEP_MAX_TOKENS : 1];             // received: a token's misses in the block's positions
-    __shared__ uint32_t s_own[2 * STEP_FEW_CLUSTER];                   // first block: of a token's misses, how many are a copying block's, by parity of the token
+    __shared__ uint32_t s_own[2 * STEP_FEW_CLUSTER];                   // first block: of those, how many it has sent, by parity of the token
     __shared__ uint32_t s_next;                                        // of the rows to be asked for, the first that no warp has taken
     __shared__ volatile uint32_t s_mine;                               // rows that are shared: the first that others have taken
     const uint32_t rank = cluster_rank(), cluster = !ASK && FEW ? STEP_FEW_CLUSTER : cluster_size(), copying = cluster - 1u;
