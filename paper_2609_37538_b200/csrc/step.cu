@@ -54,7 +54,10 @@ struct StepLayout {
 bool step_layout(StepLayout& o, uint32_t S, uint32_t K, uint32_t n_q, uint32_t nt, uint32_t copying, bool host_ids, bool ask)
 {
     // At least 32 groups a token, so that seven blocks have about the same to do: 9 tables with K = 256 30.8 us with groups of
-    // 32 positions, 27.5 with rows handed out in turn.  Larger ones are loaded in longer pieces.
+    // 32 positions, 27.5 with rows handed out in turn.  Larger ones are loaded in longer pieces.  Misses in a run of positions go
+    // to few blocks, which does not take back what asking early gives: K = 2048, two tokens, 16, 64, 256 neighbours missed of
+    // each, dealt out in turn / by groups: one table 9.9 / 9.6, 10.9 / 10.5, 15.9 / 14.2 us; eight 11.8 / 10.3, 22.1 / 20.3, 64.2 /
+    // 61.8; 32 22.4 / 21.0, 63.3 / 63.1, 228.0 / 227.1.
     o.log_group = 5u;
     while (o.log_group && K >> o.log_group < 32u) --o.log_group;
     o.groups = (K + (1u << o.log_group) - 1u) >> o.log_group;
@@ -105,6 +108,7 @@ bool step_layout(StepLayout& o, uint32_t S, uint32_t K, uint32_t n_q, uint32_t n
 }
 constexpr uint32_t NO_ITEM = 0xFFFFFFFFu;
 constexpr uint32_t NOT_MISSED = 0xFFFFFFFFu, NO_SLOT = 0xFFFFu;        // of a position; else its slot
+static_assert((NOT_MISSED & 0xFFFFu) == NO_SLOT, "a position that is not missed has no slot to store to");
 
 __device__ __forceinline__ bool wait_for(uint32_t mbar, uint32_t limit)
 {
@@ -512,8 +516,8 @@ struct Item { uint32_t n, g, x; };
 
 // A copying block finds out which of its positions are missed for certain: their ids are in no slot and in no earlier token
 // of the call.  What it does not find so (an id that seems to be in a set; a resident one that loses its slot to an earlier
-// token) is news from the first block.  The first that a warp finds is its own to ask for, and returned; the others are left in
-// lay.rest, in position order, token after token (for the other warps behind a barrier).
+// token) is news from the first block.  The first of the first token that a warp finds is its own to ask for, and returned; the others
+// are left in lay.rest, in position order, token after token (for the other warps behind a barrier).
 // What takes the time is instruction issue and bank conflicts for 32 warps.  From the call's start, 32 tables of 8192 slots,
 // K = 2048, two tokens, three copying blocks: ids and cached ids are loaded after 2.9 us, the sets are there after 3.9, the first
 // rows are asked for after 4.7, where rows that wait for their slots are asked for after 6.5.  Other ways to know: a chained index
@@ -568,6 +572,10 @@ __device__ __forceinline__ Item match(const S1ParamsT<CAP>& p, const StepLayout&
     cluster_arrive_relaxed();                            // (what this block sends is sent)
 
     // ---- every global load is issued first: cached ids, the first token's, the block's own ids ----
+    // Nothing orders the reads of cached ids before the first block's stores to them.  An id of this call that is read too early
+    // only keeps its rows from being asked for early.  One that is gone already (its slot was reserved, or it is no longer verified)
+    // makes a position look missed that an earlier token's lookup or the position's own has found: then a row is read in vain, and
+    // dropped, because the position stays NOT_MISSED.  So sets decide what is asked for, and what has been received what is stored.
     int4 t4[NV];
     int32_t xo[OWN], xe[IPT];
     const int4* g_tok = reinterpret_cast<const int4*>(p.tok + (size_t)p.table_id[ti] * S);
