@@ -80,6 +80,10 @@ class ClockSampler:
         if self.proc is None:
             return {"sm_mhz": None, "sm_max_mhz": None, "reasons": ["unavailable"]}
         time.sleep(0.15)
+        for _ in range(100):           # (on a busy host the first sample may come after a very short run: 5 s at most)
+            if self.lines or self.proc.poll() is not None:
+                break
+            time.sleep(0.05)
         self.proc.terminate()          # the exact process started above
         try:
             self.proc.wait(timeout=5)

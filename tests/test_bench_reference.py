@@ -30,3 +30,17 @@ def test_other_ranks_of_the_reference_arm_do_nothing():
     r = subprocess.run([sys.executable, os.path.join(ROOT, "bench.py"), "--impl", "reference", "--gpus", "2",
                         "--steps", "1", "--warmup", "3"], cwd=ROOT, env=env, capture_output=True, text=True, timeout=120)
     assert r.returncode == 0 and r.stdout.strip() == ""
+
+
+def test_clocks_where_the_first_sample_comes_late(tmp_path, monkeypatch):
+    """A very short run on a busy host: it is over before nvidia-smi has written its first line."""
+    tool = tmp_path / "nvidia-smi"
+    tool.write_text('#!/bin/sh\nsleep 0.6\nwhile true; do echo "1900, 1965, 200, Not Active, Not Active, Not Active, Active"; sleep 0.1; done\n')
+    tool.chmod(0o755)
+    monkeypatch.setenv("PATH", str(tmp_path) + os.pathsep + os.environ["PATH"])
+    monkeypatch.syspath_prepend(ROOT)
+    import bench
+    sampler = bench.ClockSampler(0)
+    sampler.start()
+    got = sampler.stop()
+    assert got["sm_mhz"] == 1900 and got["sm_max_mhz"] == 1965 and got["reasons"] == ["sw_power_cap"]
