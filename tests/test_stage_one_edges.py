@@ -113,14 +113,16 @@ def test_lifetimes_above_the_maximum():
         assert int(status.item()) == 0
 
 
-# clusters of eight, four and three blocks, and two kernels (state off its alignment); the small sizes of the test above too
-@pytest.mark.parametrize("n,S,K,n_q", [(2, 64, 16, 4), (1, 4096, 2048, 2), (9, 4096, 2048, 2), (32, 4096, 2048, 2), (3, 8192, 1000, 8)])
+# clusters of eight and four blocks, and two kernels (state off its alignment); the small sizes of the test above too; rows that
+# are asked for early and rows that are too long for that
+@pytest.mark.parametrize("n,S,K,n_q,rb", [(2, 64, 16, 4, 64), (1, 4096, 2048, 2, 64), (9, 4096, 2048, 2, 64), (32, 4096, 2048, 2, 64), (3, 8192, 1000, 8, 64),
+                                          (2, 64, 16, 4, 1552), (1, 4096, 2047, 2, 1552), (10, 4096, 1365, 3, 1552)])
 @pytest.mark.parametrize("aligned", [True, False])
-def test_the_last_reservation_of_a_slot_has_its_row(n, S, K, n_q, aligned):
+def test_the_last_reservation_of_a_slot_has_its_row(n, S, K, n_q, rb, aligned):
     """Lifetimes above the maximum: a slot that two tokens of a call reserve holds the row of the later one."""
     import torch
     import paper_2609_37538_b200 as avsg
-    L, context, calls, rb = 3, 40000, 3, 64
+    L, context, calls = 3, 16384, 3
     kv = avsg.pinned_empty(context * rb)
     tr.fill_kv(kv.data_ptr(), 3, 0, context, rb)
     rng = np.random.default_rng([n, S, K])
