@@ -75,8 +75,11 @@ extern "C" {
                                        (of 8192 slots) on, where rows of a table that misses
                                        more than 512 ids of a token are also taken over by
                                        blocks of others that are through (not with arriving,
-                                       timing, an own transfer geometry or a table above 8192
-                                       slots, nor with stage_one_done above three tables).
+                                       timing or an own transfer geometry, nor with
+                                       stage_one_done above three tables, nor tables above
+                                       16384 slots; of 16384 slots where n_tokens and topk
+                                       leave room for them in one SM's shared memory, up to
+                                       33 tables, and more where there are several tokens).
                                        Its blocks take whole SMs while they run: who wants
                                        room for other kernels beside the call sets a
                                        transfer geometry (100 calls of 8, 32, 64 tables
@@ -143,8 +146,9 @@ typedef struct {
     uint32_t stage_one_cluster; /* thread blocks that share one table in Stage One: 0 = chosen by
                                 the library (one block while the table fits one SM's shared
                                 memory, i.e. S <= 8192; above that the smallest thread-block
-                                cluster that holds it), or 1, 2, 4, 8.  Same results.  Not with
-                                AVSG_INDEX_PAPER; needs S / cluster >= 32                */
+                                cluster that holds it, but for calls in one kernel), or 1, 2, 4,
+                                8.  Same results.  Not with AVSG_INDEX_PAPER; needs
+                                S / cluster >= 32                                        */
 } avsg_config;
 
 typedef struct {
@@ -253,7 +257,7 @@ typedef struct {
 /* App. E (a request starts with nothing cached), Sec. 3.1-3.2 (one S-slot
  * buffer plus S state entries per request): allocates all state, every table
  * empty (id -1) and dead (lifetime -1), buffers zeroed.  *out is set only on
- * success.  Tables above 8192 slots are handled by a thread-block cluster
+ * success.  Tables above 8192 slots may be handled by a thread-block cluster
  * per table (stage_one_cluster).  Every kernel of the library is loaded here,
  * so that no later call has to wait for the device's other streams (the CUDA
  * runtime loads a kernel when it is first used, and that may wait for every
@@ -287,7 +291,7 @@ int avsg_step(avsg_ctx *ctx, const avsg_step_args *args, void *cuda_stream);
  * asynchrony), and the ids are in place when the call is made.  The outputs are there when the
  * call has finished.  Pinned buffers are read and
  * written by the kernels themselves (AVSG_XFER_SM_BALANCED or _OVERLAP, not AVSG_INDEX_PAPER nor
- * tables of several Stage One blocks); otherwise, and for more than 16384 ids that do not begin on a
+ * a Stage One of several blocks per table); otherwise, and for more than 16384 ids that do not begin on a
  * 32-byte boundary with a K that is a multiple of 8, the library stages them through its own device
  * buffers: one upload of the ids, one download per requested output. */
 int avsg_step_host(avsg_ctx *ctx, const avsg_step_args *args, void *cuda_stream);

@@ -23,6 +23,7 @@ struct avsg_ctx {
     avsg_config cfg;
     uint32_t logS = 0, logH = 0;
     uint32_t s1_cluster = 1;           // blocks that share one table in Stage One (1 = the single-block kernel)
+    bool one_kernel = false;           // both stages in one kernel, where a call allows it
     uint32_t host_status = 0;          // status bits raised on the host side (sticky like the device word)
     uint32_t list_stride = 0;          // entries per miss-list segment
     int sm_count = 0;
@@ -226,7 +227,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     // writes the outputs back, so that the calls of a stream follow one another as launches do, without an event between
     // them (measured with 32 tables: see put_outputs()).  Pageable ones, the paper-literal kernel and the comparators
     // go through copies on a side stream, and so do tables of several Stage One blocks, each of which would read all ids
-    // from the host (S = 16384 with 38, 50, 64 tables 168, 210, 263 us by copies, 219, 285, 372 in place; S = 32768, four
+    // from the host (in two kernels, S = 16384 with 38, 50, 64 tables 168, 210, 263 us by copies, 219, 285, 372 in place; S = 32768, four
     // tokens, 16 tables 146 and 306; only one to four tables were quicker in place).  So do calls of more than
     // HOST_ODD_IDS ids whose tokens do not all begin on 32-byte boundaries, which the link moves in parts of its units, while
     // a copy costs its event.  In place, begun 0, 32 and 4 bytes behind a line / by copies: 32 tables with K = 264 (four
@@ -235,9 +236,18 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     // 21, 42 / 45; 32 tables, one token 22, 18, 32 / 41.  And ids that do not begin on a word's boundary, which the copies take.
     HostOut out;
     bool host_ids = false;
+    // One kernel for both stages, where the tables' clusters fit the device (see avsg_step_kernel for what it saves).  Its
+    // blocks take whole SMs and the next grid starts behind them: a caller who wants the hits before the rows are there
+    // (stage_one_done) gets that from a call of more than a few tables only with the two kernels.
+    const bool sm_copies = c->cfg.transfer_mode == AVSG_XFER_SM_BALANCED || c->cfg.transfer_mode == AVSG_XFER_SM_OVERLAP;
+    uint32_t cluster = 0;
+    if (sm_copies && c->one_kernel && n_q <= STEP_MAX_TOKENS && !a->arriving && !c->timing && !c->geometry_set &&
+        (!a->stage_one_done || n <= STEP_EARLY_TABLES)) {
+        cluster = c->step_clusters.of(n, step_threads(c->cfg.buffer_slots, K));
+        if (cluster && !step_serves(c->cfg.buffer_slots, K, n_q, cluster)) cluster = 0;
+    }
     const bool in_place = (K % 8u == 0 && reinterpret_cast<uint64_t>(a->indices) % 32u == 0) || n_ids <= HOST_ODD_IDS;
-    if (host_io && c->cfg.index_mode != AVSG_INDEX_PAPER && c->s1_cluster == 1 && in_place &&
-        (c->cfg.transfer_mode == AVSG_XFER_SM_BALANCED || c->cfg.transfer_mode == AVSG_XFER_SM_OVERLAP)) {
+    if (host_io && c->cfg.index_mode != AVSG_INDEX_PAPER && (c->s1_cluster == 1 || cluster) && in_place && sm_copies) {
         const int32_t* ids = reinterpret_cast<uint64_t>(a->indices) % 4u == 0 ? mapped(a->indices, n_ids) : nullptr;
         out.host_slots = mapped(a->slots, n_ids);
         out.host_hit = a->hit ? mapped(a->hit, n_ids) : nullptr;
@@ -355,12 +365,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
         else CU(launch_stage_one(p, cnt < round_size ? cnt : round_size, stream));
         return AVSG_OK;
     };
-    // One kernel for both stages, where the tables' clusters fit the device (see avsg_step_kernel for what it saves).  Its
-    // blocks take whole SMs and the next grid starts behind them: a caller who wants the hits before the rows are there
-    // (stage_one_done) gets that from a call of more than a few tables only with the two kernels.
-    const uint32_t cluster = n_q <= STEP_MAX_TOKENS && (!a->stage_one_done || n <= STEP_EARLY_TABLES) ? c->step_clusters.of(n, step_threads(c->cfg.buffer_slots, K)) : 0u;
-    if (cluster && (overlap || mode == AVSG_XFER_SM_BALANCED) && c->s1_cluster == 1 && c->cfg.index_mode != AVSG_INDEX_PAPER &&
-        !a->arriving && !host_io && !c->timing && !c->geometry_set) {
+    if (cluster && !host_io) {
         auto step = [&](auto&& p) -> int {
             fill(p, 0, n);
             p.flags = nullptr; p.out = out; p.early = step_early(p); p.shared = c->d_shared;
@@ -545,6 +550,7 @@ int avsg_create(const avsg_config* cfg, avsg_ctx** out)
             for (C = 1; C <= 8 && !fits(C); C *= 2) {}
         if (C > 8 || !fits(C)) { delete c; return AVSG_EUNSUPPORTED; }
         c->s1_cluster = C;
+        c->one_kernel = cfg->index_mode != AVSG_INDEX_PAPER && (C == 1 || (cfg->stage_one_cluster == 0 && S <= STEP_MAX_SLOTS));
     }
     // always raise the kernels' dynamic shared-memory limit to the device maximum: the attribute is
     // per function, so a context with a small table must not lower it under a context with a large one

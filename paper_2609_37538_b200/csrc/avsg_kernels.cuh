@@ -90,6 +90,7 @@ constexpr uint32_t STEP_FEW_CLUSTER = 8;
 constexpr uint32_t STEP_EARLY_TABLES = 3;            // see step_early()
 constexpr uint64_t STEP_EARLY_BYTES = 2ull << 30;
 constexpr uint32_t STEP_MAX_TOKENS = 64;
+constexpr uint32_t STEP_MAX_SLOTS = 16384, STEP_MAX_IDS = 8192;      // of a table; of a token, where a table has more than 8192
 // What a table that misses far more than its cluster's blocks can have under way shares with the other blocks of the call:
 // see avsg_step_kernel.
 struct __align__(16) SharedRows {
@@ -242,6 +243,8 @@ struct StepClusters {
     }
 };
 cudaError_t step_prepare(size_t max_smem);
+// Whether the first block of a cluster has room for such a table (with up to 8192 slots it always has).
+bool step_serves(uint32_t S, uint32_t K, uint32_t n_q, uint32_t cluster);
 StepClusters step_clusters(size_t max_smem);            // after step_prepare
 // Whether the grid behind a call in one kernel may start under it (see the kernel).  Up to three tables, and up to eight
 // that reach little host memory (id_limit: rows a table's ids can reach).  Early / late, calls of K = 2048: one table 13.2 / 13.4

@@ -1,5 +1,6 @@
 // Stage One of the AVSG operator across a thread-block cluster: one table per cluster of C blocks (C = 2, 4, 8), for
-// tables that one SM's shared memory does not hold (S up to 32768 slots).
+// tables that one SM's shared memory does not hold (S up to 32768 slots; of 16384 slots those calls that avsg_step_kernel does
+// not serve).
 //
 // Same results as the single-block kernel (Algorithm 1 with the lifetime operations of Algorithm 3, the tokens of an
 // iteration in order as in Algorithm 4, the end-of-step invalidation), and the same index, bits and passes; see there.

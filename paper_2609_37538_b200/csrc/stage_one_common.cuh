@@ -80,7 +80,7 @@ __device__ __forceinline__ uint32_t decay4(uint32_t w, uint32_t d)
     return __vmaxs4(__vsubss4(w, d * 0x01010101u), 0xFFFFFFFFu);
 }
 
-// The lifetimes of a thread's SPT consecutive slots (2, 4 or 8), packed one signed byte each, four to a word; unused
+// The lifetimes of a thread's SPT consecutive slots (2, 4, 8 or 16), packed one signed byte each, four to a word; unused
 // bytes carry 0x7F (never counted, never dead).  GLOBAL: from global memory, past L1; WIDE: `at` is a multiple of SPT.
 template <int SPT, bool GLOBAL = false, bool WIDE = true>
 __device__ __forceinline__ void life_words(const int8_t* at, bool own, uint32_t (&w)[(SPT + 3) / 4])
@@ -94,6 +94,9 @@ __device__ __forceinline__ void life_words(const int8_t* at, bool own, uint32_t 
             const uint32_t v = (uint8_t)__ldcg(reinterpret_cast<const signed char*>(at) + k);
             w[k / 4] = (w[k / 4] & ~(0xFFu << (8 * (k & 3)))) | v << (8 * (k & 3));
         }
+    } else if constexpr (SPT == 16) {
+        const uint4 v = GLOBAL ? __ldcg(reinterpret_cast<const uint4*>(at)) : *reinterpret_cast<const uint4*>(at);
+        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
     } else if constexpr (SPT == 8) {
         const uint2 v = GLOBAL ? __ldcg(reinterpret_cast<const uint2*>(at)) : *reinterpret_cast<const uint2*>(at);
         w[0] = v.x; w[1] = v.y;
@@ -112,6 +115,7 @@ __device__ __forceinline__ void life_words_store(int8_t* at, bool own, const uin
 #pragma unroll
         for (int k = 0; k < SPT; ++k) at[k] = (int8_t)(w[k / 4] >> (8 * (k & 3)));
     }
+    else if constexpr (SPT == 16) *reinterpret_cast<uint4*>(at) = make_uint4(w[0], w[1], w[2], w[3]);
     else if constexpr (SPT == 8) *reinterpret_cast<uint2*>(at) = make_uint2(w[0], w[1]);
     else if constexpr (SPT == 4) *reinterpret_cast<uint32_t*>(at) = w[0];
     else *reinterpret_cast<uint16_t*>(at) = (uint16_t)w[0];
@@ -168,6 +172,66 @@ __device__ __forceinline__ void find_slots(const int32_t (&x)[M], const uint2* s
     if (open) atomicOr(status, ST_PROBE_EXHAUSTED);
 }
 
+// The same index where nodes of eight bytes do not fit (tables of 16384 slots): ids, links of two bytes, and the slots of the nodes
+// from S on, each in a place of its own; as many chains as there is room for.
+struct PackedIndex {
+    int32_t*  id;                        // [nil + 1]
+    uint16_t* link;                      // [nil + 1]
+    uint16_t* slot;                      // [nil - S]: of node S, S + 1, ...
+    uint32_t* head;                      // [heads]
+    uint32_t  heads, nil, S;
+    __device__ __forceinline__ uint32_t* chain(int32_t x) const { return head + __umulhi((uint32_t)x * 2654435769u, heads); }
+};
+
+template <int NV>
+__device__ __forceinline__ void index_slots(const int4 (&t4)[NV], const PackedIndex& ix)
+{
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        if (threadIdx.x + q * blockDim.x < ix.S / 4) {
+            const uint32_t j = 4u * (threadIdx.x + q * blockDim.x);
+            const int32_t x[4] = {t4[q].x, t4[q].y, t4[q].z, t4[q].w};
+            uint32_t next[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) next[c] = x[c] >= 0 ? atomicExch(ix.chain(x[c]), j + c) : ix.nil;
+            reinterpret_cast<int4*>(ix.id)[j / 4] = t4[q];
+            reinterpret_cast<uint2*>(ix.link)[j / 4] = make_uint2(next[0] | next[1] << 16, next[2] | next[3] << 16);
+        }
+    }
+}
+
+template <int M>
+__device__ __forceinline__ void find_slots(const int32_t (&x)[M], const PackedIndex& ix, uint32_t* status, int32_t (&slot)[M])
+{
+    uint32_t node[M];
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+        slot[k] = -1;
+        node[k] = ix.nil;
+        if (x[k] >= 0) node[k] = *ix.chain(x[k]);
+    }
+    uint32_t open = 1;
+    for (uint32_t it = 0; open && it <= ix.nil; ++it) {
+        int32_t id[M];
+        uint32_t next[M];
+#pragma unroll
+        for (int k = 0; k < M; ++k) { id[k] = ix.id[node[k]]; next[k] = ix.link[node[k]]; }
+        open = 0;
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            const bool found = id[k] == x[k];
+            slot[k] = found ? (int32_t)node[k] : slot[k];
+            node[k] = found ? ix.nil : next[k];
+            open |= node[k] ^ ix.nil;
+        }
+        open = __any_sync(0xffffffffu, open);
+    }
+    if (open) atomicOr(status, ST_PROBE_EXHAUSTED);
+#pragma unroll
+    for (int k = 0; k < M; ++k)
+        if (slot[k] >= (int32_t)ix.S) slot[k] = ix.slot[slot[k] - (int32_t)ix.S];
+}
+
 // With lifetimes above L on entry a slot that one token of a call reserves may be reserved again by a later one.  Nothing orders
 // the copies of a call's rows, so only the last reservation's row may be copied: the entries {id, slot (and more, from bit
 // LIST_SLOT_BITS on)} of a table's list whose slots hold another id by now become padding.  All threads of the block, behind a
@@ -185,16 +249,20 @@ __device__ __forceinline__ void drop_lost_rows(int2* list, uint32_t count, const
 // Bits 0 .. 3: the sign bits of a word's four bytes.
 __device__ __forceinline__ uint32_t signs(uint32_t w) { return (((w >> 7) & 0x01010101u) * 0x10204080u) >> 28; }
 
-// The thread's lifetimes to shared memory, its dead slots as bits (a byte per thread), the warp's number of them.
+// A thread's slots as bits.
+template <int SPT> struct SlotBits { using type = uint8_t; };
+template <> struct SlotBits<16> { using type = uint16_t; };
+
+// The thread's lifetimes to shared memory, its dead slots as bits, the warp's number of them.
 template <int SPT>
-__device__ __forceinline__ void store_lifetimes(int8_t* s_life, uint8_t* s_bits, uint32_t* s_ndead, bool own,
+__device__ __forceinline__ void store_lifetimes(int8_t* s_life, typename SlotBits<SPT>::type* s_bits, uint32_t* s_ndead, bool own,
                                                 const uint32_t (&w)[(SPT + 3) / 4])
 {
     uint32_t bits = 0;
 #pragma unroll
     for (int q = 0; q < (SPT + 3) / 4; ++q) bits |= signs(w[q]) << (4 * q);
     life_words_store<SPT>(s_life + threadIdx.x * SPT, own, w);
-    s_bits[threadIdx.x] = (uint8_t)bits;
+    s_bits[threadIdx.x] = (typename SlotBits<SPT>::type)bits;
     const uint32_t n = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(bits));
     if ((threadIdx.x & 31u) == 0) s_ndead[threadIdx.x >> 5] = n;
 }

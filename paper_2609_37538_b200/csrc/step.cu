@@ -45,12 +45,20 @@ struct StepLayout {
     uint32_t by_copying, by_groups;      // n / copying == n * by_copying >> 18 for every group and position; the same for groups
     uint32_t per_lane, per_token;        // words of 32 local positions to a lane; entries of a token in a block's list, at most
     uint32_t log_heads, nil;             // chains of the index; its closing node
+    uint32_t heads;                      // chains of a packed index
     uint32_t log_seen, log_asked;        // words of the copying blocks' sets: cached ids; ids of an earlier token, each
-    uint32_t node, head, life, bits, tot, ndead, cnt, sum, votes, miss, pos, dead, ids;    // first block
+    uint32_t node, link, fresh, head, life, bits, tot, ndead, cnt, sum, votes, miss, pos, dead, ids;    // first block
     uint32_t seen, asked, slots, id, mask, rest, list, their_ids;              // copying blocks
     uint32_t total;
 };
-// ask: rows are asked for early.  False if there is no room for that (without it there always is).
+// Tables above this take a packed index, and 16 slots a thread.  What bounds these is still the chain of passes on one SM, which
+// grows little with the slots: of two tokens of K = 2048 the second pass of the index, 0.9 us.  Over a cluster of its own (one
+// kernel for each stage) Stage One pays a barrier of the cluster a token instead, and Stage Two a launch and the hand-over through
+// memory: 16384 slots, in two kernels / in one, us per call: two tokens of K = 2048, 1, 4, 8, 16, 24 tables 21.4 / 12.7, 32.3 / 20.9, 44.7 /
+// 33.6, 72.9 / 62.9, 98.9 / 88.4; four tokens 33.1 / 18.9, 49.8 / 31.0, 72.1 / 53.3, 115.7 / 98.5, 160.5 / 143.3; three of K = 3000, one
+// table 33.4 / 20.4; from and to host memory, four tokens, 1, 16 tables 52.5 / 23.9, 142 / 108 (ids and outputs went by copies).
+constexpr uint32_t WIDE_SLOTS = 8192;
+// ask: rows are asked for early.  False if there is no room (without asking early there always is, up to WIDE_SLOTS).
 bool step_layout(StepLayout& o, uint32_t S, uint32_t K, uint32_t n_q, uint32_t nt, uint32_t copying, bool host_ids, bool ask)
 {
     // At least 32 groups a token, so that seven blocks have about the same to do: 9 tables with K = 256 30.8 us with groups of
@@ -69,16 +77,21 @@ bool step_layout(StepLayout& o, uint32_t S, uint32_t K, uint32_t n_q, uint32_t n
     o.nil = S + (n_q - 1u) * K;
     o.log_heads = 1u;
     while ((1u << o.log_heads) < 2u * S) ++o.log_heads;
+    o.heads = 1u << o.log_heads;
     o.log_seen = o.log_heads;                              // 64 bits an id
     o.log_asked = 2u;
     while ((1u << o.log_asked) < 2u * K) ++o.log_asked;
+    const bool packed = S > WIDE_SLOTS;
+    const uint32_t least_seen = o.log_seen - 2u;           // 16 bits an id
     const uint32_t ids = ask && host_ids ? align16(n_q * K * 4u) : 0u, room = (228u << 10) / (1024u / nt) - 2560u;
     for (;;) {
         uint32_t a = 0;
-        o.node = a;    a += align16((o.nil + 1u) * 8u);
-        o.head = a;    a += 4u << o.log_heads;
+        o.node = a;    a += align16((o.nil + 1u) * (packed ? 4u : 8u));            // nodes of the index; packed: their ids
+        o.link = a;    a += packed ? align16((o.nil + 1u) * 2u) : 0u;
+        o.fresh = a;   a += packed ? align16((n_q - 1u) * K * 2u) : 0u;
+        o.head = a;    a += 4u * o.heads;
         o.life = a;    a += align16(S);                    // lifetime per slot, one signed byte
-        o.bits = a;    a += align16(nt);                   // one bit per slot, set where it is dead (lifetime < 0)
+        o.bits = a;    a += align16(packed ? 2u * nt : nt);                        // one bit per slot, set where it is dead (lifetime < 0)
         o.tot = a;     a += 2u * 32u * 4u;                 // warps' miss totals, by parity
         o.ndead = a;   a += 2u * 32u * 4u;                 // warps' dead slots, by parity
         o.cnt = a;     a += 2u * 2u * 32u * 4u;            // warps' counts of the decay search, by parity
@@ -101,9 +114,24 @@ bool step_layout(StepLayout& o, uint32_t S, uint32_t K, uint32_t n_q, uint32_t n
         o.their_ids = a; a += ids;                         // received: the ids of a call with host buffers
         o.total = first > a ? first : a;
         if (o.total <= room) return true;
+        if (packed) {
+            // Both parts give way by themselves: the chains get what is left, down to one for eight slots, the sets half the bits each.
+            if (first > room) {
+                if (first - room > 4u * o.heads || o.heads - (first - room) / 4u < S / 8u + 4u) return false;
+                o.heads = (o.heads - (first - room) / 4u - 1u) & ~3u;
+            } else if (o.log_seen > least_seen) {
+                --o.log_seen;
+            } else if (o.log_asked > 2u && (2u << o.log_asked) > K) {
+                --o.log_asked;
+            } else {
+                return false;
+            }
+            continue;
+        }
         if (ask && a > room) return false;
         if ((1u << o.log_heads) <= S) return !ask;
         --o.log_heads;                                     // longer chains where the rest needs the room
+        o.heads /= 2u;
     }
 }
 constexpr uint32_t NO_ITEM = 0xFFFFFFFFu;
@@ -195,6 +223,8 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
                                              unsigned char* smem, const uint32_t a_mbar, const uint32_t a_sent, uint32_t* s_own)
 {
     constexpr int NV = (SPT + 3) / 4;                    // 4-slot vectors of ids / words of lifetimes per thread
+    constexpr bool PACKED = SPT > 8;                     // (such tables are a context's: no lifetimes above L)
+    constexpr uint32_t BITS = PACKED ? 16u : 8u;         // a thread's bits
     const uint32_t S = p.S, K = p.K, L = p.L, NIL = lay.nil;
     const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u, warp = tid >> 5, nw = nt >> 5;
     const uint32_t below = (1u << lane) - 1u;            // the lanes before this one
@@ -202,7 +232,9 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
     uint2*    s_node = reinterpret_cast<uint2*>(smem + lay.node);
     uint32_t* s_head = reinterpret_cast<uint32_t*>(smem + lay.head);
     int8_t*   s_life = reinterpret_cast<int8_t*>(smem + lay.life);
-    uint8_t*  s_bits = smem + lay.bits;                  // a thread's slots: set where dead
+    auto*     s_bits = reinterpret_cast<typename SlotBits<SPT>::type*>(smem + lay.bits);     // a thread's slots: set where dead
+    const PackedIndex ix = {reinterpret_cast<int32_t*>(smem + lay.node), reinterpret_cast<uint16_t*>(smem + lay.link),
+                            reinterpret_cast<uint16_t*>(smem + lay.fresh), s_head, lay.heads, NIL, S};
     uint32_t* s_tot  = reinterpret_cast<uint32_t*>(smem + lay.tot);
     uint32_t* s_ndead = reinterpret_cast<uint32_t*>(smem + lay.ndead);
     uint32_t* s_cnt  = reinterpret_cast<uint32_t*>(smem + lay.cnt);
@@ -215,8 +247,8 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
 
     // slot j is no longer dead (the count follows the bit, so that an id that comes twice is counted once)
     auto revive = [&](uint32_t j, uint32_t par) {
-        const uint32_t owner = j / SPT, bit = 1u << ((owner & 3u) * 8u + j % SPT);
-        if (atomicAnd(reinterpret_cast<uint32_t*>(s_bits) + owner / 4u, ~bit) & bit)
+        const uint32_t owner = j / SPT, in_word = 32u / BITS, bit = 1u << (owner % in_word * BITS + j % SPT);
+        if (atomicAnd(reinterpret_cast<uint32_t*>(s_bits) + owner / in_word, ~bit) & bit)
             atomicSub(&s_ndead[par + owner / 32u], 1u);
     };
     const uint32_t ipt = (K + nt - 1) / nt;              // ids per thread
@@ -233,8 +265,12 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
     // the clearing comes before the wait: under the previous kernel's tail
     const uint32_t table = p.table_id[ti], id_limit = p.id_limit[ti];
     int32_t N = p.verified_len[ti];
-    for (uint32_t i = tid; i < (1u << lay.log_heads) / 4; i += nt) reinterpret_cast<uint4*>(s_head)[i] = make_uint4(NIL, NIL, NIL, NIL);
-    if (tid == 0) s_node[NIL] = make_uint2(0xFFFFFFFEu, NIL);          // an id that nobody looks for
+    for (uint32_t i = tid; i < (PACKED ? lay.heads : 1u << lay.log_heads) / 4; i += nt) reinterpret_cast<uint4*>(s_head)[i] = make_uint4(NIL, NIL, NIL, NIL);
+    if constexpr (PACKED) {
+        if (tid == 0) { ix.id[NIL] = -2; ix.link[NIL] = (uint16_t)NIL; }
+    } else {
+        if (tid == 0) s_node[NIL] = make_uint2(0xFFFFFFFEu, NIL);      // an id that nobody looks for
+    }
     if (tid == 0) s_sum[0] = 0;
     if (ASK && tid < 2u * STEP_FEW_CLUSTER) s_own[tid] = 0;
     // Ids in host memory are there when the call is made, and nothing on the device writes them: a call that queues behind another
@@ -265,7 +301,8 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
 #pragma unroll
     for (int q = 0; q < NV; ++q)
         if (tid + q * nt < S / 4) stale_ids = stale_ids || t4[q].x >= N || t4[q].y >= N || t4[q].z >= N || t4[q].w >= N;
-    index_slots(t4, s_node, s_head, S, lay.log_heads, NIL);
+    if constexpr (PACKED) index_slots(t4, ix);
+    else index_slots(t4, s_node, s_head, S, lay.log_heads, NIL);
     uint32_t high = 0;                                   // lifetimes above L (only a caller's own state can have them)
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
@@ -277,7 +314,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
         cluster_sync();                                  // (the copying blocks have sent the ids)
         load_token(0);
     }
-    const bool unusual = __syncthreads_or(high != 0);
+    const bool unusual = __syncthreads_or(high != 0) && !PACKED;
 
     uint32_t list_off = 0, sum_miss = 0, sum_decay = 0, valid = 0;
     uint32_t shared = 0;                                 // SHARE: rows that other blocks may take (bit 31: there will be some)
@@ -304,7 +341,8 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
             valid += ok;
         }
         if (bad) atomicOr(p.status, ST_BAD_ID);                        // not fetched: reported and taken as padding
-        find_slots(xs, s_node, s_head, lay.log_heads, NIL, p.status, slot);
+        if constexpr (PACKED) find_slots(xs, ix, p.status, slot);
+        else find_slots(xs, s_node, s_head, lay.log_heads, NIL, p.status, slot);
         // with lifetimes above L on entry a slot reserved in this step may go to yet another id: its first node is stale
         if (unusual) {
 #pragma unroll
@@ -386,7 +424,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
             uint32_t bits = s_bits[tid], r, unused;
             warp_rank<SPT>(__popc(bits), below, r, unused);
             for (r += dead_before; bits && r < n_take; bits &= bits - 1u, ++r) s_dead[r] = (uint16_t)(j0 + __ffs((int)bits) - 1);
-            s_bits[tid] = (uint8_t)bits;                  // what is handed out is dead no more
+            s_bits[tid] = (typename SlotBits<SPT>::type)bits;          // what is handed out is dead no more
         }
         uint32_t left = __shfl_sync(0xffffffffu, t & 0xFFFFu, (int)warp);          // the warp's dead slots for the next token
         if (dead_before < n_take) left = left > n_take - dead_before ? left - (n_take - dead_before) : 0u;
@@ -439,13 +477,20 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
                 tell.row(g, k, share, x, j);
             }
             if (k < n_take) {
-                s_node[j].x = (uint32_t)x;
+                if constexpr (PACKED) ix.id[j] = x;
+                else s_node[j].x = (uint32_t)x;
                 s_life[j] = (int8_t)L;
                 if (share_it) list[(shared & ~SHARED_COMING) + k] = make_int2(x, j);
                 g_tok[j] = x >= N ? -1 : x;                            // speculative ids are forgotten (end of Alg. 4)
                 if (!last) {
                     const uint32_t n = S + list_off + k;
-                    s_node[n] = make_uint2((uint32_t)x, (uint32_t)j << 16 | atomicExch(&s_head[hash_id(x, lay.log_heads)], n));
+                    if constexpr (PACKED) {
+                        ix.id[n] = x;
+                        ix.slot[n - S] = (uint16_t)j;
+                        ix.link[n] = (uint16_t)atomicExch(ix.chain(x), n);
+                    } else {
+                        s_node[n] = make_uint2((uint32_t)x, (uint32_t)j << 16 | atomicExch(&s_head[hash_id(x, lay.log_heads)], n));
+                    }
                 }
             }
             O[i] = j;
@@ -469,7 +514,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
     if (stale_ids) {
         for (uint32_t q = 0; q < NV; ++q)
             for (uint32_t j = 4u * (tid + q * nt); j < 4u * (tid + q * nt) + 4u && j < S; ++j)
-                if ((int32_t)s_node[j].x >= N) g_tok[j] = -1;
+                if ((PACKED ? ix.id[j] : (int32_t)s_node[j].x) >= N) g_tok[j] = -1;
     }
     if (tid == 0) {
         TableStats* st = p.stats + table;                // (reductions: nothing waits for the old values)
@@ -897,6 +942,9 @@ template <int CAP, bool ASK, bool SHARE = false>
 const void* step_kernel(uint32_t spt, uint32_t ipt)
 {
     switch (spt) {
+        case 16: return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<16, 2, CAP, ASK, SHARE>)
+                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<16, 4, CAP, ASK, SHARE>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<16, 8, CAP, ASK, SHARE>);
         case 8:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 2, CAP, ASK, SHARE>)
                       : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 4, CAP, ASK, SHARE>)
                                  : reinterpret_cast<const void*>(avsg_step_kernel<8, 8, CAP, ASK, SHARE>);
@@ -924,8 +972,8 @@ void step_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, uint32_t n_
 // that is not left to their first launch).
 cudaError_t step_prepare(size_t max_smem)
 {
-    for (uint32_t spt : {2u, 4u, 8u})
-        for (uint32_t ipt = 2u; ipt <= spt; ipt *= 2u)                 // (K <= S)
+    for (uint32_t spt : {2u, 4u, 8u, 16u})
+        for (uint32_t ipt = 2u; ipt <= spt && ipt <= 8u; ipt *= 2u)    // (K <= S, and STEP_MAX_IDS)
             for (const void* k : {step_kernel<STEP_FEW_TABLES, true>(spt, ipt), step_kernel<STEP_FEW_TABLES, false>(spt, ipt), step_kernel<STEP_MAX_TABLES, true>(spt, ipt),
                                   step_kernel<STEP_MAX_TABLES, false>(spt, ipt), step_kernel<STEP_MAX_TABLES, false, true>(spt, ipt)}) {
                 cudaFuncAttributes fa;
@@ -935,6 +983,17 @@ cudaError_t step_prepare(size_t max_smem)
                 if (e != cudaSuccess) return e;
             }
     return cudaSuccess;
+}
+
+// Above WIDE_SLOTS: where the index has room (n_q and K decide), and not calls of few tokens with three and two blocks a table, whose
+// rows two kernels cut evenly over all SMs: K = 2048, two kernels / one, us: 36, 50, 74 tables, one token 83.9 / 83.0, 109.8 / 112.0, 154.9 /
+// 156.7; K = 1024, two tokens, 40, 64 tables 99.9 / 94.9, 149.0 / 147.3, but 64 cold ones 1103 / 1114; K = 2048, four tokens, 40, 64 tables
+// 248 / 234, 381 / 371.
+bool step_serves(uint32_t S, uint32_t K, uint32_t n_q, uint32_t cluster)
+{
+    StepLayout lay;
+    return S <= WIDE_SLOTS || (S <= STEP_MAX_SLOTS && K <= STEP_MAX_IDS && n_q + cluster >= 5u &&
+                               step_layout(lay, S, K, n_q, step_threads(S, K), cluster - 1u, false, false));
 }
 
 StepClusters step_clusters(size_t max_smem)

@@ -353,3 +353,44 @@ def test_the_default_geometry_brings_the_one_kernel_back():
         assert kernels(3) == 2, geometry
         ctx.set_transfer_geometry(0, 256)
         assert kernels(3) == 1 and kernels(74) == 1
+
+
+# Tables of 16384 slots: two, four and eight ids a thread; the fewest chains that fit (three tokens of 4096); the smallest K; many
+# tokens; the largest clusters of four, three and two blocks and one table more; four tokens of 4096, 8193 ids and one token with
+# three blocks take two kernels
+@pytest.mark.parametrize("n,K,n_q", [(1, 8192, 1), (2, 4097, 2), (8, 2048, 4), (9, 1, 8), (2, 33, 64), (3, 4096, 3), (33, 700, 1), (34, 700, 1),
+                                     (45, 600, 2), (46, 600, 2), (46, 600, 3), (74, 300, 4), (2, 4096, 4), (1, 8193, 1)])
+def test_tables_of_16384_slots(n, K, n_q):
+    import torch
+    import paper_2609_37538_b200 as avsg
+    S, L, context = 16384, 3, 30000
+    rng = np.random.default_rng([n, K, n_q])
+    kv = avsg.pinned_empty(context * RB)
+    tr.fill_kv(kv.data_ptr(), 1, 0, context, RB)
+    ctx = avsg.Context(n, S, RB, K, n_q, L)
+    orc = [OracleTable(S, RB, L) for _ in range(n)]
+    done = []
+    for c in range(7):
+        tabs = [int(t) for t in rng.permutation(n)]
+        ctx.set_transfer_mode(avsg.XFER_SM_OVERLAP if c % 2 else avsg.XFER_SM_BALANCED)
+        X = np.stack([[rng.choice([2 * K, context][c % 2] if K < context // 2 else context, K, replace=False) for _ in range(n_q)] for _ in tabs]).astype(np.int32)
+        X[:, 0, K // 2] = -1
+        N = context - 40 * c                             # shrinks: resident ids become unverified
+        if c == 5:
+            ctx.reset_async(tabs[:2])
+        host = c in (2, 4)
+        ids = torch.from_numpy(X).pin_memory() if host else torch.from_numpy(X).cuda()
+        done.append((tabs, X, N, (ctx.step_host if host else ctx.step)(tabs, ids, [kv] * n, [N] * n)))
+    torch.cuda.synchronize()
+    for c, (tabs, X, N, out) in enumerate(done):
+        for a, t in enumerate(tabs):
+            if c == 5 and a < 2:
+                orc[t].reset()
+            r = orc[t].step(X[a], N, kv.numpy(), RB)
+            assert (out.slots[a].cpu().numpy() == r.O).all() and (out.hit[a].cpu().numpy() == r.M).all(), (c, t)
+            assert (out.miss_count[a].cpu().numpy() == r.n).all(), (c, t)
+    for t in range(n):
+        assert (ctx.buffer(t).cpu().numpy() == orc[t].rows()).all(), t
+        tok, life = ctx.export_state(t)
+        assert (tok == orc[t].export_state()[0]).all() and (life == orc[t].export_state()[1]).all(), t
+    assert ctx.sync_status() == 0
