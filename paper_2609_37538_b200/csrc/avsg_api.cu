@@ -368,7 +368,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     if (cluster && !host_io) {
         auto step = [&](auto&& p) -> int {
             fill(p, 0, n);
-            p.flags = nullptr; p.out = out; p.early = step_early(p); p.shared = c->d_shared;
+            p.flags = nullptr; p.expect = n; p.out = out; p.early = step_early(p); p.shared = c->d_shared;
             CU(launch_step(p, cluster, stream));
             return AVSG_OK;
         };

@@ -369,6 +369,7 @@ def test_tables_of_16384_slots(n, K, n_q):
     tr.fill_kv(kv.data_ptr(), 1, 0, context, RB)
     ctx = avsg.Context(n, S, RB, K, n_q, L)
     orc = [OracleTable(S, RB, L) for _ in range(n)]
+    word = torch.zeros(1, dtype=torch.int64, device="cuda")
     done = []
     for c in range(7):
         tabs = [int(t) for t in rng.permutation(n)]
@@ -380,8 +381,13 @@ def test_tables_of_16384_slots(n, K, n_q):
             ctx.reset_async(tabs[:2])
         host = c in (2, 4)
         ids = torch.from_numpy(X).pin_memory() if host else torch.from_numpy(X).cuda()
-        done.append((tabs, X, N, (ctx.step_host if host else ctx.step)(tabs, ids, [kv] * n, [N] * n)))
+        early = {} if host else dict(stage_one_done=(word, c + 1) if c in (0, 1, 5) else None, want_arriving=c in (3, 5))
+        done.append((tabs, X, N, (ctx.step_host if host else ctx.step)(tabs, ids, [kv] * n, [N] * n, **early)))
+        if c == 1:
+            torch.cuda.synchronize()
+            assert int(word.item()) == 2
     torch.cuda.synchronize()
+    assert int(word.item()) == 6
     for c, (tabs, X, N, out) in enumerate(done):
         for a, t in enumerate(tabs):
             if c == 5 and a < 2:
@@ -389,6 +395,7 @@ def test_tables_of_16384_slots(n, K, n_q):
             r = orc[t].step(X[a], N, kv.numpy(), RB)
             assert (out.slots[a].cpu().numpy() == r.O).all() and (out.hit[a].cpu().numpy() == r.M).all(), (c, t)
             assert (out.miss_count[a].cpu().numpy() == r.n).all(), (c, t)
+            assert c not in (3, 5) or (out.arriving[a].cpu().numpy() == r.arriving).all(), (c, t)
     for t in range(n):
         assert (ctx.buffer(t).cpu().numpy() == orc[t].rows()).all(), t
         tok, life = ctx.export_state(t)
