@@ -74,12 +74,14 @@ extern "C" {
                                        within a table: by position, or even from 34 tables
                                        (of 8192 slots) on, where rows of a table that misses
                                        more than 512 ids of a token are also taken over by
-                                       blocks of others that are through (not with arriving,
-                                       timing or an own transfer geometry, nor with
-                                       stage_one_done above three tables, nor tables above
+                                       blocks of others that are through (not with
+                                       timing or an own transfer geometry, nor tables above
                                        16384 slots; of 16384 slots where n_tokens and topk
                                        leave room for them in one SM's shared memory, up to
-                                       33 tables, and more where there are several tokens).
+                                       33 tables, and more where there are several tokens;
+                                       with stage_one_done up to 18 tables, whose blocks
+                                       leave half of the SMs free, more of smaller ones;
+                                       with arriving up to 33, and rows of up to 1536 bytes).
                                        Its blocks take whole SMs while they run: who wants
                                        room for other kernels beside the call sets a
                                        transfer geometry (100 calls of 8, 32, 64 tables
@@ -199,7 +201,9 @@ typedef struct {
                                       avsg_step on the SAME stream with programmatic stream
                                       serialization (the operator's kernels release their
                                       dependents as soon as they run, and all their blocks
-                                      are resident by then): it polls the word, works on
+                                      are resident by then; a call in one kernel leaves it
+                                      the SMs that its own blocks do not take, at least
+                                      half): it polls the word, works on
                                       the hits, and executes griddepcontrol.wait before it
                                       touches a missed row.  avsg_step only:
                                       avsg_step_host (whose caller waits for the whole call)

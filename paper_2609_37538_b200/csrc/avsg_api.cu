@@ -237,14 +237,20 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     HostOut out;
     bool host_ids = false;
     // One kernel for both stages, where the tables' clusters fit the device (see avsg_step_kernel for what it saves).  Its
-    // blocks take whole SMs and the next grid starts behind them: a caller who wants the hits before the rows are there
-    // (stage_one_done) gets that from a call of more than a few tables only with the two kernels.
+    // blocks take whole SMs.  So a caller who wants the hits before the rows are there (stage_one_done) gets it from calls that
+    // leave half of the SMs to the kernel that starts on the hits (or are small: STEP_EARLY_TABLES), and that kernel may start
+    // at once, although the grid behind a call then finds other SMs free (from 11 GB, 16 tables 87.8 us, if it came late 82.9).
+    // K = 2048, two tokens, with both early outputs, three kernels / one: 2, 6, 8, 12, 16, 18 tables 25.4 / 14.6, 38.8 / 27.1, 45.0 /
+    // 33.1, 57.9 / 46.7, 71.7 / 60.4, 78.2 / 66.4 us; from 11 GB, 6, 16 tables 48.3 / 37.7, 96.7 / 87.4; 16384 slots, four tokens, 16
+    // tables 109.1 / 104.3.  (22 and 33 tables would gain 12 us too, with 60 and 16 SMs left.)
     const bool sm_copies = c->cfg.transfer_mode == AVSG_XFER_SM_BALANCED || c->cfg.transfer_mode == AVSG_XFER_SM_OVERLAP;
     uint32_t cluster = 0;
-    if (sm_copies && c->one_kernel && n_q <= STEP_MAX_TOKENS && !a->arriving && !c->timing && !c->geometry_set &&
-        (!a->stage_one_done || n <= STEP_EARLY_TABLES)) {
+    if (sm_copies && c->one_kernel && n_q <= STEP_MAX_TOKENS && !c->timing && !c->geometry_set) {
         cluster = c->step_clusters.of(n, step_threads(c->cfg.buffer_slots, K));
-        if (cluster && !step_serves(c->cfg.buffer_slots, K, n_q, cluster)) cluster = 0;
+        if (cluster && !step_serves(c->cfg.buffer_slots, K, n_q, cluster, c->cfg.row_bytes, a->arriving != nullptr)) cluster = 0;
+        if (a->stage_one_done && n > STEP_EARLY_TABLES &&
+            (uint64_t)n * cluster * step_threads(c->cfg.buffer_slots, K) > (uint64_t)c->sm_count / 2u * 1024u)
+            cluster = 0;
     }
     const bool in_place = (K % 8u == 0 && reinterpret_cast<uint64_t>(a->indices) % 32u == 0) || n_ids <= HOST_ODD_IDS;
     if (host_io && c->cfg.index_mode != AVSG_INDEX_PAPER && (c->s1_cluster == 1 || cluster) && in_place && sm_copies) {
@@ -368,7 +374,9 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     if (cluster && !host_io) {
         auto step = [&](auto&& p) -> int {
             fill(p, 0, n);
-            p.flags = nullptr; p.expect = n; p.out = out; p.early = step_early(p); p.shared = c->d_shared;
+            p.flags = nullptr; p.expect = n; p.out = out; p.shared = c->d_shared; p.arriving = a->arriving;
+            p.done_seq = reinterpret_cast<unsigned long long*>(a->stage_one_done);
+            p.early = a->stage_one_done || step_early(p);
             CU(launch_step(p, cluster, stream));
             return AVSG_OK;
         };

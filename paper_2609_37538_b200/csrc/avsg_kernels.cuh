@@ -115,6 +115,7 @@ struct S1ParamsT {
     int32_t*       slots;        // [n][n_q][K]
     uint8_t*       hit;          // [n][n_q][K] or null
     int32_t*       miss_count;   // [n][n_q] or null
+    uint8_t*       arriving = nullptr;          // a call in one kernel: [n][n_q][K] or null
     uint32_t S, logH, row_bytes, K, n_q, L;
     uint32_t first;              // index within the call of this launch's first table
     uint32_t n_launch;           // tables of this launch (the grid may have fewer blocks: a block then serves several)
@@ -243,8 +244,9 @@ struct StepClusters {
     }
 };
 cudaError_t step_prepare(size_t max_smem);
-// Whether the first block of a cluster has room for such a table (with up to 8192 slots it always has).
-bool step_serves(uint32_t S, uint32_t K, uint32_t n_q, uint32_t cluster);
+// Whether the first block of a cluster has room for such a table (with up to 8192 slots it always has); with the `arriving`
+// output: whether rows are asked for early.
+bool step_serves(uint32_t S, uint32_t K, uint32_t n_q, uint32_t cluster, uint32_t row_bytes, bool arriving);
 StepClusters step_clusters(size_t max_smem);            // after step_prepare
 // Whether the grid behind a call in one kernel may start under it (see the kernel).  Up to three tables, and up to eight
 // that reach little host memory (id_limit: rows a table's ids can reach).  Early / late, calls of K = 2048: one table 13.2 / 13.4

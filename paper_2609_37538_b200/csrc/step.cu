@@ -217,14 +217,17 @@ __device__ __forceinline__ void tell_at_last(const Tell tell, uint32_t n_q, uint
 // The first block of a cluster: Stage One.  SPT slots per thread (a power of two): S <= SPT * blockDim.x.  IPT: the most
 // ids a thread has of a token (K <= S, so SPT is always enough).  a_mbar: the copying blocks' mbarriers, one per token.
 // The passes are those of avsg_stage_one_kernel, which says what they are and why.  ASK: rows are asked for early.  SHARE: rows of a
-// table with very many misses may be copied by other tables' blocks.
-template <int SPT, int IPT, bool ASK, bool SHARE, int CAP>
+// table with very many misses may be copied by other tables' blocks.  ARRIVING: the output of that name is written as well: a hit
+// whose node is not its slot's own is on a slot that an earlier token of the call has reserved, which its node says (an instance of
+// its own: in a pass at the end, or as a question in every call, it costs all others more than it gives these).
+template <int SPT, int IPT, bool ASK, bool SHARE, bool ARRIVING, int CAP>
 __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const StepLayout& lay, const uint32_t ti, const uint32_t copying,
                                              unsigned char* smem, const uint32_t a_mbar, const uint32_t a_sent, uint32_t* s_own)
 {
     constexpr int NV = (SPT + 3) / 4;                    // 4-slot vectors of ids / words of lifetimes per thread
     constexpr bool PACKED = SPT > 8;                     // (such tables are a context's: no lifetimes above L)
     constexpr uint32_t BITS = PACKED ? 16u : 8u;         // a thread's bits
+    constexpr uint32_t FRESH = 1u << 15, MARK = ARRIVING ? FRESH : 0u;           // above every slot: at those that this call reserves
     const uint32_t S = p.S, K = p.K, L = p.L, NIL = lay.nil;
     const uint32_t tid = threadIdx.x, nt = blockDim.x, lane = tid & 31u, warp = tid >> 5, nw = nt >> 5;
     const uint32_t below = (1u << lane) - 1u;            // the lanes before this one
@@ -327,6 +330,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
         const size_t row = ((size_t)ti * p.n_q + g) * K;
         int32_t* O = p.slots + row;
         uint8_t* Hm = p.hit ? p.hit + row : nullptr;
+        uint8_t* A = ARRIVING ? p.arriving + row : nullptr;
 
         // ---- lookups; hits: lifetime <- L, slot and flag out (Pass 1 + Pass 2) ----
         // (pass after pass over the thread's ids, so that their reads are in flight together)
@@ -343,6 +347,12 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
         if (bad) atomicOr(p.status, ST_BAD_ID);                        // not fetched: reported and taken as padding
         if constexpr (PACKED) find_slots(xs, ix, p.status, slot);
         else find_slots(xs, s_node, s_head, lay.log_heads, NIL, p.status, slot);
+        uint32_t fresh = 0;                              // hits on slots that this call has reserved
+        if constexpr (ARRIVING) {
+#pragma unroll
+            for (int k = 0; k < IPT; ++k)
+                if (slot[k] >= (int32_t)FRESH) { slot[k] -= (int32_t)FRESH; fresh |= 1u << k; }
+        }
         // with lifetimes above L on entry a slot reserved in this step may go to yet another id: its first node is stale
         if (unusual) {
 #pragma unroll
@@ -363,6 +373,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
             if (slot[k] >= 0) s_life[slot[k]] = (int8_t)L;
             if (store) O[i0 + 32u * k] = slot[k];
             if (store && Hm) Hm[i0 + 32u * k] = slot[k] >= 0;
+            if (ARRIVING && store) A[i0 + 32u * k] = fresh >> k & 1u;
             revived = revived || was[k] < 0;
         }
         if (revived) {
@@ -486,15 +497,16 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
                     const uint32_t n = S + list_off + k;
                     if constexpr (PACKED) {
                         ix.id[n] = x;
-                        ix.slot[n - S] = (uint16_t)j;
+                        ix.slot[n - S] = (uint16_t)((uint32_t)j + MARK);
                         ix.link[n] = (uint16_t)atomicExch(ix.chain(x), n);
                     } else {
-                        s_node[n] = make_uint2((uint32_t)x, (uint32_t)j << 16 | atomicExch(&s_head[hash_id(x, lay.log_heads)], n));
+                        s_node[n] = make_uint2((uint32_t)x, ((uint32_t)j + MARK) << 16 | atomicExch(&s_head[hash_id(x, lay.log_heads)], n));
                     }
                 }
             }
             O[i] = j;
             if (Hm) Hm[i] = 0;
+            if (ARRIVING) A[i] = j >= 0;
         }
         list_off += n_take;
         if (share_it) shared += n_take;
@@ -767,7 +779,7 @@ __device__ __forceinline__ void take_shared_rows(const S1ParamsT<CAP>& p, const 
 // one, its own blocks' too, the cold calls were quicker still (45 tables 214), but a call where most tables had many misses
 // lost 5 to 20 %: the requests for claims and list entries wait behind the rows'.  Several rows of a warp at once bring an SM
 // from 20 rows a us to 28 at most.
-template <int SPT, int IPT, int CAP, bool ASK, bool SHARE>
+template <int SPT, int IPT, int CAP, bool ASK, bool SHARE, bool ARRIVING>
 __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constant__ S1ParamsT<CAP> p, const __grid_constant__ StepLayout lay)
 {
     static_assert(!ASK || !SHARE, "rows that are shared are copied in the order of the misses");
@@ -797,7 +809,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
     __syncthreads();
     cluster_arrive();
     if (rank == 0) {
-        place_tokens<SPT, IPT, ASK, SHARE>(p, lay, ti, copying, smem, smem_u32(s_mbar), smem_u32(s_sent), s_own);
+        place_tokens<SPT, IPT, ASK, SHARE, ARRIVING>(p, lay, ti, copying, smem, smem_u32(s_mbar), smem_u32(s_sent), s_own);
         __syncwarp();
         cluster_arrive();                                              // the outputs are written, everything is sent
         return;
@@ -938,19 +950,19 @@ uint32_t step_threads(uint32_t S, uint32_t K)
 
 namespace {
 
-template <int CAP, bool ASK, bool SHARE = false>
+template <int CAP, bool ASK, bool SHARE = false, bool ARRIVING = false>
 const void* step_kernel(uint32_t spt, uint32_t ipt)
 {
     switch (spt) {
-        case 16: return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<16, 2, CAP, ASK, SHARE>)
-                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<16, 4, CAP, ASK, SHARE>)
-                                 : reinterpret_cast<const void*>(avsg_step_kernel<16, 8, CAP, ASK, SHARE>);
-        case 8:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 2, CAP, ASK, SHARE>)
-                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 4, CAP, ASK, SHARE>)
-                                 : reinterpret_cast<const void*>(avsg_step_kernel<8, 8, CAP, ASK, SHARE>);
-        case 4:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<4, 2, CAP, ASK, SHARE>)
-                                 : reinterpret_cast<const void*>(avsg_step_kernel<4, 4, CAP, ASK, SHARE>);
-        default: return reinterpret_cast<const void*>(avsg_step_kernel<2, 2, CAP, ASK, SHARE>);
+        case 16: return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<16, 2, CAP, ASK, SHARE, ARRIVING>)
+                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<16, 4, CAP, ASK, SHARE, ARRIVING>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<16, 8, CAP, ASK, SHARE, ARRIVING>);
+        case 8:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 2, CAP, ASK, SHARE, ARRIVING>)
+                      : ipt <= 4 ? reinterpret_cast<const void*>(avsg_step_kernel<8, 4, CAP, ASK, SHARE, ARRIVING>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<8, 8, CAP, ASK, SHARE, ARRIVING>);
+        case 4:  return ipt <= 2 ? reinterpret_cast<const void*>(avsg_step_kernel<4, 2, CAP, ASK, SHARE, ARRIVING>)
+                                 : reinterpret_cast<const void*>(avsg_step_kernel<4, 4, CAP, ASK, SHARE, ARRIVING>);
+        default: return reinterpret_cast<const void*>(avsg_step_kernel<2, 2, CAP, ASK, SHARE, ARRIVING>);
     }
 }
 
@@ -975,7 +987,8 @@ cudaError_t step_prepare(size_t max_smem)
     for (uint32_t spt : {2u, 4u, 8u, 16u})
         for (uint32_t ipt = 2u; ipt <= spt && ipt <= 8u; ipt *= 2u)    // (K <= S, and STEP_MAX_IDS)
             for (const void* k : {step_kernel<STEP_FEW_TABLES, true>(spt, ipt), step_kernel<STEP_FEW_TABLES, false>(spt, ipt), step_kernel<STEP_MAX_TABLES, true>(spt, ipt),
-                                  step_kernel<STEP_MAX_TABLES, false>(spt, ipt), step_kernel<STEP_MAX_TABLES, false, true>(spt, ipt)}) {
+                                  step_kernel<STEP_MAX_TABLES, false>(spt, ipt), step_kernel<STEP_MAX_TABLES, false, true>(spt, ipt),
+                                  step_kernel<STEP_FEW_TABLES, true, false, true>(spt, ipt), step_kernel<STEP_MAX_TABLES, true, false, true>(spt, ipt)}) {
                 cudaFuncAttributes fa;
                 cudaError_t e = cudaFuncGetAttributes(&fa, k);
                 if (e == cudaSuccess)
@@ -989,9 +1002,11 @@ cudaError_t step_prepare(size_t max_smem)
 // rows two kernels cut evenly over all SMs: K = 2048, two kernels / one, us: 36, 50, 74 tables, one token 83.9 / 83.0, 109.8 / 112.0, 154.9 /
 // 156.7; K = 1024, two tokens, 40, 64 tables 99.9 / 94.9, 149.0 / 147.3, but 64 cold ones 1103 / 1114; K = 2048, four tokens, 40, 64 tables
 // 248 / 234, 381 / 371.
-bool step_serves(uint32_t S, uint32_t K, uint32_t n_q, uint32_t cluster)
+bool step_serves(uint32_t S, uint32_t K, uint32_t n_q, uint32_t cluster, uint32_t row_bytes, bool arriving)
 {
     StepLayout lay;
+    if (arriving && (cluster < SHARED_CLUSTER || row_bytes > 16u * ROW_CHUNKS || !step_layout(lay, S, K, n_q, step_threads(S, K), cluster - 1u, false, true)))
+        return false;
     return S <= WIDE_SLOTS || (S <= STEP_MAX_SLOTS && K <= STEP_MAX_IDS && n_q + cluster >= 5u &&
                                step_layout(lay, S, K, n_q, step_threads(S, K), cluster - 1u, false, false));
 }
@@ -1027,7 +1042,7 @@ cudaError_t launch_step(const S1ParamsT<CAP>& p, uint32_t cluster, cudaStream_t 
     cfg.numAttrs = 2;
     void* args[] = {const_cast<S1ParamsT<CAP>*>(&p), &lay};
     const uint32_t spt = p.S / nt, ipt = (p.K + nt - 1) / nt;
-    const void* kernel = ask ? step_kernel<CAP, true>(spt, ipt) : step_kernel<CAP, false>(spt, ipt);
+    const void* kernel = ask && p.arriving ? step_kernel<CAP, true, false, true>(spt, ipt) : ask ? step_kernel<CAP, true>(spt, ipt) : step_kernel<CAP, false>(spt, ipt);
     if constexpr (CAP == STEP_MAX_TABLES)
         if (share) kernel = step_kernel<CAP, false, true>(spt, ipt);
     return cudaLaunchKernelExC(&cfg, kernel, args);

@@ -401,3 +401,46 @@ def test_tables_of_16384_slots(n, K, n_q):
         tok, life = ctx.export_state(t)
         assert (tok == orc[t].export_state()[0]).all() and (life == orc[t].export_state()[1]).all(), t
     assert ctx.sync_status() == 0
+
+
+# One to eight ids and two to sixteen slots a thread; the most tables of 8192 and 1024 slots whose blocks leave half of 148 SMs free, and
+# one more; rows too long to be asked for early (three kernels)
+@pytest.mark.parametrize("n,S,K,n_q,rb", [(1, 256, 64, 4, 48), (2, 1024, 300, 3, 48), (4, 4096, 2000, 2, 48), (4, 4096, 500, 5, 48), (18, 8192, 512, 3, 48),
+                                          (19, 8192, 512, 3, 48), (37, 1024, 200, 3, 48), (38, 1024, 200, 3, 48), (3, 8192, 4000, 2, 48), (5, 8192, 4097, 1, 48),
+                                          (2, 16384, 4000, 3, 48), (4, 16384, 2000, 5, 48), (6, 16384, 8000, 1, 48), (2, 8192, 600, 3, 1552)])
+def test_early_outputs(n, S, K, n_q, rb):
+    """Ids from so few that many hits are on slots that the call has just reserved, and tables too small for all of them."""
+    import torch
+    import paper_2609_37538_b200 as avsg
+    L, context = 3, 2 * S + 100
+    rng = np.random.default_rng([n, S, K])
+    kv = avsg.pinned_empty(context * rb)
+    tr.fill_kv(kv.data_ptr(), 1, 0, context, rb)
+    ctx = avsg.Context(n, S, rb, K, n_q, L)
+    orc = [OracleTable(S, rb, L) for _ in range(n)]
+    word = torch.zeros(1, dtype=torch.int64, device="cuda")
+    done = []
+    for c in range(6):
+        X = np.empty((n, n_q, K), np.int32)
+        for t in range(n):
+            some = rng.choice(context, min(context, K + K // 2 + 8), replace=False)
+            for g in range(n_q):
+                X[t, g] = rng.choice(some, K, replace=False)
+        X[:, n_q - 1, K // 3] = -1
+        out = ctx.step(list(range(n)), torch.from_numpy(X).cuda(), [kv] * n, [context - 9 * c] * n, want_hit=c != 3,
+                       stage_one_done=(word, c + 1) if c != 2 else None, want_arriving=c != 1)
+        done.append((X, out, word.clone()))
+    torch.cuda.synchronize()
+    fresh = 0
+    for c, (X, out, w) in enumerate(done):
+        assert int(w.item()) == (2 if c == 2 else c + 1)
+        for t in range(n):
+            r = orc[t].step(X[t], context - 9 * c, kv.numpy(), rb)
+            assert (out.slots[t].cpu().numpy() == r.O).all() and (c == 3 or (out.hit[t].cpu().numpy() == r.M).all()), (c, t)
+            assert (out.miss_count[t].cpu().numpy() == r.n).all(), (c, t)
+            assert c == 1 or (out.arriving[t].cpu().numpy() == r.arriving).all(), (c, t)
+            fresh += int(((r.arriving == 1) & (r.M == 1)).sum())
+    assert n_q == 1 or fresh > 0
+    for t in range(n):
+        assert (ctx.buffer(t).cpu().numpy() == orc[t].rows()).all(), t
+    assert ctx.sync_status() == 0
