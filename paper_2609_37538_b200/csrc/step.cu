@@ -145,6 +145,17 @@ __device__ __forceinline__ bool wait_for(uint32_t mbar, uint32_t limit)
     return __all_sync(0xffffffffu, spin < limit);
 }
 
+// Programmatic dependent launch: this grid may have been started while the previous kernel of the stream was still running; nothing
+// that the device writes is read before that kernel has completed.  Only then may the next grid start under this one: let go at
+// the start, two and three grids wait behind one another, and each hears late that its turn has come (one table, K = 2048, one and
+// two tokens 7.78, 11.12 us, now 7.45, 10.72; S = K = 2048 / 4, two tokens 7.94, 7.61; S = 256 5.55, 5.26; two tables 13.3, 13.0).
+template <typename P>
+__device__ __forceinline__ void wait_for_previous(const P& p)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (p.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // What the copying blocks are told.  Where they ask for rows early: `token`, that block `to` has n misses in its positions; `miss`,
 // to the block that position i belongs to, the slot, where the position's place is and in the next entry of its list.  Where
 // they don't, the rows to copy, in the order of the misses: in turn, or (share) `share` neighbours to a block; `head`, how many of n
@@ -280,9 +291,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
     // fetches its first ones while that one's rows travel (32 tables: 5 us of link time and a round trip).
     if (!ASK && p.host_ids) load_token(0);
 
-    // Programmatic dependent launch: this grid may have been started while the previous kernel of the stream
-    // was still running; nothing that the device writes is read before that kernel has completed.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    wait_for_previous(p);
 
     const uint32_t j0 = tid * SPT;                       // first of the thread's slots
     const bool own = j0 < S;
@@ -608,7 +617,7 @@ __device__ __forceinline__ Item match(const S1ParamsT<CAP>& p, const StepLayout&
 #pragma unroll
             for (int m = 0; m < OWN; ++m) x[m] = from + m * step < all ? __ldcv(g_ids + from + m * step) : -1;
             if (first) {
-                asm volatile("griddepcontrol.wait;" ::: "memory");
+                wait_for_previous(p);
                 cluster_wait();
                 first = 0;
             }
@@ -623,10 +632,8 @@ __device__ __forceinline__ Item match(const S1ParamsT<CAP>& p, const StepLayout&
         }
         cluster_sync();
     } else {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        cluster_wait();
+        wait_for_previous(p);
     }
-    cluster_arrive_relaxed();                            // (what this block sends is sent)
 
     // ---- every global load is issued first: cached ids, the first token's, the block's own ids ----
     // Nothing orders the reads of cached ids before the first block's stores to them.  An id of this call that is read too early
@@ -635,6 +642,7 @@ __device__ __forceinline__ Item match(const S1ParamsT<CAP>& p, const StepLayout&
     // dropped, because the position stays NOT_MISSED.  So sets decide what is asked for, and what has been received what is stored.
     int4 t4[NV];
     int32_t xo[OWN], xe[IPT];
+    uint32_t xg[OWN];                                    // the tokens of xo[]
     const int4* g_tok = reinterpret_cast<const int4*>(p.tok + (size_t)p.table_id[ti] * S);
 #pragma unroll
     for (int q = 0; q < NV; ++q)
@@ -642,12 +650,12 @@ __device__ __forceinline__ Item match(const S1ParamsT<CAP>& p, const StepLayout&
     auto load_own = [&](uint32_t from) {
 #pragma unroll
         for (int m = 0; m < OWN; ++m) {
-            const uint32_t n = (from + warp + W * m) * 32u + lane;
+            const uint32_t word = from + warp + W * m, n = word * 32u + lane;
+            if (word * 32u >= mine) break;               // (most blocks have one or two words a warp: what none has costs nothing)
             xo[m] = -1;
-            if (n < mine) {
-                const Place q = place(lay, rank, copying, n);
-                if (q.i < K) xo[m] = id_at(q.g * K + q.i);
-            }
+            const Place q = place(lay, rank, copying, n);
+            xg[m] = q.g;
+            if (n < mine && q.i < K) xo[m] = id_at(q.g * K + q.i);
         }
     };
     auto load_earlier = [&](uint32_t g) {
@@ -657,6 +665,8 @@ __device__ __forceinline__ Item match(const S1ParamsT<CAP>& p, const StepLayout&
     };
     if (p.n_q > 1u) load_earlier(0);
     load_own(0);
+    if (!p.host_ids) cluster_wait();                     // (under the loads)
+    cluster_arrive_relaxed();                            // (what this block sends is sent)
     __syncthreads();                                 // the sets are empty
 #pragma unroll
     for (int q = 0; q < NV; ++q)
@@ -674,22 +684,22 @@ __device__ __forceinline__ Item match(const S1ParamsT<CAP>& p, const StepLayout&
     }
     __syncthreads();
     Item item = {NO_ITEM, 0u, 0u};
+    const uint32_t first_token = positions_of(lay, rank, lay.groups);
     for (uint32_t from = 0; from * 32u < mine; from += OWN * W) {
         if (from) load_own(from);
 #pragma unroll
         for (int m = 0; m < OWN; ++m) {
             const uint32_t word = from + warp + W * m, n = word * 32u + lane;
             if (word * 32u >= mine) break;
-            const uint32_t g = place(lay, rank, copying, n).g;
             const int32_t x = xo[m];
             bool certain = (uint32_t)x < id_limit && !set_has(s_seen, lay.log_seen, x);
-            for (uint32_t e = 0; e < g && certain; ++e) certain = !set_has(s_asked + e * asked_words, lay.log_asked, x);
+            for (uint32_t e = 0; e < xg[m] && certain; ++e) certain = !set_has(s_asked + e * asked_words, lay.log_asked, x);
             const uint32_t votes = __ballot_sync(0xffffffffu, certain);
             s_id[n] = x;
             uint32_t rest = votes;
             const uint32_t l = __ffs((int)votes) - 1u;
             // (a row of a later token is left: the queue has the tokens in order, and who holds one copies nothing until it is placed)
-            if (votes && item.n == NO_ITEM && __shfl_sync(0xffffffffu, g, (int)l) == 0) {
+            if (votes && item.n == NO_ITEM && word * 32u + l < first_token) {
                 item = {word * 32u + l, 0u, (uint32_t)__shfl_sync(0xffffffffu, x, (int)l)};
                 rest &= rest - 1u;
             }
@@ -793,7 +803,6 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
     const uint32_t rank = cluster_rank(), cluster = !ASK && FEW ? STEP_FEW_CLUSTER : cluster_size(), copying = cluster - 1u;
     const uint32_t ti = blockIdx.x / cluster, lane = threadIdx.x & 31u, W = blockDim.x >> 5, warp = threadIdx.x >> 5;
     uint32_t* s_slots = reinterpret_cast<uint32_t*>(smem + lay.slots);
-    if (p.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (SHARE && threadIdx.x == 0) s_mine = 0xFFFFFFFFu;
     if (rank != 0) {
         if (threadIdx.x < p.n_q) {
@@ -811,7 +820,10 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
     if (rank == 0) {
         place_tokens<SPT, IPT, ASK, SHARE, ARRIVING>(p, lay, ti, copying, smem, smem_u32(s_mbar), smem_u32(s_sent), s_own);
         __syncwarp();
-        cluster_arrive();                                              // the outputs are written, everything is sent
+        // Everything is sent.  Written, too, where other blocks read it; else nobody has to wait until the memory system says so (the
+        // blocks of one table's call stood 0.6 us behind their last rows: K = 2048, two tokens 10.35, now 10.19; S = 2048 7.48, 7.33).
+        if (SHARE || p.out.n_slots) cluster_arrive();
+        else cluster_arrive_relaxed();
         return;
     }
     const uint32_t cpr = p.row_bytes >> 4;
@@ -880,7 +892,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
             next();
         }
     } else {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        wait_for_previous(p);
         cluster_wait();
         cluster_arrive();
         uint32_t from = 0;                                             // the warp that is next
