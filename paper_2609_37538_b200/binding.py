@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libavsg.so: argument marshalling only.
+"""Thin binding of libavsg.so: argument marshalling only, by ctypes and, for
+the calls of every step, by an extension module (csrc/python_calls.cpp).
 
 Every step of the operator runs in the CUDA kernels behind the C ABI
 (include/avsg.h).  PyTorch supplies device tensors, pinned host tensors and
@@ -9,6 +10,7 @@ from __future__ import annotations
 
 import array
 import ctypes
+import functools
 import os
 import struct
 from typing import List, Optional, Sequence, Union
@@ -79,7 +81,20 @@ class AvsgError(RuntimeError):
         self.code = code
 
 
-_lib = None
+_lib = _calls = None
+
+
+def _python_calls():
+    """The extension module (built in-tree by build.build_library); raises if it is missing."""
+    global _calls
+    if _calls is None:
+        try:
+            from . import _python_calls as module
+        except ImportError as e:
+            raise RuntimeError("the extension module _python_calls is missing: run `python __graft_entry__.py` to build it") from e
+        module.set_binding(_addr, _c_array, _stream_handle, None, None)
+        _calls = module
+    return _calls
 
 
 def load_library():
@@ -192,6 +207,7 @@ def _current_stream() -> int:
         raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
         if raw is not None and dev is not None:
             _current_stream_fn = lambda: raw(dev())
+            _python_calls().set_binding(_addr, _c_array, _stream_handle, raw, dev)     # (the extension asks them itself from now on)
         else:
             _current_stream_fn = lambda: torch.cuda.current_stream().cuda_stream
     return _current_stream_fn()
@@ -221,6 +237,20 @@ class StepOutput:
         self.slots, self.hit, self.miss_count, self.arriving = slots, hit, miss_count, arriving
 
 
+def _address_of(function) -> int:
+    return ctypes.cast(function, ctypes.c_void_p).value
+
+
+def _set_lengths(vlen, pack_into, values) -> None:
+    """Verified lengths from any iterable of n numbers."""
+    if not isinstance(values, (list, tuple)):
+        values = list(values)                            # (an iterator can be read once only)
+    try:
+        pack_into(vlen, 0, *values)
+    except struct.error:                                 # not n integers that fit: as the element type converts them
+        vlen[:] = [int(v) for v in values]
+
+
 class PreparedCall:
     """The argument block of one recurring call (same tables, same host KV): built once, re-used per step."""
 
@@ -234,7 +264,6 @@ class PreparedCall:
         self._kv = (ctypes.c_void_p * n)(*[_addr(k) for k in kv])
         self._stride = (ctypes.c_uint64 * n)(*[int(s) for s in row_stride]) if row_stride is not None else None
         self._vlen = (ctypes.c_int32 * n)()
-        self._pack_vlen = struct.Struct("=%di" % n).pack_into
         self._rows = (ctypes.c_uint32 * n)(*[int(r) for r in kv_rows]) if kv_rows is not None else None
         a = AvsgStepArgs()
         a.n, a.n_tokens, a.topk = n, n_tokens, topk
@@ -245,6 +274,13 @@ class PreparedCall:
         a.kv_rows = ctypes.addressof(self._rows) if self._rows is not None else None
         self.args = a
         self._ref = ctypes.byref(a)
+        cell = getattr(ctx, "_cell", None)               # (a stand-in for a context has none: its library is called from here)
+        self._direct = cell is not None
+        self._native = _python_calls().Call(ctypes.addressof(a), ctypes.addressof(self._vlen), n,
+                                            ctypes.addressof(cell) if self._direct else 0,
+                                            _address_of(ctx._lib.avsg_step) if self._direct else 0,
+                                            _address_of(ctx._lib.avsg_step_host) if self._direct else 0,
+                                            functools.partial(_set_lengths, self._vlen, struct.Struct("=%di" % n).pack_into))
 
     def run(self, indices, verified_len: Sequence[int], slots, hit=None, miss_count=None, stream=None,
             host: bool = False, stage_one_done=None, arriving=None) -> None:
@@ -254,27 +290,12 @@ class PreparedCall:
         stage_one_done: None or (device int64 tensor or address, value): the word receives the value once the
         slot table, hit mask and miss counts of the whole call are final, while the missed rows still travel.
         arriving: None or a uint8 device tensor like hit: 1 where the row comes with this call's Stage Two."""
-        a = self.args
-        a.arriving = _addr(arriving) if arriving is not None else None
-        if stage_one_done is not None:
-            a.stage_one_done, a.stage_one_done_value = _addr(stage_one_done[0]), int(stage_one_done[1])
+        if self._direct:
+            rc = self._native.run(indices, verified_len, slots, hit, miss_count, stream, stage_one_done, arriving, host)
         else:
-            a.stage_one_done, a.stage_one_done_value = None, 0
-        if hasattr(verified_len, "data_ptr"):
-            a.verified_len_dev = verified_len.data_ptr()
-        else:
-            a.verified_len_dev = None
-            if not isinstance(verified_len, (list, tuple)):
-                verified_len = list(verified_len)        # (an iterator can be read once only)
-            try:
-                self._pack_vlen(self._vlen, 0, *verified_len)
-            except struct.error:                         # not n integers that fit: as the element type converts them
-                self._vlen[:] = [int(v) for v in verified_len]
-        a.indices, a.slots = _addr(indices), _addr(slots)
-        a.hit = _addr(hit) if hit is not None else None
-        a.miss_count = _addr(miss_count) if miss_count is not None else None
-        lib = self.ctx._lib
-        rc = (lib.avsg_step_host if host else lib.avsg_step)(self.ctx._h, self._ref, _stream_handle(stream))
+            at = self._native.fill(indices, verified_len, slots, hit, miss_count, stream, stage_one_done, arriving)
+            lib = self.ctx._lib
+            rc = (lib.avsg_step_host if host else lib.avsg_step)(self.ctx._h, self._ref, at or None)
         if rc != OK:
             _check(rc, "avsg_step")
 
@@ -291,11 +312,13 @@ class Context:
         cfg = AvsgConfig(num_tables, buffer_slots, row_bytes, max_topk, max_tokens, max_lifetime, transfer_mode,
                          device, index_mode, max_context, probe_retries, hash_a1, hash_a2, stage_one_cluster)
         _check(self._lib.avsg_create(ctypes.byref(cfg), ctypes.byref(self._h)), "avsg_create")
+        self._cell = ctypes.c_uint64(self._h.value)      # the handle, for prepared calls; 0 when it is closed
         self.num_tables, self.S, self.row_bytes = num_tables, buffer_slots, row_bytes
         self.max_topk, self.max_tokens, self.L, self.device = max_topk, max_tokens, max_lifetime, device
 
     def close(self) -> None:
         if getattr(self, "_h", None):
+            self._cell.value = 0
             self._lib.avsg_destroy(self._h)
             self._h = None
 
@@ -447,6 +470,9 @@ def _c_array(kind: str, values, n: int):
     return out, ctypes.addressof(out)
 
 
+_noalloc_fn = None
+
+
 def step_noalloc(tok, life, buffer, indices, kv, verified_len, *, max_lifetime: int = 16, slots, hit=None,
                  miss_count=None, status=None, row_stride=None, stream=None, kv_rows=None) -> None:
     """avsg_step_noalloc: one decode iteration on caller-owned state, for callers that cannot allocate
@@ -458,19 +484,10 @@ def step_noalloc(tok, life, buffer, indices, kv, verified_len, *, max_lifetime: 
     slots int32 like indices: CUDA tensors on the current device.  kv: one pinned host tensor (or address) per
     table.  Calls that overlap on the GPU race on the shared scratch: keep them on one stream.
     """
-    n, S = tok.shape
-    _, n_q, K = indices.shape
-    kv_arr, kv_at = _c_array("Q", [_addr(k) for k in kv], n)
-    vlen, vlen_at = _c_array("i", verified_len, n)
-    stride, stride_at = _c_array("Q", row_stride, n)
-    rows, rows_at = _c_array("I", kv_rows, n)
-    a = AvsgNoAllocArgs()
-    a.n, a.n_tokens, a.topk, a.buffer_slots = n, n_q, K, S
-    a.row_bytes, a.max_lifetime = buffer.shape[-1], max_lifetime
-    a.tok, a.life, a.buffer, a.indices = _addr(tok), _addr(life), _addr(buffer), _addr(indices)
-    a.kv_base, a.row_stride, a.verified_len, a.kv_rows = kv_at, stride_at, vlen_at, rows_at
-    a.slots = _addr(slots)
-    a.hit = _addr(hit) if hit is not None else None
-    a.miss_count = _addr(miss_count) if miss_count is not None else None
-    a.status = _addr(status) if status is not None else None
-    _check(load_library().avsg_step_noalloc(ctypes.byref(a), _stream_handle(stream)), "avsg_step_noalloc")
+    global _noalloc_fn
+    if _noalloc_fn is None:
+        _noalloc_fn = _address_of(load_library().avsg_step_noalloc)
+    rc = _python_calls().noalloc(_noalloc_fn, tok, life, buffer, indices, kv, verified_len, max_lifetime, slots, hit, miss_count,
+                                 status, row_stride, stream, kv_rows)
+    if rc != OK:
+        _check(rc, "avsg_step_noalloc")

@@ -1,12 +1,15 @@
-"""Compiles csrc/*.cu into libavsg.so (in-tree) with nvcc for sm_100a."""
+"""Compiles csrc/*.cu into libavsg.so with nvcc for sm_100a, and the binding's extension module with g++ (both in-tree)."""
 import glob
 import os
 import subprocess
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(_HERE), "include")
 LIB = os.path.join(_HERE, "libavsg.so")
+CALLS_SOURCE = os.path.join(CSRC, "python_calls.cpp")
+CALLS = os.path.join(_HERE, "_python_calls" + sysconfig.get_config_var("EXT_SUFFIX"))      # (of this Python)
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -25,8 +28,21 @@ def _stale(srcs) -> bool:
     return any(os.path.getmtime(d) > os.path.getmtime(LIB) for d in deps)
 
 
+def build_calls(force: bool = False):
+    """The extension module that makes the binding's hot calls, rebuilt when a source is newer."""
+    deps = [CALLS_SOURCE] + glob.glob(os.path.join(INCLUDE, "*.h"))
+    if force or not os.path.exists(CALLS) or any(os.path.getmtime(d) > os.path.getmtime(CALLS) for d in deps):
+        tmp = CALLS + ".tmp.%d" % os.getpid()
+        subprocess.check_call([os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-Wall", "-Wextra", "-Wno-missing-field-initializers",
+                               "-fPIC", "-shared", "-fvisibility=hidden", "-I", sysconfig.get_paths()["include"], "-I", INCLUDE,
+                               "-o", tmp, CALLS_SOURCE])
+        os.replace(tmp, CALLS)
+    return CALLS
+
+
 def build_library(force: bool = False, verbose: bool = False):
-    """Returns the path of libavsg.so, rebuilding it when a source is newer."""
+    """Returns the path of libavsg.so, rebuilding it (and the extension module) when a source is newer."""
+    build_calls(force)
     srcs = sources()
     if not srcs:
         return None

@@ -82,13 +82,14 @@ namespace {
 
 struct DeviceGuard {
     int prev = -1;
-    bool ok = true;
+    bool ok = true, other = false;
     explicit DeviceGuard(int dev)
     {
         if (cudaGetDevice(&prev) != cudaSuccess) { ok = false; return; }
-        if (prev != dev && cudaSetDevice(dev) != cudaSuccess) ok = false;
+        other = prev != dev;
+        if (other && cudaSetDevice(dev) != cudaSuccess) ok = false;
     }
-    ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
+    ~DeviceGuard() { if (other) cudaSetDevice(prev); }
 };
 
 #define CU(call) do { if ((call) != cudaSuccess) return AVSG_ECUDA; } while (0)

@@ -109,3 +109,85 @@ def test_lengths_are_taken_from_any_iterable():
         owner, at = _c_array("i", values, 3)
         assert list((ctypes.c_int32 * 3).from_address(at)) == want
     assert _c_array("I", None, 3) == (None, None)
+
+
+def test_native_calls_take_what_the_binding_takes():
+    """The extension module fills the argument blocks as ctypes would, and hands the rest to the binding's conversions."""
+    import types
+    import numpy as np
+    import pytest
+    import torch
+    from paper_2609_37538_b200 import binding as b
+    seen = []
+
+    def note(ctx, args, stream, which):
+        a = b.AvsgStepArgs.from_address(args)
+        seen.append((which, ctx, stream, {k: getattr(a, k) for k, _ in a._fields_}, list(call._vlen)))
+        return 0 if a.slots != 99 else avsg.ECAPACITY
+    fn = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p)
+    step, host = fn(lambda *a: note(*a, "step")), fn(lambda *a: note(*a, "host"))
+    cell = ctypes.c_uint64(77)
+    ctx = types.SimpleNamespace(_cell=cell, _lib=types.SimpleNamespace(avsg_step=step, avsg_step_host=host))
+    call = b.PreparedCall(ctx, [0, 1, 2], [16, 32, 48], 2, 5, kv_rows=[7, 8, 9])
+    t, n = torch.zeros(4, dtype=torch.int32), np.zeros(4, np.int32)
+    call.run(t, [1, 2, -3], n, 2**64 + 5, None, 6)
+    which, h, st, a, vlen = seen[-1]
+    assert (which, h, st, vlen) == ("step", 77, 6, [1, 2, -3]) and (a["n"], a["n_tokens"], a["topk"]) == (3, 2, 5)
+    assert (a["indices"], a["slots"], a["hit"], a["miss_count"]) == (t.data_ptr(), n.ctypes.data, 5, None)
+    assert (a["stage_one_done"], a["stage_one_done_value"], a["arriving"], a["verified_len_dev"]) == (None, 0, None, None)
+    call.run(8, t, 8, True, 0, types.SimpleNamespace(cuda_stream=11), True, (t, -1), n)
+    which, h, st, a, vlen = seen[-1]
+    assert (which, st, a["verified_len_dev"], a["hit"], a["miss_count"]) == ("host", 11, t.data_ptr(), 1, None)
+    assert (a["stage_one_done"], a["stage_one_done_value"], a["arriving"]) == (t.data_ptr(), 2**64 - 1, n.ctypes.data)
+    want = [5, -1, 7]
+    kinds = [want, tuple(want), np.array(want), np.array(want, np.float64), [5.0, -1, 7.9], [5, 2**32 - 1, 7], [np.int32(5), -1, True + 6]]
+    for values in kinds + [iter(k) for k in kinds]:
+        call.run(16, values, 16, stream=0)
+        assert seen[-1][4] == want and seen[-1][3]["verified_len_dev"] is None and seen[-1][2] is None
+    for bad in (dict(indices="x"), dict(slots=1.5), dict(hit=[]), dict(verified_len=[1, "a", 2]), dict(verified_len=[1, 2]),
+                dict(verified_len=3), dict(stage_one_done=(None, 1)), dict(stage_one_done=5)):
+        with pytest.raises((TypeError, ValueError)):
+            call.run(**{**dict(indices=8, verified_len=want, slots=8, stream=0), **bad})
+    with pytest.raises(avsg.AvsgError) as e:
+        call.run(8, want, 99, stream=0)
+    assert e.value.code == avsg.ECAPACITY
+    cell.value = 0                                       # a closed context
+    call.run(8, want, 8, stream=0)
+    assert seen[-1][1] is None
+
+    got = []
+
+    def take(args, stream):
+        a = b.AvsgNoAllocArgs.from_address(args)
+        arrays = [None if not at else list((k * a.n).from_address(at)) for at, k in ((a.kv_base, ctypes.c_uint64), (a.row_stride, ctypes.c_uint64),
+                                                                                     (a.verified_len, ctypes.c_int32), (a.kv_rows, ctypes.c_uint32))]
+        got.append(({k: getattr(a, k) for k, _ in a._fields_}, arrays, stream))
+        return avsg.EINVAL if a.max_lifetime == 7 else 0
+    keep = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p)(take)
+    before, b._noalloc_fn = b._noalloc_fn, b._address_of(keep)
+    try:
+        for n_tab in (3, 40):                            # (40: more than one call may have)
+            tok, life, rows = torch.zeros((n_tab, 64), dtype=torch.int32), torch.zeros((n_tab, 64), dtype=torch.int8), torch.zeros((n_tab, 64, 48), dtype=torch.uint8)
+            ids = torch.zeros((n_tab, 2, 5), dtype=torch.int32)
+            lens, kv = list(range(n_tab)), [16 * i for i in range(n_tab)]
+            for kvs, ls, strides, rws in ((kv, lens, None, None), (tuple(kv), np.array(lens), [48] * n_tab, iter(lens)),
+                                          (iter(kv), [float(v) for v in lens], tuple([2**64 + 48] * n_tab), [2**32 + v for v in lens])):
+                avsg.step_noalloc(tok, life, rows, ids, kvs, ls, max_lifetime=4, slots=ids, stream=9, row_stride=strides, kv_rows=rws)
+                a, arrays, st = got[-1]
+                assert (a["n"], a["n_tokens"], a["topk"], a["buffer_slots"], a["row_bytes"], a["max_lifetime"], st) == (n_tab, 2, 5, 64, 48, 4, 9)
+                assert (a["tok"], a["life"], a["buffer"], a["indices"], a["slots"]) == (tok.data_ptr(), life.data_ptr(), rows.data_ptr(), ids.data_ptr(), ids.data_ptr())
+                assert a["hit"] is None and a["miss_count"] is None and a["status"] is None
+                assert arrays == [kv, [48] * n_tab if strides else None, lens, lens if rws is not None else None]
+        some = dict(max_lifetime=4, slots=ids, stream=0)
+        avsg.step_noalloc(tok, life, rows, ids, [t] * n_tab, lens, hit=n, miss_count=5, status=t, **some)
+        assert got[-1][1][0] == [t.data_ptr()] * n_tab and (got[-1][0]["hit"], got[-1][0]["miss_count"]) == (n.ctypes.data, 5)
+        with pytest.raises(avsg.AvsgError):
+            avsg.step_noalloc(tok, life, rows, ids, kv, lens, max_lifetime=7, slots=ids, stream=0)
+        with pytest.raises(ValueError):
+            avsg.step_noalloc(tok[0], life, rows, ids, kv, lens, **some)
+        with pytest.raises(TypeError):
+            avsg.step_noalloc(tok, life, rows, ids, ["a"] * n_tab, lens, **some)
+        with pytest.raises(IndexError):
+            avsg.step_noalloc(tok, life, rows, ids, kv + [0], lens, **some)
+    finally:
+        b._noalloc_fn = before
