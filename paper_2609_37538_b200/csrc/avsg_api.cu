@@ -250,7 +250,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
         cluster = c->step_clusters.of(n, step_threads(c->cfg.buffer_slots, K));
         if (cluster && !step_serves(c->cfg.buffer_slots, K, n_q, cluster, c->cfg.row_bytes, a->arriving != nullptr)) cluster = 0;
         if (a->stage_one_done && n > STEP_EARLY_TABLES &&
-            (uint64_t)n * cluster * step_threads(c->cfg.buffer_slots, K) > (uint64_t)c->sm_count / 2u * 1024u)
+            !step_leaves_half(n, step_threads(c->cfg.buffer_slots, K), cluster, (uint32_t)c->sm_count))
             cluster = 0;
     }
     const bool in_place = (K % 8u == 0 && reinterpret_cast<uint64_t>(a->indices) % 32u == 0) || n_ids <= HOST_ODD_IDS;
@@ -377,7 +377,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
             fill(p, 0, n);
             p.flags = nullptr; p.expect = n; p.out = out; p.shared = c->d_shared; p.arriving = a->arriving;
             p.done_seq = reinterpret_cast<unsigned long long*>(a->stage_one_done);
-            p.early = a->stage_one_done || step_early(p);
+            p.early = a->stage_one_done || step_early(p, step_threads(p.S, K), cluster, (uint32_t)c->sm_count);
             CU(launch_step(p, cluster, stream));
             return AVSG_OK;
         };

@@ -248,18 +248,28 @@ cudaError_t step_prepare(size_t max_smem);
 // output: whether rows are asked for early.
 bool step_serves(uint32_t S, uint32_t K, uint32_t n_q, uint32_t cluster, uint32_t row_bytes, bool arriving);
 StepClusters step_clusters(size_t max_smem);            // after step_prepare
-// Whether the grid behind a call in one kernel may start under it (see the kernel).  Up to three tables, and up to eight
-// that reach little host memory (id_limit: rows a table's ids can reach).  Early / late, calls of K = 2048: one table 13.2 / 13.4
+// Whether the blocks of a call in one kernel leave half of the SMs to other grids.
+inline bool step_leaves_half(uint32_t n, uint32_t threads, uint32_t cluster, uint32_t sm_count)
+{
+    return (uint64_t)n * cluster * threads <= (uint64_t)sm_count / 2u * 1024u;
+}
+// Whether the grid behind a call in one kernel may start under it (see the kernel).  Up to three tables; and up to eight, or as many
+// as leave half of the SMs free with clusters of four, that reach little host memory (id_limit: rows a table's ids can
+// reach).  Early / late, calls of K = 2048: one table 13.2 / 13.4
 // us (0.08 GB) and 13.7 / 13.9 (0.6 GB); two 17.1 / 17.1, 18.0 / 18.0 (1.3 GB); three 21.4 / 21.3, 23.3 / 23.7 (1.9 GB); four 25.8 /
 // 25.8 (0.3 GB), 27.8 / 27.3 (1.3 GB), 28.9 / 28.2 (2.6 GB); six 34.4 / 34.4 (0.5 GB), 36.7 / 36.0 (1.9 GB), 39.1 / 37.2 (3.8 GB); eight 42.8 /
 // 42.8 (0.6 GB), 44.2 / 44.3 (1.3 GB), 45.2 / 44.9 (1.9 GB), 46.5 / 45.3 (2.6 GB), 58.3 / 46.7 (5.1 GB); five tables with K = 139 9.3 / 9.7.
-// More tables gain nothing by it (32 tables 113.0 / 112.9), and ids in host memory that are fetched under a call's rows slow these
+// 12, 18 tables of K = 1000 27.0 / 27.6, 37.4 / 38.0 (0.1 and 0.2 GB), 31.4 / 32.0, 44.2 / 44.9 (0.5, 0.8 GB), 33.3 / 33.8, 49.8 / 47.6 (2.1, 3.1 GB); of
+// K = 2048 37.6 / 38.1, 54.0 / 54.5, 60.0 / 60.4 and 52.9 / 53.4, 77.6 / 77.9, 89.9 / 87.4; 28 of S = 1024 13.9 / 14.1, 14.3 / 14.5, 15.2 / 15.2; but 12
+// in clusters of eight of small blocks 9.5 / 9.3 (S = 1024), 20.1 / 20.1 (2048), 18.9 / 18.9 (4096; 1.8 GB 20.0 / 19.8).
+// Where the blocks leave no room nothing is gained (32 tables 113.0 / 112.9), and ids in host memory that are fetched under a call's rows slow these
 // down (39 tables, K = 3430: 215 / 124).
 template <int CAP>
-bool step_early(const S1ParamsT<CAP>& p)
+bool step_early(const S1ParamsT<CAP>& p, uint32_t threads, uint32_t cluster, uint32_t sm_count)
 {
     if (p.n_launch <= STEP_EARLY_TABLES) return true;
-    if (p.n_launch > (uint32_t)STEP_FEW_TABLES || p.host_ids) return false;
+    if (p.host_ids || (p.n_launch > (uint32_t)STEP_FEW_TABLES && (cluster == STEP_FEW_CLUSTER || !step_leaves_half(p.n_launch, threads, cluster, sm_count))))
+        return false;
     uint64_t bytes = 0;
     for (uint32_t i = 0; i < p.n_launch; ++i) bytes += p.id_limit[i] * p.kv_stride[i];
     return bytes <= STEP_EARLY_BYTES;

@@ -125,7 +125,7 @@ extern "C" int avsg_step_noalloc(const avsg_noalloc_args* a, void* cuda_stream)
     if (cluster) {
         auto step = [&](auto&& p) -> int {               // one kernel for both stages
             if ((rc = fill(p)) != AVSG_OK) return rc;
-            p.early = step_early(p);
+            p.early = step_early(p, step_threads(p.S, p.K), cluster, (uint32_t)g_sm_count[dev]);
             p.shared = sc->shared;
             return launch_step(p, cluster, stream) == cudaSuccess ? AVSG_OK : AVSG_ECUDA;
         };
