@@ -10,7 +10,6 @@ from __future__ import annotations
 
 import array
 import ctypes
-import functools
 import os
 import struct
 from typing import List, Optional, Sequence, Union
@@ -92,7 +91,7 @@ def _python_calls():
             from . import _python_calls as module
         except ImportError as e:
             raise RuntimeError("the extension module _python_calls is missing: run `python __graft_entry__.py` to build it") from e
-        module.set_binding(_addr, _c_array, _stream_handle, None, None)
+        module.set_binding(_addr, _c_array, _set_lengths, _stream_handle, None, None)
         _calls = module
     return _calls
 
@@ -207,7 +206,7 @@ def _current_stream() -> int:
         raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
         if raw is not None and dev is not None:
             _current_stream_fn = lambda: raw(dev())
-            _python_calls().set_binding(_addr, _c_array, _stream_handle, raw, dev)     # (the extension asks them itself from now on)
+            _python_calls().set_binding(_addr, _c_array, _set_lengths, _stream_handle, raw, dev)     # (the extension asks them itself from now on)
         else:
             _current_stream_fn = lambda: torch.cuda.current_stream().cuda_stream
     return _current_stream_fn()
@@ -241,12 +240,16 @@ def _address_of(function) -> int:
     return ctypes.cast(function, ctypes.c_void_p).value
 
 
-def _set_lengths(vlen, pack_into, values) -> None:
+def _addresses(lib):
+    return _address_of(lib.avsg_step), _address_of(lib.avsg_step_host)
+
+
+def _set_lengths(vlen, values) -> None:
     """Verified lengths from any iterable of n numbers."""
     if not isinstance(values, (list, tuple)):
         values = list(values)                            # (an iterator can be read once only)
     try:
-        pack_into(vlen, 0, *values)
+        struct.pack_into("=%di" % len(vlen), vlen, 0, *values)
     except struct.error:                                 # not n integers that fit: as the element type converts them
         vlen[:] = [int(v) for v in values]
 
@@ -276,11 +279,9 @@ class PreparedCall:
         self._ref = ctypes.byref(a)
         cell = getattr(ctx, "_cell", None)               # (a stand-in for a context has none: its library is called from here)
         self._direct = cell is not None
-        self._native = _python_calls().Call(ctypes.addressof(a), ctypes.addressof(self._vlen), n,
-                                            ctypes.addressof(cell) if self._direct else 0,
-                                            _address_of(ctx._lib.avsg_step) if self._direct else 0,
-                                            _address_of(ctx._lib.avsg_step_host) if self._direct else 0,
-                                            functools.partial(_set_lengths, self._vlen, struct.Struct("=%di" % n).pack_into))
+        step, step_host = (getattr(ctx, "_addresses", None) or _addresses(ctx._lib)) if self._direct else (0, 0)
+        self._native = (_calls or _python_calls()).Call(ctypes.addressof(a), ctypes.addressof(self._vlen), n,
+                                                        ctypes.addressof(cell) if self._direct else 0, step, step_host, self._vlen)
 
     def run(self, indices, verified_len: Sequence[int], slots, hit=None, miss_count=None, stream=None,
             host: bool = False, stage_one_done=None, arriving=None) -> None:
@@ -313,6 +314,7 @@ class Context:
                          device, index_mode, max_context, probe_retries, hash_a1, hash_a2, stage_one_cluster)
         _check(self._lib.avsg_create(ctypes.byref(cfg), ctypes.byref(self._h)), "avsg_create")
         self._cell = ctypes.c_uint64(self._h.value)      # the handle, for prepared calls; 0 when it is closed
+        self._addresses = _addresses(self._lib)
         self.num_tables, self.S, self.row_bytes = num_tables, buffer_slots, row_bytes
         self.max_topk, self.max_tokens, self.L, self.device = max_topk, max_tokens, max_lifetime, device
 

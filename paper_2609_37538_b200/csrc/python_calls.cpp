@@ -20,7 +20,7 @@ namespace {
 PyObject *s_data_ptr, *s_shape;
 
 // The module's conversions, set once by the binding (set_binding).
-PyObject *b_addr, *b_array, *b_stream, *b_raw_stream, *b_device;
+PyObject *b_addr, *b_array, *b_lengths, *b_stream, *b_raw_stream, *b_device;
 
 struct Held {                            // a reference that goes with its scope
     PyObject* o;
@@ -99,7 +99,7 @@ struct Call {
     const uint64_t* ctx;                 // holds the context's handle, 0 when that is closed; null: fill() only
     StepFn step, step_host;
     Py_ssize_t n;
-    PyObject* set_lengths;               // the binding's way: any iterable of n numbers
+    PyObject* array;                     // the same, for the binding (which takes any iterable of n numbers)
 };
 
 int call_init(PyObject* self, PyObject* args, PyObject*)
@@ -107,25 +107,25 @@ int call_init(PyObject* self, PyObject* args, PyObject*)
     Call* c = reinterpret_cast<Call*>(self);
     unsigned long long block, lengths, ctx, step, step_host;
     Py_ssize_t n;
-    PyObject* set_lengths;
-    if (!PyArg_ParseTuple(args, "KKnKKKO", &block, &lengths, &n, &ctx, &step, &step_host, &set_lengths)) return -1;
+    PyObject* array;
+    if (!PyArg_ParseTuple(args, "KKnKKKO", &block, &lengths, &n, &ctx, &step, &step_host, &array)) return -1;
     c->args = reinterpret_cast<avsg_step_args*>(block);
     c->lengths = reinterpret_cast<int32_t*>(lengths);
     c->ctx = reinterpret_cast<const uint64_t*>(ctx);
     c->step = reinterpret_cast<StepFn>(step);
     c->step_host = reinterpret_cast<StepFn>(step_host);
     c->n = n;
-    Py_INCREF(set_lengths);
-    Py_XSETREF(c->set_lengths, set_lengths);
+    Py_INCREF(array);
+    Py_XSETREF(c->array, array);
     return 0;
 }
 int call_traverse(PyObject* self, visitproc visit, void* arg)
 {
     Py_VISIT(Py_TYPE(self));
-    Py_VISIT(reinterpret_cast<Call*>(self)->set_lengths);
+    Py_VISIT(reinterpret_cast<Call*>(self)->array);
     return 0;
 }
-int call_clear(PyObject* self) { Py_CLEAR(reinterpret_cast<Call*>(self)->set_lengths); return 0; }
+int call_clear(PyObject* self) { Py_CLEAR(reinterpret_cast<Call*>(self)->array); return 0; }
 void call_dealloc(PyObject* self)
 {
     PyTypeObject* type = Py_TYPE(self);
@@ -158,7 +158,7 @@ bool fill(Call* c, PyObject* const* a, uint64_t* stream)
             if (!address(a[1], &v)) return false;
             s->verified_len_dev = reinterpret_cast<const int32_t*>(v);
         } else {
-            Held done(PyObject_CallOneArg(c->set_lengths, a[1]));
+            Held done(PyObject_CallFunctionObjArgs(b_lengths, c->array, a[1], nullptr));
             if (!done.o) return false;
         }
     }
@@ -314,13 +314,14 @@ PyObject* noalloc(PyObject*, PyObject* const* a, Py_ssize_t nargs)
     return PyLong_FromLong(rc);
 }
 
-// addr, array, stream handle; raw stream and device functions, or None
+// addr, array, lengths, stream handle; raw stream and device functions, or None
 PyObject* set_binding(PyObject*, PyObject* args)
 {
-    PyObject *addr, *array, *stream, *raw, *device;
-    if (!PyArg_ParseTuple(args, "OOOOO", &addr, &array, &stream, &raw, &device)) return nullptr;
+    PyObject *addr, *array, *lengths, *stream, *raw, *device;
+    if (!PyArg_ParseTuple(args, "OOOOOO", &addr, &array, &lengths, &stream, &raw, &device)) return nullptr;
     Py_INCREF(addr); Py_XSETREF(b_addr, addr);
     Py_INCREF(array); Py_XSETREF(b_array, array);
+    Py_INCREF(lengths); Py_XSETREF(b_lengths, lengths);
     Py_INCREF(stream); Py_XSETREF(b_stream, stream);
     const bool both = raw != Py_None && device != Py_None;
     if (both) { Py_INCREF(raw); Py_INCREF(device); }
