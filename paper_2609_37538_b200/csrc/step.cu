@@ -1012,8 +1012,8 @@ cudaError_t step_prepare(size_t max_smem)
 
 // Above WIDE_SLOTS: where the index has room (n_q and K decide), and not calls of few tokens with three and two blocks a table, whose
 // rows two kernels cut evenly over all SMs: K = 2048, two kernels / one, us: 36, 50, 74 tables, one token 83.9 / 83.0, 109.8 / 112.0, 154.9 /
-// 156.7; K = 1024, two tokens, 40, 64 tables 99.9 / 94.9, 149.0 / 147.3, but 64 cold ones 1103 / 1114; K = 2048, four tokens, 40, 64 tables
-// 248 / 234, 381 / 371.
+// 156.7; K = 1024, two tokens, 40, 64 tables 99.9 / 94.9, 149.0 / 147.3, but 64 cold ones 1103 / 1114; K = 2048, three tokens, 40, 50,
+// 74 tables 200 / 190, 243 / 238, 350 / 345, 60 cold ones 810 / 810; four tokens, 40, 64 tables 248 / 234, 381 / 371.
 bool step_serves(uint32_t S, uint32_t K, uint32_t n_q, uint32_t cluster, uint32_t row_bytes, bool arriving)
 {
     StepLayout lay;
