@@ -149,12 +149,15 @@ __device__ __forceinline__ bool wait_for(uint32_t mbar, uint32_t limit)
 // that the device writes is read before that kernel has completed.  Only then may the next grid start under this one: let go at
 // the start, two and three grids wait behind one another, and each hears late that its turn has come (one table, K = 2048, one and
 // two tokens 7.78, 11.12 us, now 7.45, 10.72; S = K = 2048 / 4, two tokens 7.94, 7.61; S = 256 5.55, 5.26; two tables 13.3, 13.0).
-template <typename P>
-__device__ __forceinline__ void wait_for_previous(const P& p)
-{
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (p.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// A call with ids in host memory lets it go at the start: what that grid does before its wait is to fetch its ids, a round trip of
+// the link (K = 2048, two tokens, one, two, three tables 15.4, 18.1, 21.4 us let go behind the wait, 14.5, 17.3, 20.7 at the start).
+// The next grid comes when all blocks have let it go, so behind the wait only the copying blocks say so, and the first block of a
+// cluster at its start: behind its wait the question costs calls too that let nobody start (host ids, S = 512, K = 65, three tokens, 7, 13
+// tables 16.8, 20.1 us with it, 16.3, 19.4 without; S = 2048, K = 229, four tokens 24.6, 35.4 and 24.3, 34.7).  Nor does a branch stand
+// where ids on their way from the host are in registers, which it waits for (S = 1024, K = 1000, 5, 13 tables 23.7, 44.2 us with one,
+// 22.3, 40.4 without).
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // What the copying blocks are told.  Where they ask for rows early: `token`, that block `to` has n misses in its positions; `miss`,
 // to the block that position i belongs to, the slot, where the position's place is and in the next entry of its list.  Where
@@ -291,7 +294,7 @@ __device__ __forceinline__ void place_tokens(const S1ParamsT<CAP>& p, const Step
     // fetches its first ones while that one's rows travel (32 tables: 5 us of link time and a round trip).
     if (!ASK && p.host_ids) load_token(0);
 
-    wait_for_previous(p);
+    wait_for_previous();
 
     const uint32_t j0 = tid * SPT;                       // first of the thread's slots
     const bool own = j0 < S;
@@ -617,7 +620,7 @@ __device__ __forceinline__ Item match(const S1ParamsT<CAP>& p, const StepLayout&
 #pragma unroll
             for (int m = 0; m < OWN; ++m) x[m] = from + m * step < all ? __ldcv(g_ids + from + m * step) : -1;
             if (first) {
-                wait_for_previous(p);
+                wait_for_previous();
                 cluster_wait();
                 first = 0;
             }
@@ -632,7 +635,8 @@ __device__ __forceinline__ Item match(const S1ParamsT<CAP>& p, const StepLayout&
         }
         cluster_sync();
     } else {
-        wait_for_previous(p);
+        wait_for_previous();
+        if (p.early) let_next_start();
     }
 
     // ---- every global load is issued first: cached ids, the first token's, the block's own ids ----
@@ -803,6 +807,7 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
     const uint32_t rank = cluster_rank(), cluster = !ASK && FEW ? STEP_FEW_CLUSTER : cluster_size(), copying = cluster - 1u;
     const uint32_t ti = blockIdx.x / cluster, lane = threadIdx.x & 31u, W = blockDim.x >> 5, warp = threadIdx.x >> 5;
     uint32_t* s_slots = reinterpret_cast<uint32_t*>(smem + lay.slots);
+    if (p.early && (p.host_ids || rank == 0)) let_next_start();
     if (SHARE && threadIdx.x == 0) s_mine = 0xFFFFFFFFu;
     if (rank != 0) {
         if (threadIdx.x < p.n_q) {
@@ -892,7 +897,8 @@ __global__ void __launch_bounds__(1024, 1) avsg_step_kernel(const __grid_constan
             next();
         }
     } else {
-        wait_for_previous(p);
+        wait_for_previous();
+        if (p.early && !p.host_ids) let_next_start();
         cluster_wait();
         cluster_arrive();
         uint32_t from = 0;                                             // the warp that is next

@@ -444,3 +444,40 @@ def test_early_outputs(n, S, K, n_q, rb):
     for t in range(n):
         assert (ctx.buffer(t).cpu().numpy() == orc[t].rows()).all(), t
     assert ctx.sync_status() == 0
+
+
+@pytest.mark.parametrize("n,host,at_once", [(1, True, True), (3, True, True), (4, True, False), (1, False, False), (3, False, False)])
+def test_when_the_next_grid_may_start(n, host, at_once, tmp_path):
+    """Behind a call of up to three tables whose ids are in host memory the next grid comes while the call waits for its turn (so
+    that the next call fetches its ids in that time); behind other calls it does not."""
+    import ctypes
+    import os
+    import subprocess
+    import torch
+    import paper_2609_37538_b200 as avsg
+    from paper_2609_37538_b200 import build
+    lib = str(tmp_path / "start_marks.so")
+    subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")] + build.NVCC_FLAGS +
+                          ["-o", lib, os.path.join(os.path.dirname(os.path.abspath(__file__)), "cuda", "start_marks.cu")])
+    lib = ctypes.CDLL(lib)
+    lib.launch_hold.argtypes = [ctypes.c_uint64, ctypes.c_void_p, ctypes.c_void_p]
+    lib.launch_mark.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
+    K, n_q = 100, 2
+    kv = _kv(avsg)
+    ctx = avsg.Context(n, 1024, RB, K, n_q, 4)
+    call = ctx.prepare(list(range(n)), [kv] * n, n_q, K)
+    where = dict(pin_memory=True) if host else dict(device="cuda")
+    X = torch.empty((n, n_q, K), dtype=torch.int32, **where)
+    X.copy_(torch.arange(K, dtype=torch.int32).expand(n, n_q, K))
+    slots = torch.empty((n, n_q, K), dtype=torch.int32, **where)
+    marks = torch.zeros(2, dtype=torch.int64, device="cuda")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for ns in (1000, 5_000_000):                         # (the first time loads the kernels)
+        assert lib.launch_hold(ns, marks.data_ptr(), stream.cuda_stream) == 0
+        call.run(X, [CTX] * n, slots, stream=stream, host=host)
+        assert lib.launch_mark(marks.data_ptr() + 8, stream.cuda_stream) == 0
+        stream.synchronize()
+    held_until, started = (int(v) for v in marks.cpu())
+    assert (started < held_until) == at_once, started - held_until
+    assert ctx.sync_status() == 0
