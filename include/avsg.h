@@ -79,8 +79,11 @@ extern "C" {
                                        16384 slots; of 16384 slots where n_tokens and topk
                                        leave room for them in one SM's shared memory, up to
                                        33 tables, and more where there are several tokens;
-                                       with stage_one_done up to 18 tables, whose blocks
-                                       leave half of the SMs free, more of smaller ones;
+                                       with stage_one_done up to 18 tables, more where the
+                                       blocks are smaller than 1024 threads, but not nine
+                                       and more tables of over 2048 ids each that reach
+                                       over 3 GB of host memory together (kv_rows or the
+                                       direct index say how far they reach);
                                        with arriving up to 33, and rows of up to 1536 bytes).
                                        Its blocks take whole SMs while they run: who wants
                                        room for other kernels beside the call sets a

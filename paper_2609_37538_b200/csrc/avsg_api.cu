@@ -239,18 +239,37 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     bool host_ids = false;
     // One kernel for both stages, where the tables' clusters fit the device (see avsg_step_kernel for what it saves).  Its
     // blocks take whole SMs.  So a caller who wants the hits before the rows are there (stage_one_done) gets it from calls that
-    // leave half of the SMs to the kernel that starts on the hits (or are small: STEP_EARLY_TABLES), and that kernel may start
-    // at once, although the grid behind a call then finds other SMs free (from 11 GB, 16 tables 87.8 us, if it came late 82.9).
-    // K = 2048, two tokens, with both early outputs, three kernels / one: 2, 6, 8, 12, 16, 18 tables 25.4 / 14.6, 38.8 / 27.1, 45.0 /
-    // 33.1, 57.9 / 46.7, 71.7 / 60.4, 78.2 / 66.4 us; from 11 GB, 6, 16 tables 48.3 / 37.7, 96.7 / 87.4; 16384 slots, four tokens, 16
-    // tables 109.1 / 104.3.  (22 and 33 tables would gain 12 us too, with 60 and 16 SMs left.)
+    // leave half of the SMs to the kernel that starts on the hits (or are small: STEP_EARLY_TABLES), unless they reach far
+    // (step_reaches_far()), and that kernel may start at once.  K = 2048, two tokens, 64 Ki positions, with both early outputs, three
+    // kernels / one, 3, 8, 18 tables: calls alone 32.7 / 20.7, 58.7 / 46.0, 109.1 / 95.9 us; each with a stand-in for a consumer (see
+    // step_reaches_far()) behind it on the stream, which starts with the call, 42.8 / 31.2, 76.9 / 57.0, 138.2 / 120.1; with one on
+    // another stream while the next calls queue 40.9 / 32.6, 71.8 / 59.9, 125.3 / 109.5; if the next call waits for that one too 51.3 / 45.3,
+    // 85.3 / 69.1, 141.9 / 117.9.  What loses is this last way with a consumer that would fill the SMs besides (no shared memory): the
+    // one kernel's word comes later than a Stage One grid's, and half of the SMs are taken (K = 2048, one token, 12, 14, 16, 18 tables 60.7,
+    // 62.4, 62.3, 66.7 / 58.8, 64.4, 68.2, 71.4; small blocks, S = 1024, K = 256, 18, 31, 37 tables 41.3, 42.5, 42.1 / 36.9, 43.2, 45.9).
+    // If the kernel behind such a call came only at its end, calls without a consumer would keep their SMs from one to the next (8
+    // tables, 5.5 GB 63.6 us, then 45.4, in three kernels 58.6), but a consumer on the same stream could not start (57.1, 66.4, 72.7).
+    //
+    // id_limit_of: ids at or beyond this are never looked up or fetched: the table's host rows when the caller states them,
+    // and the size of the direct index
+    auto id_limit_of = [&](uint32_t i) -> uint32_t {
+        uint32_t lim = a->kv_rows ? a->kv_rows[i] : 0x80000000u;
+        if (c->cfg.index_mode == AVSG_INDEX_DIRECT && c->cfg.max_context < lim) lim = c->cfg.max_context;
+        return lim;
+    };
+    auto stride_of = [&](uint32_t i) -> uint64_t { return a->row_stride ? a->row_stride[i] : c->cfg.row_bytes; };
+    auto reach = [&] {
+        uint64_t bytes = 0;
+        for (uint32_t i = 0; i < n; ++i) bytes += id_limit_of(i) * stride_of(i);
+        return bytes;
+    };
     const bool sm_copies = c->cfg.transfer_mode == AVSG_XFER_SM_BALANCED || c->cfg.transfer_mode == AVSG_XFER_SM_OVERLAP;
     uint32_t cluster = 0;
     if (sm_copies && c->one_kernel && n_q <= STEP_MAX_TOKENS && !c->timing && !c->geometry_set) {
         cluster = c->step_clusters.of(n, step_threads(c->cfg.buffer_slots, K));
         if (cluster && !step_serves(c->cfg.buffer_slots, K, n_q, cluster, c->cfg.row_bytes, a->arriving != nullptr)) cluster = 0;
-        if (a->stage_one_done && n > STEP_EARLY_TABLES &&
-            !step_leaves_half(n, step_threads(c->cfg.buffer_slots, K), cluster, (uint32_t)c->sm_count))
+        if (cluster && a->stage_one_done && n > STEP_EARLY_TABLES &&
+            (!step_leaves_half(n, step_threads(c->cfg.buffer_slots, K), cluster, (uint32_t)c->sm_count) || step_reaches_far(n, n_q * K, reach())))
             cluster = 0;
     }
     const bool in_place = (K % 8u == 0 && reinterpret_cast<uint64_t>(a->indices) % 32u == 0) || n_ids <= HOST_ODD_IDS;
@@ -325,13 +344,6 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
     c->call_kv_dev.resize(n);
     for (uint32_t i = 0; i < n; ++i)
         if ((rc = resolve_kv(c, a->table_ids[i], a->kv_base[i], &c->call_kv_dev[i])) != AVSG_OK) return rc;
-    // ids at or beyond this are never looked up or fetched: the table's host rows when the caller states them,
-    // and the size of the direct index
-    auto id_limit_of = [&](uint32_t i) -> uint32_t {
-        uint32_t lim = a->kv_rows ? a->kv_rows[i] : 0x80000000u;
-        if (c->cfg.index_mode == AVSG_INDEX_DIRECT && c->cfg.max_context < lim) lim = c->cfg.max_context;
-        return lim;
-    };
     // Stage One's arguments for tables [first, first + cnt) of the call, and its launch with the small or the large block
     auto fill = [&](auto& p, uint32_t first, uint32_t cnt) {
         p.tok = c->d_tok; p.life = c->d_life; p.buffer = c->d_buffer; p.stats = c->d_stats;
@@ -363,7 +375,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
             p.verified_len[i] = a->verified_len ? a->verified_len[first + i] : 0;
             p.id_limit[i] = id_limit_of(first + i);
             p.kv_base[i] = c->call_kv_dev[first + i];
-            p.kv_stride[i] = a->row_stride ? a->row_stride[first + i] : c->cfg.row_bytes;
+            p.kv_stride[i] = stride_of(first + i);
         }
     };
     auto stage_one = [&](auto& p, uint32_t first, uint32_t cnt) -> int {
@@ -396,7 +408,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
                 p.table_id[i] = a->table_ids[first + i];
                 p.id_limit[i] = id_limit_of(first + i);
                 p.kv_base[i] = c->call_kv_dev[first + i];
-                p.kv_stride[i] = a->row_stride ? a->row_stride[first + i] : c->cfg.row_bytes;
+                p.kv_stride[i] = stride_of(first + i);
             }
             CU(launch_all_k_prepare(p, cnt, stream));
         } else if (chunk == (uint32_t)S1_MAX_TABLES) {
@@ -451,7 +463,7 @@ int step_impl(avsg_ctx* c, const avsg_step_args* a, cudaStream_t stream, bool ho
             for (uint32_t i = 0; i < n; ++i) {
                 x.table_id[i] = a->table_ids[i];
                 x.kv_base[i] = c->call_kv_dev[i];
-                x.kv_stride[i] = a->row_stride ? a->row_stride[i] : c->cfg.row_bytes;
+                x.kv_stride[i] = stride_of(i);
             }
             return launch_transfer_overlap(x, c->xfer_blocks ? c->xfer_blocks : (uint32_t)c->sm_count, c->xfer_threads, stream);
         };

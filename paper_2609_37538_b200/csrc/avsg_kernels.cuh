@@ -253,6 +253,22 @@ inline bool step_leaves_half(uint32_t n, uint32_t threads, uint32_t cluster, uin
 {
     return (uint64_t)n * cluster * threads <= (uint64_t)sm_count / 2u * 1024u;
 }
+// Whether a call that says when Stage One is done (reach: host bytes that its ids can reach) is better off with a kernel for each stage
+// though it would leave half of the SMs.  Its consumer may run on another stream while the next calls queue.  The clusters then take
+// the SMs that the consumer has left, and not those whose caches know their tables; where much has to be translated that costs more
+// than the one kernel saves.  A call and a stand-in that reads all its rows on another stream (148 blocks, with 120 KB of shared memory /
+// with none), four contexts in turn, a kernel for each stage -> one kernel: 12 tables, K = 2048, two tokens, 2.1 GB 79 -> 73 / 91 -> 79 us, 4.1
+// GB 86 -> 99 / 96 -> 80, 8.3 GB 95 -> 128 / 111 -> 91; 14 tables, 9.6 GB 106 -> 123 / 129 -> 126; 18 tables, 3.1 GB 118 -> 102 / 122 -> 107; four
+// tokens, 16 tables, 2.8 GB 183 -> 167 / 190 -> 181, 11 GB 244 -> 276 / 253 -> 288 (another box: 12 tables, 8.3 GB 94 -> 103 / 105 -> 87, 14 111 ->
+// 116 / 126 -> 114).  And 18 tables without a consumer 101 -> 92 from 3.1, 104 -> 127 from 6.2 GB.  What is given up for that: with a
+// consumer on the same stream 12 tables, 8.3 GB 104 -> 86.  With fewer ids or up to eight tables none of it is lost: 16 tables, K = 1000,
+// 11 GB 51 -> 40 / 55 -> 40; 8 tables, 5.5 GB 69 -> 59 / 66 -> 58.
+constexpr uint32_t STEP_FAR_IDS = 2048;                  // of a table
+constexpr uint64_t STEP_FAR_BYTES = 3ull << 30;
+inline bool step_reaches_far(uint32_t n, uint32_t table_ids, uint64_t reach)
+{
+    return n > (uint32_t)STEP_FEW_TABLES && table_ids > STEP_FAR_IDS && reach > STEP_FAR_BYTES;
+}
 // Whether the grid behind a call in one kernel may start under it (see the kernel).  Up to three tables; and up to eight, or as many
 // as leave half of the SMs free with clusters of four, that reach little host memory (id_limit: rows a table's ids can
 // reach).  Early / late, calls of K = 2048: one table 13.2 / 13.4

@@ -326,26 +326,33 @@ def test_rows_that_tables_share_in_a_captured_call_and_without_a_context():
     assert ctx.sync_status() == 0
 
 
-def test_the_default_geometry_brings_the_one_kernel_back():
+def _kernels(ctx, kv, n, n_q, K, word=None, want_arriving=False, kv_rows=None):
+    """The number of kernels of such a call: it is captured, and never runs."""
     import ctypes
     import torch
+    cudart = ctypes.CDLL("libcudart.so.12")
+    stream = torch.cuda.Stream()
+    X = torch.zeros((n, n_q, K), dtype=torch.int32, device="cuda")
+    slots = torch.empty_like(X)
+    arriving = torch.empty((n, n_q, K), dtype=torch.uint8, device="cuda") if want_arriving else None
+    torch.cuda.synchronize()
+    s, graph, nodes = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
+    assert cudart.cudaStreamBeginCapture(s, 2) == 0
+    ctx.prepare(list(range(n)), [kv] * n, n_q, K, kv_rows=kv_rows).run(X, [CTX] * n, slots, stream=stream, arriving=arriving,
+                                                                       stage_one_done=None if word is None else (word, 1))
+    assert cudart.cudaStreamEndCapture(s, ctypes.byref(graph)) == 0
+    assert cudart.cudaGraphGetNodes(graph, None, ctypes.byref(nodes)) == 0
+    assert cudart.cudaGraphDestroy(graph) == 0
+    return nodes.value
+
+
+def test_the_default_geometry_brings_the_one_kernel_back():
     import paper_2609_37538_b200 as avsg
     kv = _kv(avsg)
     ctx = avsg.Context(100, 256, RB, 16, 2, 4)
-    cudart = ctypes.CDLL("libcudart.so.12")
-    stream = torch.cuda.Stream()
 
-    def kernels(n):                                      # of a call that is captured
-        X = torch.zeros((n, 2, 16), dtype=torch.int32, device="cuda")
-        slots = torch.empty_like(X)
-        torch.cuda.synchronize()
-        s, graph, nodes = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
-        assert cudart.cudaStreamBeginCapture(s, 2) == 0
-        ctx.prepare(list(range(n)), [kv] * n, 2, 16).run(X, [CTX] * n, slots, stream=stream)
-        assert cudart.cudaStreamEndCapture(s, ctypes.byref(graph)) == 0
-        assert cudart.cudaGraphGetNodes(graph, None, ctypes.byref(nodes)) == 0
-        assert cudart.cudaGraphDestroy(graph) == 0
-        return nodes.value
+    def kernels(n):
+        return _kernels(ctx, kv, n, 2, 16)
 
     assert kernels(3) == 1 and kernels(74) == 1 and kernels(100) == 2
     for geometry in ((148, 256), (0, 128), (37, 64)):
@@ -481,3 +488,19 @@ def test_when_the_next_grid_may_start(n, host, at_once, tmp_path):
     held_until, started = (int(v) for v in marks.cpu())
     assert (started < held_until) == at_once, started - held_until
     assert ctx.sync_status() == 0
+
+
+# Eight tables and nine; 2048 ids a table and more; 3 GB in all and more; without `arriving` too
+@pytest.mark.parametrize("n,n_q,K,gigabytes,one", [(9, 2, 1025, 3, True), (9, 2, 1025, 3.01, False), (9, 2, 1024, 11, True), (8, 2, 1025, 11, True),
+                                                   (18, 2, 2048, 2.9, True), (18, 2, 2048, 3.1, False), (19, 2, 2048, 1, False)])
+def test_early_outputs_of_tables_that_reach_far(n, n_q, K, gigabytes, one):
+    """With stage_one_done, clusters beside a consumer on another stream lose more in translations than the one kernel saves."""
+    import torch
+    import paper_2609_37538_b200 as avsg
+    kv = _kv(avsg)
+    ctx = avsg.Context(n, 8192, RB, K, n_q, 4)
+    word = torch.zeros(1, dtype=torch.int64, device="cuda")
+    rows = [int(gigabytes * 2**30) // (n * RB)] * n
+    assert _kernels(ctx, kv, n, n_q, K, word, True, rows) == (1 if one else 3)
+    assert _kernels(ctx, kv, n, n_q, K, word, False, rows) == (1 if one else 2)
+    assert _kernels(ctx, kv, n, n_q, K, None, True, rows) == 1 and _kernels(ctx, kv, n, n_q, K, kv_rows=rows) == 1
