@@ -204,9 +204,13 @@ typedef struct {
                                       avsg_step on the SAME stream with programmatic stream
                                       serialization (the operator's kernels release their
                                       dependents as soon as they run, and all their blocks
-                                      are resident by then; a call in one kernel leaves it
-                                      the SMs that its own blocks do not take, at least
-                                      half): it polls the word, works on
+                                      are resident by then; a call in one kernel of more
+                                      than three tables leaves half of the SMs free, or,
+                                      where its blocks are smaller than 1024 threads, half
+                                      of what the SMs hold of them, which may be half of
+                                      each; on another stream a consumer shares the free
+                                      half with the next call, if that queues): it polls
+                                      the word, works on
                                       the hits, and executes griddepcontrol.wait before it
                                       touches a missed row.  avsg_step only:
                                       avsg_step_host (whose caller waits for the whole call)

@@ -248,7 +248,8 @@ cudaError_t step_prepare(size_t max_smem);
 // output: whether rows are asked for early.
 bool step_serves(uint32_t S, uint32_t K, uint32_t n_q, uint32_t cluster, uint32_t row_bytes, bool arriving);
 StepClusters step_clusters(size_t max_smem);            // after step_prepare
-// Whether the blocks of a call in one kernel leave half of the SMs to other grids.
+// Whether the blocks of a call in one kernel take no more than half of what the SMs hold of them.  Blocks of 1024 threads then leave half
+// of the SMs to other grids; smaller ones, of which an SM holds several, may stand on all SMs and leave half of each.
 inline bool step_leaves_half(uint32_t n, uint32_t threads, uint32_t cluster, uint32_t sm_count)
 {
     return (uint64_t)n * cluster * threads <= (uint64_t)sm_count / 2u * 1024u;

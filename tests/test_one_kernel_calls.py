@@ -504,3 +504,65 @@ def test_early_outputs_of_tables_that_reach_far(n, n_q, K, gigabytes, one):
     assert _kernels(ctx, kv, n, n_q, K, word, True, rows) == (1 if one else 3)
     assert _kernels(ctx, kv, n, n_q, K, word, False, rows) == (1 if one else 2)
     assert _kernels(ctx, kv, n, n_q, K, None, True, rows) == 1 and _kernels(ctx, kv, n, n_q, K, kv_rows=rows) == 1
+
+
+# Blocks of 1024 threads on half of the SMs; blocks of 512, as many as there are SMs, and of 128, more than that; a kernel for each stage
+@pytest.mark.parametrize("n,S,K,n_q,kernels", [(18, 8192, 512, 3, 1), (37, 1024, 200, 3, 1), (60, 256, 60, 4, 1), (19, 8192, 512, 3, 3)])
+def test_queued_calls_beside_a_consumer(n, S, K, n_q, kernels, tmp_path):
+    """Calls of two contexts queue behind one another; on another stream a consumer whose blocks need more than half of an SM's shared
+    memory starts on each call's resident rows when the call's word says so."""
+    import ctypes
+    import os
+    import subprocess
+    import torch
+    from cuda.bindings import driver as drv
+    import paper_2609_37538_b200 as avsg
+    from paper_2609_37538_b200 import build
+    lib = str(tmp_path / "resident_reader.so")
+    subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")] + build.NVCC_FLAGS +
+                          ["-o", lib, os.path.join(os.path.dirname(os.path.abspath(__file__)), "cuda", "resident_reader.cu")])
+    lib = ctypes.CDLL(lib)
+    vp, u32 = ctypes.c_void_p, ctypes.c_uint32
+    lib.launch_resident_reader.argtypes = [vp, vp, u32, u32, vp, u32, u32, vp, u32, vp]
+    kv, L, context, T = _kv(avsg), 3, min(CTX, 3 * S), 4
+    rng = np.random.default_rng([n, S])
+    calls, side, done = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.Event()
+    new = lambda dtype: torch.empty((T, n, n_q, K), dtype=dtype, device="cuda")
+    layers = []
+    for _ in range(2):
+        ctx = avsg.Context(n, S, RB, K, n_q, L)
+        ids = np.stack([[[rng.choice(context, K, replace=False) for _ in range(n_q)] for _ in range(n)] for _ in range(T)]).astype(np.int32)
+        base = ctx.buffer(0).data_ptr()
+        assert all(ctx.buffer(t).data_ptr() == base + t * S * RB for t in range(n))
+        layers.append((ctx, ctx.prepare(list(range(n)), [kv] * n, n_q, K), ids, torch.from_numpy(ids).cuda(), new(torch.int32), new(torch.uint8),
+                       new(torch.uint8), torch.full((T, n, n_q, K, RB), 0xEE, dtype=torch.uint8, device="cuda"),
+                       torch.zeros(1, dtype=torch.int64, device="cuda"), base))
+    word = layers[0][8]
+    assert _kernels(layers[0][0], kv, n, n_q, K, word, True) == kernels
+    assert lib.launch_resident_reader(layers[0][4].data_ptr(), layers[0][6].data_ptr(), 0, 1, layers[0][9], S, RB, layers[0][7].data_ptr(),
+                                      160 << 10, side.cuda_stream) == 0                        # (loads the kernel)
+    torch.cuda.synchronize()
+    for c in range(T):
+        calls.wait_event(done)
+        for ctx, call, ids, X, slots, hit, arriving, out, word, base in layers:
+            call.run(X[c], [context] * n, slots[c], hit[c], stream=calls, stage_one_done=(word, c + 1), arriving=arriving[c])
+        for ctx, call, ids, X, slots, hit, arriving, out, word, base in layers:
+            err, = drv.cuStreamWaitValue64(side.cuda_stream, word.data_ptr(), c + 1, drv.CUstreamWaitValue_flags.CU_STREAM_WAIT_VALUE_EQ)
+            assert err == drv.CUresult.CUDA_SUCCESS
+            assert lib.launch_resident_reader(slots[c].data_ptr(), arriving[c].data_ptr(), n * n_q * K, n_q * K, base, S, RB, out[c].data_ptr(),
+                                              160 << 10, side.cuda_stream) == 0
+        done.record(side)
+    torch.cuda.synchronize()
+    host, resident = kv.numpy().reshape(CTX, RB), 0
+    for ctx, call, ids, X, slots, hit, arriving, out, word, base in layers:
+        orc = [OracleTable(S, RB, L) for _ in range(n)]
+        for c in range(T):
+            for t in range(n):
+                r = orc[t].step(ids[c, t], context, kv.numpy(), RB)
+                assert (slots[c, t].cpu().numpy() == r.O).all() and (arriving[c, t].cpu().numpy() == r.arriving).all(), (c, t)
+                there = (r.O >= 0) & (r.arriving == 0)
+                want = np.where(there[..., None], host[ids[c, t]], 0xEE)
+                assert (out[c, t].cpu().numpy() == want).all(), (c, t)
+                resident += int(there.sum())
+        assert ctx.sync_status() == 0
+    assert resident > 0
