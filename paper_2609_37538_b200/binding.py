@@ -1,5 +1,6 @@
 """Thin binding of libavsg.so: argument marshalling only, by ctypes and, for
-the calls of every step, by an extension module (csrc/python_calls.cpp).
+the calls of every step, by an extension module (csrc/python_calls.cpp) where
+that has been built for this Python.
 
 Every step of the operator runs in the CUDA kernels behind the C ABI
 (include/avsg.h).  PyTorch supplies device tensors, pinned host tensors and
@@ -84,14 +85,16 @@ _lib = _calls = None
 
 
 def _python_calls():
-    """The extension module (built in-tree by build.build_library); raises if it is missing."""
+    """The extension module (built in-tree by build.build_library), or False: another Python than it was built for, or a
+    machine that could not build it.  The same calls are then marshalled by ctypes, 2 to 6 us slower."""
     global _calls
     if _calls is None:
         try:
             from . import _python_calls as module
-        except ImportError as e:
-            raise RuntimeError("the extension module _python_calls is missing: run `python __graft_entry__.py` to build it") from e
-        module.set_binding(_addr, _c_array, _set_lengths, _stream_handle, None, None)
+        except ImportError:
+            module = False
+        else:
+            module.set_binding(_addr, _c_array, _set_lengths, _stream_handle, None, None)
         _calls = module
     return _calls
 
@@ -206,7 +209,8 @@ def _current_stream() -> int:
         raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
         if raw is not None and dev is not None:
             _current_stream_fn = lambda: raw(dev())
-            _python_calls().set_binding(_addr, _c_array, _set_lengths, _stream_handle, raw, dev)     # (the extension asks them itself from now on)
+            if _python_calls():
+                _calls.set_binding(_addr, _c_array, _set_lengths, _stream_handle, raw, dev)     # (the extension asks them itself from now on)
         else:
             _current_stream_fn = lambda: torch.cuda.current_stream().cuda_stream
     return _current_stream_fn()
@@ -277,11 +281,12 @@ class PreparedCall:
         a.kv_rows = ctypes.addressof(self._rows) if self._rows is not None else None
         self.args = a
         self._ref = ctypes.byref(a)
-        cell = getattr(ctx, "_cell", None)               # (a stand-in for a context has none: its library is called from here)
-        self._direct = cell is not None
-        step, step_host = (getattr(ctx, "_addresses", None) or _addresses(ctx._lib)) if self._direct else (0, 0)
-        self._native = (_calls or _python_calls()).Call(ctypes.addressof(a), ctypes.addressof(self._vlen), n,
-                                                        ctypes.addressof(cell) if self._direct else 0, step, step_host, self._vlen)
+        self._cell, self._native = getattr(ctx, "_cell", None), None
+        module = _calls if _calls is not None else _python_calls()
+        if module and self._cell is not None:            # (a stand-in for a context has no cell: its library is called from here)
+            step, step_host = getattr(ctx, "_addresses", None) or _addresses(ctx._lib)
+            self._native = module.Call(ctypes.addressof(a), ctypes.addressof(self._vlen), n, ctypes.addressof(self._cell), step, step_host,
+                                       self._vlen)
 
     def run(self, indices, verified_len: Sequence[int], slots, hit=None, miss_count=None, stream=None,
             host: bool = False, stage_one_done=None, arriving=None) -> None:
@@ -291,14 +296,28 @@ class PreparedCall:
         stage_one_done: None or (device int64 tensor or address, value): the word receives the value once the
         slot table, hit mask and miss counts of the whole call are final, while the missed rows still travel.
         arriving: None or a uint8 device tensor like hit: 1 where the row comes with this call's Stage Two."""
-        if self._direct:
+        if self._native is not None:
             rc = self._native.run(indices, verified_len, slots, hit, miss_count, stream, stage_one_done, arriving, host)
         else:
-            at = self._native.fill(indices, verified_len, slots, hit, miss_count, stream, stage_one_done, arriving)
-            lib = self.ctx._lib
-            rc = (lib.avsg_step_host if host else lib.avsg_step)(self.ctx._h, self._ref, at or None)
+            rc = self._run(indices, verified_len, slots, hit, miss_count, stream, host, stage_one_done, arriving)
         if rc != OK:
             _check(rc, "avsg_step")
+
+    def _run(self, indices, verified_len, slots, hit, miss_count, stream, host, stage_one_done, arriving) -> int:
+        a = self.args
+        a.arriving = _addr(arriving) if arriving is not None else None
+        a.stage_one_done, a.stage_one_done_value = (None, 0) if stage_one_done is None else (_addr(stage_one_done[0]), int(stage_one_done[1]))
+        a.verified_len_dev = None
+        if hasattr(verified_len, "data_ptr"):
+            a.verified_len_dev = _addr(verified_len)
+        else:
+            _set_lengths(self._vlen, verified_len)
+        a.indices, a.slots = _addr(indices), _addr(slots)
+        a.hit = _addr(hit) if hit is not None else None
+        a.miss_count = _addr(miss_count) if miss_count is not None else None
+        handle = self.ctx._h if self._cell is None else self._cell.value or None
+        lib = self.ctx._lib
+        return (lib.avsg_step_host if host else lib.avsg_step)(handle, self._ref, _stream_handle(stream))
 
 
 class Context:
@@ -473,6 +492,7 @@ def _c_array(kind: str, values, n: int):
 
 
 _noalloc_fn = None
+_NOALLOC = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p)
 
 
 def step_noalloc(tok, life, buffer, indices, kv, verified_len, *, max_lifetime: int = 16, slots, hit=None,
@@ -489,7 +509,26 @@ def step_noalloc(tok, life, buffer, indices, kv, verified_len, *, max_lifetime: 
     global _noalloc_fn
     if _noalloc_fn is None:
         _noalloc_fn = _address_of(load_library().avsg_step_noalloc)
-    rc = _python_calls().noalloc(_noalloc_fn, tok, life, buffer, indices, kv, verified_len, max_lifetime, slots, hit, miss_count,
-                                 status, row_stride, stream, kv_rows)
+    module = _python_calls()
+    if module:
+        rc = module.noalloc(_noalloc_fn, tok, life, buffer, indices, kv, verified_len, max_lifetime, slots, hit, miss_count, status,
+                            row_stride, stream, kv_rows)
+    else:
+        n, S = tok.shape
+        _, n_q, K = indices.shape
+        kv_owner, kv_at = _c_array("Q", [_addr(k) for k in kv], n)
+        length_owner, lengths_at = _c_array("i", verified_len, n)
+        stride_owner, strides_at = _c_array("Q", row_stride, n)
+        rows_owner, rows_at = _c_array("I", kv_rows, n)
+        a = AvsgNoAllocArgs()
+        a.n, a.n_tokens, a.topk, a.buffer_slots = n, n_q, K, S
+        a.row_bytes, a.max_lifetime = buffer.shape[-1], max_lifetime
+        a.tok, a.life, a.buffer, a.indices = _addr(tok), _addr(life), _addr(buffer), _addr(indices)
+        a.kv_base, a.row_stride, a.verified_len, a.kv_rows = kv_at, strides_at, lengths_at, rows_at
+        a.slots = _addr(slots)
+        a.hit = _addr(hit) if hit is not None else None
+        a.miss_count = _addr(miss_count) if miss_count is not None else None
+        a.status = _addr(status) if status is not None else None
+        rc = _NOALLOC(_noalloc_fn)(ctypes.addressof(a), _stream_handle(stream))
     if rc != OK:
         _check(rc, "avsg_step_noalloc")

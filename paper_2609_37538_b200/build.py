@@ -3,6 +3,7 @@ import glob
 import os
 import subprocess
 import sysconfig
+import warnings
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
@@ -41,8 +42,17 @@ def build_calls(force: bool = False):
 
 
 def build_library(force: bool = False, verbose: bool = False):
-    """Returns the path of libavsg.so, rebuilding it (and the extension module) when a source is newer."""
-    build_calls(force)
+    """Returns the path of libavsg.so, rebuilding it (and the extension module) when a source is newer.  The library needs no
+    Python; where the module cannot be built (no C++ compiler, no Python.h) the binding goes without it."""
+    lib = _build_library(force, verbose)
+    try:
+        build_calls(force)
+    except (OSError, subprocess.CalledProcessError) as e:
+        warnings.warn("the binding's extension module was not built (%s): calls are marshalled by ctypes" % e)
+    return lib
+
+
+def _build_library(force: bool, verbose: bool):
     srcs = sources()
     if not srcs:
         return None

@@ -96,7 +96,7 @@ struct Call {
     PyObject_HEAD
     avsg_step_args* args;
     int32_t* lengths;                    // [n]
-    const uint64_t* ctx;                 // holds the context's handle, 0 when that is closed; null: fill() only
+    const uint64_t* ctx;                 // holds the context's handle, 0 when that is closed
     StepFn step, step_host;
     Py_ssize_t n;
     PyObject* array;                     // the same, for the binding (which takes any iterable of n numbers)
@@ -173,20 +173,12 @@ bool fill(Call* c, PyObject* const* a, uint64_t* stream)
     return stream_handle(a[5], stream);
 }
 
-PyObject* call_fill(PyObject* self, PyObject* const* a, Py_ssize_t nargs)
-{
-    uint64_t stream = 0;
-    if (nargs != 8) { PyErr_SetString(PyExc_TypeError, "eight arguments"); return nullptr; }
-    if (!fill(reinterpret_cast<Call*>(self), a, &stream)) return nullptr;
-    return PyLong_FromUnsignedLongLong(stream);
-}
-
-// The same arguments, then host.
+// The same arguments as fill(), then host.
 PyObject* call_run(PyObject* self, PyObject* const* a, Py_ssize_t nargs)
 {
     Call* c = reinterpret_cast<Call*>(self);
     uint64_t stream = 0;
-    if (nargs != 9 || !c->ctx) { PyErr_SetString(PyExc_TypeError, "nine arguments, of a call that has a context"); return nullptr; }
+    if (nargs != 9 || !c->ctx) { PyErr_SetString(PyExc_TypeError, "nine arguments, of a call that has been set up"); return nullptr; }
     const int host = PyObject_IsTrue(a[8]);
     if (host < 0 || !fill(c, a, &stream)) return nullptr;
     avsg_ctx* ctx = reinterpret_cast<avsg_ctx*>(*c->ctx);
@@ -199,7 +191,6 @@ PyObject* call_run(PyObject* self, PyObject* const* a, Py_ssize_t nargs)
 }
 
 PyMethodDef call_methods[] = {
-    {"fill", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(call_fill)), METH_FASTCALL, nullptr},
     {"run", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(call_run)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 PyType_Slot call_slots[] = {{Py_tp_init, reinterpret_cast<void*>(call_init)},

@@ -191,3 +191,23 @@ def test_native_calls_take_what_the_binding_takes():
             avsg.step_noalloc(tok, life, rows, ids, kv + [0], lens, **some)
     finally:
         b._noalloc_fn = before
+
+
+def test_calls_without_the_extension_module(monkeypatch):
+    """Another Python than the module was built for: the same calls by ctypes, which take and refuse the same."""
+    from paper_2609_37538_b200 import binding as b
+    monkeypatch.setattr(b, "_calls", False)
+    monkeypatch.setattr(b, "_current_stream_fn", None)
+    test_native_calls_take_what_the_binding_takes()
+    test_lengths_are_taken_from_any_iterable()
+
+
+def test_the_library_builds_without_the_extension_module(monkeypatch, tmp_path):
+    """No C++ compiler for the module, or no Python.h: the library is there all the same."""
+    import pytest
+    from paper_2609_37538_b200 import build
+    monkeypatch.setattr(build, "CALLS", str(tmp_path / "_python_calls.so"))
+    for compiler in ("/nonexistent/g++", "false"):
+        monkeypatch.setenv("CXX", compiler)
+        with pytest.warns(UserWarning, match="extension module"):
+            assert build.build_library() == build.LIB and os.path.exists(build.LIB)
