@@ -177,20 +177,23 @@ build.LIB = %(lib)r
 import paper_2609_37538_b200 as avsg
 from oracle import OracleTable
 from test_one_kernel_calls import RB, _kv
-S, K, n_q, L = 8192, 600, 3, 3
+K, n_q, L = 600, 3, 3
 kv = _kv(avsg)
 rng = np.random.default_rng(8)
-for n in (1, 20, 40, 74, 80):                            # clusters of eight, four, three, two blocks; two kernels
+# clusters of eight, four, three, two blocks; two kernels; 16 slots a thread; with the `arriving` output
+for n, S, early in ((1, 8192, False), (20, 8192, False), (40, 8192, False), (74, 8192, False), (80, 8192, False), (2, 16384, False), (20, 16384, False),
+                    (2, 8192, True), (20, 8192, True), (3, 16384, True)):
     ctx = avsg.Context(n, S, RB, K, n_q, L)
     orc = [OracleTable(S, RB, L) for _ in range(n)]
-    for host in (False, True, False):
+    for host in (False, not early, False):
         X = np.stack([[rng.choice(900, K, replace=False) for _ in range(n_q)] for _ in range(n)]).astype(np.int32)
         ids = torch.from_numpy(X).pin_memory() if host else torch.from_numpy(X).cuda()
-        out = (ctx.step_host if host else ctx.step)(list(range(n)), ids, [kv] * n, [890] * n)
+        out = (ctx.step_host if host else ctx.step)(list(range(n)), ids, [kv] * n, [890] * n, **(dict(want_arriving=True) if early else {}))
         assert ctx.sync_status() == (avsg.STATUS_WAIT_TIMEOUT if n <= 74 else 0), n
         for i in range(n):
             r = orc[i].step(X[i], 890, kv.numpy(), RB)
             assert (out.slots[i].cpu().numpy() == r.O).all() and (out.hit[i].cpu().numpy() == r.M).all(), (n, i)
+            assert not early or (out.arriving[i].cpu().numpy() == r.arriving).all(), (n, i)
     ctx.clear_status()
     for i in range(n):
         assert (ctx.export_state(i)[0] == orc[i].export_state()[0]).all(), (n, i)
@@ -362,20 +365,23 @@ def test_the_default_geometry_brings_the_one_kernel_back():
         assert kernels(3) == 1 and kernels(74) == 1
 
 
-# Tables of 16384 slots: two, four and eight ids a thread; the fewest chains that fit (three tokens of 4096); the smallest K; many
-# tokens; the largest clusters of four, three and two blocks and one table more; four tokens of 4096, 8193 ids and one token with
-# three blocks take two kernels
-@pytest.mark.parametrize("n,K,n_q", [(1, 8192, 1), (2, 4097, 2), (8, 2048, 4), (9, 1, 8), (2, 33, 64), (3, 4096, 3), (33, 700, 1), (34, 700, 1),
-                                     (45, 600, 2), (46, 600, 2), (46, 600, 3), (74, 300, 4), (2, 4096, 4), (1, 8193, 1)])
-def test_tables_of_16384_slots(n, K, n_q):
+# Tables of 16384 slots: two, four and eight ids a thread; the most ids that fit, with few and with many tokens (few chains, the largest
+# node numbers), and more; the smallest K; the most tokens; rows too long to be asked for early; the largest clusters of four, three and two
+# blocks and one table more
+@pytest.mark.parametrize("n,K,n_q,rb,kernels", [(1, 8192, 1, RB, 1), (2, 4097, 2, RB, 1), (8, 2048, 4, RB, 1), (9, 1, 8, RB, 1), (2, 33, 64, RB, 1),
+                                                (3, 4096, 3, RB, 1), (2, 4096, 4, RB, 2), (2, 256, 51, RB, 1), (2, 256, 52, RB, 2), (1, 8193, 1, RB, 2),
+                                                (9, 700, 2, 1552, 1), (33, 2100, 1, 1552, 1), (33, 700, 1, RB, 1), (34, 700, 1, RB, 2),
+                                                (45, 600, 2, RB, 1), (46, 600, 2, RB, 2), (46, 600, 3, RB, 1), (74, 300, 4, RB, 1)])
+def test_tables_of_16384_slots(n, K, n_q, rb, kernels):
     import torch
     import paper_2609_37538_b200 as avsg
     S, L, context = 16384, 3, 30000
     rng = np.random.default_rng([n, K, n_q])
-    kv = avsg.pinned_empty(context * RB)
-    tr.fill_kv(kv.data_ptr(), 1, 0, context, RB)
-    ctx = avsg.Context(n, S, RB, K, n_q, L)
-    orc = [OracleTable(S, RB, L) for _ in range(n)]
+    kv = avsg.pinned_empty(context * rb)
+    tr.fill_kv(kv.data_ptr(), 1, 0, context, rb)
+    ctx = avsg.Context(n, S, rb, K, n_q, L)
+    assert _kernels(ctx, kv, n, n_q, K) == kernels
+    orc = [OracleTable(S, rb, L) for _ in range(n)]
     word = torch.zeros(1, dtype=torch.int64, device="cuda")
     done = []
     for c in range(7):
@@ -399,7 +405,7 @@ def test_tables_of_16384_slots(n, K, n_q):
         for a, t in enumerate(tabs):
             if c == 5 and a < 2:
                 orc[t].reset()
-            r = orc[t].step(X[a], N, kv.numpy(), RB)
+            r = orc[t].step(X[a], N, kv.numpy(), rb)
             assert (out.slots[a].cpu().numpy() == r.O).all() and (out.hit[a].cpu().numpy() == r.M).all(), (c, t)
             assert (out.miss_count[a].cpu().numpy() == r.n).all(), (c, t)
             assert c not in (3, 5) or (out.arriving[a].cpu().numpy() == r.arriving).all(), (c, t)
@@ -412,10 +418,12 @@ def test_tables_of_16384_slots(n, K, n_q):
 
 # One to eight ids and two to sixteen slots a thread; the most tables of 8192 and 1024 slots whose blocks leave half of 148 SMs free, and
 # one more; rows too long to be asked for early (three kernels)
-@pytest.mark.parametrize("n,S,K,n_q,rb", [(1, 256, 64, 4, 48), (2, 1024, 300, 3, 48), (4, 4096, 2000, 2, 48), (4, 4096, 500, 5, 48), (18, 8192, 512, 3, 48),
-                                          (19, 8192, 512, 3, 48), (37, 1024, 200, 3, 48), (38, 1024, 200, 3, 48), (3, 8192, 4000, 2, 48), (5, 8192, 4097, 1, 48),
-                                          (2, 16384, 4000, 3, 48), (4, 16384, 2000, 5, 48), (6, 16384, 8000, 1, 48), (2, 8192, 600, 3, 1552)])
-def test_early_outputs(n, S, K, n_q, rb):
+@pytest.mark.parametrize("n,S,K,n_q,rb,kernels", [(1, 256, 64, 4, 48, 1), (2, 1024, 300, 3, 48, 1), (4, 4096, 2000, 2, 48, 1), (4, 4096, 500, 5, 48, 1),
+                                                  (18, 8192, 512, 3, 48, 1), (19, 8192, 512, 3, 48, 3), (37, 1024, 200, 3, 48, 1),
+                                                  (38, 1024, 200, 3, 48, 3), (3, 8192, 4000, 2, 48, 1), (5, 8192, 4097, 1, 48, 1),
+                                                  (2, 16384, 4000, 3, 48, 1), (4, 16384, 2000, 5, 48, 1), (6, 16384, 8000, 1, 48, 1),
+                                                  (2, 8192, 600, 3, 1552, 3)])
+def test_early_outputs(n, S, K, n_q, rb, kernels):
     """Ids from so few that many hits are on slots that the call has just reserved, and tables too small for all of them."""
     import torch
     import paper_2609_37538_b200 as avsg
@@ -426,6 +434,7 @@ def test_early_outputs(n, S, K, n_q, rb):
     ctx = avsg.Context(n, S, rb, K, n_q, L)
     orc = [OracleTable(S, rb, L) for _ in range(n)]
     word = torch.zeros(1, dtype=torch.int64, device="cuda")
+    assert _kernels(ctx, kv, n, n_q, K, word, True) == kernels
     done = []
     for c in range(6):
         X = np.empty((n, n_q, K), np.int32)

@@ -65,12 +65,15 @@ def _steps(S, K, n_q, cluster, L):
     assert ctx.sync_status() == 0
 
 
-def test_ids_of_one_chain():
-    """Every id hashes to the same bucket: one chain holds the whole table and the ids that come in."""
+@pytest.mark.parametrize("S", [128, 16384])
+def test_ids_of_one_chain(S):
+    """Every id hashes to the same bucket: one chain holds all of them, the table's and those that come in.  (The packed index of 16384
+    slots has up to 2 S chains; ids of the first one of so many are of the first one with fewer too.)"""
     import torch
     import paper_2609_37538_b200 as avsg
-    S, K, n_q, L = 128, 32, 4, 4
-    ids = _same_bucket_ids(S, 256, 77)
+    K, n_q, L = 32, 4, 4
+    ids = _same_bucket_ids(S, 256, 77 if S == 128 else 0)
+    assert len(ids) >= 100
     rows = int(ids.max()) + 1
     kv = avsg.pinned_empty(rows * 16)
     kv.numpy()[:] = np.random.default_rng(5).integers(0, 256, rows * 16, dtype=np.uint8)
