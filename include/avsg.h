@@ -87,11 +87,12 @@ extern "C" {
                                        with arriving up to 33, and rows of up to 1536 bytes).
                                        Its blocks take whole SMs while they run: who wants
                                        room for other kernels beside the call sets a
-                                       transfer geometry (100 calls of 8, 32, 64 tables
-                                       beside 100 GEMMs of 9.8 ms on another stream: both
-                                       through after 10.8, 17.1, 25.1 ms, with a geometry
-                                       9.6, 14.0, 25.5; alone the calls take 3.8, 12.5, 24.5
-                                       and 4.4, 12.8, 24.6).  Calls whose Stage One takes
+                                       transfer geometry (100 calls of 8, 18, 32, 64 tables
+                                       beside 100 GEMMs of 9.5 ms on another stream: both
+                                       through after 12.4, 13.5, 17.0, 22.8 ms, with a
+                                       geometry 9.9, 11.5, 12.4, 23.0; alone the calls take
+                                       3.4, 6.6, 11.1, 22.1 and 4.1, 7.4, 11.8, 22.2).
+                                       Calls whose Stage One takes
                                        more than half of the SMs are served as in
                                        AVSG_XFER_SM_OVERLAP                              */
 #define AVSG_XFER_COPY_ENGINE   1u  /* comparator: miss list read back, one async copy

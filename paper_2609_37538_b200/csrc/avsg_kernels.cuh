@@ -279,6 +279,8 @@ inline bool step_reaches_far(uint32_t n, uint32_t table_ids, uint64_t reach)
 // 12, 18 tables of K = 1000 27.0 / 27.6, 37.4 / 38.0 (0.1 and 0.2 GB), 31.4 / 32.0, 44.2 / 44.9 (0.5, 0.8 GB), 33.3 / 33.8, 49.8 / 47.6 (2.1, 3.1 GB); of
 // K = 2048 37.6 / 38.1, 54.0 / 54.5, 60.0 / 60.4 and 52.9 / 53.4, 77.6 / 77.9, 89.9 / 87.4; 28 of S = 1024 13.9 / 14.1, 14.3 / 14.5, 15.2 / 15.2; but 12
 // in clusters of eight of small blocks 9.5 / 9.3 (S = 1024), 20.1 / 20.1 (2048), 18.9 / 18.9 (4096; 1.8 GB 20.0 / 19.8).
+// (Beside 100 GEMMs on another stream 100 calls of 9, 12, 16, 18 tables are through after 12.1, 12.8, 13.1, 13.5 ms so and 11.6, 12.4, 13.0, 14.0 late;
+// beside 20 after 4.6, 5.2, 6.2, 6.8 and 5.4, 6.4, 7.4, 7.7.)
 // Where the blocks leave no room nothing is gained (32 tables 113.0 / 112.9), and ids in host memory that are fetched under a call's rows slow these
 // down (39 tables, K = 3430: 215 / 124).
 template <int CAP>
@@ -319,7 +321,8 @@ cudaError_t launch_transfer_overlap(const XferOverlapParamsBig& p, uint32_t bloc
 cudaError_t launch_transfer_positions(const PosParams& p, uint32_t blocks, uint32_t threads, cudaStream_t stream);
 
 // Optional output of a call (latency hiding, Sec. 6 with Sec. 3.6): which positions' rows come with THIS call's
-// Stage Two.  A kernel of its own between Stage One and Stage Two, so that the Stage One kernels carry no code for
+// Stage Two.  Calls in one kernel write it there (an instance of that kernel, see place_tokens()).  For the others it is a
+// kernel of its own between Stage One and Stage Two, so that the Stage One kernels carry no code for
 // an output few calls ask for (inside them it cost every call 1.7 us).  It also makes the call's "Stage One is
 // done" announcement when the caller asked for both.
 struct ArrivingParams {

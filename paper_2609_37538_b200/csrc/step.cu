@@ -56,7 +56,10 @@ struct StepLayout {
 // kernel for each stage) Stage One pays a barrier of the cluster a token instead, and Stage Two a launch and the hand-over through
 // memory: 16384 slots, in two kernels / in one, us per call: two tokens of K = 2048, 1, 4, 8, 16, 24 tables 21.4 / 12.7, 32.3 / 20.9, 44.7 /
 // 33.6, 72.9 / 62.9, 98.9 / 88.4; four tokens 33.1 / 18.9, 49.8 / 31.0, 72.1 / 53.3, 115.7 / 98.5, 160.5 / 143.3; three of K = 3000, one
-// table 33.4 / 20.4; from and to host memory, four tokens, 1, 16 tables 52.5 / 23.9, 142 / 108 (ids and outputs went by copies).
+// table 33.4 / 20.4; from and to host memory, four tokens, 1, 16 tables 52.5 / 23.9, 142 / 108 (ids and outputs went by copies).  With ids from
+// the host the first block keeps these too, where rows are asked for early, and the chains are fewer (K = 2048, four tokens 3632, not 11 824,
+// for 22 528 nodes); three tokens of 4096 and five of 2000 are not asked for early then.  Those calls, 1, 8, 33 tables: 47.3, 85.8, 228 / 22.7, 58.9,
+// 209; 50.0, 99.8, 297 / 29.3, 64.8, 272; 51.2, 97.0, 269 / 26.4, 69.9, 247.
 constexpr uint32_t WIDE_SLOTS = 8192;
 // ask: rows are asked for early.  False if there is no room (without asking early there always is, up to WIDE_SLOTS).
 bool step_layout(StepLayout& o, uint32_t S, uint32_t K, uint32_t n_q, uint32_t nt, uint32_t copying, bool host_ids, bool ask)
@@ -1019,7 +1022,8 @@ cudaError_t step_prepare(size_t max_smem)
 // Above WIDE_SLOTS: where the index has room (n_q and K decide), and not calls of few tokens with three and two blocks a table, whose
 // rows two kernels cut evenly over all SMs: K = 2048, two kernels / one, us: 36, 50, 74 tables, one token 83.9 / 83.0, 109.8 / 112.0, 154.9 /
 // 156.7; K = 1024, two tokens, 40, 64 tables 99.9 / 94.9, 149.0 / 147.3, but 64 cold ones 1103 / 1114; K = 2048, three tokens, 40, 50,
-// 74 tables 200 / 190, 243 / 238, 350 / 345, 60 cold ones 810 / 810; four tokens, 40, 64 tables 248 / 234, 381 / 371.
+// 74 tables 200 / 190, 243 / 238, 350 / 345, 60 cold ones 810 / 810; four tokens, 40, 64 tables 248 / 234, 381 / 371.  (All with device ids.
+// With host buffers two kernels also pay for copies and events; where the line would lie for these has not been measured.)
 bool step_serves(uint32_t S, uint32_t K, uint32_t n_q, uint32_t cluster, uint32_t row_bytes, bool arriving)
 {
     StepLayout lay;
